@@ -189,13 +189,28 @@ qw_status qw_get_plan(const qw_walk *w, int *depth_k, int *tile);
  * the larger tile when the cycle holds two of its chunks.  Variant 1 needs the
  * periodic cycle, N at least one chunk (any N: the last chunk wraps round), a
  * global coin, FP32 / BF16 / FP64 and k < chunk / 2, else QW_EINVAL.
- * qw_set_plan selects variant 0. */
+ * qw_set_plan selects variant 0.
+ *
+ * Variant 2 with a tile of 256 or 512 (512: FP32 / BF16): momentum-space steps.
+ * With one coin for all sites, k steps are a convolution; blocks of 32 x tile
+ * sites are transformed, multiplied by the k-step matrix of each momentum and
+ * transformed back, at a cost that does not depend on k < 16 x tile.  Needs the
+ * periodic cycle (any N, any precision) and one unitary coin (to 1e-6), else
+ * QW_EINVAL.  The result is as accurate as stepping in norm, block by block
+ * (about 2e-7 of the block's norm in float, 4e-16 in double), so an amplitude
+ * that is zero or tiny beside its neighbours is not resolved beyond that; a
+ * clipped state (qw_set_clipping) is therefore still stepped, until its box
+ * covers the cycle.  Allocates the matrices' table (at most 0.4 MB). */
 qw_status qw_set_plan_ex(qw_walk *w, int depth_k, int tile, int variant);
 qw_status qw_get_plan_ex(const qw_walk *w, int *depth_k, int *tile, int *variant);
 
 /* Time the candidate plans on this walk (CUDA events on the walk's stream,
  * reading the current state, writing only the scratch buffer, so the state is
- * unchanged) and keep the fastest.  Results are cached per (lattice shape,
+ * unchanged) and keep the fastest.  On the cycle it also times momentum-space
+ * steps (variant 2 of qw_set_plan_ex) and, where they are faster, uses them
+ * for calls of at least 128 steps (more where a launch takes longer than that
+ * many steps) on states that are not clipped; qw_describe reports them as
+ * "spectral".  Results are cached per (lattice shape,
  * precision, coin kind) in memory and, if the environment variable
  * QW_TUNE_CACHE names a file, in that JSON file.  report (may be NULL)
  * receives a one-line JSON summary, truncated to report_len bytes. */

@@ -431,6 +431,98 @@ static qw_status clear_next(qw_walk *w) {
     return QW_OK;
 }
 
+// ---------------------------------------------------------------- momentum-space steps
+// May this walk's steps be taken in momentum space?  One unitary coin for all
+// sites of a periodic cycle.  (A coin that is not unitary can make U^K large in
+// one component and small in another, which a transform would round together.)
+static bool spectral_walk(const qw_walk *w) {
+    if (w->ndim != 1 || w->bc != QW_BC_PERIODIC || links_on(w)) return false;
+    if (w->kind == CK_PERSITE || w->kind == CK_PHASE) return false;
+    const double *h = w->coin_host;   // row-major complex 2 x 2
+    for (int i = 0; i < 2; ++i)
+        for (int j = i; j < 2; ++j) {   // (C^dagger C)_ij
+            double re = 0, im = 0;
+            for (int r = 0; r < 2; ++r) {
+                const double ar = h[2 * (2 * r + i)], ai = h[2 * (2 * r + i) + 1];
+                const double br = h[2 * (2 * r + j)], bi = h[2 * (2 * r + j) + 1];
+                re += ar * br + ai * bi;
+                im += ar * bi - ai * br;
+            }
+            if (!(std::fabs(re - (i == j)) <= 1e-6 && std::fabs(im) <= 1e-6)) return false;
+        }
+    return true;
+}
+
+// The tables of a tile: allocated when a plan is set, never during a step.
+static cudaError_t spectral_prepare(qw_walk *w, int tile) {
+    cudaError_t e = cudaSuccess;
+    if (!w->spec_table && (e = dev_alloc(&w->spec_table, spectral1d_table_bytes(w->prec))) != cudaSuccess) return e;
+    if (w->spec_tw != tile) {
+        w->spec_tw = tile;
+        std::memset(&w->spec_key, 0, sizeof w->spec_key);
+        e = launch_spectral1d_twiddles(w->prec, tile, w->spec_table, w->stream);
+    }
+    return e;
+}
+
+// One launch of a.K steps from a.in to a.out; `gain` scales the output.
+static cudaError_t spectral_launch(qw_walk *w, Spec1DArgs &a, double gain) {
+    // the coin that stepping applies: the float forms round it and divide its
+    // norm back out (coin_alpha), except that the Hadamard class keeps lambda
+    // in double; the others take it as given
+    double coin[8], scale = gain;
+    std::memcpy(coin, w->coin_host, sizeof coin);
+    if (rounds_to_float(w) && w->kind != CK_SIGN_P && w->kind != CK_SIGN_M) {
+        for (double &c : coin) c = (double)(float)c;
+        scale *= std::pow(w->coin_alpha, -(double)a.K);
+    }
+    qw_walk::SpecKey key;
+    std::memset(&key, 0, sizeof key);   // padding included: keys are compared as bytes
+    std::memcpy(key.coin, coin, sizeof key.coin);
+    key.scale = scale; key.K = a.K; key.tile = a.tile; key.adjoint = a.adjoint;
+    a.table = w->spec_table;
+    if (capturing(w)) w->spec_captured = true;
+    if (w->spec_captured || std::memcmp(&key, &w->spec_key, sizeof key) != 0) {
+        cudaError_t e = launch_spectral1d_matrices(w->prec, a, coin, scale, w->stream);
+        if (e != cudaSuccess) return e;
+        std::memcpy(&w->spec_key, &key, sizeof key);
+    }
+    return launch_spectral1d(w->prec, a, w->stream);
+}
+
+// T steps in as few launches as serve best: with K = ceil(T / m) steps each, m
+// launches of ceil(n / (S - 2K)) blocks; a launch takes whole waves of CTAs
+// (two per block; one CTA per SM, or two of the small float blocks) and about
+// a quarter of a wave's time to start and drain.
+static qw_status run_spectral(qw_walk *w, int64_t T, int adj) {
+    static int sms = 0;
+    if (!sms && (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, w->device) != cudaSuccess || sms <= 0)) sms = 152;
+    const int64_t slots = (int64_t)sms * (w->spec_tile == 256 && rounds_to_float(w) ? 2 : 1);
+    const int64_t m0 = (T + w->spec_k - 1) / w->spec_k;
+    int64_t best_m = m0;
+    double best = 0;
+    for (int64_t m = m0; m < m0 + 4 && m <= T; ++m) {
+        const int64_t W = 32LL * w->spec_tile - 2 * ((T + m - 1) / m);
+        const int64_t ctas = 2 * ((w->nx + W - 1) / W);
+        const double cost = (double)m * ((double)((ctas + slots - 1) / slots) + 0.25);
+        if (m == m0 || cost < best) { best = cost; best_m = m; }
+    }
+    Spec1DArgs a{};
+    a.n = w->nx; a.tile = w->spec_tile; a.shift = w->shift; a.adjoint = adj;
+    for (int64_t rem = T, m = best_m; m > 0; --m) {
+        a.K = (int)((rem + m - 1) / m);
+        a.in = cur_view(w); a.out = next_view(w);
+        // factors of earlier launches that have not reached the state yet (norm
+        // drift, rounded gains) go into this launch's matrices
+        cudaError_t e = spectral_launch(w, a, w->drift_pending / w->gain_fb);
+        if (e != cudaSuccess) return cuda_error(w, e, "momentum-space step launch");
+        w->drift_pending = w->gain_fb = 1.0;
+        w->cur ^= 1;
+        rem -= a.K;
+    }
+    return QW_OK;
+}
+
 qw_status run_steps(qw_walk *w, int64_t T, int adj) {
     if (T < 0) return set_error(w, QW_EINVAL, "T must be >= 0");
     if (T == 0) return QW_OK;
@@ -506,9 +598,11 @@ qw_status run_steps(qw_walk *w, int64_t T, int adj) {
         if (variant != 1) K = std::min(K, 8 * teff);
         Step1DArgs a{};
         a.n = w->nx; a.shift = w->shift; a.kind = w->kind; a.coins = w->coins_dev;
+        const bool spectral = w->spec_tile && spectral_walk(w);
         for (int64_t rem = T; rem > 0;) {
             a.K = (int)std::min<int64_t>(K, rem);
             const bool clip = w->sup_mode == 2;
+            if (spectral && !clip && rem >= w->spec_min) return run_spectral(w, rem, adj);
             // the last, shorter launch of a sweep plan falls back to the tile kernel
             // if needed; a clipped launch always runs the tiles
             a.variant = (!clip && variant == 1 && sweep_ok(w, a.K, tile)) ? 1 : 0;
@@ -607,6 +701,7 @@ qw_status qw_destroy(qw_walk *w) {
     cudaFree(w->p_dev);
     cudaFree(w->staging);
     cudaFree(w->grad_scratch);
+    cudaFree(w->spec_table);
     cudaFree(w->buf3);
     cudaFree(w->pipe_p[0]);
     cudaFree(w->pipe_p[1]);
@@ -1045,9 +1140,11 @@ qw_status qw_run_host_batch(qw_walk *w, int count, const void *amp_in, int64_t i
     return QW_OK;
 }
 
+static void spectral_off(qw_walk *w) { w->spec_tile = 0; w->spec_user = false; }
+
 qw_status qw_set_plan(qw_walk *w, int depth_k, int tile) {
     if (!w) return QW_EINVAL;
-    if (depth_k == 0) { w->plan_k = 0; w->plan_tile = 0; w->plan_user = false; return QW_OK; }
+    if (depth_k == 0) { w->plan_k = 0; w->plan_tile = 0; w->plan_user = false; spectral_off(w); return QW_OK; }
     if (depth_k < 0 || tile < 0) return set_error(w, QW_EINVAL, "negative plan");
     if (w->ndim == 2) {
         if (depth_k != 1 && depth_k != 4 && depth_k != 8)
@@ -1061,11 +1158,22 @@ qw_status qw_set_plan(qw_walk *w, int depth_k, int tile) {
     if (tile && teff != tile) return set_error(w, QW_EINVAL, "tile not compiled for this precision");
     if (depth_k > 8 * teff) return set_error(w, QW_EINVAL, "k exceeds 8 * tile");
     w->plan_k = depth_k; w->plan_tile = teff; w->plan_variant = 0; w->plan_user = true;
+    spectral_off(w);
     return QW_OK;
 }
 
 qw_status qw_set_plan_ex(qw_walk *w, int depth_k, int tile, int variant) {
     if (!w) return QW_EINVAL;
+    if (variant == 2 && tile >= 256) {   // (smaller tiles: as any variant other than 1, the warp tiles)
+        if (depth_k < 1 || !spectral_walk(w) || !spectral1d_ok(w->prec, w->nx, depth_k, tile))
+            return set_error(w, QW_EINVAL, "momentum-space steps need the periodic 1D walk, one unitary coin, a tile of "
+                                           "256 (or 512: FP32/BF16) and 1 <= k < 16 x tile");
+        cudaError_t e = spectral_prepare(w, tile);
+        if (e != cudaSuccess) return cuda_error(w, e, "momentum-space tables");
+        w->plan_k = 0; w->plan_tile = 0; w->plan_variant = -1; w->plan_user = true;
+        w->spec_tile = tile; w->spec_k = depth_k; w->spec_min = 1; w->spec_user = true;
+        return QW_OK;
+    }
     if (variant != 1) {
         qw_status st = qw_set_plan(w, depth_k, tile);
         if (st == QW_OK && depth_k == 0) w->plan_variant = -1;
@@ -1077,6 +1185,7 @@ qw_status qw_set_plan_ex(qw_walk *w, int depth_k, int tile, int variant) {
                                        "1 <= k < chunk / 2");
     w->plan_k = depth_k; w->plan_tile = sweep_tile(w, tile); w->plan_variant = 1;
     w->plan_user = true;
+    spectral_off(w);
     return QW_OK;
 }
 
@@ -1085,6 +1194,7 @@ qw_status qw_get_plan_ex(const qw_walk *w, int *depth_k, int *tile, int *variant
     int k, t, v;
     effective_plan(w, k, t, v);
     if (w->ndim == 1) t = v == 1 ? sweep_tile(w, t) : tile1d(w->prec, t, w->kind, 0);
+    if (w->spec_tile && w->spec_user) { k = w->spec_k; t = w->spec_tile; v = 2; }
     *depth_k = k; *tile = t; *variant = v;
     return QW_OK;
 }
@@ -1118,15 +1228,19 @@ qw_status qw_describe(const qw_walk *w, char *buf, size_t len) {
                       (long long)w->by0, (long long)w->bh);
     else
         std::snprintf(sup, sizeof sup, "\"%s\"", w->sup_mode == 1 ? "pending" : "full");
+    char spec[96] = "";
+    if (w->spec_tile && spectral_walk(w))
+        std::snprintf(spec, sizeof spec, ", \"spectral\": {\"k\": %d, \"tile\": %d, \"from_steps\": %lld}", w->spec_k,
+                      w->spec_tile, (long long)w->spec_min);
     std::snprintf(buf, len,
                   "{\"ndim\": %d, \"sites\": %lld, \"coin_dim\": %d, \"precision\": %d, \"coin_kind\": \"%s\", "
                   "\"k\": %d, \"tile\": %d, \"path\": \"%s\", \"state_bytes\": %zu, \"clipping\": %d, "
-                  "\"support\": %s}",
+                  "\"support\": %s%s}",
                   w->ndim, (long long)w->ns, w->d, w->prec, kinds[w->kind], k, t,
                   window ? "k_step1d_window" : generic ? "generic"
                           : (w->ndim == 1 ? (var == 1 && w->sup_mode != 2 ? "k_step1d_sweep" : "k_step1d")
                                           : (k > 1 && step2d_tb_ok(w->prec, w->kind, k, w->shift) ? "k_step2d_tb" : "k_step2d")),
-                  w->state_bytes, (int)w->clip_on, sup);
+                  w->state_bytes, (int)w->clip_on, sup, spec);
     return QW_OK;
 }
 
@@ -1172,6 +1286,29 @@ void tune_load() {
         if (std::sscanf(line, " \"%127[^\"]\": [%d, %d]", key, &tile, &k) == 3) g_tune[key] = {tile, k};
     }
     std::fclose(f);
+}
+
+// Calls of fewer steps than this are stepped whatever their time: one transform
+// pair rounds about as much as this many steps.
+constexpr int SPEC_MIN_STEPS = 128;
+
+// ms of one momentum-space launch of K steps (state unchanged, a.out overwritten)
+cudaError_t time_spectral(qw_walk *w, Spec1DArgs &a, int K, float &ms) {
+    a.K = K;
+    cudaError_t e = spectral_launch(w, a, 1.0);
+    cudaEvent_t e0 = nullptr, e1 = nullptr;
+    if (e == cudaSuccess) e = cudaEventCreate(&e0);
+    if (e == cudaSuccess) e = cudaEventCreate(&e1);
+    if (e == cudaSuccess) e = cudaEventRecord(e0, w->stream);
+    const int reps = 3;
+    for (int r = 0; r < reps && e == cudaSuccess; ++r) e = spectral_launch(w, a, 1.0);
+    if (e == cudaSuccess) e = cudaEventRecord(e1, w->stream);
+    if (e == cudaSuccess) e = cudaEventSynchronize(e1);
+    if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
+    ms /= reps;
+    if (e0) cudaEventDestroy(e0);
+    if (e1) cudaEventDestroy(e1);
+    return e;
 }
 
 void tune_save() {
@@ -1238,12 +1375,64 @@ extern "C" qw_status qw_autotune(qw_walk *w, char *report, size_t report_len) {
     const std::string key = tune_key(w);
     auto it = g_tune.find(key);
     char buf[512];
+    spectral_off(w);
+    // The momentum-space form, kept beside the stepping plan under its own key
+    // (tile, fewest steps of a call worth a launch; tile 0: never), so that a
+    // tuning file written without it still serves.  ms_step: the stepping plan's.
+    auto tune_spectral = [&](float ms_step, std::string &rep) -> cudaError_t {
+        const std::string skey = key + "_spectral";
+        auto si = g_tune.find(skey);
+        cudaError_t err = cudaSuccess;
+        if (si == g_tune.end()) {
+            int tile = 0, from = 0;
+            if (ms_step > 0 && spectral_walk(w)) {
+                float best = 1e30f;
+                for (int st : {256, 512}) {
+                    const int k = 8 * st;   // a quarter of the block: half its sites are output
+                    if (!spectral1d_ok(w->prec, w->nx, k, st)) continue;
+                    if (spectral_prepare(w, st) != cudaSuccess) { (void)cudaGetLastError(); break; }
+                    Spec1DArgs a{};
+                    a.n = w->nx; a.tile = st; a.shift = w->shift;
+                    a.in = cur_view(w); a.out = next_view(w);
+                    float ms = 0.f, ms_short = 0.f;
+                    if ((err = time_spectral(w, a, k, ms)) != cudaSuccess) return err;
+                    if ((err = time_spectral(w, a, k / 8, ms_short)) != cudaSuccess) return err;
+                    if (ms / k < best) {
+                        best = ms / k;
+                        tile = st;
+                        // the shortest call that gains, and not below SPEC_MIN_STEPS
+                        from = std::max(SPEC_MIN_STEPS, (int)std::min(1e9f, std::ceil(ms_short / ms_step)));
+                    }
+                }
+                if (!(best < ms_step)) tile = 0;
+            }
+            if (ms_step > 0 && spectral_walk(w)) { g_tune[skey] = {tile, from}; tune_save(); }
+            si = g_tune.find(skey);
+        }
+        if (si != g_tune.end() && spectral_walk(w) && spectral1d_ok(w->prec, w->nx, 1, si->second.first)) {
+            if ((err = spectral_prepare(w, si->second.first)) == cudaErrorMemoryAllocation) {
+                (void)cudaGetLastError();
+                return cudaSuccess;   // no room for the tables: the stepping plan alone
+            }
+            if (err != cudaSuccess) return err;
+            w->spec_tile = si->second.first;
+            w->spec_k = w->spec_tile * 32 / 3;   // a third of the block: more steps leave too few outputs
+            w->spec_min = std::max(1, si->second.second);
+            char b[96];
+            std::snprintf(b, sizeof b, ", \"spectral\": {\"tile\": %d, \"from_steps\": %lld}", w->spec_tile, (long long)w->spec_min);
+            rep = b;
+        }
+        return cudaSuccess;
+    };
     if (it != g_tune.end()) {
         w->plan_tile = std::abs(it->second.first);   // a negative tile records the sweep kernel
         w->plan_variant = it->second.first < 0 ? 1 : 0;
         w->plan_k = it->second.second;
-        std::snprintf(buf, sizeof buf, "{\"tuned\": true, \"cached\": true, \"key\": \"%s\", \"tile\": %d, \"k\": %d}",
-                      key.c_str(), w->plan_tile, w->plan_k);
+        std::string spec;
+        cudaError_t se = tune_spectral(0.f, spec);
+        if (se != cudaSuccess) return cuda_error(w, se, "autotune");
+        std::snprintf(buf, sizeof buf, "{\"tuned\": true, \"cached\": true, \"key\": \"%s\", \"tile\": %d, \"k\": %d%s}",
+                      key.c_str(), w->plan_tile, w->plan_k, spec.c_str());
         put(buf);
         return QW_OK;
     }
@@ -1318,10 +1507,13 @@ extern "C" qw_status qw_autotune(qw_walk *w, char *report, size_t report_len) {
     w->plan_variant = best_v;
     g_tune[key] = {best_v ? -best_t : best_t, best_k};
     tune_save();
+    std::string spec;
+    err = tune_spectral(best, spec);
+    if (err != cudaSuccess) return cuda_error(w, err, "autotune");
     std::snprintf(buf, sizeof buf,
                   "{\"tuned\": true, \"cached\": false, \"key\": \"%s\", \"tile\": %d, \"k\": %d, "
-                  "\"variant\": \"%s\", \"ms_per_step\": %.6g}",
-                  key.c_str(), best_t, best_k, best_v ? "sweep" : "tiles", best);
+                  "\"variant\": \"%s\", \"ms_per_step\": %.6g%s}",
+                  key.c_str(), best_t, best_k, best_v ? "sweep" : "tiles", best, spec.c_str());
     put(buf);
     return QW_OK;
 }

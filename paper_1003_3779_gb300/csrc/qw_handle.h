@@ -82,6 +82,23 @@ struct qw_walk {
     int plan_variant = -1;   // 1D kernel: -1 automatic, 0 independent warp tiles, 1 time-skewed sweep
     bool plan_user = false;
 
+    // momentum-space steps of the cycle (k_spectral1d.cuh): calls of at least
+    // spec_min steps on an unclipped state run them in launches of up to spec_k
+    // steps on blocks of 32 * spec_tile sites (spec_tile 0: off).  The table
+    // holds the twiddles of spec_tw's tile and the matrices of spec_key; a
+    // captured call writes it on every replay, so nothing is reused after one.
+    int spec_tile = 0, spec_k = 0;
+    int64_t spec_min = 0;
+    bool spec_user = false;   // chosen by qw_set_plan_ex
+    void *spec_table = nullptr;
+    int spec_tw = 0;
+    struct SpecKey {
+        double coin[8];
+        double scale;
+        int K, tile, adjoint;
+    } spec_key = {};
+    bool spec_captured = false;
+
     // adjoint / gradient scratch
     void *grad_scratch = nullptr;
     size_t grad_scratch_bytes = 0;
@@ -159,6 +176,14 @@ int tile1d_comp(int, int, int);
 // streaming temporal blocking on the torus (step2d_tb.cu)
 bool step2d_tb_ok(int prec, int kind, int K, int shift);
 cudaError_t launch_step2d_tb(const Step2DArgs &a, const void *coinp, cudaStream_t s);
+
+// momentum-space steps of the cycle (spectral1d.cu)
+int spectral1d_groups(int tile);
+bool spectral1d_ok(int prec, int64_t n, int K, int tile);
+size_t spectral1d_table_bytes(int prec);
+cudaError_t launch_spectral1d_twiddles(int prec, int tile, void *table, cudaStream_t s);
+cudaError_t launch_spectral1d_matrices(int prec, const Spec1DArgs &a, const double *coin, double scale, cudaStream_t s);
+cudaError_t launch_spectral1d(int prec, const Spec1DArgs &a, cudaStream_t s);
 
 // per-site coin conversion kernels (qw_coins.cu)
 cudaError_t launch_convert_coins(int prec, const double *src, void *dst, int64_t count, cudaStream_t s);

@@ -348,6 +348,16 @@ struct Step1DArgs {
 cudaError_t launch_step1d(int prec, const Step1DArgs &a, const void *coinp, cudaStream_t s);
 cudaError_t launch_step1d_adjoint(int prec, const Step1DArgs &a, const void *coinp, cudaStream_t s);
 
+// K steps of a periodic cycle with one coin for all sites, in momentum space
+// (k_spectral1d.cuh); `table` holds the matrices of this K and the twiddles.
+struct Spec1DArgs {
+    View in, out;
+    int64_t n;
+    int K, tile;       // steps; block size / 32
+    int shift, adjoint;
+    void *table;
+};
+
 struct Step2DArgs {
     View in, out;
     int64_t nx, ny;
