@@ -224,7 +224,9 @@ k_step2d(View in, View out, int64_t nx, int64_t ny, int64_t segs, int64_t r0, in
     }
     const int64_t yp = (y + 1 == ny) ? 0 : y + 1;
     const int64_t ym = (y == 0) ? ny - 1 : y - 1;
-    const bool vec_ok = (row % S::VEC) == 0;  // lane sites are VEC-aligned within the row
+    // 16-byte accesses to this row and to the rows above and below: every row
+    // starts on a vector boundary only when the row length is a multiple of VEC
+    const bool vec_ok = (nx % S::VEC) == 0;
 
     if (!ADJ) {
         C a[4][R], p[4][R];

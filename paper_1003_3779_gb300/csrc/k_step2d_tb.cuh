@@ -115,7 +115,8 @@ k_step2d_tb(View in, View out, int64_t nx, int64_t ny, int64_t ox0, int64_t ow, 
     const int64_t hthis = min(H, oh - chunk * H);
     const int j0 = lane * R;                            // tile column of the lane's first site
     const int64_t xs = xo - KT + j0;                    // its global column (may wrap)
-    const bool vec = (xs >= 0) && (xs + R <= nx) && (xs % S::VEC == 0) && (R % S::VEC == 0);
+    // (rows start on 16-byte boundaries only when nx is a multiple of VEC)
+    const bool vec = (xs >= 0) && (xs + R <= nx) && (xs % S::VEC == 0) && (nx % S::VEC == 0) && (R % S::VEC == 0);
     int64_t cx[R];
 #pragma unroll
     for (int i = 0; i < R; ++i) cx[i] = wrap_index(xs + i, nx);
