@@ -34,10 +34,30 @@ __device__ __forceinline__ double block_sum(double v, double *sh) {
     return r;
 }
 
+// Is site i (linear) inside the box?  Both box axes are modulo the lattice.
+__device__ __forceinline__ bool box_has(const SupportBox &b, int64_t i) {
+    int64_t x = i, y = 0;
+    if (b.ny > 1) {
+        if (b.nx * b.ny < (int64_t(1) << 31)) { y = (uint32_t)i / (uint32_t)b.nx; x = (uint32_t)i - (uint32_t)y * (uint32_t)b.nx; }
+        else { y = i / b.nx; x = i - y * b.nx; }
+    }
+    const int64_t dx = x - b.x0, dy = y - b.y0;
+    return (dx >= 0 ? dx : dx + b.nx) < b.w && (dy >= 0 ? dy : dy + b.ny) < b.h;
+}
+template <int VEC> __device__ __forceinline__ bool box_meets(const SupportBox &b, int64_t i0) {
+    bool in = false;
+#pragma unroll
+    for (int k = 0; k < VEC; ++k) in = in || box_has(b, i0 + k);
+    return in;
+}
+
 // Each thread handles VEC consecutive sites per iteration with vector loads.
+// box: the state is zero outside it (a clipped walk), so groups of sites that
+// lie outside are not read; their P is zero and the norm's sum, in the same
+// fixed order, keeps its bits.
 template <int P, int PF32>
 __global__ void __launch_bounds__(RED_THREADS)
-k_marginals(View v, int64_t ns, void *P_out, double *partials) {
+k_marginals(View v, int64_t ns, void *P_out, double *partials, SupportBox box) {
     using S = St<P>;
     using real = typename S::real;
     __shared__ double sh[RED_THREADS / 32];
@@ -50,6 +70,15 @@ k_marginals(View v, int64_t ns, void *P_out, double *partials) {
         double p[S::VEC];
 #pragma unroll
         for (int k = 0; k < S::VEC; ++k) p[k] = 0.0;
+        if (box.w && !box_meets<S::VEC>(box, i0)) {
+#pragma unroll
+            for (int k = 0; k < S::VEC; ++k)
+                if (P_out && i0 + k < ns) {
+                    if (PF32) reinterpret_cast<float *>(P_out)[i0 + k] = 0.f;
+                    else reinterpret_cast<double *>(P_out)[i0 + k] = 0.0;
+                }
+            continue;
+        }
         if constexpr (PF32 && std::is_same<real, float>::value) {
           if (i0 + S::VEC <= ns) {
             // float amplitudes and a float P: |psi|^2 per site in float (FP64 is
@@ -110,20 +139,20 @@ __global__ void k_sum_partials(const double *partials, int n, double *out) {
 
 template <int P>
 static cudaError_t marginals_t(View v, int64_t ns, void *P_out, int pf32, double *partials, int nblocks,
-                               double *norm_dev, cudaStream_t s) {
-    if (pf32) k_marginals<P, 1><<<nblocks, RED_THREADS, 0, s>>>(v, ns, P_out, partials);
-    else k_marginals<P, 0><<<nblocks, RED_THREADS, 0, s>>>(v, ns, P_out, partials);
+                               double *norm_dev, const SupportBox &box, cudaStream_t s) {
+    if (pf32) k_marginals<P, 1><<<nblocks, RED_THREADS, 0, s>>>(v, ns, P_out, partials, box);
+    else k_marginals<P, 0><<<nblocks, RED_THREADS, 0, s>>>(v, ns, P_out, partials, box);
     k_sum_partials<<<1, 32, 0, s>>>(partials, nblocks, norm_dev);
     return cudaGetLastError();
 }
 
 cudaError_t launch_marginals(int prec, View v, int64_t ns, void *P, int p_f32, double *partials,
-                             int nblocks, double *norm_dev, cudaStream_t s) {
+                             int nblocks, double *norm_dev, const SupportBox &box, cudaStream_t s) {
     switch (prec) {
-        case P_F64: return marginals_t<P_F64>(v, ns, P, p_f32, partials, nblocks, norm_dev, s);
-        case P_F32: return marginals_t<P_F32>(v, ns, P, p_f32, partials, nblocks, norm_dev, s);
-        case P_BF16: return marginals_t<P_BF16>(v, ns, P, p_f32, partials, nblocks, norm_dev, s);
-        case P_COMP: return marginals_t<P_COMP>(v, ns, P, p_f32, partials, nblocks, norm_dev, s);
+        case P_F64: return marginals_t<P_F64>(v, ns, P, p_f32, partials, nblocks, norm_dev, box, s);
+        case P_F32: return marginals_t<P_F32>(v, ns, P, p_f32, partials, nblocks, norm_dev, box, s);
+        case P_BF16: return marginals_t<P_BF16>(v, ns, P, p_f32, partials, nblocks, norm_dev, box, s);
+        case P_COMP: return marginals_t<P_COMP>(v, ns, P, p_f32, partials, nblocks, norm_dev, box, s);
     }
     return cudaErrorInvalidValue;
 }
@@ -136,64 +165,202 @@ cudaError_t launch_marginals(int prec, View v, int64_t ns, void *P, int p_f32, d
 // clipping of a localised walk (the "line" computation window of Sec. 3,
 // which starts at the walker's site and widens by one site per step).
 //
-// Work is split into tiles of SUP_THREADS consecutive sites of one row.
-// Blocks run tiles in a probe order that starts with the first tile of row 0
-// and the last tile of the last row: a dense state fills the box there, and
-// every block that then finds the box full returns, so a dense state costs
-// about one wave of tiles, a localised one a full read.
+// The search runs with the copy of the caller's state into the walk's buffer
+// (SRC: one read and one write of the state, at the copy rate) or over the
+// buffer alone.  Each thread takes 16 bytes of every plane slot per round; a
+// block keeps the range it has seen in registers and adds it to the box once,
+// with four atomics.  (Four atomics per warp and tile on the same four words,
+// and cudaMemcpy2DAsync for the copy, took 99 us to search a dense state of
+// 10^6 sites and 1300 us to copy one of 2 GiB; now under 10 us and 650 us.)
+// Over the buffer alone, a first block looks at the first and the last 256
+// sites: a dense state fills the box there, and the search returns.
 static constexpr int SUP_THREADS = 256;
 
-__global__ void k_support_init(unsigned long long *box) {
-    box[0] = ~0ull; box[1] = 0ull; box[2] = ~0ull; box[3] = 0ull;
+// which of the vector's sites hold a nonzero amplitude (-0 is zero; a NaN is not)
+template <int SB> __device__ __forceinline__ unsigned nonzero_sites(uint4 u) {
+    if constexpr (SB == 16) return ((u.y << 1) | u.x | (u.w << 1) | u.z) != 0u;
+    else if constexpr (SB == 8) return (((u.x << 1) | (u.y << 1)) != 0u) | ((((u.z << 1) | (u.w << 1)) != 0u) << 1);
+    else return ((u.x & 0x7fff7fffu) != 0u) | (((u.y & 0x7fff7fffu) != 0u) << 1) |
+                (((u.z & 0x7fff7fffu) != 0u) << 2) | (((u.w & 0x7fff7fffu) != 0u) << 3);
 }
 
-template <int P>
-__global__ void __launch_bounds__(SUP_THREADS)
-k_support(View v, int64_t nx, int64_t ny, int64_t tiles_per_row, int64_t ntiles, unsigned long long *box) {
-    using S = St<P>;
-    const int lane = threadIdx.x & 31;
-    for (int64_t ti = blockIdx.x; ti < ntiles; ti += gridDim.x) {
-        {   // the box already spans the lattice: nothing left to find
-            const volatile unsigned long long *vb = box;
-            if (vb[0] == 0ull && vb[1] == (unsigned long long)(nx - 1) && vb[2] == 0ull &&
-                vb[3] == (unsigned long long)(ny - 1))
-                return;
+// the smallest / largest linear index and column of the sites a thread has seen
+struct Seen {
+    unsigned long long i0 = ~0ull, i1 = 0ull, x0 = ~0ull, x1 = 0ull;
+    __device__ void site(int64_t i, int64_t nx, int64_t ns) {
+        int64_t x = i;
+        if (nx < ns) x = ns < (int64_t(1) << 31) ? (int64_t)((uint32_t)i % (uint32_t)nx) : i % nx;
+        i0 = min(i0, (unsigned long long)i); i1 = max(i1, (unsigned long long)i);
+        x0 = min(x0, (unsigned long long)x); x1 = max(x1, (unsigned long long)x);
+    }
+};
+// add what the block has seen to the box
+__device__ __forceinline__ void merge_seen(Seen v, int64_t nx, unsigned long long *box) {
+    __shared__ unsigned long long sh[SUP_THREADS / 32][4];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        v.i0 = min(v.i0, __shfl_xor_sync(0xffffffffu, v.i0, o));
+        v.i1 = max(v.i1, __shfl_xor_sync(0xffffffffu, v.i1, o));
+        v.x0 = min(v.x0, __shfl_xor_sync(0xffffffffu, v.x0, o));
+        v.x1 = max(v.x1, __shfl_xor_sync(0xffffffffu, v.x1, o));
+    }
+    const int w = threadIdx.x >> 5;
+    if ((threadIdx.x & 31) == 0) { sh[w][0] = v.i0; sh[w][1] = v.i1; sh[w][2] = v.x0; sh[w][3] = v.x1; }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int k = 1; k < SUP_THREADS / 32; ++k) {
+            v.i0 = min(v.i0, sh[k][0]); v.i1 = max(v.i1, sh[k][1]);
+            v.x0 = min(v.x0, sh[k][2]); v.x1 = max(v.x1, sh[k][3]);
         }
-        const int64_t t = ti == 0 ? 0 : (ti == 1 ? ntiles - 1 : ti - 1);   // probe order
-        const int64_t y = t / tiles_per_row;
-        const int64_t x = (t - y * tiles_per_row) * SUP_THREADS + threadIdx.x;
-        bool nz = false;
-        if (x < nx) {
-            const int64_t i = y * nx + x;
-            for (int c = 0; c < v.d; ++c) {
-                const auto a = S::ld(v, c, i);
-                // (a NaN compares unequal to zero too: it counts as nonzero)
-                if constexpr (P == P_COMP)
-                    nz = nz || a.re.hi != 0.f || a.im.hi != 0.f || a.re.lo != 0.f || a.im.lo != 0.f;
-                else
-                    nz = nz || a.re != 0 || a.im != 0;
-            }
-        }
-        const unsigned m = __ballot_sync(0xffffffffu, nz);
-        if (m && lane == 0) {
-            const int64_t xw = x;   // lane 0's column; the warp's lowest / highest set lanes
-            atomicMin(&box[0], (unsigned long long)(xw + (__ffs(m) - 1)));
-            atomicMax(&box[1], (unsigned long long)(xw + (31 - __clz(m))));
-            atomicMin(&box[2], (unsigned long long)y);
-            atomicMax(&box[3], (unsigned long long)y);
+        if (v.i0 != ~0ull) {
+            atomicMin(&box[0], v.x0);
+            atomicMax(&box[1], v.x1);
+            atomicMin(&box[2], v.i0 / (unsigned long long)nx);
+            atomicMax(&box[3], v.i1 / (unsigned long long)nx);
         }
     }
 }
 
-cudaError_t launch_support(int prec, View v, int64_t nx, int64_t ny, unsigned long long *box, cudaStream_t s) {
-    k_support_init<<<1, 1, 0, s>>>(box);
-    const int64_t tpr = (nx + SUP_THREADS - 1) / SUP_THREADS, nt = tpr * ny;
-    const unsigned grid = (unsigned)std::min<int64_t>(nt, 152 * 8);
-    switch (prec) {
-        case P_F64: k_support<P_F64><<<grid, SUP_THREADS, 0, s>>>(v, nx, ny, tpr, nt, box); break;
-        case P_F32: k_support<P_F32><<<grid, SUP_THREADS, 0, s>>>(v, nx, ny, tpr, nt, box); break;
-        case P_BF16: k_support<P_BF16><<<grid, SUP_THREADS, 0, s>>>(v, nx, ny, tpr, nt, box); break;
-        case P_COMP: k_support<P_COMP><<<grid, SUP_THREADS, 0, s>>>(v, nx, ny, tpr, nt, box); break;
+// empties the box; with a state, looks at its first and last SUP_THREADS sites
+template <int SB>
+__global__ void __launch_bounds__(SUP_THREADS)
+k_support_init(const char *state, int64_t slot_bytes, int nslots, int64_t nx, int64_t ns, unsigned long long *box) {
+    if (threadIdx.x == 0) { box[0] = ~0ull; box[1] = 0ull; box[2] = ~0ull; box[3] = 0ull; }
+    if (!state) return;
+    __syncthreads();
+    Seen v;
+    for (int end = 0; end < 2; ++end) {
+        const int64_t i = end ? ns - 1 - threadIdx.x : threadIdx.x;
+        if (i < 0 || i >= ns) continue;
+        for (int c = 0; c < nslots; ++c) {
+            uint4 u = make_uint4(0, 0, 0, 0);
+            const char *p = state + c * slot_bytes + i * SB;
+            if constexpr (SB == 16) u = *reinterpret_cast<const uint4 *>(p);
+            else if constexpr (SB == 8) { const uint2 a = *reinterpret_cast<const uint2 *>(p); u.x = a.x; u.y = a.y; }
+            else u.x = *reinterpret_cast<const unsigned *>(p);
+            if (nonzero_sites<SB>(u)) v.site(i, nx, ns);
+        }
+    }
+    merge_seen(v, nx, box);
+}
+
+// SRC: src holds nslots dense planes of ns sites (16-byte aligned planes), which
+// are copied to dst; else dst is searched alone.
+template <int SB, bool SRC>
+__global__ void __launch_bounds__(SUP_THREADS)
+k_support(const char *__restrict__ src, char *__restrict__ dst, int64_t slot_bytes, int nslots, int64_t nx, int64_t ns,
+          unsigned long long *box) {
+    constexpr int SPV = 16 / SB;   // sites per 16-byte vector
+    if (!SRC) {   // the box already spans the lattice: nothing left to find
+        const volatile unsigned long long *vb = box;
+        if (vb[0] == 0ull && vb[1] == (unsigned long long)(nx - 1) && vb[2] == 0ull &&
+            vb[3] == (unsigned long long)(ns / nx - 1))
+            return;
+    }
+    const int64_t nvec = (ns + SPV - 1) / SPV;
+    Seen v;
+    for (int64_t k = (int64_t)blockIdx.x * SUP_THREADS + threadIdx.x; k < nvec; k += (int64_t)gridDim.x * SUP_THREADS) {
+        unsigned nz = 0;
+        for (int c0 = 0; c0 < nslots; c0 += 2) {   // two slots in flight (nslots is even)
+            uint4 u[2];
+#pragma unroll
+            for (int c = 0; c < 2; ++c)
+                u[c] = SRC ? __ldcs(reinterpret_cast<const uint4 *>(src + (c0 + c) * ns * SB) + k)
+                           : reinterpret_cast<const uint4 *>(dst + (c0 + c) * slot_bytes)[k];
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                if (SRC) reinterpret_cast<uint4 *>(dst + (c0 + c) * slot_bytes)[k] = u[c];
+                nz |= nonzero_sites<SB>(u[c]);
+            }
+        }
+        if (nz) {
+#pragma unroll
+            for (int i = 0; i < SPV; ++i)
+                if ((nz >> i & 1u) && k * SPV + i < ns) v.site(k * SPV + i, nx, ns);   // (not the slot's padding)
+        }
+    }
+    merge_seen(v, nx, box);
+}
+
+template <int SB>
+static cudaError_t support_t(const void *src, View v, int nslots, int64_t nx, int64_t ny, unsigned long long *box, cudaStream_t s) {
+    const int64_t ns = nx * ny, slot = v.pitch * SB;
+    const int64_t tiles = ((ns + 16 / SB - 1) / (16 / SB) + SUP_THREADS - 1) / SUP_THREADS;
+    const unsigned grid = (unsigned)std::min<int64_t>(tiles, 152 * 8);
+    char *dst = static_cast<char *>(v.p);
+    k_support_init<SB><<<1, SUP_THREADS, 0, s>>>(src ? nullptr : dst, slot, nslots, nx, ns, box);
+    if (src) k_support<SB, true><<<grid, SUP_THREADS, 0, s>>>(static_cast<const char *>(src), dst, slot, nslots, nx, ns, box);
+    else k_support<SB, false><<<grid, SUP_THREADS, 0, s>>>(nullptr, dst, slot, nslots, nx, ns, box);
+    return cudaGetLastError();
+}
+
+bool dense_copy_ok(const void *dense, int64_t ns, int slot_bytes) {
+    return (slot_bytes == 8 || slot_bytes == 16) && reinterpret_cast<uintptr_t>(dense) % 16 == 0 && ns * slot_bytes % 16 == 0;
+}
+
+cudaError_t launch_support(const void *src, View v, int nslots, int slot_bytes, int64_t nx, int64_t ny, unsigned long long *box,
+                           cudaStream_t s) {
+    switch (slot_bytes) {
+        case 16: return support_t<16>(src, v, nslots, nx, ny, box, s);
+        case 8: return support_t<8>(src, v, nslots, nx, ny, box, s);
+        case 4: return src ? cudaErrorInvalidValue : support_t<4>(nullptr, v, nslots, nx, ny, box, s);
+    }
+    return cudaErrorInvalidValue;
+}
+
+// The state out into nslots dense planes (16-byte aligned, as dense_copy_ok):
+// sites outside the box, where the state is zero, are written without a read.
+template <int SB>
+__global__ void __launch_bounds__(SUP_THREADS)
+k_store_state(const char *__restrict__ state, int64_t slot_bytes, int nslots, int64_t ns, char *__restrict__ out, SupportBox box) {
+    constexpr int SPV = 16 / SB;
+    const int64_t nvec = ns / SPV;
+    for (int64_t k = (int64_t)blockIdx.x * SUP_THREADS + threadIdx.x; k < nvec; k += (int64_t)gridDim.x * SUP_THREADS) {
+        const bool in = box.w == 0 || box_meets<SPV>(box, k * SPV);
+        for (int c0 = 0; c0 < nslots; c0 += 2) {
+            uint4 u[2] = {};
+#pragma unroll
+            for (int c = 0; c < 2; ++c)
+                if (in) u[c] = reinterpret_cast<const uint4 *>(state + (c0 + c) * slot_bytes)[k];
+#pragma unroll
+            for (int c = 0; c < 2; ++c) __stcs(reinterpret_cast<uint4 *>(out + (c0 + c) * ns * SB) + k, u[c]);
+        }
+    }
+}
+
+cudaError_t launch_store_state(View v, int nslots, int slot_bytes, int64_t ns, void *out, const SupportBox &box, cudaStream_t s) {
+    const int64_t tiles = (ns / (16 / slot_bytes) + SUP_THREADS - 1) / SUP_THREADS;
+    const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(tiles, 152 * 8));
+    const char *p = static_cast<const char *>(v.p);
+    char *o = static_cast<char *>(out);
+    if (slot_bytes == 16) k_store_state<16><<<grid, SUP_THREADS, 0, s>>>(p, v.pitch * 16, nslots, ns, o, box);
+    else if (slot_bytes == 8) k_store_state<8><<<grid, SUP_THREADS, 0, s>>>(p, v.pitch * 8, nslots, ns, o, box);
+    else return cudaErrorInvalidValue;
+    return cudaGetLastError();
+}
+
+// Zero the box of every slot (columns and rows modulo the lattice).
+template <class V>
+__global__ void __launch_bounds__(SUP_THREADS)
+k_clear_box(V *state, int64_t pitch, int nslots, SupportBox b) {
+    const int64_t n = b.w * b.h;
+    for (int64_t k = (int64_t)blockIdx.x * SUP_THREADS + threadIdx.x; k < n; k += (int64_t)gridDim.x * SUP_THREADS) {
+        const int64_t r = k / b.w;
+        int64_t x = b.x0 + (k - r * b.w), y = b.y0 + r;
+        if (x >= b.nx) x -= b.nx;
+        if (y >= b.ny) y -= b.ny;
+        for (int c = 0; c < nslots; ++c) state[c * pitch + y * b.nx + x] = V{};
+    }
+}
+
+cudaError_t launch_clear_box(View v, int nslots, int slot_bytes, const SupportBox &b, cudaStream_t s) {
+    const int64_t tiles = (b.w * b.h + SUP_THREADS - 1) / SUP_THREADS;
+    if (tiles <= 0) return cudaSuccess;
+    const unsigned grid = (unsigned)std::min<int64_t>(tiles, 152 * 8);
+    switch (slot_bytes) {
+        case 16: k_clear_box<uint4><<<grid, SUP_THREADS, 0, s>>>(static_cast<uint4 *>(v.p), v.pitch, nslots, b); break;
+        case 8: k_clear_box<uint2><<<grid, SUP_THREADS, 0, s>>>(static_cast<uint2 *>(v.p), v.pitch, nslots, b); break;
+        case 4: k_clear_box<unsigned><<<grid, SUP_THREADS, 0, s>>>(static_cast<unsigned *>(v.p), v.pitch, nslots, b); break;
         default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();

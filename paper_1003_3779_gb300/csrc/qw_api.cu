@@ -365,21 +365,21 @@ static bool capturing(const qw_walk *w) {
 }
 
 // Queue the search for the support box of the current state (qw_set_state).
-static qw_status queue_support(qw_walk *w) {
+// src: the caller's planes in the storage format, copied into the buffer on
+// the way (dense_copy_ok), or null: the buffer holds the state already.
+static qw_status queue_support(qw_walk *w, const void *src = nullptr) {
     w->next_clear = false;
-    if (!w->clip_on || capturing(w)) {
-        (void)cudaGetLastError();
-        w->sup_mode = 0;
-        return QW_OK;
-    }
-    cudaError_t e = launch_support(w->prec == QW_F64 ? P_F64 : w->prec == QW_F32 ? P_F32
-                                   : w->prec == QW_F32_BF16STORE ? P_BF16 : P_COMP,
-                                   cur_view(w), w->nx, w->ny, w->sup_dev, w->stream);
-    if (e == cudaSuccess)
+    const bool capture = capturing(w);
+    if (capture) { (void)cudaGetLastError(); w->captured = true; }
+    const bool search = w->clip_on && !capture;
+    w->sup_mode = 0;
+    if (!search && !src) return QW_OK;
+    cudaError_t e = launch_support(src, cur_view(w), w->nslots, w->slot_bytes, w->nx, w->ny, w->sup_dev, w->stream);
+    if (e == cudaSuccess && search)
         e = cudaMemcpyAsync(w->sup_host, w->sup_dev, 4 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, w->stream);
-    if (e == cudaSuccess) e = cudaEventRecord(w->sup_ev, w->stream);
-    if (e != cudaSuccess) { w->sup_mode = 0; return cuda_error(w, e, "support search"); }
-    w->sup_mode = 1;
+    if (e == cudaSuccess && search) e = cudaEventRecord(w->sup_ev, w->stream);
+    if (e != cudaSuccess) return cuda_error(w, e, src ? "state copy" : "support search");
+    w->sup_mode = search ? 1 : 0;
     return QW_OK;
 }
 
@@ -422,10 +422,19 @@ static void grow_support(qw_walk *w, int K) {
     if (w->bw >= w->nx && w->bh >= w->ny) w->sup_mode = 0;
 }
 
+// The box of the current state for the kernels that read it out (w = 0 when it
+// is not known, or when a graph replay may have changed the state).
+static SupportBox state_box(const qw_walk *w) {
+    if (w->sup_mode != 2 || w->captured) return {0, 0, 0, 0, w->nx, w->ny};
+    return {w->bx0, w->bw, w->by0, w->bh, w->nx, w->ny};
+}
+
 // Before a clipped step: the other buffer must be zero outside the box.
 static qw_status clear_next(qw_walk *w) {
     if (w->next_clear) return QW_OK;
-    cudaError_t e = cudaMemsetAsync(w->buf[w->cur ^ 1], 0, w->state_bytes, w->stream);
+    cudaError_t e = w->dirty_known && !w->captured
+                        ? launch_clear_box(next_view(w), w->nslots, w->slot_bytes, w->dirty, w->stream)
+                        : cudaMemsetAsync(w->buf[w->cur ^ 1], 0, w->state_bytes, w->stream);
     if (e != cudaSuccess) return cuda_error(w, e, "clear");
     w->next_clear = true;
     return QW_OK;
@@ -481,8 +490,8 @@ static cudaError_t spectral_launch(qw_walk *w, Spec1DArgs &a, double gain) {
     std::memcpy(key.coin, coin, sizeof key.coin);
     key.scale = scale; key.K = a.K; key.tile = a.tile; key.adjoint = a.adjoint;
     a.table = w->spec_table;
-    if (capturing(w)) w->spec_captured = true;
-    if (w->spec_captured || std::memcmp(&key, &w->spec_key, sizeof key) != 0) {
+    if (capturing(w)) w->captured = true;
+    if (w->captured || std::memcmp(&key, &w->spec_key, sizeof key) != 0) {
         cudaError_t e = launch_spectral1d_matrices(w->prec, a, coin, scale, w->stream);
         if (e != cudaSuccess) return e;
         std::memcpy(&w->spec_key, &key, sizeof key);
@@ -537,6 +546,8 @@ qw_status run_steps(qw_walk *w, int64_t T, int adj) {
         qw_status st = resolve_support(w);
         if (st != QW_OK) return st;
         if (w->sup_mode == 2 && (st = clear_next(w)) != QW_OK) return st;
+        w->dirty_known = false;
+        if (capturing(w)) { (void)cudaGetLastError(); w->captured = true; }
     }
     if (generic) {
         StepGenericArgs a{};
@@ -758,6 +769,7 @@ qw_status qw_create(int ndim, const int64_t *dims, int coin_dim, qw_boundary bc,
     double ident[32] = {0};
     for (int i = 0; i < coin_dim; ++i) ident[2 * (i * coin_dim + i)] = 1.0;
     apply_global_coin(w, ident);
+    w->dirty_known = true;   // both buffers are zero
     *out = w;
     return QW_OK;
 }
@@ -897,8 +909,13 @@ qw_status qw_set_state(qw_walk *w, const void *amp, qw_cdtype dtype, int on_devi
     const View dst = cur_view(w);
     w->gain_fb = 1.0;
     w->drift_pending = 1.0;
+    if (w->sup_mode == 2 && w->next_clear) {   // both buffers are zero outside the old box
+        w->dirty_known = true;
+        w->dirty = {w->bx0, w->bw, w->by0, w->bh, w->nx, w->ny};
+    }
     w->sup_mode = 0;
     if (direct_layout(w, dtype)) {
+        if (on_device && dense_copy_ok(amp, w->ns, w->slot_bytes)) return queue_support(w, amp);
         e = cudaMemcpy2DAsync(w->buf[w->cur], (size_t)w->pitch * w->slot_bytes, amp, plane, plane, w->d,
                               on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, w->stream);
         if (e != cudaSuccess) return cuda_error(w, e, "state copy");
@@ -937,6 +954,10 @@ qw_status qw_get_state(qw_walk *w, void *amp_out, qw_cdtype dtype, int on_device
     cudaError_t e = cudaSuccess;
     const View src = cur_view(w);
     if (direct_layout(w, dtype)) {
+        if (on_device && dense_copy_ok(amp_out, w->ns, w->slot_bytes)) {
+            e = launch_store_state(src, w->nslots, w->slot_bytes, w->ns, amp_out, state_box(w), w->stream);
+            return e == cudaSuccess ? QW_OK : cuda_error(w, e, "state copy");
+        }
         e = cudaMemcpy2DAsync(amp_out, plane, w->buf[w->cur], (size_t)w->pitch * w->slot_bytes, plane, w->d,
                               on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, w->stream);
         if (e == cudaSuccess && !on_device) e = cudaStreamSynchronize(w->stream);
@@ -997,7 +1018,7 @@ qw_status qw_probabilities(qw_walk *w, void *P_out, qw_rdtype pdtype, int on_dev
         }
     }
     e = launch_marginals(w->prec, cur_view(w), w->ns, pdst, pdtype == QW_R32, w->partials, marginal_blocks(),
-                         w->norm_dev, w->stream);
+                         w->norm_dev, state_box(w), w->stream);
     if (e != cudaSuccess) return cuda_error(w, e, "marginal launch");
     if (P_out && !on_device) {
         if ((e = cudaMemcpyAsync(P_out, w->p_dev, pb, cudaMemcpyDeviceToHost, w->stream)) != cudaSuccess)
@@ -1025,6 +1046,7 @@ qw_status qw_run_host_batch(qw_walk *w, int count, const void *amp_in, int64_t i
         return set_error(w, QW_EUNSUPPORTED, "pipelined runs take complex64 states for FP32 and complex128 for FP64");
     if (count == 0) return QW_OK;
     w->sup_mode = 0;   // arbitrary host states: every run steps the whole lattice
+    w->dirty_known = false;
     const size_t plane = (size_t)w->ns * (dtype == QW_C128 ? 16 : 8);
     const size_t pb = (size_t)w->ns * (pdtype == QW_R32 ? 4 : 8);
     cudaError_t e = cudaSuccess;
@@ -1101,7 +1123,7 @@ qw_status qw_run_host_batch(qw_walk *w, int count, const void *amp_in, int64_t i
         if ((st = run_steps(w, T, 0)) != QW_OK) break;
         void *pslot = w->pipe_p[i & 1];
         e = launch_marginals(w->prec, cur_view(w), w->ns, pslot, pdtype == QW_R32, w->partials, marginal_blocks(),
-                             w->pipe_norm + i, w->stream);
+                             w->pipe_norm + i, state_box(w), w->stream);
         if (e == cudaSuccess) e = cudaEventRecord(ev_done[i], w->stream);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(w->s_out, ev_done[i], 0);
         if (e == cudaSuccess)
@@ -1336,6 +1358,7 @@ extern "C" qw_status qw_autotune(qw_walk *w, char *report, size_t report_len) {
         put("{\"tuned\": false, \"reason\": \"the generic boundary / broken-link kernel has no plan space\"}");
         return QW_OK;
     }
+    w->next_clear = w->dirty_known = false;   // the timed launches write the other buffer
     if (w->ndim == 2) {
         // k = 1 (fused step) against the streaming kernel at k = 4 and 8
         cudaEvent_t e0, e1;

@@ -73,6 +73,13 @@ struct qw_walk {
     int sup_mode = 0;
     int64_t bx0 = 0, bw = 0, by0 = 0, bh = 0;
     bool next_clear = false;
+    // dirty_known: no step has run since the state was set, and the other buffer
+    // is zero outside the box dirty (the box of the clipped steps before that)
+    bool dirty_known = false;
+    qw::SupportBox dirty = {0, 0, 0, 0, 1, 1};
+    // a call on this handle was captured into a CUDA graph: its replays change
+    // the buffers and tables at times the host does not see
+    bool captured = false;
     unsigned long long *sup_dev = nullptr;    // 4 values (device)
     unsigned long long *sup_host = nullptr;   // 4 values (pinned)
     cudaEvent_t sup_ev = nullptr;
@@ -86,7 +93,7 @@ struct qw_walk {
     // spec_min steps on an unclipped state run them in launches of up to spec_k
     // steps on blocks of 32 * spec_tile sites (spec_tile 0: off).  The table
     // holds the twiddles of spec_tw's tile and the matrices of spec_key; a
-    // captured call writes it on every replay, so nothing is reused after one.
+    // captured call writes it on every replay, so no matrices are reused after one.
     int spec_tile = 0, spec_k = 0;
     int64_t spec_min = 0;
     bool spec_user = false;   // chosen by qw_set_plan_ex
@@ -97,7 +104,6 @@ struct qw_walk {
         double scale;
         int K, tile, adjoint;
     } spec_key = {};
-    bool spec_captured = false;
 
     // adjoint / gradient scratch
     void *grad_scratch = nullptr;

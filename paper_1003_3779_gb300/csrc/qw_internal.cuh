@@ -396,9 +396,15 @@ struct StepGenericArgs {
 };
 cudaError_t launch_step_generic(int prec, const StepGenericArgs &a, const void *coinp, cudaStream_t s);
 
+// The box outside which a state is zero: columns [x0, x0 + w) and rows
+// [y0, y0 + h), modulo the nx x ny lattice; w = 0: nothing is known.
+struct SupportBox {
+    int64_t x0, w, y0, h, nx, ny;
+};
+
 // marginals + norm
 cudaError_t launch_marginals(int prec, View v, int64_t nsites, void *P, int p_f32,
-                             double *partials, int nblocks, double *norm_dev, cudaStream_t s);
+                             double *partials, int nblocks, double *norm_dev, const SupportBox &box, cudaStream_t s);
 int marginal_blocks();
 
 // conversions between caller layout (dense planes, complex128/complex64) and storage
@@ -407,7 +413,14 @@ cudaError_t launch_import(int prec, View dst, int64_t nsites, const void *src, i
 cudaError_t launch_export(int prec, View src, int64_t nsites, void *dst, int dst_c64,
                           int64_t first_site, int64_t count, int plane, cudaStream_t s);
 cudaError_t launch_zero_state(View v, int nslots, int slot_bytes, cudaStream_t s);
-// bounding box of the nonzero amplitudes: box[0..1] columns, box[2..3] rows
-cudaError_t launch_support(int prec, View v, int64_t nx, int64_t ny, unsigned long long *box, cudaStream_t s);
+// bounding box of the nonzero amplitudes: box[0..1] columns, box[2..3] rows.
+// src: nslots dense planes in the storage format (dense_copy_ok), which are
+// copied into v on the way; or null
+bool dense_copy_ok(const void *dense, int64_t ns, int slot_bytes);
+cudaError_t launch_support(const void *src, View v, int nslots, int slot_bytes, int64_t nx, int64_t ny, unsigned long long *box,
+                           cudaStream_t s);
+// the state out into dense planes (dense_copy_ok)
+cudaError_t launch_store_state(View v, int nslots, int slot_bytes, int64_t ns, void *out, const SupportBox &box, cudaStream_t s);
+cudaError_t launch_clear_box(View v, int nslots, int slot_bytes, const SupportBox &b, cudaStream_t s);
 
 }  // namespace qw
