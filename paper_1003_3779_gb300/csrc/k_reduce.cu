@@ -142,7 +142,7 @@ static cudaError_t marginals_t(View v, int64_t ns, void *P_out, int pf32, double
                                double *norm_dev, const SupportBox &box, cudaStream_t s) {
     if (pf32) k_marginals<P, 1><<<nblocks, RED_THREADS, 0, s>>>(v, ns, P_out, partials, box);
     else k_marginals<P, 0><<<nblocks, RED_THREADS, 0, s>>>(v, ns, P_out, partials, box);
-    k_sum_partials<<<1, 32, 0, s>>>(partials, nblocks, norm_dev);
+    if (norm_dev) k_sum_partials<<<1, 32, 0, s>>>(partials, nblocks, norm_dev);
     return cudaGetLastError();
 }
 
@@ -244,13 +244,17 @@ k_support_init(const char *state, int64_t slot_bytes, int nslots, int64_t nx, in
     merge_seen(v, nx, box);
 }
 
-// SRC: src holds nslots dense planes of ns sites (16-byte aligned planes), which
-// are copied to dst; else dst is searched alone.
-template <int SB, bool SRC>
+__device__ __forceinline__ uint4 widen(uint4 u) { return u; }
+__device__ __forceinline__ uint4 widen(uint2 u) { return make_uint4(u.x, u.y, 0u, 0u); }
+
+// SRC: src holds nslots dense planes of ns sites, which are copied to dst; else
+// dst is searched alone.  V: the vector that every plane of src is aligned to,
+// 16 bytes, or 8 for complex64 planes of an odd number of sites.
+template <int SB, bool SRC, class V>
 __global__ void __launch_bounds__(SUP_THREADS)
 k_support(const char *__restrict__ src, char *__restrict__ dst, int64_t slot_bytes, int nslots, int64_t nx, int64_t ns,
           unsigned long long *box) {
-    constexpr int SPV = 16 / SB;   // sites per 16-byte vector
+    constexpr int SPV = (int)sizeof(V) / SB;   // sites per vector
     if (!SRC) {   // the box already spans the lattice: nothing left to find
         const volatile unsigned long long *vb = box;
         if (vb[0] == 0ull && vb[1] == (unsigned long long)(nx - 1) && vb[2] == 0ull &&
@@ -262,15 +266,15 @@ k_support(const char *__restrict__ src, char *__restrict__ dst, int64_t slot_byt
     for (int64_t k = (int64_t)blockIdx.x * SUP_THREADS + threadIdx.x; k < nvec; k += (int64_t)gridDim.x * SUP_THREADS) {
         unsigned nz = 0;
         for (int c0 = 0; c0 < nslots; c0 += 2) {   // two slots in flight (nslots is even)
-            uint4 u[2];
+            V u[2];
 #pragma unroll
             for (int c = 0; c < 2; ++c)
-                u[c] = SRC ? __ldcs(reinterpret_cast<const uint4 *>(src + (c0 + c) * ns * SB) + k)
-                           : reinterpret_cast<const uint4 *>(dst + (c0 + c) * slot_bytes)[k];
+                u[c] = SRC ? __ldcs(reinterpret_cast<const V *>(src + (c0 + c) * ns * SB) + k)
+                           : reinterpret_cast<const V *>(dst + (c0 + c) * slot_bytes)[k];
 #pragma unroll
             for (int c = 0; c < 2; ++c) {
-                if (SRC) reinterpret_cast<uint4 *>(dst + (c0 + c) * slot_bytes)[k] = u[c];
-                nz |= nonzero_sites<SB>(u[c]);
+                if (SRC) reinterpret_cast<V *>(dst + (c0 + c) * slot_bytes)[k] = u[c];
+                nz |= nonzero_sites<SB>(widen(u[c]));
             }
         }
         if (nz) {
@@ -282,60 +286,66 @@ k_support(const char *__restrict__ src, char *__restrict__ dst, int64_t slot_byt
     merge_seen(v, nx, box);
 }
 
-template <int SB>
+template <int SB, class V>
 static cudaError_t support_t(const void *src, View v, int nslots, int64_t nx, int64_t ny, unsigned long long *box, cudaStream_t s) {
+    constexpr int SPV = (int)sizeof(V) / SB;
     const int64_t ns = nx * ny, slot = v.pitch * SB;
-    const int64_t tiles = ((ns + 16 / SB - 1) / (16 / SB) + SUP_THREADS - 1) / SUP_THREADS;
+    const int64_t tiles = ((ns + SPV - 1) / SPV + SUP_THREADS - 1) / SUP_THREADS;
     const unsigned grid = (unsigned)std::min<int64_t>(tiles, 152 * 8);
     char *dst = static_cast<char *>(v.p);
     k_support_init<SB><<<1, SUP_THREADS, 0, s>>>(src ? nullptr : dst, slot, nslots, nx, ns, box);
-    if (src) k_support<SB, true><<<grid, SUP_THREADS, 0, s>>>(static_cast<const char *>(src), dst, slot, nslots, nx, ns, box);
-    else k_support<SB, false><<<grid, SUP_THREADS, 0, s>>>(nullptr, dst, slot, nslots, nx, ns, box);
+    if (src) k_support<SB, true, V><<<grid, SUP_THREADS, 0, s>>>(static_cast<const char *>(src), dst, slot, nslots, nx, ns, box);
+    else k_support<SB, false, V><<<grid, SUP_THREADS, 0, s>>>(nullptr, dst, slot, nslots, nx, ns, box);
     return cudaGetLastError();
 }
 
-bool dense_copy_ok(const void *dense, int64_t ns, int slot_bytes) {
-    return (slot_bytes == 8 || slot_bytes == 16) && reinterpret_cast<uintptr_t>(dense) % 16 == 0 && ns * slot_bytes % 16 == 0;
+int dense_vector(const void *dense, int64_t ns, int slot_bytes) {
+    for (int vb : {16, 8})
+        if (vb >= slot_bytes && slot_bytes >= 8 && reinterpret_cast<uintptr_t>(dense) % vb == 0 && ns * slot_bytes % vb == 0)
+            return vb;
+    return 0;
 }
 
 cudaError_t launch_support(const void *src, View v, int nslots, int slot_bytes, int64_t nx, int64_t ny, unsigned long long *box,
                            cudaStream_t s) {
-    switch (slot_bytes) {
-        case 16: return support_t<16>(src, v, nslots, nx, ny, box, s);
-        case 8: return support_t<8>(src, v, nslots, nx, ny, box, s);
-        case 4: return src ? cudaErrorInvalidValue : support_t<4>(nullptr, v, nslots, nx, ny, box, s);
-    }
+    const int vb = src ? dense_vector(src, nx * ny, slot_bytes) : 16;
+    if (slot_bytes == 16 && vb == 16) return support_t<16, uint4>(src, v, nslots, nx, ny, box, s);
+    if (slot_bytes == 8 && vb == 16) return support_t<8, uint4>(src, v, nslots, nx, ny, box, s);
+    if (slot_bytes == 8 && vb == 8) return support_t<8, uint2>(src, v, nslots, nx, ny, box, s);
+    if (slot_bytes == 4 && !src) return support_t<4, uint4>(nullptr, v, nslots, nx, ny, box, s);
     return cudaErrorInvalidValue;
 }
 
-// The state out into nslots dense planes (16-byte aligned, as dense_copy_ok):
-// sites outside the box, where the state is zero, are written without a read.
-template <int SB>
+// The state out into nslots dense planes (V as dense_vector): sites outside the
+// box, where the state is zero, are written without a read.
+template <int SB, class V>
 __global__ void __launch_bounds__(SUP_THREADS)
 k_store_state(const char *__restrict__ state, int64_t slot_bytes, int nslots, int64_t ns, char *__restrict__ out, SupportBox box) {
-    constexpr int SPV = 16 / SB;
+    constexpr int SPV = (int)sizeof(V) / SB;
     const int64_t nvec = ns / SPV;
     for (int64_t k = (int64_t)blockIdx.x * SUP_THREADS + threadIdx.x; k < nvec; k += (int64_t)gridDim.x * SUP_THREADS) {
         const bool in = box.w == 0 || box_meets<SPV>(box, k * SPV);
         for (int c0 = 0; c0 < nslots; c0 += 2) {
-            uint4 u[2] = {};
+            V u[2] = {};
 #pragma unroll
             for (int c = 0; c < 2; ++c)
-                if (in) u[c] = reinterpret_cast<const uint4 *>(state + (c0 + c) * slot_bytes)[k];
+                if (in) u[c] = reinterpret_cast<const V *>(state + (c0 + c) * slot_bytes)[k];
 #pragma unroll
-            for (int c = 0; c < 2; ++c) __stcs(reinterpret_cast<uint4 *>(out + (c0 + c) * ns * SB) + k, u[c]);
+            for (int c = 0; c < 2; ++c) __stcs(reinterpret_cast<V *>(out + (c0 + c) * ns * SB) + k, u[c]);
         }
     }
 }
 
 cudaError_t launch_store_state(View v, int nslots, int slot_bytes, int64_t ns, void *out, const SupportBox &box, cudaStream_t s) {
-    const int64_t tiles = (ns / (16 / slot_bytes) + SUP_THREADS - 1) / SUP_THREADS;
+    const int vb = dense_vector(out, ns, slot_bytes);
+    if (!vb) return cudaErrorInvalidValue;
+    const int64_t tiles = (ns / (vb / slot_bytes) + SUP_THREADS - 1) / SUP_THREADS;
     const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(tiles, 152 * 8));
     const char *p = static_cast<const char *>(v.p);
     char *o = static_cast<char *>(out);
-    if (slot_bytes == 16) k_store_state<16><<<grid, SUP_THREADS, 0, s>>>(p, v.pitch * 16, nslots, ns, o, box);
-    else if (slot_bytes == 8) k_store_state<8><<<grid, SUP_THREADS, 0, s>>>(p, v.pitch * 8, nslots, ns, o, box);
-    else return cudaErrorInvalidValue;
+    if (slot_bytes == 16) k_store_state<16, uint4><<<grid, SUP_THREADS, 0, s>>>(p, v.pitch * 16, nslots, ns, o, box);
+    else if (vb == 16) k_store_state<8, uint4><<<grid, SUP_THREADS, 0, s>>>(p, v.pitch * 8, nslots, ns, o, box);
+    else k_store_state<8, uint2><<<grid, SUP_THREADS, 0, s>>>(p, v.pitch * 8, nslots, ns, o, box);
     return cudaGetLastError();
 }
 

@@ -366,7 +366,7 @@ static bool capturing(const qw_walk *w) {
 
 // Queue the search for the support box of the current state (qw_set_state).
 // src: the caller's planes in the storage format, copied into the buffer on
-// the way (dense_copy_ok), or null: the buffer holds the state already.
+// the way (dense_vector), or null: the buffer holds the state already.
 static qw_status queue_support(qw_walk *w, const void *src = nullptr) {
     w->next_clear = false;
     const bool capture = capturing(w);
@@ -915,7 +915,7 @@ qw_status qw_set_state(qw_walk *w, const void *amp, qw_cdtype dtype, int on_devi
     }
     w->sup_mode = 0;
     if (direct_layout(w, dtype)) {
-        if (on_device && dense_copy_ok(amp, w->ns, w->slot_bytes)) return queue_support(w, amp);
+        if (on_device && dense_vector(amp, w->ns, w->slot_bytes)) return queue_support(w, amp);
         e = cudaMemcpy2DAsync(w->buf[w->cur], (size_t)w->pitch * w->slot_bytes, amp, plane, plane, w->d,
                               on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, w->stream);
         if (e != cudaSuccess) return cuda_error(w, e, "state copy");
@@ -954,7 +954,7 @@ qw_status qw_get_state(qw_walk *w, void *amp_out, qw_cdtype dtype, int on_device
     cudaError_t e = cudaSuccess;
     const View src = cur_view(w);
     if (direct_layout(w, dtype)) {
-        if (on_device && dense_copy_ok(amp_out, w->ns, w->slot_bytes)) {
+        if (on_device && dense_vector(amp_out, w->ns, w->slot_bytes)) {
             e = launch_store_state(src, w->nslots, w->slot_bytes, w->ns, amp_out, state_box(w), w->stream);
             return e == cudaSuccess ? QW_OK : cuda_error(w, e, "state copy");
         }
@@ -1018,7 +1018,7 @@ qw_status qw_probabilities(qw_walk *w, void *P_out, qw_rdtype pdtype, int on_dev
         }
     }
     e = launch_marginals(w->prec, cur_view(w), w->ns, pdst, pdtype == QW_R32, w->partials, marginal_blocks(),
-                         w->norm_dev, state_box(w), w->stream);
+                         norm_out ? w->norm_dev : nullptr, state_box(w), w->stream);
     if (e != cudaSuccess) return cuda_error(w, e, "marginal launch");
     if (P_out && !on_device) {
         if ((e = cudaMemcpyAsync(P_out, w->p_dev, pb, cudaMemcpyDeviceToHost, w->stream)) != cudaSuccess)

@@ -414,12 +414,13 @@ cudaError_t launch_export(int prec, View src, int64_t nsites, void *dst, int dst
                           int64_t first_site, int64_t count, int plane, cudaStream_t s);
 cudaError_t launch_zero_state(View v, int nslots, int slot_bytes, cudaStream_t s);
 // bounding box of the nonzero amplitudes: box[0..1] columns, box[2..3] rows.
-// src: nslots dense planes in the storage format (dense_copy_ok), which are
-// copied into v on the way; or null
-bool dense_copy_ok(const void *dense, int64_t ns, int slot_bytes);
+// src: nslots dense planes in the storage format, which are copied into v on
+// the way; or null.  dense_vector: the widest access (16 or 8 bytes) that every
+// such plane is aligned to, 0 if none (the caller then copies by other means)
+int dense_vector(const void *dense, int64_t ns, int slot_bytes);
 cudaError_t launch_support(const void *src, View v, int nslots, int slot_bytes, int64_t nx, int64_t ny, unsigned long long *box,
                            cudaStream_t s);
-// the state out into dense planes (dense_copy_ok)
+// the state out into dense planes (dense_vector > 0)
 cudaError_t launch_store_state(View v, int nslots, int slot_bytes, int64_t ns, void *out, const SupportBox &box, cudaStream_t s);
 cudaError_t launch_clear_box(View v, int nslots, int slot_bytes, const SupportBox &b, cudaStream_t s);
 
