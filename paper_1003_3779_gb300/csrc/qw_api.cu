@@ -140,30 +140,16 @@ static void tiles_of(int prec, int &a, int &b) {
     else { a = 8; b = 16; }
 }
 
-// Warps the 2D streaming kernel can keep busy at depth KT: 64-column strips
-// with KT columns of halo per side, row chunks of at least 8 KT rows.
-static int64_t tb_warps(const qw_walk *w, int KT) {
-    const int64_t W = 64 - 2 * KT;
-    return ((w->nx + W - 1) / W) * ((w->ny + 8 * KT - 1) / (8 * KT));
-}
-
 static void default_plan(const qw_walk *w, int &k, int &tile, int &variant) {
     variant = 0;
     if (w->ndim == 2) {
-        // the streaming kernel where the lattice gives it two waves of warps
-        // (8 per SM), else the fused single step
+        // the streaming kernel at its deepest wherever it runs: per step at k = 8 /
+        // k = 1, 64^2 1.9 / 6.3 us, 300 x 200 1.9 / 8.3, 1024^2 4.0 / 14.4, 2048^2
+        // 9.3 / 46, 8192^2 105 / 647 (k = 4: 2.2, 2.2, 4.7, 12.4, 174)
         tile = 0;
         k = 1;
-        if (w->bc != QW_BC_PERIODIC || links_on(w)) return;
-        static int sms = 0;
-        if (!sms) {
-            int dev = 0;
-            cudaGetDevice(&dev);
-            if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0) sms = 152;
-        }
-        const int64_t enough = (int64_t)sms * 8 * 2;
-        for (int KT : {8, 4})
-            if (step2d_tb_ok(w->prec, w->kind, KT, w->shift) && tb_warps(w, KT) >= enough) { k = KT; break; }
+        if (w->bc != QW_BC_PERIODIC || links_on(w) || w->nx < 32 || w->ny < 32) return;
+        if (step2d_tb_ok(w->prec, w->kind, 8, w->shift)) k = 8;
         return;
     }
     switch (w->prec) {
@@ -653,10 +639,12 @@ qw_status run_steps(qw_walk *w, int64_t T, int adj) {
     int K2, t2;
     effective_plan(w, K2, t2);
     if (!adj && K2 > 1 && step2d_tb_ok(w->prec, w->kind, K2, w->shift)) {
-        // whole blocks of K2 steps in the streaming kernel, the rest one step at a time
+        // whole blocks of K2 steps in the streaming kernel, then one of 4, the rest
+        // one step at a time
         Step2DArgs b = a;
         b.K = K2;
-        while (T >= K2) {
+        while (T >= K2 || (T >= 4 && step2d_tb_ok(w->prec, w->kind, 4, w->shift))) {
+            if (T < K2) b.K = K2 = 4;
             b.gain = drift_gain(w, K2, T - K2 == 0);   // applied once, to the launch's output
             b.in = cur_view(w); b.out = next_view(w);
             set_box(b);
