@@ -370,7 +370,7 @@ static qw_status queue_support(qw_walk *w, const void *src = nullptr) {
 }
 
 // Take the searched box (waits for the search only, not for later work).
-static qw_status resolve_support(qw_walk *w) {
+qw_status resolve_support(qw_walk *w) {
     if (w->sup_mode != 1) return QW_OK;
     w->sup_mode = 0;
     if (capturing(w)) { (void)cudaGetLastError(); return QW_OK; }   // step in full

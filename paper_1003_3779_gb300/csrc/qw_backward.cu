@@ -16,6 +16,15 @@
 // (the walk is unitary) instead of stored; it is re-seeded from a forward
 // checkpoint every K steps, which bounds the drift of the reconstruction to K
 // steps.
+//
+// Light cones (the computation windows of Sec. 3, of the walk and of its
+// adjoint): lambda_t is zero outside the region widened by T - t sites, and
+// psi_t outside the start's support widened by t.  The product a b, and with it
+// the gradient, is zero outside their intersection; lambda is only needed
+// where psi will still be nonzero, which is that intersection too, and psi on
+// the sites from which the rest of its segment is rebuilt.  A step runs on
+// those sites only.  On a 1024^2 torus (T = 512, K = 64, a walker on one site,
+// a 64 x 64 region) the sweep's sites fall to a tenth.
 #include <algorithm>
 #include <cmath>
 #include <string>
@@ -28,24 +37,56 @@ template <class R> __device__ __forceinline__ void expi(float a, Cx<R> &e);
 template <> __device__ __forceinline__ void expi<float>(float a, Cx<float> &e) { float s, c; sincosf(a, &s, &c); e = {c, s}; }
 template <> __device__ __forceinline__ void expi<double>(float a, Cx<double> &e) { double s, c; sincos((double)a, &s, &c); e = {c, s}; }
 
-// One backward step on the torus, one thread per site.
+// An arc of a cycle of n sites: [a, a + w) modulo n.
+struct Arc {
+    int64_t a, w;
+};
+__host__ __device__ inline bool arc_has(const Arc &r, int64_t x, int64_t n) {
+    const int64_t d = x - r.a;
+    return (d >= 0 ? d : d + n) < r.w;
+}
+// r widened by k sites on each side
+static Arc arc_widen(Arc r, int64_t k, int64_t n) {
+    if (r.w + 2 * k >= n) return {0, n};
+    return {((r.a - k) % n + n) % n, r.w + 2 * k};
+}
+// one arc that covers the intersection of p and q (w = 0: they do not meet)
+static Arc arc_cover(const Arc &p, const Arc &q, int64_t n) {
+    if (p.w >= n) return q;
+    if (q.w >= n) return p;
+    const bool qp = arc_has(p, q.a, n), pq = arc_has(q, p.a, n);
+    if (qp && pq && p.a != q.a) return p.w < q.w ? p : q;   // they may meet at both ends
+    if (qp) { const int64_t d = (q.a - p.a + n) % n; return {q.a, std::min(q.w, p.w - d)}; }
+    if (pq) { const int64_t d = (p.a - q.a + n) % n; return {p.a, std::min(p.w, q.w - d)}; }
+    return {0, 0};
+}
+
+// Where one backward step runs: the sites of the launch (cx, cy), those whose
+// psi_t is wanted (inside px, py and rx, ry), and those whose lambda_t and
+// gradient term are (also inside lx, ly).
+struct BackBox {
+    Arc cx, cy, px, py, rx, ry, lx, ly;
+};
+
+// One backward step on the torus, one thread per site of the launch's box.
+constexpr int BACK_X = 64, BACK_Y = 4;
 template <int P, int FF, int GROVER>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(BACK_X *BACK_Y)
 k_backward2d(View lam_in, View psi_in, View lam_out, View psi_out, int64_t nx, int64_t ny,
-             CoinP<typename St<P>::real> cp, const float *__restrict__ phi, typename St<P>::real *__restrict__ gseg) {
+             CoinP<typename St<P>::real> cp, const float *__restrict__ phi, typename St<P>::real *__restrict__ gseg, BackBox box) {
     using real = typename St<P>::real;
     using S = St<P>;
     using C = Cx<real>;
-    const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (v >= nx * ny) return;
-    int64_t x, y;
-    if (nx * ny < (int64_t(1) << 31)) {   // 32-bit division where it fits (uniform branch)
-        x = (int)v % (int)nx;
-        y = (int)v / (int)nx;
-    } else {
-        x = v % nx;
-        y = v / nx;
-    }
+    const int64_t ix = (int64_t)blockIdx.x * BACK_X + threadIdx.x;
+    if (ix >= box.cx.w) return;
+    int64_t x = box.cx.a + ix;
+    if (x >= nx) x -= nx;
+    for (int64_t iy = (int64_t)blockIdx.y * BACK_Y + threadIdx.y; iy < box.cy.w; iy += (int64_t)gridDim.y * BACK_Y) {
+    int64_t y = box.cy.a + iy;
+    if (y >= ny) y -= ny;
+    if (!(arc_has(box.px, x, nx) && arc_has(box.rx, x, nx) && arc_has(box.py, y, ny) && arc_has(box.ry, y, ny))) continue;
+    const bool lit = arc_has(box.lx, x, nx) && arc_has(box.ly, y, ny);
+    const int64_t v = y * nx + x;
     const int64_t xp = x + 1 == nx ? 0 : x + 1, xm = x == 0 ? nx - 1 : x - 1;
     const int64_t yp = y + 1 == ny ? 0 : y + 1, ym = y == 0 ? ny - 1 : y - 1;
     // S^dagger: field_c(v) <- field_{src c}(v + e_c); e_0 = +x, e_1 = -x, e_2 = +y, e_3 = -y
@@ -54,7 +95,7 @@ k_backward2d(View lam_in, View psi_in, View lam_out, View psi_out, int64_t nx, i
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
         const int pc = FF ? (c ^ 1) : c;
-        mu[c] = S::ld(lam_in, pc, src[c]);
+        mu[c] = lit ? S::ld(lam_in, pc, src[c]) : czero<real>();
         nu[c] = S::ld(psi_in, pc, src[c]);
     }
     // a = B^dagger mu, b = B^dagger nu
@@ -92,11 +133,14 @@ k_backward2d(View lam_in, View psi_in, View lam_out, View psi_out, int64_t nx, i
         g[k] = (a[k].im * b[k].re - a[k].re * b[k].im) * (real)2;
         C e;
         expi<real>(pk[k], e);
-        S::st(lam_out, k, v, conjmul(e, a[k]));
+        if (lit) S::st(lam_out, k, v, conjmul(e, a[k]));
         S::st(psi_out, k, v, conjmul(e, b[k]));
     }
+    if (lit) {
 #pragma unroll
-    for (int k = 0; k < 4; ++k) gseg[4 * v + k] += g[k];
+        for (int k = 0; k < 4; ++k) gseg[4 * v + k] += g[k];
+    }
+    }
 }
 
 // grad += gseg (double), gseg = 0: the end of one segment of the adjoint sweep.
@@ -108,23 +152,20 @@ __global__ void k_flush_segment(R *__restrict__ gseg, double *__restrict__ grad,
     gseg[i] = (R)0;
 }
 
-// lambda_T = 1_R psi_T, and per-block partial sums of |psi_T|^2 over R.
+// lambda_T = psi_T on the region (lam is zero elsewhere already), and per-block
+// partial sums of |psi_T|^2 over it.
 template <int P>
 __global__ void __launch_bounds__(256)
-k_seed_region(View psi, View lam, int64_t nx, int64_t ny, int64_t rx, int64_t ry, int64_t rw, int64_t rh,
-              double *partials) {
+k_seed_region(View psi, View lam, int64_t nx, int64_t rx, int64_t ry, int64_t rw, int64_t rh, double *partials) {
     using S = St<P>;
     __shared__ double sh[8];
     double acc = 0.0;
-    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < nx * ny;
-         v += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t x = v % nx, y = v / nx;
-        const bool in = x >= rx && x < rx + rw && y >= ry && y < ry + rh;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < rw * rh; i += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t r = i / rw, v = (ry + r) * nx + rx + (i - r * rw);
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
-            auto z = S::ld(psi, c, v);
-            if (in) acc += norm2d(z);
-            else z = czero<typename S::real>();
+            const auto z = S::ld(psi, c, v);
+            acc += norm2d(z);
             S::st(lam, c, v, z);
         }
     }
@@ -134,7 +175,7 @@ k_seed_region(View psi, View lam, int64_t nx, int64_t ny, int64_t rx, int64_t ry
     __syncthreads();
     if (threadIdx.x == 0) {
         double b = 0.0;
-        for (int i = 0; i < (int)(blockDim.x >> 5); ++i) b += sh[i];
+        for (int i = 0; i < 8; ++i) b += sh[i];
         partials[blockIdx.x] = b;
     }
 }
@@ -149,17 +190,17 @@ __global__ void k_sum_blocks(const double *partials, int n, double *out) {
 
 template <int P>
 static cudaError_t backward_step(const qw_walk *w, View lam_in, View psi_in, View lam_out, View psi_out,
-                                 void *gseg_v) {
+                                 void *gseg_v, const BackBox &box) {
     auto *gseg = static_cast<typename St<P>::real *>(gseg_v);
     const auto &cp = *reinterpret_cast<const CoinP<typename St<P>::real> *>(w->coinp);
-    const unsigned blocks = (unsigned)((w->ns + 255) / 256);
+    const dim3 grid((unsigned)((box.cx.w + BACK_X - 1) / BACK_X), (unsigned)std::min<int64_t>(65535, (box.cy.w + BACK_Y - 1) / BACK_Y));
     bool grover = true;
     for (int r = 0; r < 4; ++r)
         for (int c = 0; c < 4; ++c)
             grover = grover && w->coin_host[2 * (4 * r + c)] == (r == c ? -0.5 : 0.5) &&
                      w->coin_host[2 * (4 * r + c) + 1] == 0.0;
     const bool ff = w->shift == QW_SHIFT_FLIPFLOP;
-#define QW_BWD(FFV, GV) k_backward2d<P, FFV, GV><<<blocks, 256, 0, w->stream>>>(lam_in, psi_in, lam_out, psi_out, w->nx, w->ny, cp, w->phi_dev, gseg)
+#define QW_BWD(FFV, GV) k_backward2d<P, FFV, GV><<<grid, dim3(BACK_X, BACK_Y), 0, w->stream>>>(lam_in, psi_in, lam_out, psi_out, w->nx, w->ny, cp, w->phi_dev, gseg, box)
     if (ff) { if (grover) QW_BWD(1, 1); else QW_BWD(1, 0); }
     else { if (grover) QW_BWD(0, 1); else QW_BWD(0, 0); }
 #undef QW_BWD
@@ -202,6 +243,13 @@ extern "C" qw_status qw_backward(qw_walk *w, const int64_t rect[4], int64_t T, i
     double *grad = on_device ? grad_phi : reinterpret_cast<double *>(base + (nseg + 3) * sb);
     void *gseg = base + (nseg + 3) * sb + (on_device ? 0 : gbytes);
 
+    // the start's support, if it is known (else the whole torus)
+    qw_status rs = resolve_support(w);
+    if (rs != QW_OK) return rs;
+    const bool known = w->sup_mode == 2;
+    const Arc psi_x = known ? Arc{w->bx0, w->bw} : Arc{0, w->nx}, psi_y = known ? Arc{w->by0, w->bh} : Arc{0, w->ny};
+    const Arc reg_x{rect[0], rect[2]}, reg_y{rect[1], rect[3]};
+
     // forward with a checkpoint every K steps
     e = cudaMemcpyAsync(ckpt(0).p, w->buf[w->cur], sb, cudaMemcpyDeviceToDevice, w->stream);
     if (e != cudaSuccess) return cuda_error(w, e, "checkpoint");
@@ -212,12 +260,14 @@ extern "C" qw_status qw_backward(qw_walk *w, const int64_t rect[4], int64_t T, i
             return cuda_error(w, e, "checkpoint");
     }
 
-    // lambda_T and the loss
+    // lambda_T and the loss; lambda is only ever written inside its light cone,
+    // so both of its buffers start as zero
     const int nb = marginal_blocks();
+    if ((e = cudaMemsetAsync(lam[0].p, 0, 2 * sb, w->stream)) != cudaSuccess) return cuda_error(w, e, "adjoint clear");
     if (w->prec == QW_F32)
-        k_seed_region<P_F32><<<nb, 256, 0, w->stream>>>(ckpt(nseg), lam[0], w->nx, w->ny, rect[0], rect[1], rect[2], rect[3], w->partials);
+        k_seed_region<P_F32><<<nb, 256, 0, w->stream>>>(ckpt(nseg), lam[0], w->nx, rect[0], rect[1], rect[2], rect[3], w->partials);
     else
-        k_seed_region<P_F64><<<nb, 256, 0, w->stream>>>(ckpt(nseg), lam[0], w->nx, w->ny, rect[0], rect[1], rect[2], rect[3], w->partials);
+        k_seed_region<P_F64><<<nb, 256, 0, w->stream>>>(ckpt(nseg), lam[0], w->nx, rect[0], rect[1], rect[2], rect[3], w->partials);
     k_sum_blocks<<<1, 32, 0, w->stream>>>(w->partials, nb, w->norm_dev);
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_error(w, e, "region seed");
     if ((e = cudaMemsetAsync(grad, 0, gbytes, w->stream)) != cudaSuccess) return cuda_error(w, e, "gradient clear");
@@ -231,8 +281,18 @@ extern "C" qw_status qw_backward(qw_walk *w, const int64_t rect[4], int64_t T, i
         int pi = 0;
         for (int64_t t = t_hi - 1; t >= t_lo; --t) {
             View psi_out = view_of(w, pi);
-            e = w->prec == QW_F32 ? backward_step<P_F32>(w, lam[li], psi_in, lam[li ^ 1], psi_out, gseg)
-                                  : backward_step<P_F64>(w, lam[li], psi_in, lam[li ^ 1], psi_out, gseg);
+            BackBox box;
+            box.px = arc_widen(psi_x, t, w->nx); box.py = arc_widen(psi_y, t, w->ny);
+            box.lx = arc_widen(reg_x, T - t, w->nx); box.ly = arc_widen(reg_y, T - t, w->ny);
+            box.rx = arc_widen(reg_x, (T - t_lo) + (t - t_lo), w->nx);
+            box.ry = arc_widen(reg_y, (T - t_lo) + (t - t_lo), w->ny);
+            box.cx = arc_cover(box.px, box.rx, w->nx); box.cy = arc_cover(box.py, box.ry, w->ny);
+            if (box.cx.w <= 0 || box.cy.w <= 0) {   // no site matters any more at this time or before
+                li ^= 1; psi_in = psi_out; pi ^= 1;
+                continue;
+            }
+            e = w->prec == QW_F32 ? backward_step<P_F32>(w, lam[li], psi_in, lam[li ^ 1], psi_out, gseg, box)
+                                  : backward_step<P_F64>(w, lam[li], psi_in, lam[li ^ 1], psi_out, gseg, box);
             if (e != cudaSuccess) return cuda_error(w, e, "backward step");
             li ^= 1;
             psi_in = psi_out;

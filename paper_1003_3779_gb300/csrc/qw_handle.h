@@ -145,6 +145,9 @@ inline View next_view(const qw_walk *w) { return view_of(w, w->cur ^ 1); }
 // the other buffer and flips w->cur; used by qw_step and the adjoint.
 qw_status run_steps(qw_walk *w, int64_t T, int adj);
 
+// Takes the box that qw_set_state searched (waits for the search).
+qw_status resolve_support(qw_walk *w);
+
 // Launch helpers implemented in the per-precision translation units.
 cudaError_t launch_step1d_f32(const Step1DArgs &, const void *, int, cudaStream_t);
 cudaError_t launch_step1d_f64(const Step1DArgs &, const void *, int, cudaStream_t);
