@@ -14,18 +14,6 @@
 
 namespace qw {
 
-struct GenGeom {
-    int ndim;
-    int64_t nx, ny, ns;
-    int shift, bc;
-    const uint8_t *links;
-    uint32_t rthr, rk0, rk1, rstep;   // links broken at random at this step (rthr 0: none)
-    // tiled kernels: block (bx, by) runs tile ((tx0 + bx) mod ntx, (ty0 + by) mod nty)
-    // of the ntx x nty tiles of the lattice (all of them, or those around the
-    // light-cone window of a localised state)
-    int tx0, ntx, ty0, nty;
-};
-
 // Words 0 and 1 of Philox4x32 with 10 rounds (Salmon, Moraes, Dror and Shaw, SC
 // 2011) for counter (c0, c1, c2, c3) and key (k0, k1): each round multiplies c0
 // and c2 by 0xD2511F53 and 0xCD9E8D57 and mixes the product halves with c1, c3

@@ -140,6 +140,8 @@ static void tiles_of(int prec, int &a, int &b) {
     else { a = 8; b = 16; }
 }
 
+static bool tile2d_walk(const qw_walk *w);
+
 static void default_plan(const qw_walk *w, int &k, int &tile, int &variant) {
     variant = 0;
     if (w->ndim == 2) {
@@ -149,7 +151,8 @@ static void default_plan(const qw_walk *w, int &k, int &tile, int &variant) {
         tile = 0;
         k = 1;
         if (w->bc != QW_BC_PERIODIC || links_on(w) || w->nx < 32 || w->ny < 32) return;
-        if (step2d_tb_ok(w->prec, w->kind, 8, w->shift)) k = 8;
+        // Phase coins run in tiles: 300 x 200 1.4 / 8.3, 1024^2 8.1 / 16.7 (k = 4: 9.3)
+        if (step2d_tb_ok(w->prec, w->kind, 8, w->shift) || tile2d_walk(w)) k = 8;
         return;
     }
     switch (w->prec) {
@@ -370,7 +373,7 @@ static qw_status queue_support(qw_walk *w, const void *src = nullptr) {
 }
 
 // Take the searched box (waits for the search only, not for later work).
-qw_status resolve_support(qw_walk *w) {
+static qw_status resolve_support(qw_walk *w) {
     if (w->sup_mode != 1) return QW_OK;
     w->sup_mode = 0;
     if (capturing(w)) { (void)cudaGetLastError(); return QW_OK; }   // step in full
@@ -384,6 +387,21 @@ qw_status resolve_support(qw_walk *w) {
     if (w->bh >= w->ny) { w->by0 = 0; w->bh = w->ny; }
     w->sup_mode = (w->bw < w->nx || w->bh < w->ny) ? 2 : 0;
     return QW_OK;
+}
+
+qw_status start_support(qw_walk *w, SupportBox &box) {
+    const bool on = w->clip_on;
+    qw_status st = QW_OK;
+    if (!on) {
+        w->clip_on = true;
+        st = queue_support(w);
+        w->clip_on = false;
+    }
+    if (st == QW_OK) st = resolve_support(w);
+    box = {0, 0, 0, 0, w->nx, w->ny};
+    if (w->sup_mode == 2) box = {w->bx0, w->bw, w->by0, w->bh, w->nx, w->ny};
+    if (!on) w->sup_mode = 0;
+    return st;
 }
 
 // The box after K more steps: one site more on each side per step, modulo the
@@ -518,6 +536,54 @@ static qw_status run_spectral(qw_walk *w, int64_t T, int adj) {
     return QW_OK;
 }
 
+// ---------------------------------------------------------------- 2D tiles
+// Steps per launch with links or edges: more steps re-read less, but leave a
+// smaller share of the tile as output.  Per step at p = 0.05, 1 (a launch per
+// step) / 4 / 5 / 6 / 8: 300 x 200 6.2 / 2.1 / 2.1 / 1.8 / 2.1 us, 1024^2 14.4 /
+// 11.8 / 11.2 / 10.6 / 12.6, 2048 x 1500 40.6 / 29.7 / 28.0 / 28.7 / 31.8, 4096^2
+// 188 / 146 / 144 / 143 / 156.
+constexpr int TILE2D_LINK_STEPS = 6;
+// Largest output box that takes tiles where the streaming kernel runs too: at
+// k = 8, tiles / streaming, 300 x 200 1.34 / 1.87 us per step, 512^2 2.08 / 2.32,
+// 1024^2 6.4 / 3.9 (shared memory against registers).
+constexpr int64_t TILE2D_SITES = 300000;
+// Does the tile kernel (k_tile2d.cuh) run this walk's forward steps?
+static bool tile2d_walk(const qw_walk *w) {
+    return w->ndim == 2 && w->prec == QW_F32 && w->kind != CK_PERSITE && w->nx < (int64_t(1) << 30) &&
+           w->ny < (int64_t(1) << 18) && w->ns < (int64_t(1) << 32) &&
+           !(w->shift == QW_SHIFT_DIAGONAL && (w->bc != QW_BC_PERIODIC || links_on(w)));
+}
+
+// The outputs of K steps along an axis of n sites: the support [b0, b0 + bw)
+// widened by K (modulo n, or cut at the ends); clip = false: the whole axis.
+static void output_range(bool clip, int64_t b0, int64_t bw, int64_t n, int K, bool periodic, int64_t &o0, int64_t &ow) {
+    o0 = 0; ow = n;
+    if (!clip) return;
+    int64_t a = b0, l = bw;
+    grow_axis(a, l, n, K, periodic);
+    o0 = a; ow = l;
+}
+
+static void tile2d_box(const qw_walk *w, int K, Tile2DArgs &a) {
+    const bool per = w->bc == QW_BC_PERIODIC, clip = w->sup_mode == 2;
+    output_range(clip, w->bx0, w->bw, w->nx, K, per, a.ox0, a.ow);
+    output_range(clip, w->by0, w->bh, w->ny, K, per, a.oy0, a.oh);
+}
+
+// One launch of K steps from the current buffer to the other (links: broken
+// links or an edge, whose random draws start at rstep).
+static cudaError_t tile2d_launch(qw_walk *w, int K, bool links, uint32_t rstep, double gain) {
+    Tile2DArgs a{};
+    a.in = cur_view(w); a.out = next_view(w);
+    a.g = GenGeom{2, w->nx, w->ny, w->ns, w->shift, w->bc, w->has_links ? w->links_dev : nullptr, w->link_thr,
+                  (uint32_t)w->link_seed, (uint32_t)(w->link_seed >> 32), rstep, 0, 1, 0, 1};
+    a.K = K; a.gain = gain;
+    const bool phase = w->kind == CK_PHASE;
+    a.phi = phase ? w->phi_dev : nullptr;
+    tile2d_box(w, K, a);
+    return launch_tile2d(w->shift, phase ? w->base_kind : w->kind, links, a, w->coinp, w->stream);
+}
+
 qw_status run_steps(qw_walk *w, int64_t T, int adj) {
     if (T < 0) return set_error(w, QW_EINVAL, "T must be >= 0");
     if (T == 0) return QW_OK;
@@ -548,7 +614,19 @@ qw_status run_steps(qw_walk *w, int64_t T, int adj) {
         const bool win_ok = w->ndim == 1 && !adj && w->bc != QW_BC_PERIODIC &&
                             (w->shift == QW_SHIFT_MOVING || w->shift == QW_SHIFT_FLIPFLOP) && w->nx < (int64_t(1) << 30);
         const int64_t win_cap = win_ok ? window_capacity(w->prec) : 0;
+        const bool tiles = !adj && tile2d_walk(w);
         for (int64_t t = 0; t < T; ++t) {
+            if (tiles) {
+                const int k = (int)std::min<int64_t>(TILE2D_LINK_STEPS, T - t);
+                const double gain = drift_gain(w, k, t + k == T);
+                if ((e = tile2d_launch(w, k, true, (uint32_t)w->link_step, gain)) != cudaSuccess)
+                    return cuda_error(w, e, "tile step launch");
+                if (w->link_thr) w->link_step += k;
+                grow_support(w, k);
+                w->cur ^= 1;
+                t += k - 1;
+                continue;
+            }
             if (win_ok && w->sup_mode == 2) {
                 int ns = (int)std::min<int64_t>(T - t, WINDOW_MAX_STEPS);
                 auto width = [&](int k) {
@@ -638,20 +716,34 @@ qw_status run_steps(qw_walk *w, int64_t T, int adj) {
     };
     int K2, t2;
     effective_plan(w, K2, t2);
-    if (!adj && K2 > 1 && step2d_tb_ok(w->prec, w->kind, K2, w->shift)) {
-        // whole blocks of K2 steps in the streaming kernel, then one of 4, the rest
-        // one step at a time
-        Step2DArgs b = a;
-        b.K = K2;
-        while (T >= K2 || (T >= 4 && step2d_tb_ok(w->prec, w->kind, 4, w->shift))) {
-            if (T < K2) b.K = K2 = 4;
-            b.gain = drift_gain(w, K2, T - K2 == 0);   // applied once, to the launch's output
-            b.in = cur_view(w); b.out = next_view(w);
-            set_box(b);
-            if ((e = launch_step2d_tb(b, cp, w->stream)) != cudaSuccess) return cuda_error(w, e, "2D blocked step launch");
-            grow_support(w, K2);
+    if (!adj && K2 > 1) {
+        // K2 steps per launch: tiles on small boxes and for the coins the streaming
+        // kernel does not run, else the streaming kernel, whose remainders of 4 to
+        // 7 steps take a launch of 4
+        const bool tile = tile2d_walk(w);
+        while (T > 0) {
+            int k = (int)std::min<int64_t>(K2, T);
+            const int kt = k >= 8 ? 8 : 4;
+            const bool tb = k >= 4 && step2d_tb_ok(w->prec, w->kind, kt, w->shift);
+            Tile2DArgs box{};
+            tile2d_box(w, k, box);
+            const bool use_tile = tile && (!tb || box.ow * box.oh <= TILE2D_SITES);
+            if (!use_tile && !tb) break;
+            if (!use_tile) k = kt;
+            const double gain = drift_gain(w, k, T - k == 0);   // applied once, to the launch's output
+            if (use_tile) {
+                e = tile2d_launch(w, k, false, 0, gain);
+            } else {
+                Step2DArgs b = a;
+                b.K = k; b.gain = gain;
+                b.in = cur_view(w); b.out = next_view(w);
+                set_box(b);
+                e = launch_step2d_tb(b, cp, w->stream);
+            }
+            if (e != cudaSuccess) return cuda_error(w, e, "2D blocked step launch");
+            grow_support(w, k);
             w->cur ^= 1;
-            T -= K2;
+            T -= k;
         }
     }
     for (int64_t t = 0; t < T; ++t) {
@@ -829,6 +921,7 @@ qw_status qw_set_coin_phases(qw_walk *w, const double *base, const float *phi, i
     if (e != cudaSuccess) return cuda_error(w, e, "phase copy");
     apply_global_coin(w, base);   // the kernels read the base coin from here
     if (w->ndim == 2) {
+        w->base_kind = w->kind;
         w->kind = CK_PHASE;
         return QW_OK;
     }

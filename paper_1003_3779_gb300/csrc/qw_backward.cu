@@ -243,11 +243,12 @@ extern "C" qw_status qw_backward(qw_walk *w, const int64_t rect[4], int64_t T, i
     double *grad = on_device ? grad_phi : reinterpret_cast<double *>(base + (nseg + 3) * sb);
     void *gseg = base + (nseg + 3) * sb + (on_device ? 0 : gbytes);
 
-    // the start's support, if it is known (else the whole torus)
-    qw_status rs = resolve_support(w);
+    // the start's support (the whole torus if nothing is known), searched here
+    // when the steps are not clipped: the sweep's sites do not depend on that
+    SupportBox start;
+    qw_status rs = start_support(w, start);
     if (rs != QW_OK) return rs;
-    const bool known = w->sup_mode == 2;
-    const Arc psi_x = known ? Arc{w->bx0, w->bw} : Arc{0, w->nx}, psi_y = known ? Arc{w->by0, w->bh} : Arc{0, w->ny};
+    const Arc psi_x = start.w ? Arc{start.x0, start.w} : Arc{0, w->nx}, psi_y = start.w ? Arc{start.y0, start.h} : Arc{0, w->ny};
     const Arc reg_x{rect[0], rect[2]}, reg_y{rect[1], rect[3]};
 
     // forward with a checkpoint every K steps

@@ -22,6 +22,7 @@ struct qw_walk {
 
     // coin
     int kind = qw::CK_REAL;
+    int base_kind = qw::CK_REAL;           // CK_PHASE on the torus: the class of the base coin
     double coin_host[32] = {0};            // global / base coin, row-major complex
     double coin_alpha = 1.0;               // sqrt(tr(C_f^dagger C_f) / d) of the rounded coin
     // Hadamard-class coin lambda * diag(a, c) H diag(1, s) (1D moving shift)
@@ -145,8 +146,9 @@ inline View next_view(const qw_walk *w) { return view_of(w, w->cur ^ 1); }
 // the other buffer and flips w->cur; used by qw_step and the adjoint.
 qw_status run_steps(qw_walk *w, int64_t T, int adj);
 
-// Takes the box that qw_set_state searched (waits for the search).
-qw_status resolve_support(qw_walk *w);
+// The support box of the current state (w = 0: the whole lattice, or not known):
+// the one the clipped steps track, or, with clipping off, one searched now.
+qw_status start_support(qw_walk *w, SupportBox &box);
 
 // Launch helpers implemented in the per-precision translation units.
 cudaError_t launch_step1d_f32(const Step1DArgs &, const void *, int, cudaStream_t);
@@ -193,6 +195,10 @@ size_t spectral1d_table_bytes(int prec);
 cudaError_t launch_spectral1d_twiddles(int prec, int tile, void *table, cudaStream_t s);
 cudaError_t launch_spectral1d_matrices(int prec, const Spec1DArgs &a, const double *coin, double scale, cudaStream_t s);
 cudaError_t launch_spectral1d(int prec, const Spec1DArgs &a, cudaStream_t s);
+
+// K steps in shared-memory tiles (tile2d.cu, FP32); kind: the global coin, or
+// with a.phi the base coin of the phases; links: broken links or an edge
+cudaError_t launch_tile2d(int shift, int kind, bool links, const Tile2DArgs &a, const void *coinp, cudaStream_t s);
 
 // per-site coin conversion kernels (qw_coins.cu)
 cudaError_t launch_convert_coins(int prec, const double *src, void *dst, int64_t count, cudaStream_t s);

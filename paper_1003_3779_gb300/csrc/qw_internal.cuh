@@ -402,6 +402,31 @@ struct SupportBox {
     int64_t x0, w, y0, h, nx, ny;
 };
 
+// lattice, boundary and links of the generic kernels
+struct GenGeom {
+    int ndim;
+    int64_t nx, ny, ns;
+    int shift, bc;
+    const uint8_t *links;
+    uint32_t rthr, rk0, rk1, rstep;   // links broken at random at this step (rthr 0: none)
+    // tiled kernels: block (bx, by) runs tile ((tx0 + bx) mod ntx, (ty0 + by) mod nty)
+    // of the ntx x nty tiles of the lattice (all of them, or those around the
+    // light-cone window of a localised state)
+    int tx0, ntx, ty0, nty;
+};
+
+// K steps of a 2D walk in shared-memory tiles (k_tile2d.cuh)
+constexpr int TILE2D_MAX_STEPS = 12;
+struct Tile2DArgs {
+    View in, out;
+    GenGeom g;                      // lattice, boundary, links; rstep: of the first step
+    int64_t ox0, ow, oy0, oh;       // output box, modulo the lattice
+    int K;
+    const float *phi;
+    double gain;                    // factor of the launch's output
+};
+
+
 // marginals + norm
 cudaError_t launch_marginals(int prec, View v, int64_t nsites, void *P, int p_f32,
                              double *partials, int nblocks, double *norm_dev, const SupportBox &box, cudaStream_t s);
