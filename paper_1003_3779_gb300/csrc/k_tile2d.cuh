@@ -111,8 +111,11 @@ k_tile2d(View in, View out, GenGeom g, int64_t ox0, int64_t ow, int64_t oy0, int
     const int TX = EX - 2 * K, TY = EY - 2 * K;
     // the tile's first site (wrapped); its site (i, j) is lattice site (x0 + i, y0 + j)
     const int64_t bx = (int64_t)blockIdx.x * TX, by = (int64_t)blockIdx.y * TY;
-    auto wrap = [](int64_t a, int64_t n) { a %= n; return a < 0 ? a + n : a; };
-    const int64_t x0 = wrap(ox0 + bx - K, g.nx), y0 = wrap(oy0 + by - K, g.ny);
+    auto wrap = [](int64_t a, int64_t n, int e) {   // a is at most one period outside [0, n) where n >= e
+        if (n < e) a %= n;
+        return a < 0 ? a + n : (a >= n ? a - n : a);
+    };
+    const int64_t x0 = wrap(ox0 + bx - K, g.nx, EX), y0 = wrap(oy0 + by - K, g.ny, EY);
     const int i = (int)threadIdx.x % EX, j0 = (int)threadIdx.x / EX;   // site n of this thread: (i, j0 + n TH / EX)
     constexpr int DJ = TH / EX;
     int64_t gx = x0 + i;

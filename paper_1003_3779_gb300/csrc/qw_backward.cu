@@ -30,6 +30,7 @@
 #include <string>
 
 #include "qw_handle.h"
+#include "k_step2d.cuh"
 
 namespace qw {
 
@@ -41,7 +42,7 @@ template <> __device__ __forceinline__ void expi<double>(float a, Cx<double> &e)
 struct Arc {
     int64_t a, w;
 };
-__host__ __device__ inline bool arc_has(const Arc &r, int64_t x, int64_t n) {
+static bool arc_has(const Arc &r, int64_t x, int64_t n) {
     const int64_t d = x - r.a;
     return (d >= 0 ? d : d + n) < r.w;
 }
@@ -60,86 +61,167 @@ static Arc arc_cover(const Arc &p, const Arc &q, int64_t n) {
     if (pq) { const int64_t d = (p.a - q.a + n) % n; return {p.a, std::min(p.w, q.w - d)}; }
     return {0, 0};
 }
+// how far x lies outside the arc: x is in the arc widened by k if and only if
+// this is at most k
+__device__ __forceinline__ int64_t arc_distance(const Arc &r, int64_t x, int64_t n) {
+    int64_t d = x - r.a;
+    if (d < 0) d += n;
+    return d < r.w ? 0 : min(d - r.w + 1, n - d);
+}
 
-// Where one backward step runs: the sites of the launch (cx, cy), those whose
-// psi_t is wanted (inside px, py and rx, ry), and those whose lambda_t and
-// gradient term are (also inside lx, ly).
-struct BackBox {
-    Arc cx, cy, px, py, rx, ry, lx, ly;
+// One launch of K backward steps, t0 + K -> t0.
+struct BackArgs {
+    View lam_in, psi_in, lam_out, psi_out;
+    int64_t nx, ny;
+    int64_t cx, cw, cy, ch;          // the box of output sites (a cover of those that matter)
+    Arc psi_x, psi_y, reg_x, reg_y;  // the start's support and the region
+    int64_t t0, T, reach;            // psi_t0 is wanted up to `reach` sites from the region
+    int K;
+    const float *phi;
+    void *gseg;
 };
 
-// One backward step on the torus, one thread per site of the launch's box.
-constexpr int BACK_X = 64, BACK_Y = 4;
+// Slot of plane c in the in-place update (k_tile2d.cuh), backward: the step from
+// s to s + 1 steps before the launch's start reads plane c (flip-flop: c xor 1)
+// at v + e_c, and plane c of v is written to the slot that was read.
+template <int FF> __device__ __forceinline__ void back_slot(int c, int s, int &track, int &dx, int &dy) {
+    const int k = FF ? (s & 1 ? 0 : 1) : s + 1;
+    track = FF && !(s & 1) ? c ^ 1 : c;
+    dx = k * dir_dx<0>(c);
+    dy = k * dir_dy<0>(c);
+}
+
+// K backward steps in a tile of both fields in shared memory: one launch, one
+// read of the phases (and their sines) and one update of the accumulator per K
+// steps.  On the workload above the sweep took 512 launches of 4.0 us (6.2 us
+// with the gaps between them), now 83 of 16 us.  64 registers a thread (a few
+// spilled) for two CTAs per SM: 26 -> 16 us per launch.  What bounds it: latency
+// for narrow windows, 128 bytes of shared memory per site and step for wide ones.
+// Largest box that takes 8 steps per launch rather than 4; the whole gradient of
+// the workload above at 0 / 40000 / 70000 / 120000 / no limit: 4.28 / 4.19 / 4.17
+// / 4.12 / 4.24 ms.
+constexpr int64_t BACK_DEEP_SITES = 120000;
+constexpr int BACK_E = 32, BACK_TH = 512, BACK_NS = BACK_E * BACK_E / BACK_TH;   // tile, threads, sites per thread
 template <int P, int FF, int GROVER>
-__global__ void __launch_bounds__(BACK_X *BACK_Y)
-k_backward2d(View lam_in, View psi_in, View lam_out, View psi_out, int64_t nx, int64_t ny,
-             CoinP<typename St<P>::real> cp, const float *__restrict__ phi, typename St<P>::real *__restrict__ gseg, BackBox box) {
+__global__ void __launch_bounds__(BACK_TH, P == P_F32 ? 2 : 1)
+k_backward2d(BackArgs a, CoinP<typename St<P>::real> cp) {
     using real = typename St<P>::real;
     using S = St<P>;
     using C = Cx<real>;
-    const int64_t ix = (int64_t)blockIdx.x * BACK_X + threadIdx.x;
-    if (ix >= box.cx.w) return;
-    int64_t x = box.cx.a + ix;
-    if (x >= nx) x -= nx;
-    for (int64_t iy = (int64_t)blockIdx.y * BACK_Y + threadIdx.y; iy < box.cy.w; iy += (int64_t)gridDim.y * BACK_Y) {
-    int64_t y = box.cy.a + iy;
-    if (y >= ny) y -= ny;
-    if (!(arc_has(box.px, x, nx) && arc_has(box.rx, x, nx) && arc_has(box.py, y, ny) && arc_has(box.ry, y, ny))) continue;
-    const bool lit = arc_has(box.lx, x, nx) && arc_has(box.ly, y, ny);
-    const int64_t v = y * nx + x;
-    const int64_t xp = x + 1 == nx ? 0 : x + 1, xm = x == 0 ? nx - 1 : x - 1;
-    const int64_t yp = y + 1 == ny ? 0 : y + 1, ym = y == 0 ? ny - 1 : y - 1;
-    // S^dagger: field_c(v) <- field_{src c}(v + e_c); e_0 = +x, e_1 = -x, e_2 = +y, e_3 = -y
-    const int64_t src[4] = {y * nx + xp, y * nx + xm, yp * nx + x, ym * nx + x};
-    C mu[4], nu[4];
+    struct alignas(2 * sizeof(real)) Slot { real re, im; };
+    constexpr int E = BACK_E, M = E - 1;
+    extern __shared__ __align__(16) unsigned char bsm[];
+    Slot *lam = reinterpret_cast<Slot *>(bsm), *psi = lam + 4 * E * E;   // [track][y][x]
+    const int O = E - 2 * a.K;
+    auto wrap = [](int64_t q, int64_t n) {   // q is at most about a period outside [0, n): no division
+        while (q < 0) q += n;
+        while (q >= n) q -= n;
+        return q;
+    };
+    const int64_t bx = (int64_t)blockIdx.x * O - a.K, by = (int64_t)blockIdx.y * O - a.K;
+    const int i = (int)threadIdx.x % E, j0 = (int)threadIdx.x / E;
+    const int64_t x = wrap(a.cx + bx + i, a.nx);
+    const int64_t far_x = arc_distance(a.psi_x, x, a.nx), near_x = arc_distance(a.reg_x, x, a.nx);
+    C e[BACK_NS][4];
+    real g[BACK_NS][4];
+    int64_t v[BACK_NS];
+    int far[BACK_NS], near[BACK_NS];
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-        const int pc = FF ? (c ^ 1) : c;
-        mu[c] = lit ? S::ld(lam_in, pc, src[c]) : czero<real>();
-        nu[c] = S::ld(psi_in, pc, src[c]);
-    }
-    // a = B^dagger mu, b = B^dagger nu
-    C a[4], b[4];
-    if (GROVER) {   // real symmetric: B^dagger = B = (1/2) J - I
-        C sm = cadd(cadd(mu[0], mu[1]), cadd(mu[2], mu[3]));
-        C sn = cadd(cadd(nu[0], nu[1]), cadd(nu[2], nu[3]));
-        sm = rmul(cp.re[1], sm);
-        sn = rmul(cp.re[1], sn);
+    for (int n = 0; n < BACK_NS; ++n) {
+        const int j = j0 + n * (BACK_TH / E);
+        const int64_t y = wrap(a.cy + by + j, a.ny);
+        v[n] = y * a.nx + x;
+        // distances (cut at 2^30) from the start's support and from the region
+        far[n] = (int)min((int64_t)1 << 30, max(far_x, arc_distance(a.psi_y, y, a.ny)));
+        near[n] = (int)min((int64_t)1 << 30, max(near_x, arc_distance(a.reg_y, y, a.ny)));
 #pragma unroll
-        for (int k = 0; k < 4; ++k) { a[k] = csub(sm, mu[k]); b[k] = csub(sn, nu[k]); }
-    } else {
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            C aa = conjmul(C{cp.re[k], cp.im[k]}, mu[0]);
-            C bb = conjmul(C{cp.re[k], cp.im[k]}, nu[0]);
-#pragma unroll
-            for (int r = 1; r < 4; ++r) {
-                const C br{cp.re[4 * r + k], cp.im[4 * r + k]};
-                aa = cadd(aa, conjmul(br, mu[r]));
-                bb = cadd(bb, conjmul(br, nu[r]));
-            }
-            a[k] = aa;
-            b[k] = bb;
+        for (int c = 0; c < 4; ++c) {
+            const C l = S::ld(a.lam_in, c, v[n]), p = S::ld(a.psi_in, c, v[n]);
+            lam[(c * E + j) * E + i] = {l.re, l.im};
+            psi[(c * E + j) * E + i] = {p.re, p.im};
+            g[n][c] = (real)0;
         }
-    }
-    const float4 ph = reinterpret_cast<const float4 *>(phi)[v];
-    const float pk[4] = {ph.x, ph.y, ph.z, ph.w};
-    real g[4];
+        const float4 ph = reinterpret_cast<const float4 *>(a.phi)[v[n]];
+        const float pk[4] = {ph.x, ph.y, ph.z, ph.w};
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        // -2 Im(conj(a) b) in the compute precision; the segment's running sum
-        // stays in that precision and is added into the double gradient once per
-        // segment of K steps (double arithmetic is slow on this part)
-        g[k] = (a[k].im * b[k].re - a[k].re * b[k].im) * (real)2;
-        C e;
-        expi<real>(pk[k], e);
-        if (lit) S::st(lam_out, k, v, conjmul(e, a[k]));
-        S::st(psi_out, k, v, conjmul(e, b[k]));
+        for (int c = 0; c < 4; ++c) expi<real>(pk[c], e[n][c]);
     }
-    if (lit) {
+    __syncthreads();
+    for (int s = 0; s < a.K; ++s) {
+        const int64_t t = a.t0 + a.K - 1 - s;   // this step forms time t
 #pragma unroll
-        for (int k = 0; k < 4; ++k) gseg[4 * v + k] += g[k];
+        for (int n = 0; n < BACK_NS; ++n) {
+            const int j = j0 + n * (BACK_TH / E);
+            C mu[4], nu[4];
+            int at[4];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                int tr, dx, dy;
+                back_slot<FF>(c, s, tr, dx, dy);
+                at[c] = (tr * E + ((j + dy) & M)) * E + ((i + dx) & M);
+                mu[c] = {lam[at[c]].re, lam[at[c]].im};
+                nu[c] = {psi[at[c]].re, psi[at[c]].im};
+            }
+            // p = B^dagger mu, q = B^dagger nu
+            C p[4], q[4];
+            if (GROVER) {   // real symmetric: B^dagger = B = (1/2) J - I
+                C sm = cadd(cadd(mu[0], mu[1]), cadd(mu[2], mu[3]));
+                C sn = cadd(cadd(nu[0], nu[1]), cadd(nu[2], nu[3]));
+                sm = rmul(cp.re[1], sm);
+                sn = rmul(cp.re[1], sn);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) { p[k] = csub(sm, mu[k]); q[k] = csub(sn, nu[k]); }
+            } else {
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    C aa = conjmul(C{cp.re[k], cp.im[k]}, mu[0]);
+                    C bb = conjmul(C{cp.re[k], cp.im[k]}, nu[0]);
+#pragma unroll
+                    for (int r = 1; r < 4; ++r) {
+                        const C br{cp.re[4 * r + k], cp.im[4 * r + k]};
+                        aa = cadd(aa, conjmul(br, mu[r]));
+                        bb = cadd(bb, conjmul(br, nu[r]));
+                    }
+                    p[k] = aa;
+                    q[k] = bb;
+                }
+            }
+            // the gradient term, where psi_t and lambda_t may both be nonzero
+            // (elsewhere a field is zero, or was not rebuilt).  -2 Im(conj(p) q)
+            // in the compute precision, as is the segment's running sum, which is
+            // added into the double gradient once per segment of K steps (double
+            // arithmetic is slow on this part)
+            const bool lit = far[n] <= t && near[n] <= a.T - t;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                if (lit) g[n][k] += (p[k].im * q[k].re - p[k].re * q[k].im) * (real)2;
+                const C l = conjmul(e[n][k], p[k]), w = conjmul(e[n][k], q[k]);
+                lam[at[k]] = {l.re, l.im};
+                psi[at[k]] = {w.re, w.im};
+            }
+        }
+        __syncthreads();
     }
+    if (i < a.K || i >= E - a.K || bx + i >= a.cw) return;
+#pragma unroll
+    for (int n = 0; n < BACK_NS; ++n) {
+        const int j = j0 + n * (BACK_TH / E);
+        if (j < a.K || j >= E - a.K || by + j >= a.ch) continue;
+        const bool lit = near[n] <= a.T - a.t0;
+        if (lit && far[n] < a.t0 + a.K) {
+            real *gs = static_cast<real *>(a.gseg) + 4 * v[n];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) gs[k] += g[n][k];
+        }
+        if (far[n] > a.t0 || near[n] > a.reach) continue;
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            int tr, dx, dy;
+            back_slot<FF>(c, a.K - 1, tr, dx, dy);
+            const int at = (tr * E + ((j + dy) & M)) * E + ((i + dx) & M);
+            if (lit) S::st(a.lam_out, c, v[n], C{lam[at].re, lam[at].im});
+            S::st(a.psi_out, c, v[n], C{psi[at].re, psi[at].im});
+        }
     }
 }
 
@@ -188,23 +270,28 @@ __global__ void k_sum_blocks(const double *partials, int n, double *out) {
     if (threadIdx.x == 0) *out = v;
 }
 
+template <int P> constexpr size_t back_smem() { return (size_t)2 * 4 * BACK_E * BACK_E * 2 * sizeof(typename St<P>::real); }
+
+template <int P, int FF, int GROVER>
+static cudaError_t go_backward(const qw_walk *w, const BackArgs &a) {
+    auto kern = k_backward2d<P, FF, GROVER>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)back_smem<P>());
+    if (e != cudaSuccess) return e;
+    const int O = BACK_E - 2 * a.K;
+    const dim3 grid((unsigned)((a.cw + O - 1) / O), (unsigned)((a.ch + O - 1) / O));
+    kern<<<grid, BACK_TH, back_smem<P>(), w->stream>>>(a, *reinterpret_cast<const CoinP<typename St<P>::real> *>(w->coinp));
+    return cudaGetLastError();
+}
+
 template <int P>
-static cudaError_t backward_step(const qw_walk *w, View lam_in, View psi_in, View lam_out, View psi_out,
-                                 void *gseg_v, const BackBox &box) {
-    auto *gseg = static_cast<typename St<P>::real *>(gseg_v);
-    const auto &cp = *reinterpret_cast<const CoinP<typename St<P>::real> *>(w->coinp);
-    const dim3 grid((unsigned)((box.cx.w + BACK_X - 1) / BACK_X), (unsigned)std::min<int64_t>(65535, (box.cy.w + BACK_Y - 1) / BACK_Y));
+static cudaError_t backward_steps(const qw_walk *w, const BackArgs &a) {
     bool grover = true;
     for (int r = 0; r < 4; ++r)
         for (int c = 0; c < 4; ++c)
             grover = grover && w->coin_host[2 * (4 * r + c)] == (r == c ? -0.5 : 0.5) &&
                      w->coin_host[2 * (4 * r + c) + 1] == 0.0;
-    const bool ff = w->shift == QW_SHIFT_FLIPFLOP;
-#define QW_BWD(FFV, GV) k_backward2d<P, FFV, GV><<<grid, dim3(BACK_X, BACK_Y), 0, w->stream>>>(lam_in, psi_in, lam_out, psi_out, w->nx, w->ny, cp, w->phi_dev, gseg, box)
-    if (ff) { if (grover) QW_BWD(1, 1); else QW_BWD(1, 0); }
-    else { if (grover) QW_BWD(0, 1); else QW_BWD(0, 0); }
-#undef QW_BWD
-    return cudaGetLastError();
+    if (w->shift == QW_SHIFT_FLIPFLOP) return grover ? go_backward<P, 1, 1>(w, a) : go_backward<P, 1, 0>(w, a);
+    return grover ? go_backward<P, 0, 1>(w, a) : go_backward<P, 0, 0>(w, a);
 }
 
 }  // namespace qw
@@ -280,24 +367,32 @@ extern "C" qw_status qw_backward(qw_walk *w, const int64_t rect[4], int64_t T, i
         const int64_t t_hi = std::min((s + 1) * K, T), t_lo = s * K;
         View psi_in = ckpt(s + 1);
         int pi = 0;
-        for (int64_t t = t_hi - 1; t >= t_lo; --t) {
-            View psi_out = view_of(w, pi);
-            BackBox box;
-            box.px = arc_widen(psi_x, t, w->nx); box.py = arc_widen(psi_y, t, w->ny);
-            box.lx = arc_widen(reg_x, T - t, w->nx); box.ly = arc_widen(reg_y, T - t, w->ny);
-            box.rx = arc_widen(reg_x, (T - t_lo) + (t - t_lo), w->nx);
-            box.ry = arc_widen(reg_y, (T - t_lo) + (t - t_lo), w->ny);
-            box.cx = arc_cover(box.px, box.rx, w->nx); box.cy = arc_cover(box.py, box.ry, w->ny);
-            if (box.cx.w <= 0 || box.cy.w <= 0) {   // no site matters any more at this time or before
-                li ^= 1; psi_in = psi_out; pi ^= 1;
-                continue;
+        for (int64_t t = t_hi; t > t_lo;) {
+            BackArgs a{};
+            // 8 steps per launch where their tiles (16 x 16 outputs of 32 x 32) are
+            // about one per SM, else 4 (24 x 24): the fewer sites for the halo
+            for (int k : {8, 4}) {
+                a.K = (int)std::min<int64_t>(k, t - t_lo);
+                a.t0 = t - a.K;
+                a.reach = (T - t_lo) + (a.t0 - t_lo);
+                const Arc cx = arc_cover(arc_widen(psi_x, t - 1, w->nx), arc_widen(reg_x, a.reach, w->nx), w->nx);
+                const Arc cy = arc_cover(arc_widen(psi_y, t - 1, w->ny), arc_widen(reg_y, a.reach, w->ny), w->ny);
+                a.cx = cx.a; a.cw = cx.w; a.cy = cy.a; a.ch = cy.w;
+                if (a.cw * a.ch <= BACK_DEEP_SITES) break;
             }
-            e = w->prec == QW_F32 ? backward_step<P_F32>(w, lam[li], psi_in, lam[li ^ 1], psi_out, gseg, box)
-                                  : backward_step<P_F64>(w, lam[li], psi_in, lam[li ^ 1], psi_out, gseg, box);
-            if (e != cudaSuccess) return cuda_error(w, e, "backward step");
+            a.lam_in = lam[li]; a.lam_out = lam[li ^ 1];
+            a.psi_in = psi_in; a.psi_out = view_of(w, pi);
+            a.nx = w->nx; a.ny = w->ny;
+            a.psi_x = psi_x; a.psi_y = psi_y; a.reg_x = reg_x; a.reg_y = reg_y;
+            a.T = T; a.phi = w->phi_dev; a.gseg = gseg;
+            if (a.cw > 0 && a.ch > 0) {   // (else the cones do not meet: the gradient is zero)
+                e = w->prec == QW_F32 ? backward_steps<P_F32>(w, a) : backward_steps<P_F64>(w, a);
+                if (e != cudaSuccess) return cuda_error(w, e, "backward step");
+            }
             li ^= 1;
-            psi_in = psi_out;
+            psi_in = a.psi_out;
             pi ^= 1;
+            t = a.t0;
         }
         const int64_t n4 = 4 * w->ns;
         const unsigned fb = (unsigned)((n4 + 255) / 256);
