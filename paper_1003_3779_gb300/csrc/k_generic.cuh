@@ -32,6 +32,54 @@ __device__ __forceinline__ uint2 philox_words01(uint32_t c0, uint32_t c1, uint32
     return make_uint2(c0, c1);
 }
 
+// The draw of philox_words01 for one site and many steps.  Counter (v, 0, step,
+// 0), v < 2^32: the first two of the ten rounds leave c0 = site.h ^ step.u,
+// c1 = site.l, c2 = site.b ^ step.v, c3 = step.w, with parts that depend on the
+// site or on the step alone; the last two only form what words 0 and 1 need.
+struct PhiloxSite { uint32_t h, l, b; };
+struct PhiloxStep { uint32_t u, v, w; };
+constexpr uint32_t PHILOX_M0 = 0xD2511F53u, PHILOX_M1 = 0xCD9E8D57u, PHILOX_W0 = 0x9E3779B9u, PHILOX_W1 = 0xBB67AE85u;
+__device__ __forceinline__ void mul_wide(uint32_t a, uint32_t b, uint32_t &hi, uint32_t &lo) {
+    const uint64_t p = (uint64_t)a * b;
+    hi = (uint32_t)(p >> 32);
+    lo = (uint32_t)p;
+}
+__device__ __forceinline__ PhiloxSite philox_site(uint32_t v, uint32_t k1) {
+    uint32_t h, l;
+    PhiloxSite s;
+    mul_wide(PHILOX_M0, v, h, s.b);
+    mul_wide(PHILOX_M1, h ^ k1, h, l);
+    s.h = h; s.l = l;
+    return s;
+}
+__device__ __forceinline__ PhiloxStep philox_step(uint32_t step, uint32_t k0, uint32_t k1) {
+    uint32_t h, l, h2;
+    PhiloxStep t;
+    mul_wide(PHILOX_M1, step, h, l);
+    mul_wide(PHILOX_M0, h ^ k0, h2, t.w);
+    t.u = l ^ (k0 + PHILOX_W0);
+    t.v = h2 ^ (k1 + PHILOX_W1);
+    return t;
+}
+__device__ __forceinline__ uint2 philox_draw(const PhiloxSite &s, const PhiloxStep &t, uint32_t k0, uint32_t k1) {
+    uint32_t c0 = s.h ^ t.u, c1 = s.l, c2 = s.b ^ t.v, c3 = t.w;
+#pragma unroll
+    for (uint32_t r = 2; r < 8; ++r) {
+        uint32_t h0, l0, h1, l1;
+        mul_wide(PHILOX_M0, c0, h0, l0);
+        mul_wide(PHILOX_M1, c2, h1, l1);
+        c0 = h1 ^ c1 ^ (k0 + r * PHILOX_W0);
+        c2 = h0 ^ c3 ^ (k1 + r * PHILOX_W1);
+        c1 = l1;
+        c3 = l0;
+    }
+    const uint32_t l1 = PHILOX_M1 * c2;
+    c2 = __umulhi(PHILOX_M0, c0) ^ c3 ^ (k1 + 8u * PHILOX_W1);
+    uint32_t h, l;
+    mul_wide(PHILOX_M1, c2, h, l);
+    return make_uint2(h ^ l1 ^ (k0 + 9u * PHILOX_W0), l);
+}
+
 // Is the link from (lx, ly) to its +axis neighbour broken at random at this
 // step?  The site's two links share one draw: word `axis` below the threshold.
 __device__ __forceinline__ bool random_closed(const GenGeom &g, int axis, int64_t lx, int64_t ly) {
@@ -295,69 +343,6 @@ k_step_generic_tile(View in, View out, GenGeom g, CoinP<typename St<P>::real> cp
             if (st == 0) val = ph[SHIFT == QW_SHIFT_MOVING ? co : (co ^ 1)][nby][nbx];
             else if (st == 1) val = ph[SHIFT == QW_SHIFT_MOVING ? (co ^ 1) : co][ey][ex];
             S::st(out, co, v, rmul(gain, val));
-        }
-    }
-}
-
-// The same on the cycle: a block owns GT1_X sites, phi of them and a one-site
-// halo in shared memory, the state of links x0 - 1 .. x0 + GT1_X - 1 once.
-// 1D coins: 0 moves to x - 1, 1 to x + 1; a site's link (to x + 1) is word 0 of
-// its draw.
-constexpr int GT1_X = 1024;
-
-template <int P, int SHIFT, int CK>
-__global__ void __launch_bounds__(GT_THREADS)
-k_step_generic_tile1d(View in, View out, GenGeom g, CoinP<typename St<P>::real> cp,
-                      const Cx<typename St<P>::real> *__restrict__ coins, const float *__restrict__ phi,
-                      typename St<P>::real gain) {
-    using real = typename St<P>::real;
-    using S = St<P>;
-    using C = Cx<real>;
-    constexpr int EX = GT1_X + 2;
-    __shared__ C ph[2][EX];
-    __shared__ unsigned char ls[GT1_X + 1];      // links owned by x0 - 1 .. x0 + GT1_X - 1
-    const int nx = (int)g.nx;                    // < 2^31 (launcher)
-    int tx = g.tx0 + (int)blockIdx.x;
-    if (tx >= g.ntx) tx -= g.ntx;
-    const int x0 = tx * GT1_X;
-    for (int ex = threadIdx.x; ex < EX; ex += GT_THREADS) {
-        int gx = x0 - 1 + ex;
-        gx = gx < 0 ? gx + nx : (gx >= nx ? gx % nx : gx);
-        const C a0 = S::ld(in, 0, gx), a1 = S::ld(in, 1, gx);
-        C e[2];
-        if (CK == CK_PHASE) gen_phases<real>(phi, gx, 2, e);
-#pragma unroll
-        for (int r = 0; r < 2; ++r) {
-            C val = czero<real>();
-            val = cfma(gen_entry<CK, real>(cp, coins, e, 2, gx, r, 0), a0, val);
-            val = cfma(gen_entry<CK, real>(cp, coins, e, 2, gx, r, 1), a1, val);
-            ph[r][ex] = val;
-        }
-        if (ex <= GT1_X) {
-            uint32_t rnd = 0u;
-            if (g.rthr) rnd = philox_words01((uint32_t)gx, 0u, g.rstep, 0u, g.rk0, g.rk1).x;
-            ls[ex] = link_state(g, 0, gx, 0, rnd);
-        }
-    }
-    __syncthreads();
-    for (int tx = threadIdx.x; tx < GT1_X; tx += GT_THREADS) {
-        const int x = x0 + tx;
-        if (x >= nx) break;
-        const int ex = tx + 1;
-#pragma unroll
-        for (int co = 0; co < 2; ++co) {
-            int nb, st;
-            if (SHIFT == QW_SHIFT_MOVING) {   // from x + 1 (coin 0) or x - 1 (coin 1), same coin
-                nb = co == 0 ? ex + 1 : ex - 1;
-                st = co == 0 ? ls[ex] : ls[ex - 1];
-            } else {                          // from x - 1 (coin 0) or x + 1 (coin 1), coin co ^ 1
-                nb = co == 0 ? ex - 1 : ex + 1;
-                st = co == 0 ? ls[ex - 1] : ls[ex];
-            }
-            C val = czero<real>();
-            if (st == 0) val = ph[SHIFT == QW_SHIFT_MOVING ? co : (co ^ 1)][nb];
-            else if (st == 1) val = ph[SHIFT == QW_SHIFT_MOVING ? (co ^ 1) : co][ex];
-            S::st(out, co, x, rmul(gain, val));
         }
     }
 }

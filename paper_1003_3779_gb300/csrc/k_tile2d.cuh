@@ -47,54 +47,6 @@ template <int SH> __device__ __forceinline__ void tile_slot(int p, int t, int &t
     }
 }
 
-// The draw of philox_words01 for one site and many steps.  Counter (v, 0, step,
-// 0), v < 2^32: the first two of the ten rounds leave c0 = site.h ^ step.u,
-// c1 = site.l, c2 = site.b ^ step.v, c3 = step.w, with parts that depend on the
-// site or on the step alone; the last two only form what words 0 and 1 need.
-struct PhiloxSite { uint32_t h, l, b; };
-struct PhiloxStep { uint32_t u, v, w; };
-constexpr uint32_t PHILOX_M0 = 0xD2511F53u, PHILOX_M1 = 0xCD9E8D57u, PHILOX_W0 = 0x9E3779B9u, PHILOX_W1 = 0xBB67AE85u;
-__device__ __forceinline__ void mul_wide(uint32_t a, uint32_t b, uint32_t &hi, uint32_t &lo) {
-    const uint64_t p = (uint64_t)a * b;
-    hi = (uint32_t)(p >> 32);
-    lo = (uint32_t)p;
-}
-__device__ __forceinline__ PhiloxSite philox_site(uint32_t v, uint32_t k1) {
-    uint32_t h, l;
-    PhiloxSite s;
-    mul_wide(PHILOX_M0, v, h, s.b);
-    mul_wide(PHILOX_M1, h ^ k1, h, l);
-    s.h = h; s.l = l;
-    return s;
-}
-__device__ __forceinline__ PhiloxStep philox_step(uint32_t step, uint32_t k0, uint32_t k1) {
-    uint32_t h, l, h2;
-    PhiloxStep t;
-    mul_wide(PHILOX_M1, step, h, l);
-    mul_wide(PHILOX_M0, h ^ k0, h2, t.w);
-    t.u = l ^ (k0 + PHILOX_W0);
-    t.v = h2 ^ (k1 + PHILOX_W1);
-    return t;
-}
-__device__ __forceinline__ uint2 philox_draw(const PhiloxSite &s, const PhiloxStep &t, uint32_t k0, uint32_t k1) {
-    uint32_t c0 = s.h ^ t.u, c1 = s.l, c2 = s.b ^ t.v, c3 = t.w;
-#pragma unroll
-    for (uint32_t r = 2; r < 8; ++r) {
-        uint32_t h0, l0, h1, l1;
-        mul_wide(PHILOX_M0, c0, h0, l0);
-        mul_wide(PHILOX_M1, c2, h1, l1);
-        c0 = h1 ^ c1 ^ (k0 + r * PHILOX_W0);
-        c2 = h0 ^ c3 ^ (k1 + r * PHILOX_W1);
-        c1 = l1;
-        c3 = l0;
-    }
-    const uint32_t l1 = PHILOX_M1 * c2;
-    c2 = __umulhi(PHILOX_M0, c0) ^ c3 ^ (k1 + 8u * PHILOX_W1);
-    uint32_t h, l;
-    mul_wide(PHILOX_M1, c2, h, l);
-    return make_uint2(h ^ l1 ^ (k0 + 9u * PHILOX_W0), l);
-}
-
 // PH: per-site phase factors before the coin CK.
 template <int P, int SH, int CK, bool PH, bool LINKS, int EX, int EY, int TH>
 __global__ void __launch_bounds__(TH)
@@ -128,6 +80,7 @@ k_tile2d(View in, View out, GenGeom g, int64_t ox0, int64_t ow, int64_t oy0, int
     SiteCoin<real> sc[PH ? NS : 1];
     unsigned char fixed[LINKS ? NS : 1];        // links closed or absorbing at every step
     PhiloxSite rnd[LINKS ? NS : 1];
+    int any = 0;
 #pragma unroll
     for (int n = 0; n < NS; ++n) {
         const int j = j0 + n * DJ;
@@ -141,10 +94,12 @@ k_tile2d(View in, View out, GenGeom g, int64_t ox0, int64_t ow, int64_t oy0, int
         if constexpr (LINKS) {
             fixed[n] = (unsigned char)(link_state(g, 0, (int)gx, (int)gy, 0xffffffffu) |
                                        (link_state(g, 1, (int)gx, (int)gy, 0xffffffffu) << 2));
+            any |= fixed[n];
             rnd[n] = philox_site((uint32_t)v, g.rk1);
         }
     }
-    __syncthreads();
+    // does any link of the tile ever close (or absorb)?
+    const bool settle = __syncthreads_or(any) || (LINKS && g.rthr);
     // slot of plane c of site (i, j) at step t
     auto slot = [&](int c, int t, int si, int sj) {
         int tr, dx, dy;
@@ -188,10 +143,11 @@ k_tile2d(View in, View out, GenGeom g, int64_t ox0, int64_t ow, int64_t oy0, int
         if constexpr (LINKS) {
             // a site settles its +x and +y links: what each end sends across one
             // that is closed changes places, and is lost on an absorbing one
-            __syncthreads();
+            if (settle) __syncthreads();
 #pragma unroll
             for (int n = 0; n < NS; ++n) {
                 const int j = j0 + n * DJ;
+                if (!settle) break;
 #pragma unroll
                 for (int axis = 0; axis < 2; ++axis) {
                     const unsigned s = st[n] >> (2 * axis) & 3u;

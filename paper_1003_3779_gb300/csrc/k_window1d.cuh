@@ -1,145 +1,136 @@
-// k_window1d.cuh -- many generic steps of a 1D walk whose light cone is still
-// narrow, in one CTA: the line computation window of Sec. 3 (a walker started
-// at MP steps only the sites [l_i, r_i] its light cone has reached, which
-// widen by one site per step on each side and stop at the ends of the line).
+// k_window1d.cuh -- K generic forward steps of the 1D walk per launch: the segment
+// and the line of Sec. 3, broken links, on the whole lattice or on the
+// computation window of a localised walk (a walker started at MP steps only the
+// sites [l_i, r_i] its light cone has reached).
 //
-// On the segment and the line such a window is a few thousand sites for
-// hundreds of steps, so a launch per step costs far more than the step.  One
-// CTA keeps the window's state in shared memory, in the walk's storage format,
-// and runs up to WIN_MAX_STEPS steps with a barrier between the coin phase and
-// the shift phase of each.  Each step is the one k_step_generic_tile1d makes:
-// the same coin row per site (gen_entry), the same link states (link_state,
-// with the step's Philox draw), the same pull rule and the same drift gain, so
-// the state after the launch equals that of the per-step launches bit for bit.
-// Sites outside the support box are zero and stay zero until the box reaches
-// them; the window is the box after the launch's steps.
+// The 1D form of k_tile2d.cuh: a CTA keeps E sites in shared memory, in the
+// walk's storage format, updates them in place for K steps (an amplitude stays
+// in its slot while the lattice moves under it; a closed link swaps two slots)
+// and writes the E - 2K sites whose light cone lies inside.  Every step applies
+// the full coin row, the step's drift gain and the step's link draws, whatever
+// the window, so clipped and full steps agree bit for bit.
+//
+// One step per launch of the whole lattice costs its round trip through HBM, and
+// one CTA for a whole window is bound by one SM's issue (0.58 us per step for
+// windows of up to 2049 sites); tiles of 256 sites spread a window over many SMs.
 #pragma once
 #include "k_generic.cuh"
 
 namespace qw {
 
-constexpr int WIN_THREADS = 1024;
-constexpr int WIN_MAX_STEPS = 256;               // steps per launch
-constexpr size_t WIN_SMEM_BYTES = 200 * 1024;   // dynamic shared memory of the window CTA
-
 // drift gains of the launch's steps, in the compute real
 template <class R>
 struct WinGains {
-    R v[WIN_MAX_STEPS];
+    R v[WINDOW_MAX_STEPS];
 };
 
-// Shared-memory layout for a window of wn sites: phi of sites w0 - 1 .. w0 + wn
-// (2 coin values each), the state (d = 2 coins, SLOTS_PER_COIN slots each, of
-// SLOT_BYTES per site) and one link-state byte per owner w0 - 1 .. w0 + wn - 1.
-template <int P>
-constexpr size_t win_ph_bytes(int64_t wn) { return ((size_t)2 * (wn + 2) * sizeof(Cx<typename St<P>::real>) + 15) / 16 * 16; }
-template <int P>
-constexpr size_t win_state_bytes(int64_t wn) {
-    return ((size_t)2 * St<P>::SLOTS_PER_COIN * St<P>::SLOT_BYTES * wn + 15) / 16 * 16;
-}
-template <int P>
-constexpr size_t win_smem(int64_t wn) { return win_ph_bytes<P>(wn) + win_state_bytes<P>(wn) + (size_t)wn + 2; }
-// the widest window that fits WIN_SMEM_BYTES
-template <int P>
-constexpr int64_t win_capacity() {
-    int64_t wn = (int64_t)(WIN_SMEM_BYTES / (2 * sizeof(Cx<typename St<P>::real>) +
-                                            2 * St<P>::SLOTS_PER_COIN * St<P>::SLOT_BYTES + 1));
-    while (wn > 0 && win_smem<P>(wn) > WIN_SMEM_BYTES) --wn;
-    return wn;
+// Slot of plane p at step t, as tile_slot of the 2D tiles: coin 0 moves to
+// x - 1, coin 1 to x + 1.
+template <int SH> __device__ __forceinline__ void win_slot(int p, int t, int &track, int &dx) {
+    const int e = p == 0 ? -1 : 1;
+    if (SH == QW_SHIFT_FLIPFLOP) {
+        const int odd = t & 1;
+        track = p ^ odd;
+        dx = odd ? e : 0;
+    } else {
+        track = p;
+        dx = -t * e;
+    }
 }
 
-// nsteps forward steps of the walk on the segment or the line (no wrap): the
-// input's support box is [b0, b0 + bw); the window [w0, w0 + wn) is that box
-// after nsteps steps (cut at the ends), read from `in` and written to `out`.
-// LINKS: fixed or random broken links, whose states are drawn per step into
-// shared memory; without them a link is open unless it is the edge link
-// (owned by site n - 1, and seen by site 0 from its left), whose state is the
-// boundary's, so nothing is stored.
-template <int P, int SHIFT, int CK, bool LINKS>
-__global__ void __launch_bounds__(WIN_THREADS)
+// Outputs: [o0, o0 + ow) modulo g.nx.
+template <int P, int SH, int CK, int E, int TH>
+__global__ void __launch_bounds__(TH)
 k_step1d_window(View in, View out, GenGeom g, CoinP<typename St<P>::real> cp,
-                const Cx<typename St<P>::real> *__restrict__ coins, const float *__restrict__ phi, int b0, int bw,
-                int nsteps, int w0, int wn, WinGains<typename St<P>::real> gains) {
-    using real = typename St<P>::real;
+                const Cx<typename St<P>::real> *__restrict__ coins, int o0, int ow, int K,
+                WinGains<typename St<P>::real> gains) {
     using S = St<P>;
+    using real = typename S::real;
     using C = Cx<real>;
+    constexpr int NS = E / TH, M = E - 1;
+    static_assert(NS * TH == E && (E & M) == 0, "tile shape");
     extern __shared__ __align__(16) unsigned char wsm[];
-    C *ph0 = reinterpret_cast<C *>(wsm);                  // phi, coin 0, of site w0 - 1 + i at i
-    C *ph1 = ph0 + (wn + 2);                              // coin 1
-    const View sv{wsm + win_ph_bytes<P>(wn), (int64_t)wn, 2};   // the window's state, site w0 + i at i
-    unsigned char *ls = wsm + win_ph_bytes<P>(wn) + win_state_bytes<P>(wn);   // owner w0 - 1 + i at i
-    const int n = (int)g.nx;                              // < 2^30 (launcher)
-    const int nt = (int)blockDim.x;
-    // the edge link's state without broken links: reflecting (segment) or absorbing (line)
-    const unsigned char edge = g.bc == QW_BC_SEGMENT ? 1 : 2;
-
-    for (int i = threadIdx.x; i < wn; i += nt) {
+    const View sv{wsm, E, 2};
+    const int n = (int)g.nx, O = E - 2 * K;                     // n < 2^30 (launcher)
+    const int b = (int)blockIdx.x * O - K;                      // tile site i is output b + i
+    auto site = [&](int i) {
+        int64_t x = (int64_t)o0 + b + i;                        // in [-K, 2n + E)
+        if (n < E) { x %= n; return (int)(x < 0 ? x + n : x); }
+        if (x < 0) x += n;
+        if (x >= n) x -= n;
+        return (int)(x >= n ? x - n : x);
+    };
+    C m[CK == CK_PERSITE ? NS : 1][4];
+    unsigned char fixed[NS];
+    PhiloxSite rnd[NS];
+    int any = 0;
 #pragma unroll
-        for (int c = 0; c < 2; ++c) S::st(sv, c, i, S::ld(in, c, (int64_t)w0 + i));
-    }
-    __syncthreads();
-    for (int t = 0; t < nsteps; ++t) {
-        // outputs of this step: the box after it
-        const int o0 = max(0, b0 - (t + 1)), o1 = min(n, b0 + bw + t + 1);
-        const uint32_t rstep = g.rstep + (uint32_t)t;
-        // phase 1: phi of sites o0 - 1 .. o1 (zero off the lattice and outside
-        // the window, where the state is zero) and, with broken links, the links
-        // owned by o0 - 1 .. o1 - 1
-        for (int x = o0 - 1 + (int)threadIdx.x; x <= o1; x += nt) {
-            const int i = x - w0 + 1;
-            C v0 = czero<real>(), v1 = czero<real>();
-            if (x >= 0 && x < n && x >= w0 && x < w0 + wn) {
-                const C a0 = S::ld(sv, 0, x - w0), a1 = S::ld(sv, 1, x - w0);
-                C e[2];
-                if (CK == CK_PHASE) gen_phases<real>(phi, x, 2, e);
-                v0 = cfma(gen_entry<CK, real>(cp, coins, e, 2, x, 0, 0), a0, v0);
-                v0 = cfma(gen_entry<CK, real>(cp, coins, e, 2, x, 0, 1), a1, v0);
-                v1 = cfma(gen_entry<CK, real>(cp, coins, e, 2, x, 1, 0), a0, v1);
-                v1 = cfma(gen_entry<CK, real>(cp, coins, e, 2, x, 1, 1), a1, v1);
-            }
-            ph0[i] = v0;
-            ph1[i] = v1;
-            if (LINKS && x < o1) {
-                // site 0's left link is the edge link, owned by site n - 1
-                const int owner = x < 0 ? n - 1 : x;
-                uint32_t rnd = 0u;
-                if (g.rthr) rnd = philox_words01((uint32_t)owner, 0u, rstep, 0u, g.rk0, g.rk1).x;
-                ls[i] = link_state(g, 0, owner, 0, rnd);
-            }
+    for (int k = 0; k < NS; ++k) {
+        const int i = (int)threadIdx.x + k * TH, x = site(i);
+#pragma unroll
+        for (int c = 0; c < 2; ++c) S::st(sv, c, i, S::ld(in, c, x));
+        if constexpr (CK == CK_PERSITE) {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) m[k][e] = coins[4 * (int64_t)x + e];
         }
-        __syncthreads();
-        // phase 2: each output site pulls its two amplitudes (as the 1D tile)
+        fixed[k] = link_state(g, 0, x, 0, 0xffffffffu);
+        any |= fixed[k];
+        rnd[k] = philox_site((uint32_t)x, g.rk1);
+    }
+    // does any link of the tile ever close (or absorb)?
+    const bool settle = __syncthreads_or(any) || g.rthr;
+    for (int t = 0; t < K; ++t) {
         const real gain = gains.v[t];
-        for (int x = o0 + (int)threadIdx.x; x < o1; x += nt) {
-            const int ex = x - w0 + 1;
-            // states of the links to the right (owned by x) and to the left (owned by x - 1)
-            const int sr = LINKS ? ls[ex] : (x == n - 1 ? edge : 0);
-            const int sl = LINKS ? ls[ex - 1] : (x == 0 ? edge : 0);
-            C out2[2];
+        const bool one = is_one(gain);
+        int st[NS];
+        PhiloxStep ps;
+        if (g.rthr) ps = philox_step(g.rstep + (uint32_t)t, g.rk0, g.rk1);
 #pragma unroll
-            for (int co = 0; co < 2; ++co) {
-                int nb, st;
-                if (SHIFT == QW_SHIFT_MOVING) {   // from x + 1 (coin 0) or x - 1 (coin 1), same coin
-                    nb = co == 0 ? ex + 1 : ex - 1;
-                    st = co == 0 ? sr : sl;
-                } else {                          // from x - 1 (coin 0) or x + 1 (coin 1), coin co ^ 1
-                    nb = co == 0 ? ex - 1 : ex + 1;
-                    st = co == 0 ? sl : sr;
-                }
-                const int from = SHIFT == QW_SHIFT_MOVING ? co : (co ^ 1);   // coin of the arriving value
-                C val = czero<real>();
-                if (st == 0) val = from == 0 ? ph0[nb] : ph1[nb];
-                else if (st == 1) val = from == 0 ? ph1[ex] : ph0[ex];   // reflected: the other coin of x
-                out2[co] = rmul(gain, val);
-            }
-            S::st(sv, 0, x - w0, out2[0]);
-            S::st(sv, 1, x - w0, out2[1]);
+        for (int k = 0; k < NS; ++k) {
+            const int i = (int)threadIdx.x + k * TH;
+            int t0, d0, t1, d1;
+            win_slot<SH>(0, t, t0, d0);
+            win_slot<SH>(1, t, t1, d1);
+            const int s0 = (i + d0) & M, s1 = (i + d1) & M;
+            const C a0 = S::ld(sv, t0, s0), a1 = S::ld(sv, t1, s1);
+            auto entry = [&](int e) { return CK == CK_PERSITE ? m[CK == CK_PERSITE ? k : 0][e] : C{cp.re[e], cp.im[e]}; };
+            C v0 = cfma(entry(1), a1, cfma(entry(0), a0, czero<real>()));
+            C v1 = cfma(entry(3), a1, cfma(entry(2), a0, czero<real>()));
+            if (!one) { v0 = rmul(gain, v0); v1 = rmul(gain, v1); }
+            S::st(sv, t0, s0, v0);
+            S::st(sv, t1, s1, v1);
+            st[k] = fixed[k];
+            if (g.rthr && philox_draw(rnd[k], ps, g.rk0, g.rk1).x < g.rthr) st[k] = 1;
         }
         __syncthreads();
-    }
-    for (int i = threadIdx.x; i < wn; i += nt) {
+        // each site settles the link to its right neighbour
+        if (settle) {
 #pragma unroll
-        for (int c = 0; c < 2; ++c) S::st(out, c, (int64_t)w0 + i, S::ld(sv, c, i));
+            for (int k = 0; k < NS; ++k) {
+                if (!st[k]) continue;
+                const int i = (int)threadIdx.x + k * TH;
+                int t1, d1, t0, d0;
+                win_slot<SH>(1, t, t1, d1);
+                win_slot<SH>(0, t, t0, d0);
+                const int q = (i + d1) & M, r = (i + 1 + d0) & M;
+                const C u = st[k] == 1 ? S::ld(sv, t1, q) : czero<real>(), w = st[k] == 1 ? S::ld(sv, t0, r) : czero<real>();
+                S::st(sv, t1, q, w);
+                S::st(sv, t0, r, u);
+            }
+            __syncthreads();
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < NS; ++k) {
+        const int i = (int)threadIdx.x + k * TH;
+        if (i < K || i >= E - K || b + i >= ow) continue;
+        const int x = site(i);
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            int tr, d;
+            win_slot<SH>(c, K, tr, d);
+            S::st(out, c, x, S::ld(sv, tr, (i + d) & M));
+        }
     }
 }
 

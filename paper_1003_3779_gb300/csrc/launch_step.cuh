@@ -24,6 +24,13 @@ template <> struct Tiles1D<P_COMP> { static constexpr int A = 4, B = 8, DEF = 4;
 template <int P> struct Tile2D { static constexpr int R = 32 / St<P>::SLOT_BYTES < 1 ? 1 : 32 / St<P>::SLOT_BYTES; };
 template <> struct Tile2D<P_COMP> { static constexpr int R = 4; };
 
+// A third, short tile for narrow light-cone windows: an FP64 warp gets half a
+// lane a clock from its scheduler, so a window runs faster on many short tiles
+// (2001-site Hadamard cycle from one site, T = 1000: tiles of 8 sites per lane in
+// blocks of four warps 2.3 ms, of 4 sites in blocks of one 0.82 ms, of 2 sites 0.59).
+template <int P> struct WindowTile1D { static constexpr int R = 0; };
+template <> struct WindowTile1D<P_F64> { static constexpr int R = 2; };
+
 template <int P, int CK, int FF, int ADJ>
 static void go1d_k1(const Step1DArgs &a, const CoinP<typename St<P>::real> &cp, cudaStream_t s) {
     using real = typename St<P>::real;
@@ -62,8 +69,11 @@ static void go1d(const Step1DArgs &a, const CoinP<typename St<P>::real> &cp, cud
     const bool win = a.oend > a.obeg;   // a light-cone window, else the whole cycle
     const int64_t ob = win ? a.obeg : 0, oe = win ? a.oend : a.n;
     const int64_t nwarps = (oe - ob + W - 1) / W;
-    const int64_t blocks = (nwarps + 3) / 4;
-    k_step1d<P, R, CK, FF, ADJ><<<(unsigned)blocks, 128, 0, s>>>(
+    // a window of few tiles: one warp per block, so that each has a scheduler of
+    // its own
+    const int wpb = win && nwarps <= 4 * 152 ? 1 : 4;
+    const int64_t blocks = (nwarps + wpb - 1) / wpb;
+    k_step1d<P, R, CK, FF, ADJ><<<(unsigned)blocks, 32 * wpb, 0, s>>>(
         a.in, a.out, a.n, a.K, W, ob, oe, nwarps, cp,
         static_cast<const Cx<typename St<P>::real> *>(a.coins),
         real_from_double<typename St<P>::real>(a.pre0), real_from_double<typename St<P>::real>(a.pre1),
@@ -156,8 +166,9 @@ bool sweep_ok(int64_t n, int K, int kind, int tile) {
     return B > 0 && n >= B && K >= 2 && K <= B / 2 - 1;
 }
 
-// Largest K the 1D kernel accepts for tile R: at least half the tile is output.
-inline int max_k_1d(int R) { return 8 * R; }
+// Largest K the 1D kernel accepts for tile R: at least half the tile is output
+// (a quarter of the short window tile).
+inline int max_k_1d(int R) { return R == 2 ? 24 : 8 * R; }
 
 template <int P>
 int tile1d_effective(int tile, int kind, int adj) {
@@ -180,6 +191,13 @@ cudaError_t step1d_t(const Step1DArgs &a0, const void *coinp, int adj, cudaStrea
             if (sweep_tile<P>(a.n, a.tile) == ST::B)
                 return adj ? go1d_sweep_kind<P, ST::B, 1>(a, cp, s) : go1d_sweep_kind<P, ST::B, 0>(a, cp, s);
             return adj ? go1d_sweep_kind<P, ST::A, 1>(a, cp, s) : go1d_sweep_kind<P, ST::A, 0>(a, cp, s);
+        }
+    }
+    if constexpr (WindowTile1D<P>::R > 0) {
+        constexpr int R = WindowTile1D<P>::R;
+        if (a.tile == R && a.oend > a.obeg && a.kind != CK_PERSITE && a.K >= 1 && a.K <= max_k_1d(R)) {
+            const bool ok = adj ? go1d_kind<P, R, 1>(a, cp, s) : go1d_kind<P, R, 0>(a, cp, s);
+            return ok ? cudaGetLastError() : cudaErrorInvalidValue;
         }
     }
     a.tile = tile1d_effective<P>(a.tile, a.kind, adj);
@@ -299,13 +317,14 @@ static void gogen(const StepGenericArgs &a, const CoinP<typename St<P>::real> &c
         real_from_double<typename St<P>::real>(a.gain));
 }
 
-// The tiled forms serve the forward step on the axis lattice (1D and 2D; any
-// coin, boundary and links); the grid's y extent limits ny to 65535 tiles.
+// The tiled form serves the forward step on the 2D axis lattice (any coin,
+// boundary and links); the grid's y extent limits ny to 65535 tiles.  (1D forward
+// steps run k_step1d_window.)
 template <int P>
 static bool generic_tile_ok(const StepGenericArgs &a) {
     if (a.adjoint || !(a.shift == QW_SHIFT_MOVING || a.shift == QW_SHIFT_FLIPFLOP) || a.nx >= (int64_t(1) << 30))
         return false;
-    return a.ndim == 1 || (a.ny + gt_y<P>() - 1) / gt_y<P>() <= 65535;
+    return a.ndim == 2 && (a.ny + gt_y<P>() - 1) / gt_y<P>() <= 65535;
 }
 
 template <int P, int CK>
@@ -315,18 +334,6 @@ static void gotile(const StepGenericArgs &a, const CoinP<typename St<P>::real> &
     GenGeom g{a.ndim, a.nx, a.ny, a.nx * a.ny, a.shift, a.bc, a.links, a.rthr, a.rk0, a.rk1, a.rstep, 0, 1, 0, 1};
     const auto gain = real_from_double<real>(a.gain);
     const auto *coins = static_cast<const Cx<real> *>(a.coins);
-    if (a.ndim == 1) {
-        if constexpr (CK == CK_COMPLEX || CK == CK_PERSITE || CK == CK_PHASE) {   // (the 1D tiles take these)
-            tile_range(a.bx0, a.bw, a.nx, GT1_X, per, g.tx0, g.ntx);
-            const unsigned grid = (unsigned)g.ntx;
-            g.ntx = (int)((a.nx + GT1_X - 1) / GT1_X);
-            if (a.shift == QW_SHIFT_MOVING)
-                k_step_generic_tile1d<P, QW_SHIFT_MOVING, CK><<<grid, GT_THREADS, 0, s>>>(a.in, a.out, g, cp, coins, a.phi, gain);
-            else
-                k_step_generic_tile1d<P, QW_SHIFT_FLIPFLOP, CK><<<grid, GT_THREADS, 0, s>>>(a.in, a.out, g, cp, coins, a.phi, gain);
-        }
-        return;
-    }
     int gx = 0, gy = 0;
     tile_range(a.bx0, a.bw, a.nx, GT_X, per, g.tx0, gx);
     tile_range(a.by0, a.bw > 0 ? a.bh : 0, a.ny, gt_y<P>(), per, g.ty0, gy);
@@ -343,13 +350,12 @@ template <int P>
 cudaError_t generic_t(const StepGenericArgs &a, const void *coinp, cudaStream_t s) {
     const auto &cp = *static_cast<const CoinP<typename St<P>::real> *>(coinp);
     if (generic_tile_ok<P>(a)) {
-        const bool d2 = a.ndim == 2;   // the 2D tiles specialise the global coin classes
         switch (a.kind) {
             case CK_PERSITE: gotile<P, CK_PERSITE>(a, cp, s); break;
             case CK_PHASE: gotile<P, CK_PHASE>(a, cp, s); break;
-            case CK_GROVER: d2 ? gotile<P, CK_GROVER>(a, cp, s) : gotile<P, CK_COMPLEX>(a, cp, s); break;
-            case CK_HH: d2 ? gotile<P, CK_HH>(a, cp, s) : gotile<P, CK_COMPLEX>(a, cp, s); break;
-            case CK_REAL: d2 ? gotile<P, CK_REAL>(a, cp, s) : gotile<P, CK_COMPLEX>(a, cp, s); break;
+            case CK_GROVER: gotile<P, CK_GROVER>(a, cp, s); break;
+            case CK_HH: gotile<P, CK_HH>(a, cp, s); break;
+            case CK_REAL: gotile<P, CK_REAL>(a, cp, s); break;
             default: gotile<P, CK_COMPLEX>(a, cp, s); break;   // other global coins as a full matrix
         }
         return cudaGetLastError();
@@ -362,48 +368,52 @@ cudaError_t generic_t(const StepGenericArgs &a, const void *coinp, cudaStream_t 
     return cudaGetLastError();
 }
 
-// The 1D window kernel (a clipped forward walk on the segment or the line,
-// nsteps steps in one CTA); gains[i] is the drift gain of step i, a.rstep the
-// random-link step of the first.  cudaErrorInvalidValue if the window after
-// the steps is wider than win_capacity<P>() or nsteps is out of [1, WIN_MAX_STEPS].
-template <int P, int CK, int SHIFT>
-static cudaError_t gowin_shift(const StepGenericArgs &a, const CoinP<typename St<P>::real> &cp, const double *gains,
-                               int nsteps, cudaStream_t s) {
+// 1D generic forward steps: nsteps (at most WINDOW_MAX_STEPS) from the state in
+// a.in on the output range [o0, o0 + ow) modulo nx; gains[i] is the drift gain of
+// step i, a.rstep the random-link step of the first.  Ranges of up to
+// WINDOW_SITES sites take tiles of 256, wider ones tiles of 2048, whose halos are
+// a smaller share (a line of 2^20 sites from its middle, T = 1024, FP32: 593 us in
+// one CTA, now under 150; the whole 2^27 line: 0.66 ms per step one by one).
+template <int P, int CK, int SH, int E, int TH>
+static cudaError_t gowin(const StepGenericArgs &a, const CoinP<typename St<P>::real> &cp, const double *gains, int nsteps,
+                         int64_t o0, int64_t ow, cudaStream_t s) {
     using real = typename St<P>::real;
-    const int64_t w0 = std::max<int64_t>(0, a.bx0 - nsteps), w1 = std::min<int64_t>(a.nx, a.bx0 + a.bw + nsteps);
-    const int64_t wn = w1 - w0;
-    if (nsteps < 1 || nsteps > WIN_MAX_STEPS || wn < 1 || wn > win_capacity<P>() || a.bc == QW_BC_PERIODIC)
-        return cudaErrorInvalidValue;
     GenGeom g{a.ndim, a.nx, a.ny, a.nx * a.ny, a.shift, a.bc, a.links, a.rthr, a.rk0, a.rk1, a.rstep, 0, 1, 0, 1};
     WinGains<real> gv{};
     for (int i = 0; i < nsteps; ++i) gv.v[i] = real_from_double<real>(gains[i]);
-    const bool links = a.links != nullptr || a.rthr != 0;
-    auto kfn = links ? k_step1d_window<P, SHIFT, CK, true> : k_step1d_window<P, SHIFT, CK, false>;
-    // (set on every launch: the attribute is the current device's, and a launch runs up to 256 steps)
-    cudaError_t e = cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)WIN_SMEM_BYTES);
+    auto kfn = k_step1d_window<P, SH, CK, E, TH>;
+    constexpr size_t smem = (size_t)E * 2 * St<P>::SLOTS_PER_COIN * St<P>::SLOT_BYTES;
+    // (set on every launch that needs it: the attribute is the current device's)
+    cudaError_t e = smem > 48 * 1024 ? cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) : cudaSuccess;
     if (e != cudaSuccess) return e;
-    kfn<<<1, WIN_THREADS, win_smem<P>(wn), s>>>(a.in, a.out, g, cp, static_cast<const Cx<real> *>(a.coins), a.phi,
-                                                 (int)a.bx0, (int)a.bw, nsteps, (int)w0, (int)wn, gv);
+    const int64_t blocks = (ow + E - 2 * nsteps - 1) / (E - 2 * nsteps);
+    kfn<<<(unsigned)blocks, TH, smem, s>>>(a.in, a.out, g, cp, static_cast<const Cx<real> *>(a.coins), (int)o0, (int)ow,
+                                           nsteps, gv);
     return cudaGetLastError();
 }
 
 template <int P, int CK>
-static cudaError_t gowin(const StepGenericArgs &a, const CoinP<typename St<P>::real> &cp, const double *gains, int nsteps,
-                         cudaStream_t s) {
-    if (a.shift == QW_SHIFT_MOVING) return gowin_shift<P, CK, QW_SHIFT_MOVING>(a, cp, gains, nsteps, s);
-    if (a.shift == QW_SHIFT_FLIPFLOP) return gowin_shift<P, CK, QW_SHIFT_FLIPFLOP>(a, cp, gains, nsteps, s);
+static cudaError_t gowin_shift(const StepGenericArgs &a, const CoinP<typename St<P>::real> &cp, const double *gains, int nsteps,
+                               int64_t o0, int64_t ow, cudaStream_t s) {
+    const bool narrow = ow <= WINDOW_SITES;
+    if (a.shift == QW_SHIFT_MOVING)
+        return narrow ? gowin<P, CK, QW_SHIFT_MOVING, 256, 256>(a, cp, gains, nsteps, o0, ow, s)
+                      : gowin<P, CK, QW_SHIFT_MOVING, 2048, 512>(a, cp, gains, nsteps, o0, ow, s);
+    if (a.shift == QW_SHIFT_FLIPFLOP)
+        return narrow ? gowin<P, CK, QW_SHIFT_FLIPFLOP, 256, 256>(a, cp, gains, nsteps, o0, ow, s)
+                      : gowin<P, CK, QW_SHIFT_FLIPFLOP, 2048, 512>(a, cp, gains, nsteps, o0, ow, s);
     return cudaErrorInvalidValue;
 }
 
 template <int P>
-cudaError_t window1d_t(const StepGenericArgs &a, const void *coinp, const double *gains, int nsteps, cudaStream_t s) {
+cudaError_t window1d_t(const StepGenericArgs &a, const void *coinp, const double *gains, int nsteps, int64_t o0, int64_t ow,
+                       cudaStream_t s) {
     const auto &cp = *static_cast<const CoinP<typename St<P>::real> *>(coinp);
-    if (a.ndim != 1 || a.adjoint || a.nx >= (int64_t(1) << 30)) return cudaErrorInvalidValue;
-    switch (a.kind) {   // the coins of the 1D tiles: global coins as the full matrix
-        case CK_PERSITE: return gowin<P, CK_PERSITE>(a, cp, gains, nsteps, s);
-        case CK_PHASE: return gowin<P, CK_PHASE>(a, cp, gains, nsteps, s);
-        default: return gowin<P, CK_COMPLEX>(a, cp, gains, nsteps, s);
-    }
+    if (a.ndim != 1 || a.adjoint || a.nx >= (int64_t(1) << 30) || nsteps < 1 || nsteps > WINDOW_MAX_STEPS || ow < 1)
+        return cudaErrorInvalidValue;
+    // (phase coins are expanded to per-site matrices in 1D); global coins as the full matrix
+    return a.kind == CK_PERSITE ? gowin_shift<P, CK_PERSITE>(a, cp, gains, nsteps, o0, ow, s)
+                                : gowin_shift<P, CK_COMPLEX>(a, cp, gains, nsteps, o0, ow, s);
 }
 
 }  // namespace qw
@@ -421,10 +431,9 @@ cudaError_t window1d_t(const StepGenericArgs &a, const void *coinp, const double
         return generic_t<PREC>(a, cp, s);                                                               \
     }                                                                                                   \
     cudaError_t launch_window1d_##SUFFIX(const StepGenericArgs &a, const void *cp, const double *gains,  \
-                                         int nsteps, cudaStream_t s) {                                  \
-        return window1d_t<PREC>(a, cp, gains, nsteps, s);                                               \
+                                         int nsteps, int64_t o0, int64_t ow, cudaStream_t s) {          \
+        return window1d_t<PREC>(a, cp, gains, nsteps, o0, ow, s);                                       \
     }                                                                                                   \
-    int64_t window1d_capacity_##SUFFIX() { return win_capacity<PREC>(); }                               \
     int tile1d_##SUFFIX(int tile, int kind, int adj) { return tile1d_effective<PREC>(tile, kind, adj); } \
     bool sweep_ok_##SUFFIX(int64_t n, int K, int kind, int tile) { return sweep_ok<PREC>(n, K, kind, tile); } \
     int sweep_tile_##SUFFIX(int64_t n, int tile) { return sweep_tile<PREC>(n, tile); }                   \

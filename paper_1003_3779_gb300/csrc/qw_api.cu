@@ -76,24 +76,15 @@ static cudaError_t step2d(int prec, const Step2DArgs &a, const void *cp, int adj
     }
     return cudaErrorInvalidValue;
 }
-static cudaError_t stepwin(int prec, const StepGenericArgs &a, const void *cp, const double *gains, int nsteps,
-                           cudaStream_t s) {
+static cudaError_t stepwin(int prec, const StepGenericArgs &a, const void *cp, const double *gains, int nsteps, int64_t o0,
+                           int64_t ow, cudaStream_t s) {
     switch (prec) {
-        case QW_F64: return launch_window1d_f64(a, cp, gains, nsteps, s);
-        case QW_F32: return launch_window1d_f32(a, cp, gains, nsteps, s);
-        case QW_F32_BF16STORE: return launch_window1d_bf16(a, cp, gains, nsteps, s);
-        case QW_F32_COMP: return launch_window1d_comp(a, cp, gains, nsteps, s);
+        case QW_F64: return launch_window1d_f64(a, cp, gains, nsteps, o0, ow, s);
+        case QW_F32: return launch_window1d_f32(a, cp, gains, nsteps, o0, ow, s);
+        case QW_F32_BF16STORE: return launch_window1d_bf16(a, cp, gains, nsteps, o0, ow, s);
+        case QW_F32_COMP: return launch_window1d_comp(a, cp, gains, nsteps, o0, ow, s);
     }
     return cudaErrorInvalidValue;
-}
-static int64_t window_capacity(int prec) {
-    switch (prec) {
-        case QW_F64: return window1d_capacity_f64();
-        case QW_F32: return window1d_capacity_f32();
-        case QW_F32_BF16STORE: return window1d_capacity_bf16();
-        case QW_F32_COMP: return window1d_capacity_comp();
-    }
-    return 0;
 }
 
 static cudaError_t stepgen(int prec, const StepGenericArgs &a, const void *cp, cudaStream_t s) {
@@ -292,7 +283,7 @@ static double feedback_gain(qw_walk *w, double ideal, bool update = true) {
 // be biased: round-to-nearest of x * (1 - 2^-24) is always x - ulp(x).
 static double take_drift(qw_walk *w, int steps, bool last) {
     if (w->kind == CK_PERSITE || w->kind == CK_PHASE || w->coin_alpha == 1.0) return 1.0;
-    w->drift_pending *= std::pow(w->coin_alpha, -(double)steps);
+    w->drift_pending *= steps == 1 ? 1.0 / w->coin_alpha : std::pow(w->coin_alpha, -(double)steps);
     if (!last && std::fabs(w->drift_pending - 1.0) < 1.0 / 65536) return 1.0;
     const double applied = rounds_to_float(w) ? (double)(float)w->drift_pending : w->drift_pending;
     w->drift_pending /= applied;
@@ -442,6 +433,40 @@ static qw_status clear_next(qw_walk *w) {
     if (e != cudaSuccess) return cuda_error(w, e, "clear");
     w->next_clear = true;
     return QW_OK;
+}
+
+// ---------------------------------------------------------------- clipped 1D launches
+// Tile and depth of the warp tiles on a window of `width` sites, where the plan
+// leaves them open (the sweep, which windows do not run): the choice with the
+// least time per step, from a launch's fixed cost (about 4800 clocks from one
+// launch to the next) and per step the longer of a warp's own chain and the
+// issue of the warps that share its scheduler (an FP64 instruction holds a
+// scheduler for 64 clocks, a double-float operation is about 12 instructions).
+// With the sweep's depth of 8 and 256 sites per warp, the 2001-site FP64 cycle kept
+// three SMs busy for 17 us per launch of 8 steps.
+constexpr int WINDOW_TILE_F64 = 2;   // (WindowTile1D)
+static int max_k_of_tile(int tile) { return tile == WINDOW_TILE_F64 ? 24 : 8 * tile; }
+static void window_plan(const qw_walk *w, int64_t width, int64_t T, int adj, int &tile, int &k) {
+    int tiles[3] = {0, 0, 0};
+    tiles_of(w->prec, tiles[0], tiles[1]);
+    for (int &t : tiles)
+        if (t) t = tile1d(w->prec, t, w->kind, adj);
+    if (w->prec == QW_F64 && w->kind != CK_PERSITE) tiles[2] = WINDOW_TILE_F64;
+    const double unit = w->prec == QW_F64 ? 64 : (w->prec == QW_F32_COMP ? 12 : 1);
+    const double ops = w->kind == CK_SIGN_P || w->kind == CK_SIGN_M ? 4 : (w->kind == CK_REAL ? 8 : 16);
+    const int64_t schedulers = 4 * 152;
+    double best = -1;
+    for (int r : tiles) {
+        if (!r) continue;
+        for (int kk = 8; kk <= max_k_of_tile(r); kk += 8) {
+            const int K = (int)std::min<int64_t>(kk, T);
+            const int64_t W = std::max<int64_t>(1, 32LL * r - 2 * K - 3);
+            const int64_t warps = (width + 2 * K + W - 1) / W;
+            const double chain = r * ops * unit, step = std::max(chain + 40, (double)((warps + schedulers - 1) / schedulers) * chain);
+            const double cost = (4800 + K * step) / K;
+            if (best < 0 || cost < best) { best = cost; tile = r; k = K; }
+        }
+    }
 }
 
 // ---------------------------------------------------------------- momentum-space steps
@@ -609,11 +634,9 @@ qw_status run_steps(qw_walk *w, int64_t T, int adj) {
         a.rthr = w->link_thr;
         a.rk0 = (uint32_t)w->link_seed; a.rk1 = (uint32_t)(w->link_seed >> 32);
         if (w->kind == CK_SIGN_P || w->kind == CK_SIGN_M) a.kind = CK_COMPLEX;   // generic reads the matrix
-        // a clipped forward walk on the segment or the line: as many steps as keep
-        // the box (after them) within one CTA's window go into one launch
-        const bool win_ok = w->ndim == 1 && !adj && w->bc != QW_BC_PERIODIC &&
-                            (w->shift == QW_SHIFT_MOVING || w->shift == QW_SHIFT_FLIPFLOP) && w->nx < (int64_t(1) << 30);
-        const int64_t win_cap = win_ok ? window_capacity(w->prec) : 0;
+        // 1D forward steps: many per launch, on the support box widened by them
+        const bool line = w->ndim == 1 && !adj && (w->shift == QW_SHIFT_MOVING || w->shift == QW_SHIFT_FLIPFLOP) &&
+                          w->nx < (int64_t(1) << 30);
         const bool tiles = !adj && tile2d_walk(w);
         for (int64_t t = 0; t < T; ++t) {
             if (tiles) {
@@ -627,27 +650,22 @@ qw_status run_steps(qw_walk *w, int64_t T, int adj) {
                 t += k - 1;
                 continue;
             }
-            if (win_ok && w->sup_mode == 2) {
-                int ns = (int)std::min<int64_t>(T - t, WINDOW_MAX_STEPS);
-                auto width = [&](int k) {
-                    return std::min<int64_t>(w->nx, w->bx0 + w->bw + k) - std::max<int64_t>(0, w->bx0 - k);
-                };
-                while (ns > 0 && width(ns) > win_cap) --ns;
-                if (ns > 0) {
-                    double gains[WINDOW_MAX_STEPS];
-                    for (int i = 0; i < ns; ++i) gains[i] = drift_gain(w, 1, t + i + 1 == T);
-                    a.rstep = (uint32_t)w->link_step;   // the first step's; step i draws rstep + i
-                    if (w->link_thr) w->link_step += ns;
-                    a.gain = 1.0;
-                    a.in = cur_view(w); a.out = next_view(w);
-                    a.bx0 = w->bx0; a.bw = w->bw; a.by0 = 0; a.bh = 1;
-                    if ((e = stepwin(w->prec, a, cp, gains, ns, w->stream)) != cudaSuccess)
-                        return cuda_error(w, e, "window step launch");
-                    grow_support(w, ns);
-                    w->cur ^= 1;
-                    t += ns - 1;
-                    continue;
-                }
+            if (line) {
+                const int k = (int)std::min<int64_t>(WINDOW_MAX_STEPS, T - t);
+                double gains[WINDOW_MAX_STEPS];
+                for (int i = 0; i < k; ++i) gains[i] = drift_gain(w, 1, t + i + 1 == T);
+                a.rstep = (uint32_t)w->link_step;   // the first step's; step i draws rstep + i
+                if (w->link_thr) w->link_step += k;
+                a.gain = 1.0;
+                a.in = cur_view(w); a.out = next_view(w);
+                int64_t o0, ow;
+                output_range(w->sup_mode == 2, w->bx0, w->bw, w->nx, k, w->bc == QW_BC_PERIODIC, o0, ow);
+                if ((e = stepwin(w->prec, a, cp, gains, k, o0, ow, w->stream)) != cudaSuccess)
+                    return cuda_error(w, e, "window step launch");
+                grow_support(w, k);
+                w->cur ^= 1;
+                t += k - 1;
+                continue;
             }
             // random links: a forward step draws the mask of its index, then counts
             // up; the adjoint counts down first, so it undoes the last forward step
@@ -682,7 +700,8 @@ qw_status run_steps(qw_walk *w, int64_t T, int adj) {
             // if needed; a clipped launch always runs the tiles
             a.variant = (!clip && variant == 1 && sweep_ok(w, a.K, tile)) ? 1 : 0;
             a.tile = a.variant == 1 ? tile : teff;
-            if (a.variant == 0) a.K = std::min(a.K, 8 * teff);
+            if (clip && variant == 1 && !w->plan_user) window_plan(w, w->bw, rem, adj, a.tile, a.K);
+            if (a.variant == 0) a.K = std::min(a.K, max_k_of_tile(a.tile));
             launch_gains_1d(w, a.K, adj, a, true, rem - a.K == 0);
             a.in = cur_view(w); a.out = next_view(w);
             a.obeg = a.oend = 0;
@@ -1319,12 +1338,11 @@ qw_status qw_describe(const qw_walk *w, char *buf, size_t len) {
     const bool generic = w->bc != QW_BC_PERIODIC || links_on(w) ||
                          (w->ndim == 2 && (w->kind == CK_PERSITE ||
                                            (w->kind == CK_PHASE && !(w->prec == QW_F32 || w->prec == QW_F64))));
-    // a clipped walk on the segment or the line whose box (one step on) fits the
-    // window CTA runs its steps in the window kernel
+    // a clipped walk on the segment or the line whose box (one step on) takes the
+    // small tiles of the window kernel
     const bool window = generic && w->ndim == 1 && w->bc != QW_BC_PERIODIC && w->sup_mode == 2 &&
                         (w->shift == QW_SHIFT_MOVING || w->shift == QW_SHIFT_FLIPFLOP) && w->nx < (int64_t(1) << 30) &&
-                        std::min<int64_t>(w->nx, w->bx0 + w->bw + 1) - std::max<int64_t>(0, w->bx0 - 1) <=
-                            window_capacity(w->prec);
+                        std::min<int64_t>(w->nx, w->bx0 + w->bw + 1) - std::max<int64_t>(0, w->bx0 - 1) <= WINDOW_SITES;
     char sup[96];
     if (w->sup_mode == 2)
         std::snprintf(sup, sizeof sup, "[%lld, %lld, %lld, %lld]", (long long)w->bx0, (long long)w->bw,

@@ -402,6 +402,10 @@ struct SupportBox {
     int64_t x0, w, y0, h, nx, ny;
 };
 
+// k_step1d_window: steps per launch, and the widest output range that takes its
+// small tiles
+constexpr int WINDOW_MAX_STEPS = 64;
+constexpr int64_t WINDOW_SITES = 8192;
 // lattice, boundary and links of the generic kernels
 struct GenGeom {
     int ndim;
