@@ -561,6 +561,32 @@ static qw_status run_spectral(qw_walk *w, int64_t T, int adj) {
     return QW_OK;
 }
 
+// Momentum-space steps of the torus: as many of T as its kernels take (all, or
+// with the Grover coin all but an odd one).
+static bool spectral2d_walk(const qw_walk *w) {
+    return w->ndim == 2 && w->bc == QW_BC_PERIODIC && !links_on(w) && spectral2d_ok(w->prec, w->kind, w->shift);
+}
+static qw_status run_spectral2d(qw_walk *w, int64_t &T, int adj) {
+    const bool even = w->kind == CK_GROVER;
+    int64_t rem = even ? T & ~int64_t(1) : T;
+    const Spec2Plan p = spectral2d_plan(w->nx, w->ny, rem, even);
+    if (p.K < 2) return QW_OK;
+    Step2DArgs a{};
+    a.nx = w->nx; a.ny = w->ny; a.shift = w->shift; a.kind = w->kind;
+    while (rem >= 2) {
+        a.K = (int)std::min<int64_t>(p.K, rem);
+        a.gain = take_drift(w, 0, true) / w->gain_fb;   // (these coins are exact in float: what earlier steps left)
+        w->gain_fb = 1.0;
+        a.in = cur_view(w); a.out = next_view(w);
+        cudaError_t e = launch_spectral2d(a, adj, w->spec_table, w->stream);
+        if (e != cudaSuccess) return cuda_error(w, e, "momentum-space step launch");
+        w->cur ^= 1;
+        rem -= a.K;
+        T -= a.K;
+    }
+    return QW_OK;
+}
+
 // ---------------------------------------------------------------- 2D tiles
 // Steps per launch with links or edges: more steps re-read less, but leave a
 // smaller share of the tile as output.  Per step at p = 0.05, 1 (a launch per
@@ -733,6 +759,10 @@ qw_status run_steps(qw_walk *w, int64_t T, int adj) {
         if (w->sup_mode == 2) { b.bx0 = w->bx0; b.bw = w->bw; b.by0 = w->by0; b.bh = w->bh; }
         else { b.bx0 = b.by0 = b.bh = 0; b.bw = 0; }
     };
+    if (w->spec2 && w->sup_mode != 2 && T >= w->spec_min && spectral2d_walk(w)) {
+        const qw_status st = run_spectral2d(w, T, adj);
+        if (st != QW_OK) return st;
+    }
     int K2, t2;
     effective_plan(w, K2, t2);
     if (!adj && K2 > 1) {
@@ -1262,7 +1292,7 @@ qw_status qw_run_host_batch(qw_walk *w, int count, const void *amp_in, int64_t i
     return QW_OK;
 }
 
-static void spectral_off(qw_walk *w) { w->spec_tile = 0; w->spec_user = false; }
+static void spectral_off(qw_walk *w) { w->spec_tile = 0; w->spec_user = w->spec2 = false; }
 
 qw_status qw_set_plan(qw_walk *w, int depth_k, int tile) {
     if (!w) return QW_EINVAL;
@@ -1350,6 +1380,8 @@ qw_status qw_describe(const qw_walk *w, char *buf, size_t len) {
     else
         std::snprintf(sup, sizeof sup, "\"%s\"", w->sup_mode == 1 ? "pending" : "full");
     char spec[96] = "";
+    if (w->spec2 && spectral2d_walk(w))
+        std::snprintf(spec, sizeof spec, ", \"spectral\": {\"from_steps\": %lld}", (long long)w->spec_min);
     if (w->spec_tile && spectral_walk(w))
         std::snprintf(spec, sizeof spec, ", \"spectral\": {\"k\": %d, \"tile\": %d, \"from_steps\": %lld}", w->spec_k,
                       w->spec_tile, (long long)w->spec_min);
@@ -1432,6 +1464,40 @@ cudaError_t time_spectral(qw_walk *w, Spec1DArgs &a, int K, float &ms) {
     return e;
 }
 
+// ms of SPEC2_TUNE_STEPS steps of the torus in momentum space (0: no room for
+// them); the state is unchanged, the other buffer overwritten.
+constexpr int SPEC2_TUNE_STEPS = 256, SPEC2_MIN_STEPS = 64;
+cudaError_t tune_spectral2d(qw_walk *w, float &ms) {
+    ms = 0.f;
+    const Spec2Plan p = spectral2d_plan(w->nx, w->ny, SPEC2_TUNE_STEPS, true);
+    if (p.K < 2) return cudaSuccess;
+    if (!w->spec_table) {
+        if (dev_alloc(&w->spec_table, spectral2d_workspace(w->nx, w->ny)) != cudaSuccess) {
+            (void)cudaGetLastError();
+            w->spec_table = nullptr;
+            return cudaSuccess;   // no room: the stepping plan alone
+        }
+        const cudaError_t e = launch_spectral2d_tables(w->spec_table, w->stream);
+        if (e != cudaSuccess) return e;
+    }
+    Step2DArgs a{};
+    a.nx = w->nx; a.ny = w->ny; a.shift = w->shift; a.kind = w->kind; a.K = p.K; a.gain = 1.0;
+    a.in = cur_view(w); a.out = next_view(w);
+    cudaEvent_t e0 = nullptr, e1 = nullptr;
+    cudaError_t e = launch_spectral2d(a, 0, w->spec_table, w->stream);
+    if (e == cudaSuccess) e = cudaEventCreate(&e0);
+    if (e == cudaSuccess) e = cudaEventCreate(&e1);
+    if (e == cudaSuccess) e = cudaEventRecord(e0, w->stream);
+    if (e == cudaSuccess) e = launch_spectral2d(a, 0, w->spec_table, w->stream);
+    if (e == cudaSuccess) e = cudaEventRecord(e1, w->stream);
+    if (e == cudaSuccess) e = cudaEventSynchronize(e1);
+    if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
+    ms *= (float)SPEC2_TUNE_STEPS / p.K;
+    if (e0) cudaEventDestroy(e0);
+    if (e1) cudaEventDestroy(e1);
+    return e;
+}
+
 void tune_save() {
     const char *path = std::getenv("QW_TUNE_CACHE");
     if (!path) return;
@@ -1487,8 +1553,18 @@ extern "C" qw_status qw_autotune(qw_walk *w, char *report, size_t report_len) {
         cudaEventDestroy(e1);
         if (err != cudaSuccess) return cuda_error(w, err, "autotune");
         w->plan_k = best_k; w->plan_tile = 0; w->plan_user = true;
-        char b2[256];
-        std::snprintf(b2, sizeof b2, "{\"tuned\": true, \"ndim\": 2, \"k\": %d, \"ms_per_step\": %.6g}", best_k, best);
+        char b2[256], sp[64] = "";
+        spectral_off(w);
+        if (spectral2d_walk(w)) {
+            float ms = 0.f;
+            if ((err = tune_spectral2d(w, ms)) != cudaSuccess) return cuda_error(w, err, "autotune");
+            if (ms > 0 && ms < best * SPEC2_TUNE_STEPS) {
+                w->spec2 = true;
+                w->spec_min = std::max<int64_t>(SPEC2_MIN_STEPS, (int64_t)std::ceil(ms / best));
+                std::snprintf(sp, sizeof sp, ", \"spectral\": {\"from_steps\": %lld}", (long long)w->spec_min);
+            }
+        }
+        std::snprintf(b2, sizeof b2, "{\"tuned\": true, \"ndim\": 2, \"k\": %d, \"ms_per_step\": %.6g%s}", best_k, best, sp);
         put(b2);
         return QW_OK;
     }

@@ -98,6 +98,9 @@ struct qw_walk {
     int spec_tile = 0, spec_k = 0;
     int64_t spec_min = 0;
     bool spec_user = false;   // chosen by qw_set_plan_ex
+    // ... of the torus (k_spectral2d.cuh): calls of at least spec_min steps; the
+    // table is then the workspace of the transforms
+    bool spec2 = false;
     void *spec_table = nullptr;
     int spec_tw = 0;
     struct SpecKey {
@@ -189,6 +192,18 @@ size_t spectral1d_table_bytes(int prec);
 cudaError_t launch_spectral1d_twiddles(int prec, int tile, void *table, cudaStream_t s);
 cudaError_t launch_spectral1d_matrices(int prec, const Spec1DArgs &a, const double *coin, double scale, cudaStream_t s);
 cudaError_t launch_spectral1d(int prec, const Spec1DArgs &a, cudaStream_t s);
+
+// momentum-space steps of the torus (spectral2d.cu, FP32): the Grover coin, in
+// even numbers of steps, and H (x) H on the diagonal lattice
+struct Spec2Plan {
+    int K = 0;        // steps per launch (0: none fits)
+    double ms = 0;    // estimated time of all launches
+};
+bool spectral2d_ok(int prec, int kind, int shift);
+size_t spectral2d_workspace(int64_t nx, int64_t ny);
+Spec2Plan spectral2d_plan(int64_t nx, int64_t ny, int64_t T, bool even);
+cudaError_t launch_spectral2d_tables(void *work, cudaStream_t s);
+cudaError_t launch_spectral2d(const Step2DArgs &a, int adjoint, void *work, cudaStream_t s);
 
 // K steps in shared-memory tiles (tile2d.cu, FP32); kind: the global coin, or
 // with a.phi the base coin of the phases; links: broken links or an edge

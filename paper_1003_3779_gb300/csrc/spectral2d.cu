@@ -1,0 +1,222 @@
+// spectral2d.cu -- tables and launchers of the momentum-space torus kernels
+// (k_spectral2d.cuh), FP32.
+#include <algorithm>
+#include <cmath>
+#include <type_traits>
+
+#include "qw_handle.h"
+#include "k_spectral2d.cuh"
+
+namespace qw {
+
+// twiddles of every stage length, and the axis tables of both lengths
+__global__ void k_spec2_twiddles(S2 *tw) {
+    const int id = blockIdx.x * blockDim.x + threadIdx.x;
+    if (id < 32 || id >= SPEC2_TW) return;
+    const int n = 1 << (31 - __clz(id)), i = id - n, k = i / (n / 16), b = i % (n / 16);
+    double s, c;
+    sincospi(-2.0 * k * b / n, &s, &c);
+    tw[id] = {(float)c, (float)s};
+}
+__global__ void k_spec2_axis(Spec2Axis *ax, int L) {
+    const int p = blockIdx.x * blockDim.x + threadIdx.x, n = 1 << L;
+    if (p >= n) return;
+    const double k = (double)spec2_freq(L, p) / n;   // momentum / (2 pi)
+    double s, c, h, g;
+    sincospi(2.0 * k, &s, &c);
+    sincospi(k, &h, &g);
+    h *= h;
+    g *= g;
+    Spec2Axis a;
+    a.s = (float)s;
+    a.sh = (float)h; a.sl = (float)(h - a.sh);
+    a.ch = (float)g; a.cl = (float)(g - a.ch);
+    a.pad = 0.f;
+    ax[p] = a;
+}
+// rows of (diag(e^{-ik}, e^{ik}) H)^K, or of its adjoint, by place
+__global__ void k_spec2_tensor(SpecPair<float> *t, int L, int K, int adj) {
+    const int p = blockIdx.x * blockDim.x + threadIdx.x, n = 1 << L;
+    if (p >= n) return;
+    using Z = Cx<double>;
+    double s, c;
+    sincospi(2.0 * spec2_freq(L, p) / n, &s, &c);
+    const double r = 0.70710678118654752440;
+    const Z u[4] = {{c * r, -s * r}, {c * r, -s * r}, {c * r, s * r}, {-c * r, -s * r}};
+    Z m[4] = {u[0], u[1], u[2], u[3]};
+    auto mul = [](const Z (&a)[4], const Z (&b)[4], Z (&o)[4]) {
+        for (int i = 0; i < 2; ++i)
+            for (int j = 0; j < 2; ++j) o[2 * i + j] = cfma(a[2 * i + 1], b[2 + j], cmul(a[2 * i], b[j]));
+    };
+    for (int bit = 30 - __clz(K); bit >= 0; --bit) {
+        Z q[4];
+        mul(m, m, q);
+        if (K >> bit & 1) mul(q, u, m);
+        else for (int i = 0; i < 4; ++i) m[i] = q[i];
+    }
+    if (adj) {
+        const Z b = m[1];
+        m[1] = {m[2].re, -m[2].im};
+        m[2] = {b.re, -b.im};
+        m[0].im = -m[0].im;
+        m[3].im = -m[3].im;
+    }
+    for (int i = 0; i < 2; ++i)
+        t[2 * p + i] = {{(float)m[2 * i].re, (float)m[2 * i].im}, {(float)m[2 * i + 1].re, (float)m[2 * i + 1].im}};
+}
+
+// tables: twiddles, the axes (places of 2^LX, then 2^LY), their 2 x 2 matrices
+struct Spec2Tables {
+    S2 *tw;
+    Spec2Axis *ax, *ay;
+    SpecPair<float> *tx, *ty;
+};
+static Spec2Tables tables(void *base) {
+    Spec2Tables t;
+    char *p = static_cast<char *>(base);
+    t.tw = reinterpret_cast<S2 *>(p); p += sizeof(S2) * SPEC2_TW;
+    t.tx = reinterpret_cast<SpecPair<float> *>(p); p += sizeof(SpecPair<float>) * 2 << SPEC2_MAX_LX;
+    t.ty = reinterpret_cast<SpecPair<float> *>(p); p += sizeof(SpecPair<float>) * 2 << SPEC2_MAX_LX;
+    t.ax = reinterpret_cast<Spec2Axis *>(p); p += sizeof(Spec2Axis) << SPEC2_MAX_LX;
+    t.ay = reinterpret_cast<Spec2Axis *>(p);
+    return t;
+}
+static constexpr size_t TABLE_BYTES = sizeof(S2) * SPEC2_TW + ((2 * sizeof(SpecPair<float>) * 2) << SPEC2_MAX_LX) +
+                                      ((2 * sizeof(Spec2Axis)) << SPEC2_MAX_LX);
+
+bool spectral2d_ok(int prec, int kind, int shift) {
+    return prec == QW_F32 && (kind == CK_GROVER || (kind == CK_HH && shift == QW_SHIFT_DIAGONAL));
+}
+
+// How an axis of n sites is cut for K steps: the transform length, halo, outputs
+// per block and blocks.
+struct AxisCut {
+    int L = 0, h = 0;
+    int64_t w = 0, blocks = 0;
+    double points() const { return (double)blocks * (1 << L) * (L + 4); }   // (work: points times stages)
+};
+static AxisCut cut_axis(int64_t n, int K, int maxL) {
+    for (int L = SPEC2_MIN_L; L <= maxL; ++L)
+        if (n == (int64_t)1 << L) return {L, 0, n, 1};   // a cycle of its own
+    AxisCut best;
+    for (int L = SPEC2_MIN_L; L <= maxL; ++L) {
+        const int64_t w = ((int64_t)1 << L) - 2 * K;
+        if (w < 1) continue;
+        AxisCut c{L, K, std::min(w, n), (n + w - 1) / w};
+        if (!best.L || c.points() < best.points()) best = c;
+    }
+    return best;
+}
+
+// Workspace: the blocks of one batch, at least one of the largest that is planned.
+size_t spectral2d_workspace(int64_t nx, int64_t ny) {
+    const size_t want = (size_t)nx * ny * 32 * 4;
+    return TABLE_BYTES + std::min<size_t>(size_t(1) << 30, std::max<size_t>(size_t(1) << 26, want));
+}
+
+Spec2Plan spectral2d_plan(int64_t nx, int64_t ny, int64_t T, bool even) {
+    // m launches of about T / m steps; a launch costs its points (about 7e8 point
+    // stages per millisecond) and 20 us for its kernels
+    Spec2Plan best;
+    const size_t room = spectral2d_workspace(nx, ny) - TABLE_BYTES;
+    for (int64_t m = 1; m <= 64 && m <= T; ++m) {
+        int64_t K = (T + m - 1) / m;
+        if (even) K += K & 1;
+        if (K > 4000) continue;
+        const AxisCut x = cut_axis(nx, (int)K, SPEC2_MAX_LX), y = cut_axis(ny, (int)K, SPEC2_MAX_LY);
+        if (!x.L || !y.L || ((size_t)32 << (x.L + y.L)) > room) continue;
+        const double pts = (double)x.blocks * y.blocks * std::ldexp(1.0, x.L + y.L) * (x.L + y.L + 8);
+        const double cost = (double)m * (pts / 7e8 + 0.02);
+        if (best.K == 0 || cost < best.ms) { best.K = (int)K; best.ms = cost; }
+    }
+    return best;
+}
+
+cudaError_t launch_spectral2d_tables(void *work, cudaStream_t s) {
+    k_spec2_twiddles<<<SPEC2_TW / 256, 256, 0, s>>>(tables(work).tw);
+    return cudaGetLastError();
+}
+
+template <int L> static cudaError_t rows(const Spec2Args &a, bool inverse, cudaStream_t s) {
+    constexpr int R = spec2_rows<L>(), TH = (1 << L) / 16 * R;
+    constexpr size_t smem = spec2_row_smem<L>();
+    auto kern = inverse ? k_spec2_rows_inverse<L> : k_spec2_rows_forward<L>;
+    cudaError_t e = smem > 48 * 1024 ? cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) : cudaSuccess;
+    if (e != cudaSuccess) return e;
+    const int64_t n = (int64_t)a.nb * 4 * (inverse ? a.wy : (int64_t)1 << a.LY);
+    kern<<<(unsigned)((n + R - 1) / R), TH, smem, s>>>(a);
+    return cudaGetLastError();
+}
+static cudaError_t rows_any(const Spec2Args &a, bool inverse, cudaStream_t s) {
+    switch (a.LX) {
+        case 8: return rows<8>(a, inverse, s);
+        case 9: return rows<9>(a, inverse, s);
+        case 10: return rows<10>(a, inverse, s);
+        case 11: return rows<11>(a, inverse, s);
+        case 12: return rows<12>(a, inverse, s);
+        case 13: return rows<13>(a, inverse, s);
+    }
+    return cudaErrorInvalidValue;
+}
+template <int L, int MODE> static cudaError_t columns(const Spec2Args &a, const Spec2Coin &c, cudaStream_t s) {
+    constexpr size_t smem = spec2_col_smem<L>();
+    auto kern = k_spec2_columns<L, MODE>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    kern<<<(unsigned)((int64_t)a.nb * (1 << a.LX) / spec2_cols<L>()), spec2_cols<L>() * 4 * (1 << L) / 16, smem, s>>>(a, c);
+    return cudaGetLastError();
+}
+template <int L> static cudaError_t columns_mode(int mode, const Spec2Args &a, const Spec2Coin &c, cudaStream_t s) {
+    switch (mode) {
+        case QW_SHIFT_MOVING: return columns<L, QW_SHIFT_MOVING>(a, c, s);
+        case QW_SHIFT_FLIPFLOP: return columns<L, QW_SHIFT_FLIPFLOP>(a, c, s);
+        case QW_SHIFT_DIAGONAL: return columns<L, QW_SHIFT_DIAGONAL>(a, c, s);
+        case SPEC2_TENSOR: return columns<L, SPEC2_TENSOR>(a, c, s);
+    }
+    return cudaErrorInvalidValue;
+}
+
+// K steps (even for the Grover coin) from a.in to a.out; work: the workspace,
+// with the twiddles in place.
+cudaError_t launch_spectral2d(const Step2DArgs &a, int adjoint, void *work, cudaStream_t s) {
+    const bool tensor = a.kind == CK_HH;
+    const AxisCut x = cut_axis(a.nx, a.K, SPEC2_MAX_LX), y = cut_axis(a.ny, a.K, SPEC2_MAX_LY);
+    if (!x.L || !y.L || a.K < 2 || (!tensor && (a.K & 1))) return cudaErrorInvalidValue;
+    const Spec2Tables t = tables(work);
+    Spec2Args g{};
+    g.in = a.in; g.out = a.out; g.nx = a.nx; g.ny = a.ny;
+    g.wx = x.w; g.wy = y.w; g.hx = x.h; g.hy = y.h; g.nbx = (int)x.blocks; g.LX = x.L; g.LY = y.L;
+    g.z = reinterpret_cast<S2 *>(static_cast<char *>(work) + TABLE_BYTES);
+    g.tw = t.tw;
+    g.scale = (float)(a.gain * std::ldexp(1.0, -(x.L + y.L)));
+    Spec2Coin c{t.ax, t.ay, t.tx, t.ty, a.K, adjoint ? -1.f : 1.f};
+    if (tensor) {
+        k_spec2_tensor<<<(1 << x.L) / 32, 32, 0, s>>>(t.tx, x.L, a.K, adjoint);
+        k_spec2_tensor<<<(1 << y.L) / 32, 32, 0, s>>>(t.ty, y.L, a.K, adjoint);
+    } else {
+        k_spec2_axis<<<(1 << x.L) / 32, 32, 0, s>>>(t.ax, x.L);
+        k_spec2_axis<<<(1 << y.L) / 32, 32, 0, s>>>(t.ay, y.L);
+    }
+    cudaError_t e = cudaGetLastError();
+    const int64_t blocks = x.blocks * y.blocks;
+    const size_t each = (size_t)32 << (x.L + y.L), room = spectral2d_workspace(a.nx, a.ny) - TABLE_BYTES;
+    const int64_t batch = std::max<int64_t>(1, std::min<int64_t>(blocks, (int64_t)(room / each)));
+    for (int64_t b = 0; b < blocks && e == cudaSuccess; b += batch) {
+        g.b0 = (int)b;
+        g.nb = (int)std::min(batch, blocks - b);
+        e = rows_any(g, false, s);
+        const int mode = tensor ? SPEC2_TENSOR : a.shift;
+        if (e == cudaSuccess) switch (y.L) {
+            case 8: e = columns_mode<8>(mode, g, c, s); break;
+            case 9: e = columns_mode<9>(mode, g, c, s); break;
+            case 10: e = columns_mode<10>(mode, g, c, s); break;
+            case 11: e = columns_mode<11>(mode, g, c, s); break;
+            case 12: e = columns_mode<12>(mode, g, c, s); break;
+            default: e = cudaErrorInvalidValue;
+        }
+        if (e == cudaSuccess) e = rows_any(g, true, s);
+    }
+    return e;
+}
+
+}  // namespace qw
