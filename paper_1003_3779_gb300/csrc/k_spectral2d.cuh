@@ -53,6 +53,16 @@ __host__ __device__ inline int spec2_freq(int L, int p) {   // momentum at place
     }
     return f;
 }
+__host__ __device__ inline int spec2_place(int L, int f) {   // place of momentum f
+    int n = 1 << L, p = 0;
+    while (n > 1) {
+        const int r = n >= 16 ? 16 : n, m = n / r;
+        p += f % r * m;
+        f /= r;
+        n = m;
+    }
+    return p;
+}
 __device__ __forceinline__ int spec2_at(int p) { return p + (p >> 4); }   // one pad slot per 16
 
 template <int INV, class R> __device__ __forceinline__ void dft8(Cx<R> (&x)[8]) {
@@ -170,10 +180,20 @@ struct Spec2Args {
     View in, out;
     int64_t nx, ny, wx, wy;
     int hx, hy, nbx, b0, nb, LX, LY;
+    int split;       // the y axis is a cycle of 2^(LY+1): block g transforms (row r +- row r + 2^LY) w^{gr}
     S2 *z;
     const S2 *tw;
     float scale;
 };
+
+// w_n^r, r < n/2, from the stage's twiddles: w_n^{bk} is at n + k n/16 + b, b < n/16
+__device__ __forceinline__ C2 spec2_root(const S2 *tw, int n, int r) {
+    const int m = n / 16, q = r / m;                    // r = q m + b: w^r = w^b w16^q
+    const C2 w = spec_tw(tw, n + m + r % m);            // k = 1: w^b
+    float s, c;
+    sincospif(-0.125f * (float)q, &s, &c);
+    return cmul(w, C2{c, s});
+}
 
 template <int L> constexpr int spec2_rows() { return L >= 12 ? 1 : 4096 >> L; }   // rows per CTA
 template <int L> constexpr size_t spec2_row_smem() { return (size_t)spec2_rows<L>() * ((1 << L) * 17 / 16) * sizeof(S2); }
@@ -188,15 +208,20 @@ k_spec2_rows_forward(Spec2Args a) {
     const int NY = 1 << a.LY;
     const int64_t id = (int64_t)blockIdx.x * spec2_rows<L>() + rr;   // (block, plane, row), a whole number of CTAs
     const int r = (int)(id % NY), c = (int)(id / NY % 4), b = a.b0 + (int)(id / NY / 4);
-    int64_t x0 = ((b % a.nbx) * a.wx - a.hx) % a.nx, y = ((b / a.nbx) * a.wy - a.hy + r) % a.ny;
+    int64_t x0 = ((b % a.nbx) * a.wx - a.hx) % a.nx, y = a.split ? r : ((b / a.nbx) * a.wy - a.hy + r) % a.ny;
     if (x0 < 0) x0 += a.nx;
     if (y < 0) y += a.ny;
+    const C2 w = a.split ? spec2_root(a.tw, 2 * NY, r) : C2{1.f, 0.f};
     C2 x[16];
 #pragma unroll
     for (int i = 0; i < 16; ++i) {
         int64_t s = x0 + t + i * TH;
         if (s >= a.nx) s = a.nx >= N ? s - a.nx : s % a.nx;
         x[i] = St<P_F32>::ld(a.in, c, y * a.nx + s);
+        if (a.split) {
+            const C2 q = St<P_F32>::ld(a.in, c, (y + NY) * a.nx + s);
+            x[i] = b == 0 ? cadd(x[i], q) : spec_twiddle<0>(csub(x[i], q), w);
+        }
     }
     spec2_forward<L>(x, sm, a.tw, t);
     __syncthreads();
@@ -214,14 +239,25 @@ k_spec2_rows_inverse(Spec2Args a) {
     S2 *sm = reinterpret_cast<S2 *>(ssm) + rr * (N * 17 / 16);
     const int64_t rows = (int64_t)a.nb * 4 * a.wy, id = min((int64_t)blockIdx.x * spec2_rows<L>() + rr, rows - 1);
     const int64_t r = id % a.wy;                                     // output row of the block
-    const int c = (int)(id / a.wy % 4), bl = (int)(id / a.wy / 4), b = a.b0 + bl;
-    const S2 *z = a.z + (((int64_t)bl * 4 + c) * (1 << a.LY) + a.hy + r) * N;
+    const int c = (int)(id / a.wy % 4), bl = (int)(id / a.wy / 4), b = a.b0 + bl, NY = 1 << a.LY;
+    const S2 *z = a.z + (((int64_t)(a.split ? 0 : bl) * 4 + c) * NY + a.hy + r) * N;
+    if (!a.split) {
 #pragma unroll
-    for (int i = 0; i < 16; ++i) sm[spec2_at(t + i * TH)] = z[t + i * TH];
+        for (int i = 0; i < 16; ++i) sm[spec2_at(t + i * TH)] = z[t + i * TH];
+    } else {   // rows r and r + 2^LY are even +- odd w^{-r}
+        const C2 w = spec2_root(a.tw, 2 * NY, (int)r);
+        const S2 *o = z + (int64_t)4 * NY * N;
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            const S2 e = z[t + i * TH], q = o[t + i * TH];
+            const C2 u = spec_twiddle<1>(C2{q.re, q.im}, w);
+            sm[spec2_at(t + i * TH)] = bl == 0 ? S2{e.re + u.re, e.im + u.im} : S2{e.re - u.re, e.im - u.im};
+        }
+    }
     __syncthreads();
     C2 x[16];
     spec2_inverse<L>(x, sm, a.tw, t);
-    const int64_t x0 = (b % a.nbx) * a.wx, y = (b / a.nbx) * a.wy + r;
+    const int64_t x0 = (b % a.nbx) * a.wx, y = a.split ? r + (int64_t)bl * NY : (b / a.nbx) * a.wy + r;
     if (y >= a.ny || (int64_t)blockIdx.x * spec2_rows<L>() + rr >= rows) return;
     const int64_t w = min(a.wx, a.nx - x0);
 #pragma unroll
@@ -257,70 +293,85 @@ template <int MODE> __device__ __forceinline__ void spec2_coin(C2 (&v)[4], const
     }
 }
 
-template <int MODE> __device__ __forceinline__ void spec2_power(const Spec2Coin &k, int px, int py, C2 (&v)[4]) {
-    if constexpr (MODE == SPEC2_TENSOR) {
-        const SpecPair<float> a0 = k.tx[2 * px], a1 = k.tx[2 * px + 1], b0 = k.ty[2 * py], b1 = k.ty[2 * py + 1];
-        C2 u[4];   // coin c = 2 j + k: j moves in x, k in y
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            u[q] = cfma(a0.b, v[2 + q], cmul(a0.a, v[q]));
-            u[2 + q] = cfma(a1.b, v[2 + q], cmul(a1.a, v[q]));
-        }
-#pragma unroll
-        for (int j = 0; j < 2; ++j) {
-            v[2 * j] = cfma(b0.b, u[2 * j + 1], cmul(b0.a, u[2 * j]));
-            v[2 * j + 1] = cfma(b1.b, u[2 * j + 1], cmul(b1.a, u[2 * j]));
-        }
+// The coefficients of one momentum: e = E, and s_K and 2 s_{K/2}^2 (the same for
+// ky and -ky).
+struct Spec2Factor {
+    float sK, f2;
+};
+// sin^2(w'/2) and the sign of s_K (see above)
+template <int MODE> __device__ __forceinline__ Spec2Factor spec2_factor(const Spec2Coin &k, const Spec2Axis &X, const Spec2Axis &Y) {
+    const ff one = ff_from(1.f), two = ff_from(2.f);
+    ff u;          // sin^2(w'/2), w' = w or pi - w, in [0, pi/2]
+    float sgn;     // s_K(w) = sgn s_K(w')   (K even)
+    if constexpr (MODE == QW_SHIFT_DIAGONAL) {
+        const bool nx = X.sh > X.ch, ny = Y.sh > Y.ch;   // cos kx, cos ky < 0
+        const ff hx = nx ? ff{X.ch, X.cl} : ff{X.sh, X.sl}, hy = ny ? ff{Y.ch, Y.cl} : ff{Y.sh, Y.sl};
+        u = hx + hy - two * (hx * hy);
+        sgn = nx == ny ? -1.f : 1.f;
     } else {
-        const Spec2Axis X = k.ax[px], Y = k.ay[py];
-        const ff one = ff_from(1.f), two = ff_from(2.f);
-        ff u;          // sin^2(w'/2), w' = w or pi - w, in [0, pi/2]
-        float sgn;     // s_K(w) = sgn s_K(w')   (K even)
-        C2 e[4];
-        if constexpr (MODE == QW_SHIFT_DIAGONAL) {
-            const bool nx = X.sh > X.ch, ny = Y.sh > Y.ch;   // cos kx, cos ky < 0
-            const ff hx = nx ? ff{X.ch, X.cl} : ff{X.sh, X.sl}, hy = ny ? ff{Y.ch, Y.cl} : ff{Y.sh, Y.sl};
-            u = hx + hy - two * (hx * hy);
-            sgn = nx == ny ? -1.f : 1.f;
-            const float gx = nx ? -1.f : 1.f, gy = ny ? -1.f : 1.f;
-            const C2 ex{-2.f * gx * hx.hi, -X.s}, ey{-2.f * gy * hy.hi, -Y.s};   // e^{-ik} - (its sign at w' = 0)
-            const C2 p = cmul(ex, ey), q = conjmul(ey, ex);                      // ex ey, ex conj(ey)
-            e[0] = {gx * ey.re + gy * ex.re + p.re, gx * ey.im + gy * ex.im + p.im};
-            e[1] = {gx * ey.re + gy * ex.re + q.re, -gx * ey.im + gy * ex.im + q.im};
-            e[2] = {e[1].re, -e[1].im};
-            e[3] = {e[0].re, -e[0].im};
-        } else {
-            const bool neg = X.sh + Y.sh > 1.f;              // cos kx + cos ky < 0
-            const ff hx = neg ? ff{X.ch, X.cl} : ff{X.sh, X.sl}, hy = neg ? ff{Y.ch, Y.cl} : ff{Y.sh, Y.sl};
-            u = hx + hy;
-            u = {0.5f * u.hi, 0.5f * u.lo};
-            const float g = neg ? -1.f : 1.f;
-            sgn = MODE == QW_SHIFT_FLIPFLOP ? g : -g;
-            const float dir = MODE == QW_SHIFT_FLIPFLOP ? 1.f : -1.f;   // moving: D_0 = e^{-ikx}; flip-flop: e^{ikx}
-            e[0] = {-2.f * g * hx.hi, dir * X.s};
-            e[1] = {e[0].re, -e[0].im};
-            e[2] = {-2.f * g * hy.hi, dir * Y.s};
-            e[3] = {e[2].re, -e[2].im};
+        const bool neg = X.sh + Y.sh > 1.f;              // cos kx + cos ky < 0
+        const ff hx = neg ? ff{X.ch, X.cl} : ff{X.sh, X.sl}, hy = neg ? ff{Y.ch, Y.cl} : ff{Y.sh, Y.sl};
+        u = hx + hy;
+        u = {0.5f * u.hi, 0.5f * u.lo};
+        sgn = (MODE == QW_SHIFT_FLIPFLOP) == neg ? -1.f : 1.f;
+    }
+    const ff c = one - two * u, s2 = two * two * u * (one - u);   // cos w', sin^2 w'
+    ff C = c, S = one;                                            // of n = 1
+    const int m = k.K / 2;
+    for (int bit = 30 - __clz(m); bit >= 0; --bit) {
+        const ff C1 = two * (C * C) - one;
+        S = two * (S * C);
+        C = C1;
+        if (m >> bit & 1) {
+            const ff C2n = C * c - S * s2;
+            S = S * c + C;
+            C = C2n;
         }
-        const ff c = one - two * u, s2 = two * two * u * (one - u);   // cos w', sin^2 w'
-        ff C = c, S = one;                                            // of n = 1
-        const int m = k.K / 2;
-        for (int bit = 30 - __clz(m); bit >= 0; --bit) {
-            const ff C1 = two * (C * C) - one;
-            S = two * (S * C);
-            C = C1;
-            if (m >> bit & 1) {
-                const ff C2n = C * c - S * s2;
-                S = S * c + C;
-                C = C2n;
-            }
-        }
-        const float sK = k.sign * sgn * 2.f * (S * C).hi, f2 = 2.f * (S * S).hi;
-        C2 x1[4], x2[4];
-        spec2_coin<MODE>(v, e, x1);
-        spec2_coin<MODE>(x1, e, x2);
+    }
+    return {k.sign * sgn * 2.f * (S * C).hi, 2.f * (S * S).hi};
+}
+// U^K v at the momentum (X, Y), or with flip at (kx, -ky)
+template <int MODE>
+__device__ __forceinline__ void spec2_apply(const Spec2Axis &X, const Spec2Axis &Y, bool flip, Spec2Factor f, C2 (&v)[4]) {
+    C2 e[4];
+    const float ys = flip ? -Y.s : Y.s;
+    if constexpr (MODE == QW_SHIFT_DIAGONAL) {
+        const bool nx = X.sh > X.ch, ny = Y.sh > Y.ch;
+        const float hx = nx ? X.ch : X.sh, hy = ny ? Y.ch : Y.sh, gx = nx ? -1.f : 1.f, gy = ny ? -1.f : 1.f;
+        const C2 ex{-2.f * gx * hx, -X.s}, ey{-2.f * gy * hy, -ys};   // e^{-ik} - (its sign at w' = 0)
+        const C2 p = cmul(ex, ey), q = conjmul(ey, ex);               // ex ey, ex conj(ey)
+        e[0] = {gx * ey.re + gy * ex.re + p.re, gx * ey.im + gy * ex.im + p.im};
+        e[1] = {gx * ey.re + gy * ex.re + q.re, -gx * ey.im + gy * ex.im + q.im};
+        e[2] = {e[1].re, -e[1].im};
+        e[3] = {e[0].re, -e[0].im};
+    } else {
+        const bool neg = X.sh + Y.sh > 1.f;
+        const float g = neg ? -1.f : 1.f;
+        const float dir = MODE == QW_SHIFT_FLIPFLOP ? 1.f : -1.f;     // moving: D_0 = e^{-ikx}; flip-flop: e^{ikx}
+        e[0] = {-2.f * g * (neg ? X.ch : X.sh), dir * X.s};
+        e[1] = {e[0].re, -e[0].im};
+        e[2] = {-2.f * g * (neg ? Y.ch : Y.sh), dir * ys};
+        e[3] = {e[2].re, -e[2].im};
+    }
+    C2 x1[4], x2[4];
+    spec2_coin<MODE>(v, e, x1);
+    spec2_coin<MODE>(x1, e, x2);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) v[q] = rfma(f2, x2[q], rfma(sK, x1[q], v[q]));
+    for (int q = 0; q < 4; ++q) v[q] = rfma(f.f2, x2[q], rfma(f.sK, x1[q], v[q]));
+}
+// H (x) H on the diagonal lattice
+__device__ __forceinline__ void spec2_tensor(const Spec2Coin &k, int px, int py, C2 (&v)[4]) {
+    const SpecPair<float> a0 = k.tx[2 * px], a1 = k.tx[2 * px + 1], b0 = k.ty[2 * py], b1 = k.ty[2 * py + 1];
+    C2 u[4];   // coin c = 2 j + k: j moves in x, k in y
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        u[q] = cfma(a0.b, v[2 + q], cmul(a0.a, v[q]));
+        u[2 + q] = cfma(a1.b, v[2 + q], cmul(a1.a, v[q]));
+    }
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        v[2 * j] = cfma(b0.b, u[2 * j + 1], cmul(b0.a, u[2 * j]));
+        v[2 * j + 1] = cfma(b1.b, u[2 * j + 1], cmul(b1.a, u[2 * j]));
     }
 }
 
@@ -345,16 +396,51 @@ k_spec2_columns(Spec2Args a, Spec2Coin coin) {
     for (int i = 0; i < 16; ++i) { const S2 v = z[(int64_t)(t + i * TH) * NX]; x[i] = {v.re, v.im}; }
     spec2_forward<L>(x, sm, a.tw, t);
     __syncthreads();
-#pragma unroll 1
-    for (int q = 0; q < 4; ++q) {
-        const int id = (int)threadIdx.x + q * (4 * C * TH), k = id % C, p = id / C;
-        S2 *m = all + k * spec2_col_stride<L>() + spec2_at(p);
-        C2 v[4];
+    auto get = [&](int k, int p, C2 (&v)[4]) {
+        const S2 *m = all + k * spec2_col_stride<L>() + spec2_at(p);
 #pragma unroll
         for (int d = 0; d < 4; ++d) v[d] = {m[d * PL].re, m[d * PL].im};
-        spec2_power<MODE>(coin, p0 + k, p, v);
+    };
+    auto put = [&](int k, int p, const C2 (&v)[4]) {
+        S2 *m = all + k * spec2_col_stride<L>() + spec2_at(p);
 #pragma unroll
         for (int d = 0; d < 4; ++d) m[d * PL] = {v[d].re, v[d].im};
+    };
+    const int odd = a.split ? a.b0 + bl : 0;             // the odd momenta of a split axis
+    if constexpr (MODE == SPEC2_TENSOR) {
+#pragma unroll 1
+        for (int q = 0; q < 4; ++q) {
+            const int id = (int)threadIdx.x + q * (4 * C * TH), k = id % C, p = id / C;
+            C2 v[4];
+            get(k, p, v);
+            spec2_tensor(coin, p0 + k, odd * N + p, v);
+            put(k, p, v);
+        }
+    } else {
+        // the pairs ky, -ky share their factors: one of each pair has the last
+        // digit of its place in the lower half; f = 0 and N / 2 are their own
+        // partners (of the odd momenta, 2f + 1, none is)
+        constexpr int R = L % 4 ? 1 << (L % 4) : 16, H = R / 2;
+#pragma unroll 1
+        for (int q = 0; q < 2; ++q) {
+            const int id = (int)threadIdx.x + q * (4 * C * TH), k = id % C, h = id / C, p = h / H * R + h % H;
+            const int f = spec2_freq(L, p), g = odd ? N - 1 - f : (N - f) % N;
+            const int p2 = f == 0 && !odd ? spec2_place(L, N / 2) : spec2_place(L, g);
+            const Spec2Axis X = coin.ax[p0 + k], Y = coin.ay[odd * N + p];
+            const Spec2Factor fac = spec2_factor<MODE>(coin, X, Y);
+            C2 v[4];
+            get(k, p, v);
+            spec2_apply<MODE>(X, Y, false, fac, v);
+            put(k, p, v);
+            get(k, p2, v);
+            if (f == 0 && !odd) {
+                const Spec2Axis Z = coin.ay[p2];
+                spec2_apply<MODE>(X, Z, false, spec2_factor<MODE>(coin, X, Z), v);
+            } else {
+                spec2_apply<MODE>(X, Y, true, fac, v);
+            }
+            put(k, p2, v);
+        }
     }
     __syncthreads();
     spec2_inverse<L>(x, sm, a.tw, t);

@@ -578,7 +578,7 @@ static qw_status run_spectral2d(qw_walk *w, int64_t &T, int adj) {
         a.gain = take_drift(w, 0, true) / w->gain_fb;   // (these coins are exact in float: what earlier steps left)
         w->gain_fb = 1.0;
         a.in = cur_view(w); a.out = next_view(w);
-        cudaError_t e = launch_spectral2d(a, adj, w->spec_table, w->stream);
+        cudaError_t e = launch_spectral2d(a, p.K, adj, w->spec_table, w->stream);
         if (e != cudaSuccess) return cuda_error(w, e, "momentum-space step launch");
         w->cur ^= 1;
         rem -= a.K;
@@ -1484,11 +1484,11 @@ cudaError_t tune_spectral2d(qw_walk *w, float &ms) {
     a.nx = w->nx; a.ny = w->ny; a.shift = w->shift; a.kind = w->kind; a.K = p.K; a.gain = 1.0;
     a.in = cur_view(w); a.out = next_view(w);
     cudaEvent_t e0 = nullptr, e1 = nullptr;
-    cudaError_t e = launch_spectral2d(a, 0, w->spec_table, w->stream);
+    cudaError_t e = launch_spectral2d(a, p.K, 0, w->spec_table, w->stream);
     if (e == cudaSuccess) e = cudaEventCreate(&e0);
     if (e == cudaSuccess) e = cudaEventCreate(&e1);
     if (e == cudaSuccess) e = cudaEventRecord(e0, w->stream);
-    if (e == cudaSuccess) e = launch_spectral2d(a, 0, w->spec_table, w->stream);
+    if (e == cudaSuccess) e = launch_spectral2d(a, p.K, 0, w->spec_table, w->stream);
     if (e == cudaSuccess) e = cudaEventRecord(e1, w->stream);
     if (e == cudaSuccess) e = cudaEventSynchronize(e1);
     if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);

@@ -203,7 +203,7 @@ bool spectral2d_ok(int prec, int kind, int shift);
 size_t spectral2d_workspace(int64_t nx, int64_t ny);
 Spec2Plan spectral2d_plan(int64_t nx, int64_t ny, int64_t T, bool even);
 cudaError_t launch_spectral2d_tables(void *work, cudaStream_t s);
-cudaError_t launch_spectral2d(const Step2DArgs &a, int adjoint, void *work, cudaStream_t s);
+cudaError_t launch_spectral2d(const Step2DArgs &a, int cut_K, int adjoint, void *work, cudaStream_t s);
 
 // K steps in shared-memory tiles (tile2d.cu, FP32); kind: the global coin, or
 // with a.phi the base coin of the phases; links: broken links or an edge

@@ -18,10 +18,16 @@ __global__ void k_spec2_twiddles(S2 *tw) {
     sincospi(-2.0 * k * b / n, &s, &c);
     tw[id] = {(float)c, (float)s};
 }
-__global__ void k_spec2_axis(Spec2Axis *ax, int L) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x, n = 1 << L;
-    if (p >= n) return;
-    const double k = (double)spec2_freq(L, p) / n;   // momentum / (2 pi)
+// momentum / (2 pi) at place p; split: places of the even momenta of a cycle of
+// 2^(L+1), then of the odd ones
+__device__ __forceinline__ double spec2_momentum(int L, int p, int split) {
+    const int n = 1 << L;
+    return split ? (2.0 * spec2_freq(L, p % n) + p / n) / (2 * n) : (double)spec2_freq(L, p) / n;
+}
+__global__ void k_spec2_axis(Spec2Axis *ax, int L, int split) {
+    const int p = blockIdx.x * blockDim.x + threadIdx.x;
+    if (p >= 1 << (L + split)) return;
+    const double k = spec2_momentum(L, p, split);
     double s, c, h, g;
     sincospi(2.0 * k, &s, &c);
     sincospi(k, &h, &g);
@@ -35,12 +41,12 @@ __global__ void k_spec2_axis(Spec2Axis *ax, int L) {
     ax[p] = a;
 }
 // rows of (diag(e^{-ik}, e^{ik}) H)^K, or of its adjoint, by place
-__global__ void k_spec2_tensor(SpecPair<float> *t, int L, int K, int adj) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x, n = 1 << L;
-    if (p >= n) return;
+__global__ void k_spec2_tensor(SpecPair<float> *t, int L, int split, int K, int adj) {
+    const int p = blockIdx.x * blockDim.x + threadIdx.x;
+    if (p >= 1 << (L + split)) return;
     using Z = Cx<double>;
     double s, c;
-    sincospi(2.0 * spec2_freq(L, p) / n, &s, &c);
+    sincospi(2.0 * spec2_momentum(L, p, split), &s, &c);
     const double r = 0.70710678118654752440;
     const Z u[4] = {{c * r, -s * r}, {c * r, -s * r}, {c * r, s * r}, {-c * r, -s * r}};
     Z m[4] = {u[0], u[1], u[2], u[3]};
@@ -91,27 +97,36 @@ bool spectral2d_ok(int prec, int kind, int shift) {
 // How an axis of n sites is cut for K steps: the transform length, halo, outputs
 // per block and blocks.
 struct AxisCut {
-    int L = 0, h = 0;
+    int L = 0, h = 0, split = 0;
     int64_t w = 0, blocks = 0;
     double points() const { return (double)blocks * (1 << L) * (L + 4); }   // (work: points times stages)
 };
-static AxisCut cut_axis(int64_t n, int K, int maxL) {
+static AxisCut cut_axis(int64_t n, int K, int maxL, bool may_split = false) {
     for (int L = SPEC2_MIN_L; L <= maxL; ++L)
-        if (n == (int64_t)1 << L) return {L, 0, n, 1};   // a cycle of its own
+        if (n == (int64_t)1 << L) return {L, 0, 0, n, 1};   // a cycle of its own
+    if (may_split && n == (int64_t)2 << maxL) return {maxL, 0, 1, n / 2, 2};   // ... in two halves
     AxisCut best;
     for (int L = SPEC2_MIN_L; L <= maxL; ++L) {
         const int64_t w = ((int64_t)1 << L) - 2 * K;
         if (w < 1) continue;
-        AxisCut c{L, K, std::min(w, n), (n + w - 1) / w};
+        AxisCut c{L, K, 0, std::min(w, n), (n + w - 1) / w};
         if (!best.L || c.points() < best.points()) best = c;
     }
     return best;
 }
 
+// both axes, and whether a batch of them fits the workspace (the halves of a split
+// column are combined on the way back, so they are one batch: one block of rows)
+static bool cut_axes(int64_t nx, int64_t ny, int K, size_t room, AxisCut &x, AxisCut &y) {
+    x = cut_axis(nx, K, SPEC2_MAX_LX);
+    y = cut_axis(ny, K, SPEC2_MAX_LY, x.blocks == 1);
+    return x.L && y.L && ((size_t)32 << (x.L + y.L + y.split)) <= room;
+}
+
 // Workspace: the blocks of one batch, at least one of the largest that is planned.
 size_t spectral2d_workspace(int64_t nx, int64_t ny) {
     const size_t want = (size_t)nx * ny * 32 * 4;
-    return TABLE_BYTES + std::min<size_t>(size_t(1) << 30, std::max<size_t>(size_t(1) << 26, want));
+    return TABLE_BYTES + std::min<size_t>(size_t(1) << 31, std::max<size_t>(size_t(1) << 26, want));
 }
 
 Spec2Plan spectral2d_plan(int64_t nx, int64_t ny, int64_t T, bool even) {
@@ -123,8 +138,8 @@ Spec2Plan spectral2d_plan(int64_t nx, int64_t ny, int64_t T, bool even) {
         int64_t K = (T + m - 1) / m;
         if (even) K += K & 1;
         if (K > 4000) continue;
-        const AxisCut x = cut_axis(nx, (int)K, SPEC2_MAX_LX), y = cut_axis(ny, (int)K, SPEC2_MAX_LY);
-        if (!x.L || !y.L || ((size_t)32 << (x.L + y.L)) > room) continue;
+        AxisCut x, y;
+        if (!cut_axes(nx, ny, (int)K, room, x, y)) continue;
         const double pts = (double)x.blocks * y.blocks * std::ldexp(1.0, x.L + y.L) * (x.L + y.L + 8);
         const double cost = (double)m * (pts / 7e8 + 0.02);
         if (best.K == 0 || cost < best.ms) { best.K = (int)K; best.ms = cost; }
@@ -176,31 +191,31 @@ template <int L> static cudaError_t columns_mode(int mode, const Spec2Args &a, c
     return cudaErrorInvalidValue;
 }
 
-// K steps (even for the Grover coin) from a.in to a.out; work: the workspace,
-// with the twiddles in place.
-cudaError_t launch_spectral2d(const Step2DArgs &a, int adjoint, void *work, cudaStream_t s) {
+// a.K steps (even for the Grover coin) from a.in to a.out, on the blocks of a
+// launch of cut_K >= a.K; work: the workspace, with the twiddles in place.
+cudaError_t launch_spectral2d(const Step2DArgs &a, int cut_K, int adjoint, void *work, cudaStream_t s) {
     const bool tensor = a.kind == CK_HH;
-    const AxisCut x = cut_axis(a.nx, a.K, SPEC2_MAX_LX), y = cut_axis(a.ny, a.K, SPEC2_MAX_LY);
-    if (!x.L || !y.L || a.K < 2 || (!tensor && (a.K & 1))) return cudaErrorInvalidValue;
+    const size_t room = spectral2d_workspace(a.nx, a.ny) - TABLE_BYTES;
+    AxisCut x, y;
+    if (a.K < 2 || a.K > cut_K || (!tensor && (a.K & 1)) || !cut_axes(a.nx, a.ny, cut_K, room, x, y)) return cudaErrorInvalidValue;
     const Spec2Tables t = tables(work);
     Spec2Args g{};
     g.in = a.in; g.out = a.out; g.nx = a.nx; g.ny = a.ny;
-    g.wx = x.w; g.wy = y.w; g.hx = x.h; g.hy = y.h; g.nbx = (int)x.blocks; g.LX = x.L; g.LY = y.L;
+    g.wx = x.w; g.wy = y.w; g.hx = x.h; g.hy = y.h; g.nbx = (int)x.blocks; g.LX = x.L; g.LY = y.L; g.split = y.split;
     g.z = reinterpret_cast<S2 *>(static_cast<char *>(work) + TABLE_BYTES);
     g.tw = t.tw;
-    g.scale = (float)(a.gain * std::ldexp(1.0, -(x.L + y.L)));
+    g.scale = (float)(a.gain * std::ldexp(1.0, -(x.L + y.L + y.split)));
     Spec2Coin c{t.ax, t.ay, t.tx, t.ty, a.K, adjoint ? -1.f : 1.f};
     if (tensor) {
-        k_spec2_tensor<<<(1 << x.L) / 32, 32, 0, s>>>(t.tx, x.L, a.K, adjoint);
-        k_spec2_tensor<<<(1 << y.L) / 32, 32, 0, s>>>(t.ty, y.L, a.K, adjoint);
+        k_spec2_tensor<<<(1 << x.L) / 32, 32, 0, s>>>(t.tx, x.L, 0, a.K, adjoint);
+        k_spec2_tensor<<<(1 << (y.L + y.split)) / 32, 32, 0, s>>>(t.ty, y.L, y.split, a.K, adjoint);
     } else {
-        k_spec2_axis<<<(1 << x.L) / 32, 32, 0, s>>>(t.ax, x.L);
-        k_spec2_axis<<<(1 << y.L) / 32, 32, 0, s>>>(t.ay, y.L);
+        k_spec2_axis<<<(1 << x.L) / 32, 32, 0, s>>>(t.ax, x.L, 0);
+        k_spec2_axis<<<(1 << (y.L + y.split)) / 32, 32, 0, s>>>(t.ay, y.L, y.split);
     }
     cudaError_t e = cudaGetLastError();
     const int64_t blocks = x.blocks * y.blocks;
-    const size_t each = (size_t)32 << (x.L + y.L), room = spectral2d_workspace(a.nx, a.ny) - TABLE_BYTES;
-    const int64_t batch = std::max<int64_t>(1, std::min<int64_t>(blocks, (int64_t)(room / each)));
+    const int64_t batch = std::min<int64_t>(blocks, (int64_t)(room / ((size_t)32 << (x.L + y.L))));
     for (int64_t b = 0; b < blocks && e == cudaSuccess; b += batch) {
         g.b0 = (int)b;
         g.nb = (int)std::min(batch, blocks - b);

@@ -63,7 +63,8 @@ def check(qw, psi0, coin, T, shift=0, adjoint=False, force=True):
 GROVER, HH = inputs.grover(), inputs.hadamard2()
 
 
-@pytest.mark.parametrize("dims", [(256, 256), (512, 1024), (1024, 256), (2048, 512), (300, 200), (1000, 700), (257, 1025)])
+@pytest.mark.parametrize("dims", [(256, 256), (512, 1024), (1024, 256), (2048, 512), (300, 200), (1000, 700), (257, 1025), (256, 8192),
+                                  (300, 8192), (8192, 300)])
 @pytest.mark.parametrize("coin,shift", [("grover", 0), ("grover", 1), ("grover", 2), ("hh", 2)])
 @pytest.mark.parametrize("adjoint", [False, True])
 def test_sizes_shifts_and_directions(qw, dims, coin, shift, adjoint):
