@@ -293,7 +293,9 @@ static cudaError_t support_t(const void *src, View v, int nslots, int64_t nx, in
     const int64_t tiles = ((ns + SPV - 1) / SPV + SUP_THREADS - 1) / SUP_THREADS;
     const unsigned grid = (unsigned)std::min<int64_t>(tiles, 152 * 8);
     char *dst = static_cast<char *>(v.p);
-    k_support_init<SB><<<1, SUP_THREADS, 0, s>>>(src ? nullptr : dst, slot, nslots, nx, ns, box);
+    // (the first look saves reading a dense state, but costs 2 us: not for small ones)
+    const bool look = !src && nslots * ns * SB > (int64_t(32) << 20);
+    k_support_init<SB><<<1, SUP_THREADS, 0, s>>>(look ? dst : nullptr, slot, nslots, nx, ns, box);
     if (src) k_support<SB, true, V><<<grid, SUP_THREADS, 0, s>>>(static_cast<const char *>(src), dst, slot, nslots, nx, ns, box);
     else k_support<SB, false, V><<<grid, SUP_THREADS, 0, s>>>(nullptr, dst, slot, nslots, nx, ns, box);
     return cudaGetLastError();

@@ -93,9 +93,15 @@ k_step1d_window(View in, View out, GenGeom g, CoinP<typename St<P>::real> cp,
             win_slot<SH>(1, t, t1, d1);
             const int s0 = (i + d0) & M, s1 = (i + d1) & M;
             const C a0 = S::ld(sv, t0, s0), a1 = S::ld(sv, t1, s1);
-            auto entry = [&](int e) { return CK == CK_PERSITE ? m[CK == CK_PERSITE ? k : 0][e] : C{cp.re[e], cp.im[e]}; };
-            C v0 = cfma(entry(1), a1, cfma(entry(0), a0, czero<real>()));
-            C v1 = cfma(entry(3), a1, cfma(entry(2), a0, czero<real>()));
+            C v0, v1;
+            if constexpr (CK == CK_REAL) {   // (the full row's products with its zero imaginary parts left out)
+                v0 = rfma(cp.re[1], a1, rfma(cp.re[0], a0, czero<real>()));
+                v1 = rfma(cp.re[3], a1, rfma(cp.re[2], a0, czero<real>()));
+            } else {
+                auto entry = [&](int e) { return CK == CK_PERSITE ? m[CK == CK_PERSITE ? k : 0][e] : C{cp.re[e], cp.im[e]}; };
+                v0 = cfma(entry(1), a1, cfma(entry(0), a0, czero<real>()));
+                v1 = cfma(entry(3), a1, cfma(entry(2), a0, czero<real>()));
+            }
             if (!one) { v0 = rmul(gain, v0); v1 = rmul(gain, v1); }
             S::st(sv, t0, s0, v0);
             S::st(sv, t1, s1, v1);

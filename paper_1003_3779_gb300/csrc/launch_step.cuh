@@ -392,15 +392,21 @@ static cudaError_t gowin(const StepGenericArgs &a, const CoinP<typename St<P>::r
     return cudaGetLastError();
 }
 
+// the small tile: 256 sites; 64 in FP64, where a tile is bound by its SM's two
+// lanes a clock (and takes at most 16 steps, see window1d_steps)
+template <int P> struct WindowTile { static constexpr int E = 256; };
+template <> struct WindowTile<P_F64> { static constexpr int E = 64; };
+
 template <int P, int CK>
 static cudaError_t gowin_shift(const StepGenericArgs &a, const CoinP<typename St<P>::real> &cp, const double *gains, int nsteps,
                                int64_t o0, int64_t ow, cudaStream_t s) {
-    const bool narrow = ow <= WINDOW_SITES;
+    constexpr int E = WindowTile<P>::E;
+    const bool narrow = ow <= WINDOW_SITES && 4 * nsteps <= E;
     if (a.shift == QW_SHIFT_MOVING)
-        return narrow ? gowin<P, CK, QW_SHIFT_MOVING, 256, 256>(a, cp, gains, nsteps, o0, ow, s)
+        return narrow ? gowin<P, CK, QW_SHIFT_MOVING, E, E>(a, cp, gains, nsteps, o0, ow, s)
                       : gowin<P, CK, QW_SHIFT_MOVING, 2048, 512>(a, cp, gains, nsteps, o0, ow, s);
     if (a.shift == QW_SHIFT_FLIPFLOP)
-        return narrow ? gowin<P, CK, QW_SHIFT_FLIPFLOP, 256, 256>(a, cp, gains, nsteps, o0, ow, s)
+        return narrow ? gowin<P, CK, QW_SHIFT_FLIPFLOP, E, E>(a, cp, gains, nsteps, o0, ow, s)
                       : gowin<P, CK, QW_SHIFT_FLIPFLOP, 2048, 512>(a, cp, gains, nsteps, o0, ow, s);
     return cudaErrorInvalidValue;
 }
@@ -411,9 +417,12 @@ cudaError_t window1d_t(const StepGenericArgs &a, const void *coinp, const double
     const auto &cp = *static_cast<const CoinP<typename St<P>::real> *>(coinp);
     if (a.ndim != 1 || a.adjoint || a.nx >= (int64_t(1) << 30) || nsteps < 1 || nsteps > WINDOW_MAX_STEPS || ow < 1)
         return cudaErrorInvalidValue;
-    // (phase coins are expanded to per-site matrices in 1D); global coins as the full matrix
-    return a.kind == CK_PERSITE ? gowin_shift<P, CK_PERSITE>(a, cp, gains, nsteps, o0, ow, s)
-                                : gowin_shift<P, CK_COMPLEX>(a, cp, gains, nsteps, o0, ow, s);
+    // (phase coins are expanded to per-site matrices in 1D)
+    switch (a.kind) {
+        case CK_PERSITE: return gowin_shift<P, CK_PERSITE>(a, cp, gains, nsteps, o0, ow, s);
+        case CK_REAL: return gowin_shift<P, CK_REAL>(a, cp, gains, nsteps, o0, ow, s);
+        default: return gowin_shift<P, CK_COMPLEX>(a, cp, gains, nsteps, o0, ow, s);
+    }
 }
 
 }  // namespace qw

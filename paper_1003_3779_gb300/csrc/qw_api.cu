@@ -659,7 +659,7 @@ qw_status run_steps(qw_walk *w, int64_t T, int adj) {
         a.links = w->has_links ? w->links_dev : nullptr; a.adjoint = adj;
         a.rthr = w->link_thr;
         a.rk0 = (uint32_t)w->link_seed; a.rk1 = (uint32_t)(w->link_seed >> 32);
-        if (w->kind == CK_SIGN_P || w->kind == CK_SIGN_M) a.kind = CK_COMPLEX;   // generic reads the matrix
+        if (w->kind == CK_SIGN_P || w->kind == CK_SIGN_M) a.kind = CK_REAL;   // generic reads the matrix
         // 1D forward steps: many per launch, on the support box widened by them
         const bool line = w->ndim == 1 && !adj && (w->shift == QW_SHIFT_MOVING || w->shift == QW_SHIFT_FLIPFLOP) &&
                           w->nx < (int64_t(1) << 30);
@@ -677,7 +677,8 @@ qw_status run_steps(qw_walk *w, int64_t T, int adj) {
                 continue;
             }
             if (line) {
-                const int k = (int)std::min<int64_t>(WINDOW_MAX_STEPS, T - t);
+                const int64_t wide = w->sup_mode == 2 ? w->bw + 2 * WINDOW_MAX_STEPS : w->nx;
+                const int k = (int)std::min<int64_t>(window1d_steps(w->prec, wide), T - t);
                 double gains[WINDOW_MAX_STEPS];
                 for (int i = 0; i < k; ++i) gains[i] = drift_gain(w, 1, t + i + 1 == T);
                 a.rstep = (uint32_t)w->link_step;   // the first step's; step i draws rstep + i

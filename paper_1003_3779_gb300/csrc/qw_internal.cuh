@@ -406,6 +406,8 @@ struct SupportBox {
 // small tiles
 constexpr int WINDOW_MAX_STEPS = 64;
 constexpr int64_t WINDOW_SITES = 8192;
+// steps per launch for an output range of ow sites: a quarter of the small tile
+inline int window1d_steps(int prec, int64_t ow) { return prec == P_F64 && ow <= WINDOW_SITES ? 16 : WINDOW_MAX_STEPS; }
 // lattice, boundary and links of the generic kernels
 struct GenGeom {
     int ndim;
