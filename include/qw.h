@@ -444,7 +444,12 @@ int qw_batch_cta_walks(const qw_batch *b);
 
 /* Time the batch for k in {8, ..., 128} and both variants (each timing runs
  * the whole batch from its initial states) and keep the fastest; report as
- * for qw_autotune. */
+ * for qw_autotune.  An FP32 batch whose walks all have unitary coins and at most
+ * 8191 steps is also timed in momentum space ("spectral" in the report): each
+ * walk's final state in one transform, as accurate in norm as stepping (about
+ * 3e-7), exactly zero outside the light cone and on the sites of the other
+ * parity; walks with a coin entry within 2^-18 of modulus 1 are stepped beside
+ * it.  Where that is faster, qw_batch_step runs it until a plan is set. */
 qw_status qw_batch_autotune(qw_batch *b, char *report, size_t report_len);
 
 /* Probabilities of all walks, concatenated in walk order (walk i starts at

@@ -31,6 +31,7 @@
 // no waits other than __syncthreads / __syncwarp: nothing spins.
 #include <algorithm>
 #include <cmath>
+#include <complex>
 #include <cstring>
 #include <new>
 #include <numeric>
@@ -452,6 +453,92 @@ k_batch_sweep(BatchArgs a) {
     }
 }
 
+// ---------------------------------------------------------------- near-diagonal walks
+// Beside the batch's transforms (spectral_batch.cu): walks whose coin has an
+// entry within 2^-18 of modulus 1 go on being stepped in float, so that every
+// plan gives the same for them.  (Their amplitudes hardly change over the walk, so
+// float rounding is systematic and P up to 2e-4 off after 4096 steps, whatever
+// the order of the steps; a double-float batch is the form that resolves them.)
+// A few walks on a CTA each would be the batch's critical path, so all of them
+// take NEAR_STEPS steps per launch on tiles of NEAR_E sites, a site per thread,
+// updated in place in shared memory as in k_window1d.cuh (4096 walks, about 15 of
+// them near-diagonal: 1.7 ms with a register tile of 512 sites per warp).
+constexpr int NEAR_STEPS = 64, NEAR_E = 256;
+constexpr int NEAR_W = NEAR_E - 2 * NEAR_STEPS;   // outputs per tile
+
+__global__ void k_near_start(BatchArgs a, const int *__restrict__ ids) {
+    const WalkDesc d = a.walks[ids[blockIdx.y]];
+    float2 *s = static_cast<float2 *>(a.buf0) + d.base, *o = static_cast<float2 *>(a.buf1) + d.base;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < d.pitch; i += (int64_t)gridDim.x * blockDim.x) {
+        const bool here = i == d.x0;
+        s[i] = here ? make_float2(a.cs[0], a.cs[1]) : make_float2(0.f, 0.f);
+        s[d.pitch + i] = here ? make_float2(a.cs[2], a.cs[3]) : make_float2(0.f, 0.f);
+        o[i] = o[d.pitch + i] = make_float2(0.f, 0.f);
+    }
+}
+
+// steps [t0, t0 + NEAR_STEPS) of every walk: block blockIdx.x takes a tile of the
+// cone after them
+template <int CK>
+__global__ void __launch_bounds__(NEAR_E)
+k_near_steps(BatchArgs a, const int *__restrict__ ids, int t0) {
+    __shared__ float2 sm[2][NEAR_E];
+    const WalkDesc d = a.walks[ids[blockIdx.y]];
+    if (t0 >= d.T) return;
+    const int k = (int)min((int64_t)NEAR_STEPS, d.T - t0), i = (int)threadIdx.x, M = NEAR_E - 1;
+    const int64_t r = t0 + k, width = min(d.n, 2 * r + 1), b = (int64_t)blockIdx.x * NEAR_W;
+    if (b >= width) return;
+    const float2 *in = static_cast<const float2 *>(t0 / NEAR_STEPS & 1 ? a.buf1 : a.buf0) + d.base;
+    float2 *out = static_cast<float2 *>(t0 / NEAR_STEPS & 1 ? a.buf0 : a.buf1) + d.base;
+    // thread i's site: output b + i - NEAR_STEPS of [x0 - r, x0 + r] (or of the cycle), modulo n
+    int64_t x = ((width < d.n ? d.x0 - r : 0) + b + i - NEAR_STEPS) % d.n;
+    if (x < 0) x += d.n;
+    sm[0][i] = in[x];
+    sm[1][i] = in[d.pitch + x];
+    CoinP<float> cp;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) { cp.re[e] = d.c[2 * e]; cp.im[e] = d.c[2 * e + 1]; }
+    __syncthreads();
+    for (int t = 0; t < k; ++t) {   // coin 0 moves to x - 1: slot x + t of plane 0; coin 1: slot x - t
+        const int s0 = (i + t) & M, s1 = (i - t) & M;
+        const float2 u = sm[0][s0], v = sm[1][s1];
+        Cx<float> p0, p1;
+        coin2<CK>(cp, (const Cx<float> *)nullptr, Cx<float>{u.x, u.y}, Cx<float>{v.x, v.y}, p0, p1);
+        sm[0][s0] = make_float2(p0.re, p0.im);
+        sm[1][s1] = make_float2(p1.re, p1.im);
+        __syncthreads();
+    }
+    if (i < NEAR_STEPS || i >= NEAR_E - NEAR_STEPS || b + i - NEAR_STEPS >= width) return;
+    const float g = t0 + k >= d.T ? d.g_last : d.g_main;
+    const float2 u = sm[0][(i + k) & M], v = sm[1][(i - k) & M];
+    out[x] = make_float2(g * u.x, g * u.y);
+    out[d.pitch + x] = make_float2(g * v.x, g * v.y);
+}
+
+__global__ void __launch_bounds__(1024) k_near_finish(BatchArgs a, const int *__restrict__ ids) {
+    __shared__ double red[32];
+    const int w = ids[blockIdx.x];
+    const WalkDesc d = a.walks[w];
+    const int cur = (int)((d.T + NEAR_STEPS - 1) / NEAR_STEPS & 1);
+    const View v{static_cast<float2 *>(cur ? a.buf1 : a.buf0) + d.base, d.pitch, 2};
+    double acc = 0.0;
+    for (int64_t x = threadIdx.x; x < d.n; x += blockDim.x) {
+        double pd;
+        a.P[d.poff + x] = site_prob<P_F32>(v, x, pd);
+        acc += pd;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double tot = 0.0;
+        for (int i = 0; i < 32; ++i) tot += red[i];
+        a.norms[w] = tot;
+        a.final_buf[w] = cur;
+    }
+}
+
 }  // namespace qw
 
 using namespace qw;
@@ -480,6 +567,18 @@ struct qw_batch {
     int grid = 0, grid1 = 0;            // persistent grid of each variant (one wave)
     float cs[4] = {0, 0, 0, 0};
     float cs_lo[4] = {0, 0, 0, 0};
+    // momentum space (spectral_batch.cu), chosen by the autotuner: the walks by
+    // transform length, their count per length, the tables
+    bool spectral = false;
+    SpecWalk *spec_walks = nullptr;
+    int spec_count[SPEC_BATCH_CLASSES] = {0};
+    void *spec_table = nullptr;
+    // ... and its near-diagonal walks, which are stepped on a stream beside it
+    int *near_ids = nullptr;
+    int near_count = 0;
+    int64_t near_T = 0, near_n = 0;     // the longest of them, the largest cycle
+    cudaStream_t side = nullptr;
+    cudaEvent_t fork = nullptr, join = nullptr;
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
     bool ran = false;
@@ -526,6 +625,31 @@ static cudaError_t launch_batch_kernel(qw_batch *b, const BatchArgs &a, cudaStre
     return cudaSuccess;
 }
 
+// The transforms on s, the near-diagonal walks beside them.
+static cudaError_t batch_launch_spectral(qw_batch *b, const BatchArgs &a, cudaStream_t s) {
+    cudaError_t e = cudaSuccess;
+    if (b->near_count) {
+        e = cudaEventRecord(b->fork, s);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(b->side, b->fork, 0);
+        if (e != cudaSuccess) return e;
+        const unsigned n = (unsigned)b->near_count;
+        k_near_start<<<dim3(16, n), 256, 0, b->side>>>(a, b->near_ids);
+        for (int64_t t = 0; t < b->near_T; t += NEAR_STEPS) {
+            const int64_t width = std::min(b->near_n, 2 * (t + NEAR_STEPS) + 1);
+            const dim3 grid((unsigned)((width + NEAR_W - 1) / NEAR_W), n);
+            if (b->kind == CK_REAL) k_near_steps<CK_REAL><<<grid, NEAR_E, 0, b->side>>>(a, b->near_ids, (int)t);
+            else k_near_steps<CK_COMPLEX><<<grid, NEAR_E, 0, b->side>>>(a, b->near_ids, (int)t);
+        }
+        k_near_finish<<<n, 1024, 0, b->side>>>(a, b->near_ids);
+        e = cudaGetLastError();
+        if (e == cudaSuccess) e = cudaEventRecord(b->join, b->side);
+        if (e != cudaSuccess) return e;
+    }
+    e = launch_batch_spectral(b->spec_walks, b->spec_count, b->buf[0], b->P_dev, b->norms_dev, b->final_dev, b->spec_table, s);
+    if (e == cudaSuccess && b->near_count) e = cudaStreamWaitEvent(s, b->join, 0);
+    return e;
+}
+
 static cudaError_t batch_launch(qw_batch *b, cudaStream_t s) {
     BatchArgs a{};
     a.walks = b->walks_dev; a.order = b->order_dev; a.nwalks = b->nwalks;
@@ -534,6 +658,7 @@ static cudaError_t batch_launch(qw_batch *b, cudaStream_t s) {
     std::memcpy(a.cs, b->cs, sizeof a.cs);
     std::memcpy(a.cs_lo, b->cs_lo, sizeof a.cs_lo);
     a.nbig = b->nbig;
+    if (b->spectral) return batch_launch_spectral(b, a, s);
     cudaError_t e = cudaMemsetAsync(b->counter, 0, 2 * sizeof(int), s);
     if (e != cudaSuccess) return e;
     if (b->prec == QW_F32_COMP) {   // warp tiles only (no double-float sweep)
@@ -567,6 +692,91 @@ static void drop_graph(qw_batch *b) {
     b->graph = nullptr;
 }
 
+// Back to stepping: a plan was set.
+static void batch_spectral_off(qw_batch *b) {
+    if (!b->spectral) return;
+    cudaStreamSynchronize(b->stream);
+    drop_graph(b);
+    b->spectral = false;
+}
+
+// The walks of the batch in momentum space, if all of them can run there: FP32,
+// T + 1 <= 8192, a unitary coin (to 1e-6); near-diagonal ones are set aside for
+// k_near_steps.  The coin is the one that stepping
+// applies, rounded to float; its nearest e^{i delta} SU(2) is taken, as stepping
+// divides the norm's drift back out.  false: not all, or no memory.
+static bool batch_spectral_prepare(qw_batch *b) {
+    if (b->spec_walks) return true;
+    if (b->prec != QW_F32) return false;
+    std::vector<SpecWalk> by[SPEC_BATCH_CLASSES];
+    std::vector<int> near;
+    b->near_T = b->near_n = 0;
+    for (int i = 0; i < b->nwalks; ++i) {
+        const WalkDesc &d = b->walks[i];
+        const int L = batch_spectral_length(d.T);
+        if (!L) return false;
+        typedef std::complex<double> Z;
+        Z c[4];
+        for (int e = 0; e < 4; ++e) c[e] = Z(d.c[2 * e], d.c[2 * e + 1]);
+        for (int p = 0; p < 2; ++p)
+            for (int q = 0; q < 2; ++q) {
+                const Z g = std::conj(c[p]) * c[q] + std::conj(c[2 + p]) * c[2 + q] - (p == q ? 1.0 : 0.0);
+                if (!(std::abs(g) <= 1e-6)) return false;
+            }
+        if (std::max(std::abs(c[0]), std::abs(c[1])) >= 1.0 - 0x1p-18) {
+            near.push_back(i);
+            b->near_T = std::max(b->near_T, d.T);
+            b->near_n = std::max(b->near_n, d.n);
+            continue;
+        }
+        const double delta = std::arg(c[0] * c[3] - c[1] * c[2]) / 2;
+        const Z u = std::polar(1.0, -delta);
+        Z alpha = (c[0] * u + std::conj(c[3] * u)) / 2.0, beta = (c[1] * u - std::conj(c[2] * u)) / 2.0;
+        const double norm = std::sqrt(std::norm(alpha) + std::norm(beta));
+        alpha /= norm;
+        beta /= norm;
+        SpecWalk w{};
+        w.n = d.n; w.x0 = d.x0; w.base = d.base; w.pitch = d.pitch; w.poff = d.poff;
+        w.T = (int)d.T; w.id = i;
+        const double a[2] = {alpha.real(), alpha.imag()}, b2 = std::norm(beta);
+        for (int e = 0; e < 2; ++e) { w.ah[e] = (float)a[e]; w.al[e] = (float)(a[e] - (double)w.ah[e]); }
+        w.b[0] = (float)beta.real(); w.b[1] = (float)beta.imag();
+        w.b2h = (float)b2; w.b2l = (float)(b2 - (double)w.b2h);
+        const Z ph = std::polar(1.0, std::remainder(delta * (double)d.T, 2 * M_PI));
+        for (int e = 0; e < 2; ++e) {
+            const Z s = ph * Z(b->cs[2 * e], b->cs[2 * e + 1]);
+            w.c[2 * e] = (float)s.real(); w.c[2 * e + 1] = (float)s.imag();
+        }
+        by[L - 8].push_back(w);
+    }
+    std::vector<SpecWalk> all;
+    for (int k = SPEC_BATCH_CLASSES - 1; k >= 0; --k) {
+        b->spec_count[k] = (int)by[k].size();
+        all.insert(all.end(), by[k].begin(), by[k].end());
+    }
+    if (near.size() > 65535) return false;   // (the grid's second dimension)
+    cudaError_t e = dev_alloc((void **)&b->spec_walks, sizeof(SpecWalk) * std::max<size_t>(1, all.size()));
+    b->near_count = (int)near.size();
+    if (e == cudaSuccess && !near.empty()) {
+        if (!b->near_ids) e = dev_alloc((void **)&b->near_ids, sizeof(int) * near.size());
+        if (e == cudaSuccess) e = cudaMemcpy(b->near_ids, near.data(), sizeof(int) * near.size(), cudaMemcpyHostToDevice);
+        if (e == cudaSuccess && !b->side) e = cudaStreamCreateWithFlags(&b->side, cudaStreamNonBlocking);
+        if (e == cudaSuccess && !b->fork) e = cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming);
+        if (e == cudaSuccess && !b->join) e = cudaEventCreateWithFlags(&b->join, cudaEventDisableTiming);
+    }
+    if (e == cudaSuccess && !b->spec_table) {
+        e = dev_alloc(&b->spec_table, batch_spectral_table_bytes());
+        if (e == cudaSuccess) e = launch_batch_spectral_tables(b->spec_table, b->stream);
+    }
+    if (e == cudaSuccess) e = cudaMemcpy(b->spec_walks, all.data(), sizeof(SpecWalk) * all.size(), cudaMemcpyHostToDevice);
+    if (e != cudaSuccess) {
+        (void)cudaGetLastError();
+        cudaFree(b->spec_walks);
+        b->spec_walks = nullptr;
+    }
+    return e == cudaSuccess;
+}
+
 extern "C" {
 
 qw_status qw_batch_destroy(qw_batch *b) {
@@ -582,6 +792,12 @@ qw_status qw_batch_destroy(qw_batch *b) {
     cudaFree(b->norms_dev);
     cudaFree(b->counter);
     cudaFree(b->final_dev);
+    cudaFree(b->spec_walks);
+    cudaFree(b->spec_table);
+    cudaFree(b->near_ids);
+    if (b->side) cudaStreamDestroy(b->side);
+    if (b->fork) cudaEventDestroy(b->fork);
+    if (b->join) cudaEventDestroy(b->join);
     if (b->cap) cudaStreamDestroy(b->cap);
     delete b;
     return QW_OK;
@@ -714,6 +930,7 @@ qw_status qw_batch_set_plan(qw_batch *b, int depth_k) {
     if (!b) return QW_EINVAL;
     if (depth_k < 1 || depth_k > batch_kmax(b->prec))
         return batch_fail(b, QW_EINVAL, "k must be in [1, " + std::to_string(batch_kmax(b->prec)) + "]");
+    batch_spectral_off(b);
     if (depth_k != b->K) {
         cudaStreamSynchronize(b->stream);
         drop_graph(b);   // the captured launch carries k
@@ -751,6 +968,7 @@ qw_status qw_batch_set_cta_walks(qw_batch *b, int n) {
     if (!b) return QW_EINVAL;
     if (n < 0) return batch_fail(b, QW_EINVAL, "the number of CTA walks must be >= 0");
     n = std::min(n, b->nwalks);
+    batch_spectral_off(b);
     if (n != b->nbig) {
         cudaStreamSynchronize(b->stream);
         drop_graph(b);   // the captured launch carries the split
@@ -772,6 +990,7 @@ qw_status qw_batch_get_plan_ex(const qw_batch *b, int *depth_k, int *tile, int *
 qw_status qw_batch_autotune(qw_batch *b, char *report, size_t report_len) {
     if (!b) return QW_EINVAL;
     const int ks[] = {8, 16, 24, 32, 48, 64, 96, 128};
+    batch_spectral_off(b);
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
@@ -818,15 +1037,28 @@ qw_status qw_batch_autotune(qw_batch *b, char *report, size_t report_len) {
         if (!time_plan(ms)) break;
         if (ms < best) { best = ms; best_k = k; best_v = 1; best_n = n1; }
     }
+    qw_batch_set_cta_walks(b, best_n);
+    if (e == cudaSuccess && qw_batch_set_plan_ex(b, best_k, best_v) != QW_OK) e = cudaErrorUnknown;
+    // momentum space, over the stepping plan that stays set beneath it (the runs
+    // above have left every site outside the walks' cones zero)
+    if (e == cudaSuccess && batch_spectral_prepare(b)) {
+        cudaStreamSynchronize(b->stream);
+        drop_graph(b);
+        b->spectral = true;
+        float ms = 0.f;
+        if (time_plan(ms)) {
+            if (ms < best) best = ms;
+            else batch_spectral_off(b);
+        }
+    }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    qw_batch_set_cta_walks(b, best_n);
     if (e != cudaSuccess) return e == cudaErrorUnknown ? QW_ECUDA : batch_cuda(b, e, "batch autotune");
-    qw_batch_set_plan_ex(b, best_k, best_v);
     if (report && report_len) {
         std::snprintf(report, report_len,
                       "{\"tuned\": true, \"k\": %d, \"tile\": %d, \"variant\": \"%s\", \"cta_walks\": %d, "
-                      "\"ms\": %.6g}", best_k, batch_tile(b->prec), best_v ? "window_sweep" : "tiles", best_v ? b->nbig : b->nwalks, best);
+                      "\"spectral\": %s, \"ms\": %.6g}", best_k, batch_tile(b->prec), best_v ? "window_sweep" : "tiles",
+                      best_v ? b->nbig : b->nwalks, b->spectral ? "true" : "false", best);
     }
     return QW_OK;
 }

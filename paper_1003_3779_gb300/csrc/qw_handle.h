@@ -205,6 +205,21 @@ Spec2Plan spectral2d_plan(int64_t nx, int64_t ny, int64_t T, bool even);
 cudaError_t launch_spectral2d_tables(void *work, cudaStream_t s);
 cudaError_t launch_spectral2d(const Step2DArgs &a, int cut_K, int adjoint, void *work, cudaStream_t s);
 
+// a batch of localised walks in momentum space (spectral_batch.cu, FP32)
+struct SpecWalk {
+    int64_t n, x0, base, pitch, poff;   // as WalkDesc
+    int T, id;
+    float ah[2], al[2];                 // alpha (re, im), high and low parts
+    float b[2], b2h, b2l;               // beta; |beta|^2 in two parts
+    float c[4];                         // coin state times e^{i delta T}
+};
+constexpr int SPEC_BATCH_CLASSES = 6;   // transform lengths 2^8 .. 2^13
+int batch_spectral_length(int64_t T);   // log2 of the transform length, 0: T too long
+size_t batch_spectral_table_bytes();
+cudaError_t launch_batch_spectral_tables(void *table, cudaStream_t s);
+cudaError_t launch_batch_spectral(const SpecWalk *walks, const int *count, void *state, float *P, double *norms, int *final_buf,
+                                  const void *table, cudaStream_t s);
+
 // K steps in shared-memory tiles (tile2d.cu, FP32); kind: the global coin, or
 // with a.phi the base coin of the phases; links: broken links or an edge
 cudaError_t launch_tile2d(int shift, int kind, bool links, const Tile2DArgs &a, const void *coinp, cudaStream_t s);
