@@ -256,10 +256,16 @@ k_support(const char *__restrict__ src, char *__restrict__ dst, int64_t slot_byt
           unsigned long long *box) {
     constexpr int SPV = (int)sizeof(V) / SB;   // sites per vector
     if (!SRC) {   // the box already spans the lattice: nothing left to find
-        const volatile unsigned long long *vb = box;
-        if (vb[0] == 0ull && vb[1] == (unsigned long long)(nx - 1) && vb[2] == 0ull &&
-            vb[3] == (unsigned long long)(ns / nx - 1))
-            return;
+        // (one thread looks for the block: other blocks are adding to the box, and
+        // threads that saw different boxes would part before the shuffles below)
+        __shared__ int full;
+        if (threadIdx.x == 0) {
+            const volatile unsigned long long *vb = box;
+            full = vb[0] == 0ull && vb[1] == (unsigned long long)(nx - 1) && vb[2] == 0ull &&
+                   vb[3] == (unsigned long long)(ns / nx - 1);
+        }
+        __syncthreads();
+        if (full) return;
     }
     const int64_t nvec = (ns + SPV - 1) / SPV;
     Seen v;

@@ -115,3 +115,23 @@ def test_reused_handle_equals_a_fresh_one(qw, dims, bc, prec):
         w2.close()
     assert np.array_equal(got, fresh(dev.cpu().numpy(), 11))
     w.close()
+
+
+@pytest.mark.parametrize("dims", [(1 << 20,), (1000003,), (1024, 1024), (4096, 512)])
+@pytest.mark.parametrize("prec,dtype", [("f64", torch.complex64), ("comp", torch.complex64), ("f32", torch.complex128),
+                                        ("bf16", torch.complex64)])
+def test_dense_states_fill_the_box(qw, dims, prec, dtype):
+    """Converted states are searched in the buffer, by blocks that stop once the
+    box is full, while others still add to it: the box is the whole lattice, and
+    every run of the same state ends in the same bits."""
+    g = torch.Generator(device="cuda").manual_seed(len(dims))
+    psi = torch.randn((2 * len(dims),) + tuple(reversed(dims)), dtype=dtype, device="cuda", generator=g)
+    psi /= psi.abs().square().sum().sqrt()
+    w, first = make(qw, dims, prec), None
+    for _ in range(25):
+        w.set_state(psi).step(3)
+        assert w.describe()["support"] == "full"
+        out = qw.qw_get_state(w.h, torch.empty_like(psi))
+        first = out if first is None else first
+        assert torch.equal(out, first)
+    w.close()
