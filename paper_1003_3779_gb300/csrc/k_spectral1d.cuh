@@ -26,15 +26,22 @@
 // repeated squaring.
 //
 // Measured, stepping (autotuned) -> momentum space, per qw_step call:
-//   n = 2^27 FP32, T = 4096: Hadamard class 73.7 -> 5.0 ms, complex coin 313 ->
-//   5.0 ms; T = 1000: 18.1 -> 2.1 ms (G = 1), 76.4 -> 2.1 ms
-//   n = 1000003 FP32 complex, T = 1000: 0.86 -> 0.034 ms
-//   n = 2^20 FP64 real, T = 1000: 18.9 -> 0.58 ms; double-float: 6.2 -> 0.65 ms
-// What bounds it (FP32): shared-memory and L1 traffic, about 1.1 MB per CTA.
+//   n = 2^27 FP32, T = 4096: Hadamard class 73.7 -> 4.3 ms, complex coin 313 ->
+//   4.3 ms; T = 1000: 18.1 -> 2.1 ms (G = 1), 76.4 -> 2.1 ms
+//   n = 1000003 FP32 complex, T = 1000: 0.86 -> 0.031 ms
+//   n = 2^20 FP64 real, T = 1000: 18.9 -> 0.57 ms; double-float: 6.2 -> 0.65 ms
+// What bounds it (FP32, G = 2, 2^24 sites): latency.  One CTA fills an SM (139 KB
+// of shared memory, all registers), so the loads of its block, the matrices and
+// the barriers are only hidden by its own warps: issue 50 %, long scoreboard the
+// first stall, DRAM 10 %.  Hence one plane per thread (1024 threads of 64
+// registers; with both planes per thread, 512 of 128: issue 35 %, 5.0 ms), the
+// next block's sites prefetched into L2 (4.8 ms without; two CTAs of G = 1 cover
+// for each other, and gain nothing from it), and spec_reload.  FP64: its pipe.
 //
-// Layout of the transform.  256 threads hold 4096 points of both planes, 16 per
-// thread and plane, in registers.  4096 = 16 x 16 x 16 (Cooley and Tukey, 1965):
-// with j = t + 256 i, t = u + 16 v and p = a + 16 b + 256 c,
+// Layout of the transform.  512 threads hold 4096 points of both planes, 16 per
+// thread, in registers: the lower half of a warp plane 0, the upper half plane 1
+// at the same points, so that the 2 x 2 matrices take the other plane's value by
+// a shuffle.  4096 = 16 x 16 x 16 (Cooley and Tukey, 1965): with j = t + 256 i, t = u + 16 v and p = a + 16 b + 256 c,
 //   X[p] = sum_u w16^{uc} w256^{ub} sum_v w16^{vb} w4096^{ta} sum_i w16^{ia} x[j],
 // so each sum is a 16-point transform inside a thread.  Between the first two
 // the data change threads through shared memory (one block barrier); the second
@@ -55,13 +62,16 @@ template <int P> struct SpecReal { using type = float; };
 template <> struct SpecReal<P_F64> { using type = double; };
 template <> struct SpecReal<P_COMP> { using type = double; };
 
-constexpr int SPEC_GROUP = 256;                       // threads per 4096 points
+constexpr int SPEC_GROUP = 256;                       // threads per 4096 points of one plane
+constexpr int SPEC_THREADS = 2 * SPEC_GROUP;          // ... of both planes
 constexpr int SPEC_POINTS = 4096;                     // points per group and plane
 constexpr int SPEC_ROW = 16 * 17;                     // one padded 16 x 16 tile
 constexpr int SPEC_TW1 = 0;                           // twiddle tables, in elements: w4096^{ta} [a][t],
 constexpr int SPEC_TW2 = 16 * 256;                    // w256^{ub} [b][u],
 constexpr int SPEC_TWG = SPEC_TW2 + 16 * 16;          // w8192^{j} [i][t]
 constexpr int SPEC_TW = SPEC_TWG + 16 * 256;
+
+constexpr int SPEC_AHEAD = 152;                       // CTAs in flight (G = 2: one per SM)
 
 template <class R> struct alignas(4 * sizeof(R)) SpecPair { Cx<R> a, b; };
 template <class R> struct alignas(2 * sizeof(R)) SpecCx { R re, im; };
@@ -98,6 +108,11 @@ template <class R> __device__ __forceinline__ Cx<R> spec_tw(const SpecCx<R> *__r
     const SpecCx<R> w = t[i];
     return {w.re, w.im};
 }
+
+// The twiddles of the way back are those of the way forth, at the same
+// addresses: without this the compiler keeps them in registers in between, and
+// spills (190 bytes per thread at 64 registers).
+template <class T> __device__ __forceinline__ void spec_reload(const T *&p) { asm volatile("" : "+l"(p)); }
 
 // 4-point transform in place, w4 = -i (forward) or +i (inverse)
 template <int INV, class R> __device__ __forceinline__ void dft4(Cx<R> &x0, Cx<R> &x1, Cx<R> &x2, Cx<R> &x3) {
@@ -140,7 +155,7 @@ template <class R> __device__ __forceinline__ void order16(Cx<R> (&x)[16]) {   /
 
 __device__ __forceinline__ void spec_group_barrier(int G, int g) {
     if (G == 1) __syncthreads();
-    else asm volatile("bar.sync %0, %1;" ::"r"(g + 1), "n"(SPEC_GROUP) : "memory");
+    else asm volatile("bar.sync %0, %1;" ::"r"(g + 1), "n"(SPEC_THREADS) : "memory");
 }
 
 // forward transform of one plane: x[i] = x(t + 256 i) -> x[c] = X(a + 16 b + 256 c)
@@ -212,15 +227,15 @@ __device__ __forceinline__ void spec_inv2(Cx<R> (&x)[16], const SpecCx<R> *sm, c
 // Block blockIdx.x / 2 of W = 2 (G * 4096 - K) output sites, parity blockIdx.x & 1.
 // table: U^K / B in the order the threads hold the momenta, then the twiddles.
 template <int P, int G>
-__global__ void __launch_bounds__(G *SPEC_GROUP, (G == 1 && sizeof(typename SpecReal<P>::type) == 4) ? 2 : 1)
+__global__ void __launch_bounds__(G *SPEC_THREADS, (G == 1 && sizeof(typename SpecReal<P>::type) == 4) ? 2 : 1)
 k_spectral1d(View in, View out, int64_t n, int K, int64_t W, const void *__restrict__ table) {
     using R = typename SpecReal<P>::type;
     using C = Cx<R>;
     extern __shared__ __align__(16) unsigned char ssm[];
-    const int g = G == 1 ? 0 : (int)threadIdx.x / SPEC_GROUP;   // uniform per warp
-    const int t = (int)threadIdx.x % SPEC_GROUP;
-    SpecCx<R> *sm0 = reinterpret_cast<SpecCx<R> *>(ssm) + (size_t)g * 2 * 16 * SPEC_ROW;
-    SpecCx<R> *sm1 = sm0 + 16 * SPEC_ROW;
+    const int g = G == 1 ? 0 : (int)threadIdx.x / SPEC_THREADS;   // uniform per warp
+    const int h = (int)threadIdx.x >> 4 & 1;                      // the thread's plane
+    const int t = ((int)threadIdx.x % SPEC_THREADS >> 5) * 16 + ((int)threadIdx.x & 15);
+    SpecCx<R> *sm = reinterpret_cast<SpecCx<R> *>(ssm) + (size_t)(2 * g + h) * 16 * SPEC_ROW;
     const auto *mat = static_cast<const SpecPair<R> *>(table);
     const auto *tw = reinterpret_cast<const SpecCx<R> *>(static_cast<const char *>(table) + spec_matrix_bytes<R>(G));
     const int q = (int)(blockIdx.x & 1);
@@ -235,89 +250,69 @@ k_spectral1d(View in, View out, int64_t n, int K, int64_t W, const void *__restr
         if (s >= n) s = once ? s - n : s % n;
         return s;
     };
-    C f0[16], f1[16];
+    if constexpr (G == 2) {
+        // the block that this SM takes next, into L2: 16 sites of plane q per thread
+        const int64_t o1 = (int64_t)((blockIdx.x + SPEC_AHEAD) >> 1) * W, s1 = o1 - K + 16 * (int64_t)threadIdx.x;
+        if (o1 < n && s1 >= 0 && s1 < n)
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(static_cast<const char *>(in.p) + (q * in.pitch + s1) * St<P>::SLOT_BYTES));
+    }
+    C f[16];
     if constexpr (G == 1) {
 #pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            const int64_t s = site(t + 256 * i);
-            f0[i] = spec_ld<P>(in, 0, s);
-            f1[i] = spec_ld<P>(in, 1, s);
-        }
+        for (int i = 0; i < 16; ++i) f[i] = spec_ld<P>(in, h, site(t + 256 * i));
     } else {
 #pragma unroll
         for (int i = 0; i < 16; ++i) {
-            const int64_t s = site(t + 256 * i), r = site(t + 256 * i + SPEC_POINTS);
-            const C a0 = spec_ld<P>(in, 0, s), a1 = spec_ld<P>(in, 1, s);
-            const C b0 = spec_ld<P>(in, 0, r), b1 = spec_ld<P>(in, 1, r);
-            if (g == 0) {
-                f0[i] = cadd(a0, b0);
-                f1[i] = cadd(a1, b1);
-            } else {
-                const C w = spec_tw(tw + SPEC_TWG, i * 256 + t);
-                f0[i] = spec_twiddle<0>(csub(a0, b0), w);
-                f1[i] = spec_twiddle<0>(csub(a1, b1), w);
-            }
+            const C a = spec_ld<P>(in, h, site(t + 256 * i)), b = spec_ld<P>(in, h, site(t + 256 * i + SPEC_POINTS));
+            f[i] = g == 0 ? cadd(a, b) : spec_twiddle<0>(csub(a, b), spec_tw(tw + SPEC_TWG, i * 256 + t));
         }
     }
-    spec_fwd1(f0, sm0, tw, t);
-    spec_fwd1(f1, sm1, tw, t);
+    spec_fwd1(f, sm, tw, t);
     spec_group_barrier(G, g);
-    spec_fwd2(f0, sm0, tw, t);
-    spec_fwd2(f1, sm1, tw, t);
+    spec_fwd2(f, sm, tw, t);
+    // row h of the matrix: the other plane's value is 16 lanes away
 #pragma unroll
     for (int c = 0; c < 16; ++c) {
-        const SpecPair<R> r0 = mat[((g * 16 + c) * 2) * SPEC_GROUP + t], r1 = mat[((g * 16 + c) * 2 + 1) * SPEC_GROUP + t];
-        const C y0 = cfma(r0.b, f1[c], cmul(r0.a, f0[c]));
-        const C y1 = cfma(r1.b, f1[c], cmul(r1.a, f0[c]));
-        f0[c] = y0;
-        f1[c] = y1;
+        const SpecPair<R> r = mat[((g * 16 + c) * 2 + h) * SPEC_GROUP + t];
+        const C o{__shfl_xor_sync(0xffffffffu, f[c].re, 16), __shfl_xor_sync(0xffffffffu, f[c].im, 16)};
+        const C z0 = h == 0 ? f[c] : o, z1 = h == 0 ? o : f[c];
+        f[c] = cfma(r.b, z1, cmul(r.a, z0));
     }
     __syncwarp();   // the forward transposes' last reads of the tiles, before they are rewritten
-    spec_inv1(f0, sm0, tw, t);
-    spec_inv1(f1, sm1, tw, t);
+    spec_reload(tw);
+    spec_inv1(f, sm, tw, t);
     spec_group_barrier(G, g);
-    spec_inv2(f0, sm0, tw, t);
-    spec_inv2(f1, sm1, tw, t);
+    spec_inv2(f, sm, tw, t);
     // point j is site out0 - K + o, o = 2j + q + (K mod 2); outputs have K <= o < K + wthis
-    auto put = [&](int j, C v0, C v1) {
+    auto put = [&](int j, C v) {
         const int64_t o = 2 * (int64_t)j + q + (K & 1) - K;
-        if (o < 0 || o >= wthis) return;
-        spec_st<P>(out, 0, out0 + o, v0);
-        spec_st<P>(out, 1, out0 + o, v1);
+        if (o >= 0 && o < wthis) spec_st<P>(out, h, out0 + o, v);
     };
     if constexpr (G == 1) {
 #pragma unroll
-        for (int i = 0; i < 16; ++i) put(t + 256 * i, f0[i], f1[i]);
+        for (int i = 0; i < 16; ++i) put(t + 256 * i, f[i]);
     } else {
         // x[j] = z0 + z1 w8192^{-j}, x[j + 4096] = z0 - z1 w8192^{-j}: group 0 forms
         // them for i < 8, group 1 for i >= 8, after swapping the other half
         if (g == 1) {
 #pragma unroll
-            for (int i = 0; i < 16; ++i) {
-                const C w = spec_tw(tw + SPEC_TWG, i * 256 + t);
-                f0[i] = spec_twiddle<1>(f0[i], w);
-                f1[i] = spec_twiddle<1>(f1[i], w);
-            }
+            for (int i = 0; i < 16; ++i) f[i] = spec_twiddle<1>(f[i], spec_tw(tw + SPEC_TWG, i * 256 + t));
         }
         __syncthreads();   // every read of the tiles is done
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
-            const C s0 = g == 0 ? f0[8 + k] : f0[k], s1 = g == 0 ? f1[8 + k] : f1[k];
-            sm0[k * 256 + t] = {s0.re, s0.im};
-            sm1[k * 256 + t] = {s1.re, s1.im};
+            const C s = g == 0 ? f[8 + k] : f[k];
+            sm[k * 256 + t] = {s.re, s.im};
         }
         __syncthreads();
-        const SpecCx<R> *p0 = reinterpret_cast<const SpecCx<R> *>(ssm) + (size_t)(g ^ 1) * 2 * 16 * SPEC_ROW;
-        const SpecCx<R> *p1 = p0 + 16 * SPEC_ROW;
+        const SpecCx<R> *p = reinterpret_cast<const SpecCx<R> *>(ssm) + (size_t)(2 * (g ^ 1) + h) * 16 * SPEC_ROW;
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
-            const C m0 = g == 0 ? f0[k] : f0[8 + k], m1 = g == 0 ? f1[k] : f1[8 + k];
-            const C o0{p0[k * 256 + t].re, p0[k * 256 + t].im}, o1{p1[k * 256 + t].re, p1[k * 256 + t].im};
-            const C z00 = g == 0 ? m0 : o0, z10 = g == 0 ? o0 : m0;   // group 0's and group 1's value, plane 0
-            const C z01 = g == 0 ? m1 : o1, z11 = g == 0 ? o1 : m1;   // ... plane 1
+            const C m = g == 0 ? f[k] : f[8 + k], o{p[k * 256 + t].re, p[k * 256 + t].im};
+            const C z0 = g == 0 ? m : o, z1 = g == 0 ? o : m;   // group 0's and group 1's value
             const int j = t + 256 * (g == 0 ? k : 8 + k);
-            put(j, cadd(z00, z10), cadd(z01, z11));
-            put(j + SPEC_POINTS, csub(z00, z10), csub(z01, z11));
+            put(j, cadd(z0, z1));
+            put(j + SPEC_POINTS, csub(z0, z1));
         }
     }
 }

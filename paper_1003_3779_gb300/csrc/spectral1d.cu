@@ -149,7 +149,7 @@ static cudaError_t go_spectral(const Spec1DArgs &a, cudaStream_t s) {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     const int64_t W = 2 * ((int64_t)G * SPEC_POINTS - a.K), blocks = (a.n + W - 1) / W * 2;
-    kern<<<(unsigned)blocks, G * SPEC_GROUP, smem, s>>>(a.in, a.out, a.n, a.K, W, a.table);
+    kern<<<(unsigned)blocks, G * SPEC_THREADS, smem, s>>>(a.in, a.out, a.n, a.K, W, a.table);
     return cudaGetLastError();
 }
 
