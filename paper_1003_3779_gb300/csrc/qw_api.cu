@@ -1303,6 +1303,7 @@ qw_status qw_set_plan(qw_walk *w, int depth_k, int tile) {
         if (depth_k != 1 && depth_k != 4 && depth_k != 8)
             return set_error(w, QW_EINVAL, "2D plans take k = 1, 4 or 8");
         w->plan_k = depth_k; w->plan_tile = 0; w->plan_user = true;
+        spectral_off(w);
         return QW_OK;
     }
     int dk, dt, dv;

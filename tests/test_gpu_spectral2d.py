@@ -106,3 +106,17 @@ def test_against_the_oracle_and_short_calls(qw):
     w.set_state(psi1).step(90)
     v.set_state(psi1).step(90)
     assert np.array_equal(w.state(), v.state())
+
+
+def test_a_plan_set_after_autotune_steps(qw):
+    """qw_set_plan takes the momentum-space steps back: the same bits as the plan
+    on a handle that was never tuned."""
+    psi0 = inputs.random_state((4, 128, 128), seed=4, dtype=np.complex64)
+    w = qw.Walk((128, 128), prec="f32").set_coin(inputs.grover()).set_state(psi0)
+    w.autotune()
+    w.set_plan(8)
+    v = qw.Walk((128, 128), prec="f32").set_coin(inputs.grover()).set_plan(8)
+    assert "spectral" not in w.describe()
+    assert np.array_equal(w.set_state(psi0).step(200).state(np.complex64), v.set_state(psi0).step(200).state(np.complex64))
+    w.close()
+    v.close()
