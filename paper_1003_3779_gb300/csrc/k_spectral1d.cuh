@@ -109,10 +109,10 @@ template <class R> __device__ __forceinline__ Cx<R> spec_tw(const SpecCx<R> *__r
     return {w.re, w.im};
 }
 
-// The twiddles of the way back are those of the way forth, at the same
-// addresses: without this the compiler keeps them in registers in between, and
-// spills (190 bytes per thread at 64 registers).
-template <class T> __device__ __forceinline__ void spec_reload(const T *&p) { asm volatile("" : "+l"(p)); }
+// The way back reads the twiddles (and in k_spec2_columns writes the addresses)
+// of the way forth: without this the compiler keeps them in registers in
+// between, and spills (190 bytes per thread here, 104 there, at 64 registers).
+template <class T> __device__ __forceinline__ void spec_reload(T *&p) { asm volatile("" : "+l"(p)); }
 
 // 4-point transform in place, w4 = -i (forward) or +i (inverse)
 template <int INV, class R> __device__ __forceinline__ void dft4(Cx<R> &x0, Cx<R> &x1, Cx<R> &x2, Cx<R> &x3) {

@@ -443,6 +443,7 @@ k_spec2_columns(Spec2Args a, Spec2Coin coin) {
         }
     }
     __syncthreads();
+    if constexpr (L >= 10) spec_reload(z);   // (shorter columns have the registers)
     spec2_inverse<L>(x, sm, a.tw, t);
 #pragma unroll
     for (int i = 0; i < 16; ++i) {
