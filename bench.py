@@ -2,14 +2,16 @@
 
 Workload (one "step" of the benchmark = one pass of the whole path): the 1D walk
 on a cycle of N = 2^27 sites with the SU(2) coin theta = pi/4 (phases 0), a
-seeded random normalised state (complex64), T = 4096 walk steps with the
-temporal-blocking depth chosen by the autotuner, then the coin marginals
-P(x) and the norm.  Per benchmark step: the state is re-seeded from a resident
-device copy (set_state), stepped T times (fused coin + shift kernels, k steps
-per HBM round trip) and reduced to P (float32) and the norm (double).
+seeded random normalised state (complex64), T = 4096 walk steps with the plan
+chosen by the autotuner, then the coin marginals P(x).  Per benchmark step: the
+state is re-seeded from a resident device copy (set_state), advanced by T steps
+(in momentum space block by block, or by fused coin + shift kernels with k steps
+per HBM round trip, whichever the autotuner timed as faster) and reduced to P
+(float32).
 
 Metric: site-coin-updates/s = N * d * T / time (d = 2), whole job over all ranks.
-Also reported: the roofline of the dominant kernel (live CUDA-event timing),
+Also reported: the roofline of the dominant kernel (live CUDA-event timing), that
+of the stepping kernel on the same workload,
 the FP64 / bf16-storage / compensated forms on the same input with their L1
 distance to the FP64 result, an end-to-end number through the C ABI with host
 buffers, the SM clocks during the timed region, and the FP64 CPU oracle timed
@@ -115,8 +117,11 @@ class ClockSampler:
             self.f = open(self.path, "w")
             self.proc = subprocess.Popen(
                 ["nvidia-smi", "-i", str(self.gpu), f"--query-gpu={self.FIELDS}",
-                 "--format=csv,noheader,nounits", "-lms", "200"], stdout=self.f,
+                 "--format=csv,noheader,nounits", "-lms", "20"], stdout=self.f,
                 stderr=subprocess.DEVNULL)
+            deadline = time.perf_counter() + 3.0
+            while os.path.getsize(self.path) == 0 and time.perf_counter() < deadline:
+                time.sleep(0.01)
         except Exception:
             self.proc = None
         return self
@@ -331,34 +336,90 @@ COIN_CLASS_WORK = {"hadamard_class": (4, 4.0, "FADD"), "real": (8, 12.0, "FMUL/F
                    "complex": (16, 28.0, "FMUL/FFMA")}
 
 
+def time_walk(qw, w, dev0, stream):
+    """Seconds of one qw_step(T_STEPS) from dev0, by CUDA events, after a warm-up."""
+    import torch
+    for timed in (False, True):
+        qw.qw_set_state(w.h, dev0)
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record(stream)
+        qw.qw_step(w.h, T_STEPS)
+        b.record(stream)
+        torch.cuda.synchronize()
+    return a.elapsed_time(b) / 1e3
+
+
+def stepping_roofline(desc, K, tile, t_step, hbm_gbs, sm_max_mhz, peak_src):
+    """Roofline of the 1D stepping kernel that ran T_STEPS steps in t_step seconds."""
+    launches = math.ceil(T_STEPS / K)
+    avg_launch_s, k_eff = t_step / launches, T_STEPS / launches   # (k_eff: steps per launch, average)
+    if desc["coin_kind"] == "hadamard_class":
+        # 4 additions per site-step (a0 +- a1, re and im); one FP32 add per lane per clock
+        flops_site_step, flops_per_lane_clk, op = 4.0, 1, "FADD"
+    else:
+        # 8 FMAs per site-step (real 2x2 coin on complex amplitudes) = 16 flops
+        flops_site_step, flops_per_lane_clk, op = 16.0, 2, "FFMA"
+    bytes_launch = 32.0 * N_SITES                         # 2 planes x 8 B read + written
+    alu_peak = SMS * FP32_LANES * flops_per_lane_clk * sm_max_mhz * 1e6 / 1e12   # TFLOP/s
+    ach_tflops = flops_site_step * N_SITES * k_eff / avg_launch_s / 1e12
+    ach_gbs = bytes_launch / avg_launch_s / 1e9
+    alu_frac, hbm_frac = ach_tflops / alu_peak, ach_gbs / hbm_gbs
+    traffic = ncu_traffic(desc["path"], tile)
+    if alu_frac >= hbm_frac:
+        roof = {"bound": "alu", "achieved": ach_tflops, "peak": alu_peak, "unit": "TFLOP/s",
+                "frac": alu_frac, "traffic": traffic,
+                "peak_source": f"{SMS} SMs (device attribute) x 128 FP32 lanes x {flops_per_lane_clk} flop "
+                               f"({op}) x {sm_max_mhz:.0f} MHz (derived)",
+                "hbm_view": {"achieved_gbs": ach_gbs, "peak_gbs": hbm_gbs, "frac": hbm_frac,
+                             "peak_source": f"{peak_src} HBM copy"}}
+    else:
+        roof = {"bound": "hbm", "achieved": ach_gbs, "peak": hbm_gbs, "unit": "GB/s",
+                "frac": hbm_frac, "traffic": traffic, "peak_source": f"{peak_src} HBM copy",
+                "alu_view": {"achieved_tflops": ach_tflops, "peak_tflops": alu_peak, "frac": alu_frac}}
+    roof.update({"kernel": "%s<f32,R=%d,%s coin>" % (desc["path"], tile, desc["coin_kind"]), "k": K,
+                 "flops_per_site_step": flops_site_step, "avg_launch_ms": avg_launch_s * 1e3,
+                 "ms_per_T_steps": t_step * 1e3,
+                 "site_coin_updates_per_s": 2.0 * N_SITES * T_STEPS / t_step,
+                 "effective_bytes_per_site_step": bytes_launch / N_SITES / k_eff})
+    return roof
+
+
+def spectral_work(spec):
+    """Work of T_STEPS steps in momentum space: (launches, flops per site, bytes
+    per site).  A launch of K steps transforms both planes of blocks of B = 16 x
+    tile sites of one parity, forth and back (5 B log2 B flops each), multiplies
+    each momentum by a 2 x 2 complex matrix (28 flops) and keeps B - K sites; it
+    reads and writes the state once (32 bytes per site)."""
+    launches = math.ceil(T_STEPS / spec["k"])
+    K, B = math.ceil(T_STEPS / launches), 16 * spec["tile"]
+    return launches, launches * (4 * 5 * B * math.log2(B) + 28 * B) / (B - K), launches * 32.0
+
+
 def coin_class_leg(qw, C, dev0, stream, sm_max_mhz, hbm_gbs):
     """The benchmark workload (N = 2^27, T = 4096, FP32, same state) with another
-    SU(2) coin: autotuned plan, CUDA events around qw_step, and the kernel's
-    roofline against the FP32 instruction issue rate of its coin class."""
+    SU(2) coin: autotuned plan, CUDA events around qw_step; beside it the best
+    stepping plan, whose roofline is the FP32 instruction issue rate at its coin
+    class's instructions per site-step."""
     import torch
     w = qw.Walk((N_SITES,), prec="f32").set_coin(C).set_state(dev0)
     tune = json.loads(w.autotune())
     K, tile, var = w.plan_ex()
     desc = w.describe()
-    qw.qw_set_state(w.h, dev0)
-    qw.qw_step(w.h, 2 * K)
-    qw.qw_set_state(w.h, dev0)
-    a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-    a.record(stream)
-    qw.qw_step(w.h, T_STEPS)
-    b.record(stream)
-    torch.cuda.synchronize()
-    t = a.elapsed_time(b) / 1e3
+    t_auto = time_walk(qw, w, dev0, stream)
     norm = w.norm()
+    w.set_plan_ex(K, tile, var)          # the best stepping plan alone
+    t = time_walk(qw, w, dev0, stream)
     w.close()
     inst, flops, op = COIN_CLASS_WORK[desc["coin_kind"]]
     launches = math.ceil(T_STEPS / K)
     issue_peak = SMS * FP32_LANES * sm_max_mhz * 1e6            # FP32 instructions / s
     ach_inst = inst * N_SITES * T_STEPS / t
-    return {"site_coin_updates_per_s": 2.0 * N_SITES * T_STEPS / t, "ms_per_T_steps": t * 1e3,
-            "coin_kind": desc["coin_kind"], "kernel": desc["path"], "k": K, "tile": tile,
-            "avg_launch_ms": t * 1e3 / launches, "norm_err": abs(norm - 1.0), "autotune": tune,
-            "roofline": {"bound": "alu", "achieved": ach_inst / 1e12, "peak": issue_peak / 1e12,
+    return {"site_coin_updates_per_s": 2.0 * N_SITES * T_STEPS / t_auto, "ms_per_T_steps": t_auto * 1e3,
+            "coin_kind": desc["coin_kind"], "momentum_space": desc.get("spectral"), "norm_err": abs(norm - 1.0),
+            "autotune": tune,
+            "stepping": {"site_coin_updates_per_s": 2.0 * N_SITES * T_STEPS / t, "ms_per_T_steps": t * 1e3,
+                         "kernel": desc["path"], "k": K, "tile": tile, "avg_launch_ms": t * 1e3 / launches},
+            "roofline_stepping": {"bound": "alu", "achieved": ach_inst / 1e12, "peak": issue_peak / 1e12,
                          "unit": "T FP32-instructions/s", "frac": ach_inst / issue_peak,
                          "instructions_per_site_step": inst, "op": op,
                          "achieved_tflops": flops * N_SITES * T_STEPS / t / 1e12,
@@ -448,11 +509,14 @@ def run_gpu(args, rank, world, local):
         tune = json.loads(w.autotune())
     K, tile, _variant = w.plan_ex()
     desc = w.describe()
-    launches_step = math.ceil(T_STEPS / K)
+    spec = desc.get("spectral")
+    if spec and T_STEPS < spec["from_steps"]:
+        spec = None
+    launches_step = spectral_work(spec)[0] if spec else math.ceil(T_STEPS / K)
 
-    # one benchmark step launches the support search of qw_set_state (2 kernels:
-    # a dense state returns after one wave), the step kernels (launches_step)
-    # and the marginals with the norm (2 kernels)
+    # one benchmark step launches the copy of qw_set_state, which also searches
+    # the support (2 kernels), the step kernels (launches_step or more) and the
+    # marginals (1 kernel)
     def one_step(ev_a=None, ev_b=None):
         qw.qw_set_state(w.h, dev0)
         if ev_a is not None:
@@ -462,15 +526,17 @@ def run_gpu(args, rank, world, local):
             ev_b.record(stream)
         qw.qw_probabilities(w.h, P_dev, want_norm=False)
 
-    for _ in range(args.warmup):
-        one_step()
-    torch.cuda.synchronize()
     evs = [(torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True))
            for _ in range(args.steps)]
     start, stop = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-    barrier(dist, local)
-    torch.cuda.synchronize()
+    # (the clock sampler runs before the warm-up starts: the timed region can be
+    # shorter than its start-up)
     with ClockSampler(local) as clk:
+        for _ in range(args.warmup):
+            one_step()
+        torch.cuda.synchronize()
+        barrier(dist, local)
+        torch.cuda.synchronize()
         start.record(stream)
         for i in range(args.steps):
             one_step(*evs[i])
@@ -484,53 +550,43 @@ def run_gpu(args, rank, world, local):
     units = 2.0 * N_SITES * T_STEPS * args.steps
     value = aggregate_throughput(units, tmax, world)
 
-    # roofline of the dominant kernel (the temporal-blocking step kernel)
-    avg_launch_s = step_kernel_s / (args.steps * launches_step)
-    k_eff = T_STEPS / launches_step                       # steps per launch (average)
-    if desc["coin_kind"] == "hadamard_class":
-        # 4 additions per site-step (a0 +- a1, re and im); one FP32 add per lane per clock
-        flops_site_step, flops_per_lane_clk, op = 4.0, 1, "FADD"
-    else:
-        # 8 FMAs per site-step (real 2x2 coin on complex amplitudes) = 16 flops
-        flops_site_step, flops_per_lane_clk, op = 16.0, 2, "FFMA"
-    flops_launch = flops_site_step * N_SITES * k_eff
-    bytes_launch = 32.0 * N_SITES                         # 2 planes x 8 B read + written
-    alu_peak = SMS * FP32_LANES * flops_per_lane_clk * sm_max_mhz * 1e6 / 1e12   # TFLOP/s
-    ach_tflops = flops_launch / avg_launch_s / 1e12
-    ach_gbs = bytes_launch / avg_launch_s / 1e9
-    alu_frac, hbm_frac = ach_tflops / alu_peak, ach_gbs / hbm_gbs
-    traffic = ncu_traffic(desc["path"], tile)
-    if alu_frac >= hbm_frac:
-        roof = {"bound": "alu", "achieved": ach_tflops, "peak": alu_peak, "unit": "TFLOP/s",
-                "frac": alu_frac, "traffic": traffic,
-                "peak_source": f"{SMS} SMs (device attribute) x 128 FP32 lanes x {flops_per_lane_clk} flop "
-                               f"({op}) x {sm_max_mhz:.0f} MHz (derived)",
-                "hbm_view": {"achieved_gbs": ach_gbs, "peak_gbs": hbm_gbs, "frac": hbm_frac,
-                             "peak_source": f"{peak_src} HBM copy"}}
-    else:
-        roof = {"bound": "hbm", "achieved": ach_gbs, "peak": hbm_gbs, "unit": "GB/s",
-                "frac": hbm_frac, "traffic": traffic, "peak_source": f"{peak_src} HBM copy",
-                "alu_view": {"achieved_tflops": ach_tflops, "peak_tflops": alu_peak, "frac": alu_frac}}
-    roof.update({"kernel": "%s<f32,R=%d,%s coin>" % (desc["path"], tile, desc["coin_kind"]), "k": K,
-                 "flops_per_site_step": flops_site_step,
-                 "avg_launch_ms": avg_launch_s * 1e3,
-                 "effective_bytes_per_site_step": bytes_launch / N_SITES / k_eff})
+    # roofline of the dominant kernel, and of the stepping kernel on the same work
+    t_step = step_kernel_s / args.steps
+    w1 = w if not spec else qw.Walk((N_SITES,), prec="f32").set_coin(C).set_plan_ex(K, tile, _variant)
+    stepping = stepping_roofline(desc, K, tile, time_walk(qw, w1, dev0, stream) if spec else t_step, hbm_gbs, sm_max_mhz,
+                                 peak_src)
+    roof = stepping
+    if spec:
+        _, flops_site, bytes_site = spectral_work(spec)
+        peak = SMS * FP32_LANES * 2 * sm_max_mhz * 1e6 / 1e12
+        ach, gbs = flops_site * N_SITES / t_step / 1e12, bytes_site * N_SITES / t_step / 1e9
+        roof = {"bound": "alu" if ach / peak >= gbs / hbm_gbs else "hbm",
+                "achieved": ach, "peak": peak, "unit": "TFLOP/s", "frac": ach / peak, "traffic": None,
+                "peak_source": f"{SMS} SMs (device attribute) x 128 FP32 lanes x 2 flop (FFMA) x {sm_max_mhz:.0f} MHz (derived)",
+                "hbm_view": {"achieved_gbs": gbs, "peak_gbs": hbm_gbs, "frac": gbs / hbm_gbs,
+                             "peak_source": f"{peak_src} HBM copy"},
+                "kernel": f"k_spectral1d<f32, tile {spec['tile']}>", "k": math.ceil(T_STEPS / launches_step),
+                "flops_per_site": flops_site, "avg_launch_ms": t_step * 1e3 / launches_step,
+                "note": "latency-bound: one CTA fills an SM (issue 50 % under ncu)"}
 
     # k = 1 (one step per HBM round trip): the plain fused step against the HBM roof
-    plan_saved = w.plan_ex()
-    w.set_plan(1, 0)
-    qw.qw_set_state(w.h, dev0)
+    plan_saved = w1.plan_ex()
+    w1.set_plan(1, 0)
+    qw.qw_set_state(w1.h, dev0)
     e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-    qw.qw_step(w.h, 8)
+    qw.qw_step(w1.h, 8)
     e0.record(stream)
-    qw.qw_step(w.h, 64)
+    qw.qw_step(w1.h, 64)
     e1.record(stream)
     torch.cuda.synchronize()
     k1_s = e0.elapsed_time(e1) / 1e3 / 64
     roof_k1 = {"bound": "hbm", "achieved": 32.0 * N_SITES / k1_s / 1e9, "peak": hbm_gbs,
                "unit": "GB/s", "frac": 32.0 * N_SITES / k1_s / 1e9 / hbm_gbs,
                "frac_of_8000": 32.0 * N_SITES / k1_s / 1e9 / 8000.0}
-    w.set_plan_ex(*plan_saved)
+    if w1 is w:
+        w.set_plan_ex(*plan_saved)
+    else:
+        w1.close()
 
     # end to end through the C ABI with host buffers (pinned), rank-local; measured
     # right after the device-timed steps, before the other legs allocate and free
@@ -626,10 +682,11 @@ def run_gpu(args, rank, world, local):
                                           "frac_of_measured": gbs / hbm_gbs, "frac_of_8000": gbs / 8000.0}
             w2.close()
         # the rows beyond the periodic lattice walk, same lattice and state: the
-        # generic kernel with a segment boundary and 5 % of the links closed
-        # (fixed mask, 2 more bytes per site-step), or with links closed at
-        # random afresh at every step (p = 0.05, Philox in the kernel, no mask
-        # traffic); the diagonal lattice is timed above with the axis lattice
+        # tiled kernel with a segment boundary and 5 % of the links closed (fixed
+        # mask), or with links closed at random afresh at every step (p = 0.05,
+        # Philox in the kernel, no mask traffic).  It runs several steps per HBM
+        # round trip: the rates in bytes are effective ones, at the bytes of one
+        # step per round trip
         mask = (torch.rand((2, L * L), generator=torch.Generator().manual_seed(3)) < 0.05).to(torch.uint8).cuda()
         for name, kw, setup, nbytes in (
                 ("segment_fixed_links_5pct", dict(bc=qw.BC_SEGMENT),
@@ -648,8 +705,8 @@ def run_gpu(args, rank, world, local):
             ts = a.elapsed_time(b) / 1e3 / 64
             gbs = nbytes * L * L / ts / 1e9
             torus[name] = {"site_coin_updates_per_s": 4.0 * L * L / ts, "ms_per_step": ts * 1e3,
-                           "kernel": w2.describe()["path"], "algorithmic_bytes_per_site_step": nbytes,
-                           "hbm_gbs": gbs, "frac_of_measured": gbs / hbm_gbs, "norm": w2.norm()}
+                           "kernel": w2.describe()["path"], "bytes_per_site_step_at_k1": nbytes,
+                           "effective_gbs": gbs, "frac_of_measured": gbs / hbm_gbs, "norm": w2.norm()}
             w2.close()
         del z, mask
         # the paper's own timed case, the 1D segment (reflecting ends, no broken
@@ -664,7 +721,7 @@ def run_gpu(args, rank, world, local):
         ts = a.elapsed_time(b) / 1e3 / 64
         torus["cycle_2e27_segment_hadamard"] = {
             "site_coin_updates_per_s": 2.0 * N_SITES / ts, "ms_per_step": ts * 1e3, "kernel": ws.describe()["path"],
-            "algorithmic_bytes_per_site_step": 32.0, "hbm_gbs": 32.0 * N_SITES / ts / 1e9,
+            "bytes_per_site_step_at_k1": 32.0, "effective_gbs": 32.0 * N_SITES / ts / 1e9,
             "frac_of_measured": 32.0 * N_SITES / ts / 1e9 / hbm_gbs, "norm": ws.norm()}
         ws.close()
 
@@ -717,9 +774,10 @@ def run_gpu(args, rank, world, local):
             issue_peak = SMS * FP32_LANES * sm_max_mhz * 1e6 / 1e12
             batch[pname] = {"dense_site_coin_updates_per_s": dense / tb,
                             "active_site_coin_updates_per_s": active / tb, "ms_per_batch": tb * 1e3,
-                            "k": tune_b["k"], "variant": tune_b.get("variant"), "cta_walks": tune_b.get("cta_walks"),
+                            "k": tune_b["k"], "variant": tune_b.get("variant"),
+                            "momentum_space": bool(tune_b.get("spectral")), "cta_walks": tune_b.get("cta_walks"),
                             "max_norm_err": float(np.abs(nb_ - 1).max())}
-            if pname != "comp":
+            if pname != "comp" and not tune_b.get("spectral"):
                 batch[pname]["alu_view"] = {"achieved_tinst_per_s": inst_rate, "peak_tinst_per_s": issue_peak,
                                             "frac": inst_rate / issue_peak,
                                             "note": "8 FP32 instructions per active site-step (real coin)"}
@@ -756,19 +814,18 @@ def run_gpu(args, rank, world, local):
         tg = ev[0].elapsed_time(ev[1]) / 1e3 / reps
         tf = ev[2].elapsed_time(ev[3]) / 1e3
         tb = max(tg - tf, 1e-9)
-        # the adjoint sweep per site-step (FP32): reads lambda and psi (32 B each),
-        # phi (16 B) and the segment accumulator (16 B), writes lambda', psi' and
-        # the accumulator (32 + 32 + 16 B)
-        bwd_bytes = 176.0 * Lg * Lg * Tg
+        # a backward launch of 8 steps (FP32) reads lambda and psi (32 B each), phi
+        # and the segment accumulator (16 B each) and writes lambda', psi' and the
+        # accumulator (32 + 32 + 16 B): 176 B per site, if every site is lit
+        bwd_bytes = 176.0 / 8 * Lg * Lg * Tg
         grad_leg = {"ms": tg * 1e3, "loss": lossg, "forward_ms": tf * 1e3, "adjoint_ms": tb * 1e3,
                     "site_steps_per_s": 2.0 * Tg * Lg * Lg / tg,
-                    "roofline": {"bound": "hbm", "kernel": "k_backward2d<f32, Grover>", "achieved": bwd_bytes / tb / 1e9,
-                                 "peak": hbm_gbs, "unit": "GB/s", "frac": bwd_bytes / tb / 1e9 / hbm_gbs,
-                                 "algorithmic_bytes_per_site_step": 176,
-                                 "note": "adjoint time = the qw_backward call minus its forward phase timed alone; "
-                                         "the sweep's working set (lambda and psi in and out, 4 x 32 MiB, phi and "
-                                         "the accumulator, 16 MiB each) is about the L2 size, so part of it is "
-                                         "served from L2 and frac can exceed 1"},
+                    "hbm_view": {"kernel": "k_backward2d<f32, Grover>", "achieved_gbs": bwd_bytes / tb / 1e9,
+                                 "peak_gbs": hbm_gbs, "frac": bwd_bytes / tb / 1e9 / hbm_gbs,
+                                 "algorithmic_bytes_per_site_step": 176 / 8,
+                                 "note": "adjoint time = the qw_backward call minus its forward phase timed alone; the "
+                                         "launches run on the sites that the start or the region can reach, the bytes "
+                                         "count the whole lattice"},
                     "note": "forward T steps (light-cone clipped from the localised start) with checkpoints + T "
                             "adjoint steps; CUDA events"}
         wg.close()
@@ -808,7 +865,7 @@ def run_gpu(args, rank, world, local):
             torch.cuda.synchronize()
             ts = a.elapsed_time(b) / 1e3
             forms[name] = {"value": 2.0 * N_SITES * T_STEPS / ts, "unit": UNIT, "k": Kf,
-                           "tile": tf, "norm": nf}
+                           "tile": tf, "momentum_space": wf.describe().get("spectral"), "norm": nf}
             if name == "f64":
                 ref = Pf
             else:
@@ -847,8 +904,9 @@ def run_gpu(args, rank, world, local):
     w.close()
     return {
         "value": value, "elapsed": tmax, "norm": norm, "roofline": roof, "roofline_k1": roof_k1,
+        "roofline_stepping": stepping, "spectral": spec,
         "forms": forms, "accuracy": accuracy, "e2e": e2e, "clocks": clk.summary(), "tune": tune,
-        "K": K, "tile": tile, "launches": args.steps * (launches_step + 4), "dist": dist,
+        "K": K, "tile": tile, "launches": args.steps * (launches_step + 3), "dist": dist,
         "torus": torus, "batch": batch, "grad": grad_leg, "graph": graph_leg,
         "coin_classes": coin_classes, "coin_kind": desc["coin_kind"], "localized": localized,
     }
@@ -887,7 +945,7 @@ def run_case(args):
         return
     if args.case == "line":
         # the paper's line walk: Hadamard coin from the centre of a line of
-        # --n-sites sites (absorbing ends), --steps steps, clipped (the window CTA)
+        # --n-sites sites (absorbing ends), --steps steps, clipped (the window kernel)
         n = args.n_sites
         z = torch.zeros((2, n), dtype=torch.complex64, device="cuda")
         z[0, n // 2] = 2 ** -0.5
@@ -1050,12 +1108,15 @@ def main():
                    "sites": N_SITES, "coin_dim": 2, "T": T_STEPS,
                    "k": r["K"], "tile": r["tile"], "parallelism": f"replicas{world}",
                    "coin_class": r["coin_kind"] + " (theta = pi/4 with zero phases is lambda * M, M a "
-                                                  "+-1 matrix: four additions per site-step; the real and "
-                                                  "complex SU(2) classes are in coin_classes)",
+                                                  "+-1 matrix: four additions per site-step when stepped; the "
+                                                  "real and complex SU(2) classes are in coin_classes)",
+                   "momentum_space": r["spectral"],
+                   "updates": "N * d * T per step; in momentum space the T steps are one exact convolution per block, "
+                              "not T passes (roofline_stepping: the same workload stepped)",
                    "l2": "inputs larger than L2 (2 GiB state, 129 MB L2); no flush needed",
-                   "step": "set_state (device copy) + T=4096 walk steps + marginals/norm"},
+                   "step": "set_state (device copy) + T=4096 walk steps + marginals"},
         "clocks": r["clocks"], "e2e": r["e2e"], "gpu_launches": r["launches"],
-        "roofline": r["roofline"], "roofline_k1": r["roofline_k1"], "cpu_baseline": cpu,
+        "roofline": r["roofline"], "roofline_stepping": r["roofline_stepping"], "roofline_k1": r["roofline_k1"], "cpu_baseline": cpu,
         "accuracy": r["accuracy"], "forms": r["forms"], "torus_8192": r["torus"],
         "batch_4096": r["batch"], "region_grad_1024": r["grad"], "graph": r["graph"],
         "coin_classes": r["coin_classes"], "localized_start": r["localized"],

@@ -198,7 +198,9 @@ qw_status qw_get_plan(const qw_walk *w, int *depth_k, int *tile);
  * periodic cycle (any N, any precision) and one unitary coin (to 1e-6), else
  * QW_EINVAL.  The result is as accurate as stepping in norm, block by block
  * (about 2e-7 of the block's norm in float, 4e-16 in double), so an amplitude
- * that is zero or tiny beside its neighbours is not resolved beyond that; a
+ * that is zero or tiny beside its neighbours is not resolved beyond that, and a
+ * NaN or an infinity reaches every site whose block holds it (all sites on the
+ * torus), not its light cone alone; a
  * clipped state (qw_set_clipping) is therefore still stepped, until its box
  * covers the cycle.  Allocates the matrices' table (at most 0.4 MB). */
 qw_status qw_set_plan_ex(qw_walk *w, int depth_k, int tile, int variant);
@@ -227,17 +229,18 @@ qw_status qw_autotune(qw_walk *w, char *report, size_t report_len);
  * state's nonzero amplitudes on the GPU, and every step kernel then runs only
  * on that box widened by its steps, until the box covers the lattice: on the
  * cycle and the torus the box wraps; on the segment and the line it stops at
- * the ends (with broken links too), and in 1D, while the box after the next
- * steps fits one CTA's shared memory (about 6200 sites in FP32), up to 256
- * steps run in one launch with the state on chip (qw_describe's path
- * "k_step1d_window").  The adjoint with a boundary or broken
+ * the ends (with broken links too); there in 1D up to 64 steps run in one
+ * launch, on tiles that shrink with the box (qw_describe's path
+ * "k_step1d_window" while it is at most about 8192 sites).  The adjoint with a boundary or broken
  * links, and per-site coins on the torus, run kernels that step the whole
  * lattice; the box still widens with them.  The first qw_step or
  * qw_step_adjoint after qw_set_state waits for the search (not for other
  * queued work); while the walk's stream is being captured into a CUDA graph
- * nothing waits: the search is skipped and the steps run on the whole lattice.  A dense state costs about one wave of the search.  Every
- * amplitude equals that of stepping the whole lattice with the same plan, bit
- * for bit (a zero may differ in sign).  on = 0 turns it off
+ * nothing waits: the search is skipped and the steps run on the whole lattice.
+ * The search rides on the copy of a device state that is in the storage format;
+ * else it reads the buffer.  Every amplitude equals that of stepping the whole
+ * lattice with the same plan, bit for bit (a zero may differ in sign; clipped
+ * states are never taken to momentum space).  on = 0 turns it off
  * (the current state is then stepped in full); on = 1 takes effect at the next
  * qw_set_state.  qw_describe reports the box ("support": [x0, w, y0, h],
  * columns [x0, x0 + w) and rows [y0, y0 + h) modulo the lattice, "full" or
