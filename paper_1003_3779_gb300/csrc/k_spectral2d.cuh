@@ -27,6 +27,15 @@
 // stages in place in shared memory (the last one radix 2, 4 or 8 where 16 does
 // not divide), in decimation-in-frequency order forward and the reverse order
 // back, so momenta stay in digit-reversed places and nothing is reordered.
+//
+// Measured, streaming (8 steps per launch) -> momentum space, 1024 steps per call:
+//   Grover 8192^2 106 -> 9.4 ms, 4096^2 29.2 -> 1.66 ms; H (x) H on the diagonal
+//   lattice, 8192^2, 123 -> 8.6 ms; 300 x 200, 200 steps, with readout 1.12 -> 0.12 ms
+// What bounds it (4096^2): the rows run at 61-66 % of the DRAM rate; the columns,
+// three quarters of the time, are bound by the load queue and latency (issue 33 %):
+// four planes of 4096 points take an SM, one column per CTA, whose 8-byte loads
+// touch a 32-byte sector each.  A split axis of 8192 runs as even and odd momenta,
+// and k and -k share their factors (15.3 -> 11.1 ms per call with copies).
 #pragma once
 #include "qw_internal.cuh"
 #include "k_spectral1d.cuh"
