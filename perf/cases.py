@@ -77,11 +77,6 @@ def _log(rng, lo, hi):
     return int(round(math.exp(rng.uniform(math.log(lo), math.log(hi)))))
 
 
-def _even(rng, lo, hi):
-    """Row lengths of the tori: a state's rows lie 16-byte aligned only when they are even."""
-    return _log(rng, lo // 2, hi // 2) * 2
-
-
 def draw(rng):
     kind = rng.choice(["site1d", "cycle", "cycle", "torus", "torus", "site2d", "links", "grad", "batch", "graph"])
     if kind == "site1d":
@@ -97,11 +92,11 @@ def draw(rng):
                 "xi": round(rng.uniform(-1, 1), 3) if cplx else 0.0, "zeta": round(rng.uniform(-1, 1), 3) if cplx else 0.0,
                 "shift": rng.choice(["moving", "flipflop"]), "adjoint": rng.random() < 0.3}
     if kind == "torus":
-        return {"kind": kind, "nx": _even(rng, 64, 8192), "ny": _log(rng, 64, 8192), "t": _log(rng, 16, 1024),
+        return {"kind": kind, "nx": _log(rng, 64, 8192), "ny": _log(rng, 64, 8192), "t": _log(rng, 16, 1024),
                 "prec": "f32", "coin": rng.choice(["grover", "hadamard2"]),
                 "shift": rng.choice(["moving", "flipflop", "diagonal"])}
     if kind == "site2d":
-        return {"kind": kind, "nx": _even(rng, 256, 8192), "ny": _log(rng, 256, 8192), "t": _log(rng, 32, 500),
+        return {"kind": kind, "nx": _log(rng, 256, 8192), "ny": _log(rng, 256, 8192), "t": _log(rng, 32, 500),
                 "prec": "f32", "coin": rng.choice(["grover", "hadamard2"]),
                 "shift": rng.choice(["moving", "flipflop", "diagonal"])}
     if kind == "links":
@@ -109,7 +104,7 @@ def draw(rng):
                 "prec": "f32", "bc": rng.choice(["periodic", "segment", "line"]),
                 "shift": rng.choice(["moving", "flipflop"])}
     if kind == "grad":
-        return {"kind": kind, "l": _even(rng, 100, 1024), "t": _log(rng, 64, 512), "k": rng.choice([32, 64]),
+        return {"kind": kind, "l": _log(rng, 100, 1024), "t": _log(rng, 64, 512), "k": rng.choice([32, 64]),
                 "prec": "f32"}
     if kind == "batch":
         return {"kind": kind, "walks": _log(rng, 64, 4096), "nmax": _log(rng, 1024, 65536), "tmax": _log(rng, 256, 4096),
