@@ -77,6 +77,7 @@ struct BackArgs {
     Arc psi_x, psi_y, reg_x, reg_y;  // the start's support and the region
     int64_t t0, T, reach;            // psi_t0 is wanted up to `reach` sites from the region
     int K;
+    unsigned nbx;                    // tiles per row of tiles (the grid is one-dimensional: tall tori)
     const float *phi;
     void *gseg;
 };
@@ -118,7 +119,8 @@ k_backward2d(BackArgs a, CoinP<typename St<P>::real> cp) {
         while (q >= n) q -= n;
         return q;
     };
-    const int64_t bx = (int64_t)blockIdx.x * O - a.K, by = (int64_t)blockIdx.y * O - a.K;
+    const unsigned row = blockIdx.x / a.nbx;
+    const int64_t bx = (int64_t)(blockIdx.x - row * a.nbx) * O - a.K, by = (int64_t)row * O - a.K;
     const int i = (int)threadIdx.x % E, j0 = (int)threadIdx.x / E;
     const int64_t x = wrap(a.cx + bx + i, a.nx);
     const int64_t far_x = arc_distance(a.psi_x, x, a.nx), near_x = arc_distance(a.reg_x, x, a.nx);
@@ -273,13 +275,15 @@ __global__ void k_sum_blocks(const double *partials, int n, double *out) {
 template <int P> constexpr size_t back_smem() { return (size_t)2 * 4 * BACK_E * BACK_E * 2 * sizeof(typename St<P>::real); }
 
 template <int P, int FF, int GROVER>
-static cudaError_t go_backward(const qw_walk *w, const BackArgs &a) {
+static cudaError_t go_backward(const qw_walk *w, BackArgs a) {
     auto kern = k_backward2d<P, FF, GROVER>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)back_smem<P>());
     if (e != cudaSuccess) return e;
     const int O = BACK_E - 2 * a.K;
-    const dim3 grid((unsigned)((a.cw + O - 1) / O), (unsigned)((a.ch + O - 1) / O));
-    kern<<<grid, BACK_TH, back_smem<P>(), w->stream>>>(a, *reinterpret_cast<const CoinP<typename St<P>::real> *>(w->coinp));
+    const int64_t nbx = (a.cw + O - 1) / O, blocks = nbx * ((a.ch + O - 1) / O);
+    if (blocks >= (int64_t(1) << 31)) return cudaErrorInvalidConfiguration;
+    a.nbx = (unsigned)nbx;
+    kern<<<(unsigned)blocks, BACK_TH, back_smem<P>(), w->stream>>>(a, *reinterpret_cast<const CoinP<typename St<P>::real> *>(w->coinp));
     return cudaGetLastError();
 }
 
