@@ -418,9 +418,12 @@ static void grow_support(qw_walk *w, int K) {
 }
 
 // The box of the current state for the kernels that read it out (w = 0 when it
-// is not known, or when a graph replay may have changed the state).
+// is not known, when a graph replay may have changed the state, or when the
+// readout itself is being captured: its replays read whatever the state is then).
 static SupportBox state_box(const qw_walk *w) {
-    if (w->sup_mode != 2 || w->captured) return {0, 0, 0, 0, w->nx, w->ny};
+    const SupportBox whole = {0, 0, 0, 0, w->nx, w->ny};
+    if (w->sup_mode != 2 || w->captured) return whole;
+    if (capturing(w)) { (void)cudaGetLastError(); return whole; }
     return {w->bx0, w->bw, w->by0, w->bh, w->nx, w->ny};
 }
 
