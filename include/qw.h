@@ -202,7 +202,8 @@ qw_status qw_get_plan(const qw_walk *w, int *depth_k, int *tile);
  * NaN or an infinity reaches every site whose block holds it (all sites on the
  * torus), not its light cone alone; a
  * clipped state (qw_set_clipping) is therefore still stepped, until its box
- * covers the cycle.  Allocates the matrices' table (at most 0.4 MB). */
+ * covers the cycle.  Allocates the tile's table of matrices (at most 0.4 MB), which
+ * the handle keeps. */
 qw_status qw_set_plan_ex(qw_walk *w, int depth_k, int tile, int variant);
 qw_status qw_get_plan_ex(const qw_walk *w, int *depth_k, int *tile, int *variant);
 

@@ -494,15 +494,15 @@ static bool spectral_walk(const qw_walk *w) {
     return true;
 }
 
-// The tables of a tile: allocated when a plan is set, never during a step.
+// The table of a tile: allocated when a plan is set, never during a step.
 static cudaError_t spectral_prepare(qw_walk *w, int tile) {
-    cudaError_t e = cudaSuccess;
-    if (!w->spec_table && (e = dev_alloc(&w->spec_table, spectral1d_table_bytes(w->prec))) != cudaSuccess) return e;
-    if (w->spec_tw != tile) {
-        w->spec_tw = tile;
-        std::memset(&w->spec_key, 0, sizeof w->spec_key);
-        e = launch_spectral1d_twiddles(w->prec, tile, w->spec_table, w->stream);
-    }
+    void *&table = w->spec_tables[spectral1d_groups(tile) - 1];
+    if (table) return cudaSuccess;
+    void *t = nullptr;
+    cudaError_t e = dev_alloc(&t, spectral1d_table_bytes(w->prec, tile));
+    if (e == cudaSuccess) e = launch_spectral1d_twiddles(w->prec, tile, t, w->stream);
+    if (e == cudaSuccess) table = t;
+    else cudaFree(t);
     return e;
 }
 
@@ -521,7 +521,7 @@ static cudaError_t spectral_launch(qw_walk *w, Spec1DArgs &a, double gain) {
     std::memset(&key, 0, sizeof key);   // padding included: keys are compared as bytes
     std::memcpy(key.coin, coin, sizeof key.coin);
     key.scale = scale; key.K = a.K; key.tile = a.tile; key.adjoint = a.adjoint;
-    a.table = w->spec_table;
+    a.table = w->spec_tables[spectral1d_groups(a.tile) - 1];
     if (capturing(w)) w->captured = true;
     if (w->captured || std::memcmp(&key, &w->spec_key, sizeof key) != 0) {
         cudaError_t e = launch_spectral1d_matrices(w->prec, a, coin, scale, w->stream);
@@ -846,6 +846,7 @@ qw_status qw_destroy(qw_walk *w) {
     cudaFree(w->staging);
     cudaFree(w->grad_scratch);
     cudaFree(w->spec_table);
+    for (void *t : w->spec_tables) cudaFree(t);
     cudaFree(w->buf3);
     cudaFree(w->pipe_p[0]);
     cudaFree(w->pipe_p[1]);

@@ -92,17 +92,19 @@ struct qw_walk {
 
     // momentum-space steps of the cycle (k_spectral1d.cuh): calls of at least
     // spec_min steps on an unclipped state run them in launches of up to spec_k
-    // steps on blocks of 32 * spec_tile sites (spec_tile 0: off).  The table
-    // holds the twiddles of spec_tw's tile and the matrices of spec_key; a
-    // captured call writes it on every replay, so no matrices are reused after one.
+    // steps on blocks of 32 * spec_tile sites (spec_tile 0: off).  Each tile has
+    // a table of its own, which stays as long as the handle: captured calls go on
+    // reading its twiddles when the other tile is in use.  The matrices of
+    // spec_key are in its tile's table; a captured call writes them on every
+    // replay, so no matrices are reused after one.
     int spec_tile = 0, spec_k = 0;
     int64_t spec_min = 0;
     bool spec_user = false;   // chosen by qw_set_plan_ex
-    // ... of the torus (k_spectral2d.cuh): calls of at least spec_min steps; the
-    // table is then the workspace of the transforms
+    void *spec_tables[2] = {nullptr, nullptr};   // by spectral1d_groups(tile) - 1
+    // ... of the torus (k_spectral2d.cuh): calls of at least spec_min steps, in
+    // the workspace spec_table
     bool spec2 = false;
     void *spec_table = nullptr;
-    int spec_tw = 0;
     struct SpecKey {
         double coin[8];
         double scale;
@@ -188,7 +190,7 @@ cudaError_t launch_step2d_tb(const Step2DArgs &a, const void *coinp, cudaStream_
 // momentum-space steps of the cycle (spectral1d.cu)
 int spectral1d_groups(int tile);
 bool spectral1d_ok(int prec, int64_t n, int K, int tile);
-size_t spectral1d_table_bytes(int prec);
+size_t spectral1d_table_bytes(int prec, int tile);
 cudaError_t launch_spectral1d_twiddles(int prec, int tile, void *table, cudaStream_t s);
 cudaError_t launch_spectral1d_matrices(int prec, const Spec1DArgs &a, const double *coin, double scale, cudaStream_t s);
 cudaError_t launch_spectral1d(int prec, const Spec1DArgs &a, cudaStream_t s);

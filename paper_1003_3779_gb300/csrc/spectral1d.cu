@@ -177,8 +177,9 @@ bool spectral1d_ok(int prec, int64_t n, int K, int tile) {
     return K >= 1 && K < 16 * tile && (n + W - 1) / W < (int64_t(1) << 30);
 }
 
-size_t spectral1d_table_bytes(int prec) {
-    return spec_double(prec) ? spec_table_bytes<double>(1) : spec_table_bytes<float>(2);
+size_t spectral1d_table_bytes(int prec, int tile) {
+    const int G = spectral1d_groups(tile);
+    return spec_double(prec) ? spec_table_bytes<double>(G) : spec_table_bytes<float>(G);
 }
 
 cudaError_t launch_spectral1d_twiddles(int prec, int tile, void *table, cudaStream_t s) {

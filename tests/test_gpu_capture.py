@@ -49,3 +49,28 @@ def test_captured_readout_reads_the_whole_state(qw, dims):
     assert maxabs(out.cpu().numpy(), want) < amp_tol("f32", 24)
     assert maxabs(P.cpu().numpy(), (np.abs(want) ** 2).sum(0)) < 2 * amp_tol("f32", 24)
     w.close()
+
+
+def test_captured_momentum_space_call_survives_another_tile(qw):
+    """A momentum-space call captured with one tile, replayed after the handle ran
+    with the other (tolerance: one launch, as in test_gpu_spectral)."""
+    import torch
+    n, s = 30001, torch.cuda.Stream()
+    psi0 = inputs.random_state((2, n), seed=9)
+    psi = torch.from_numpy(psi0).to("cuda", torch.complex64)
+    C = inputs.su2(0.7)
+    with torch.cuda.stream(s):
+        for tile, other in ((256, 512), (512, 256)):
+            w = qw.Walk((n,), prec="f32").set_coin(C).set_plan_ex(512, tile, 2).set_state(psi)
+            w.step(300)
+            want = w.state()
+            assert maxabs(want, oracle.evolve(psi0, C, 300)) <= (300 * 4 / np.sqrt(n) + 94) * U["f32"]
+            g = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(g, stream=s):
+                w.set_state(psi)
+                w.step(300)
+            w.set_plan_ex(512, other, 2).set_state(psi).step(211).step(100)   # two launches: the captured buffers again
+            g.replay()
+            s.synchronize()
+            assert np.array_equal(w.state(), want)
+            w.close()
