@@ -596,6 +596,15 @@ static qw_status batch_cuda(qw_batch *b, cudaError_t e, const char *where) {
     return batch_fail(b, e == cudaErrorMemoryAllocation ? QW_ENOMEM : QW_ECUDA, m);
 }
 
+// Host data to the device on the batch's stream, complete on return.  (cudaMemcpy
+// orders nothing against a non-blocking stream, and from pageable memory it may
+// return before the copy has reached the device.)
+static cudaError_t batch_upload(qw_batch *b, void *dst, const void *src, size_t bytes) {
+    cudaError_t e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, b->stream);
+    const cudaError_t f = cudaStreamSynchronize(b->stream);   // (also after an error: src is the caller's to free)
+    return e != cudaSuccess ? e : f;
+}
+
 static int batch_slot_bytes(int prec) { return prec == QW_F32_BF16STORE ? 4 : 8; }
 static int batch_slots(int prec) { return prec == QW_F32_COMP ? 4 : 2; }    // plane slots per walk
 static int batch_tile(int prec) { return prec == QW_F32_COMP ? BATCH_R_COMP : BATCH_R; }
@@ -759,7 +768,7 @@ static bool batch_spectral_prepare(qw_batch *b) {
     b->near_count = (int)near.size();
     if (e == cudaSuccess && !near.empty()) {
         if (!b->near_ids) e = dev_alloc((void **)&b->near_ids, sizeof(int) * near.size());
-        if (e == cudaSuccess) e = cudaMemcpy(b->near_ids, near.data(), sizeof(int) * near.size(), cudaMemcpyHostToDevice);
+        if (e == cudaSuccess) e = batch_upload(b, b->near_ids, near.data(), sizeof(int) * near.size());
         if (e == cudaSuccess && !b->side) e = cudaStreamCreateWithFlags(&b->side, cudaStreamNonBlocking);
         if (e == cudaSuccess && !b->fork) e = cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming);
         if (e == cudaSuccess && !b->join) e = cudaEventCreateWithFlags(&b->join, cudaEventDisableTiming);
@@ -768,7 +777,7 @@ static bool batch_spectral_prepare(qw_batch *b) {
         e = dev_alloc(&b->spec_table, batch_spectral_table_bytes());
         if (e == cudaSuccess) e = launch_batch_spectral_tables(b->spec_table, b->stream);
     }
-    if (e == cudaSuccess) e = cudaMemcpy(b->spec_walks, all.data(), sizeof(SpecWalk) * all.size(), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = batch_upload(b, b->spec_walks, all.data(), sizeof(SpecWalk) * all.size());
     if (e != cudaSuccess) {
         (void)cudaGetLastError();
         cudaFree(b->spec_walks);
@@ -889,8 +898,8 @@ qw_status qw_batch_create(int nwalks, const int64_t *N, const int64_t *T, const 
     if (e == cudaSuccess) e = dev_alloc((void **)&b->counter, 2 * sizeof(int));
     if (e == cudaSuccess) e = dev_alloc((void **)&b->final_dev, sizeof(int) * nwalks);
     set_gains(b, b->K);
-    if (e == cudaSuccess) e = cudaMemcpy(b->walks_dev, b->walks.data(), sizeof(WalkDesc) * nwalks, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(b->order_dev, b->order.data(), sizeof(int) * nwalks, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = batch_upload(b, b->walks_dev, b->walks.data(), sizeof(WalkDesc) * nwalks);
+    if (e == cudaSuccess) e = batch_upload(b, b->order_dev, b->order.data(), sizeof(int) * nwalks);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking);
     if (e != cudaSuccess) {
         qw_status st = e == cudaErrorMemoryAllocation ? QW_ENOMEM : QW_ECUDA;
@@ -936,7 +945,7 @@ qw_status qw_batch_set_plan(qw_batch *b, int depth_k) {
         drop_graph(b);   // the captured launch carries k
         b->K = depth_k;
         set_gains(b, depth_k);
-        cudaError_t e = cudaMemcpy(b->walks_dev, b->walks.data(), sizeof(WalkDesc) * b->nwalks, cudaMemcpyHostToDevice);
+        cudaError_t e = batch_upload(b, b->walks_dev, b->walks.data(), sizeof(WalkDesc) * b->nwalks);
         if (e != cudaSuccess) return batch_cuda(b, e, "batch plan");
     }
     return QW_OK;
