@@ -536,8 +536,10 @@ static cudaError_t spectral_launch(qw_walk *w, Spec1DArgs &a, double gain) {
 // (two per block; one CTA per SM, or two of the small float blocks) and about
 // a quarter of a wave's time to start and drain.
 static qw_status run_spectral(qw_walk *w, int64_t T, int adj) {
-    static int sms = 0;
-    if (!sms && (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, w->device) != cudaSuccess || sms <= 0)) sms = 152;
+    static const int sms = [w] {   // (every device here is the same part)
+        int n = 0;
+        return cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, w->device) == cudaSuccess && n > 0 ? n : 152;
+    }();
     const int64_t slots = (int64_t)sms * (w->spec_tile == 256 && rounds_to_float(w) ? 2 : 1);
     const int64_t m0 = (T + w->spec_k - 1) / w->spec_k;
     int64_t best_m = m0;

@@ -31,17 +31,20 @@ static cudaError_t go2d_tb(const Step2DArgs &a, const CoinP<float> &cp, cudaStre
     // its scheduler, whichever is longer.  Chunks of at least 64 rows kept 88
     // warps busy on a 500 x 500 window; KT = 8, per step, before -> now: 300 x 200
     // 6.1 -> 1.9 us, 1024^2 6.0 -> 4.0 us, 2048^2 11.1 -> 9.3 us.
-    // (looked up once per instance; every device here is the same part)
-    static int64_t resident = 0, schedulers = 0;
-    if (!resident) {
+    // (looked up once per instance, by whichever thread is first; every device here
+    // is the same part)
+    struct Chip {
+        int64_t resident, schedulers;   // warps of this instance that the device holds; schedulers
+    };
+    static const Chip chip = [&] {
         int dev = 0, sms = 0, per_sm = 0;
         cudaGetDevice(&dev);
         if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) sms = 1;
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 128, smem) != cudaSuccess || per_sm < 1)
             per_sm = 1;
-        schedulers = (int64_t)sms * 4;
-        resident = schedulers * per_sm;
-    }
+        return Chip{(int64_t)sms * 4 * per_sm, (int64_t)sms * 4};
+    }();
+    const int64_t resident = chip.resident, schedulers = chip.schedulers;
     int64_t H = oh;
     double best = -1;
     const bool fills = nstrips * ((oh + 8 * KT - 1) / (8 * KT)) >= resident;

@@ -9,18 +9,18 @@ namespace qw {
 template <int P, int SH, int CK, bool PH, bool LINKS, int EX, int EY, int TH>
 struct TileShape {
     static constexpr size_t smem = (size_t)EX * EY * 4 * 2 * sizeof(typename St<P>::real);
-    // CTAs of this shape the device holds at once (looked up once; every device here is the same part)
+    // CTAs of this shape the device holds at once (looked up once, by whichever
+    // thread is first; every device here is the same part)
     static int64_t slots() {
-        static int64_t n = 0;
-        if (!n) {
+        static const int64_t n = [] {
             auto kern = k_tile2d<P, SH, CK, PH, LINKS, EX, EY, TH>;
             int dev = 0, sms = 0, per_sm = 0;
             cudaGetDevice(&dev);
             if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) sms = 1;
             cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, TH, smem) != cudaSuccess || per_sm < 1) per_sm = 1;
-            n = (int64_t)sms * per_sm;
-        }
+            return (int64_t)sms * per_sm;
+        }();
         return n;
     }
     static dim3 grid(const Tile2DArgs &a) {
