@@ -626,6 +626,12 @@ static void tile2d_box(const qw_walk *w, int K, Tile2DArgs &a) {
     output_range(clip, w->by0, w->bh, w->ny, K, per, a.oy0, a.oh);
 }
 
+// Does a launch of up to k steps of the torus onto `sites` output sites run in tiles?
+// (On small boxes, and for the coins that the streaming kernel does not run.)
+static bool tile2d_runs(const qw_walk *w, int k, int64_t sites) {
+    return tile2d_walk(w) && (!(k >= 4 && step2d_tb_ok(w->prec, w->kind, k >= 8 ? 8 : 4, w->shift)) || sites <= TILE2D_SITES);
+}
+
 // One launch of K steps from the current buffer to the other (links: broken
 // links or an edge, whose random draws start at rstep).
 static cudaError_t tile2d_launch(qw_walk *w, int K, bool links, uint32_t rstep, double gain) {
@@ -772,17 +778,15 @@ qw_status run_steps(qw_walk *w, int64_t T, int adj) {
     int K2, t2;
     effective_plan(w, K2, t2);
     if (!adj && K2 > 1) {
-        // K2 steps per launch: tiles on small boxes and for the coins the streaming
-        // kernel does not run, else the streaming kernel, whose remainders of 4 to
-        // 7 steps take a launch of 4
-        const bool tile = tile2d_walk(w);
+        // K2 steps per launch: tiles (tile2d_runs), else the streaming kernel, whose
+        // remainders of 4 to 7 steps take a launch of 4
         while (T > 0) {
             int k = (int)std::min<int64_t>(K2, T);
             const int kt = k >= 8 ? 8 : 4;
             const bool tb = k >= 4 && step2d_tb_ok(w->prec, w->kind, kt, w->shift);
             Tile2DArgs box{};
             tile2d_box(w, k, box);
-            const bool use_tile = tile && (!tb || box.ow * box.oh <= TILE2D_SITES);
+            const bool use_tile = tile2d_runs(w, k, box.ow * box.oh);
             if (!use_tile && !tb) break;
             if (!use_tile) k = kt;
             const double gain = drift_gain(w, k, T - k == 0);   // applied once, to the launch's output
@@ -1533,7 +1537,8 @@ extern "C" qw_status qw_autotune(qw_walk *w, char *report, size_t report_len) {
     }
     w->next_clear = w->dirty_known = false;   // the timed launches write the other buffer
     if (w->ndim == 2) {
-        // k = 1 (fused step) against the streaming kernel at k = 4 and 8
+        // k = 1 (fused step) against k = 4 and 8 in the kernel that those steps run
+        // in on the whole torus: the streaming kernel, or the tiles
         cudaEvent_t e0, e1;
         cudaEventCreate(&e0);
         cudaEventCreate(&e1);
@@ -1544,10 +1549,16 @@ extern "C" qw_status qw_autotune(qw_walk *w, char *report, size_t report_len) {
         float best = 1e30f;
         int best_k = 1;
         cudaError_t err = cudaSuccess;
+        const int sup = w->sup_mode;
+        w->sup_mode = 0;   // (time whole launches, whatever is known of the state)
         for (int k : {1, 4, 8}) {
-            if (k > 1 && !step2d_tb_ok(w->prec, w->kind, k, w->shift)) continue;
+            const bool tile = k > 1 && tile2d_runs(w, k, w->ns);
+            if (k > 1 && !tile && !step2d_tb_ok(w->prec, w->kind, k, w->shift)) continue;
             a.K = k;
-            auto launch = [&]() { return k == 1 ? step2d(w->prec, a, w->coinp, 0, w->stream) : launch_step2d_tb(a, w->coinp, w->stream); };
+            auto launch = [&]() {
+                if (tile) return tile2d_launch(w, k, false, 0, 1.0);
+                return k == 1 ? step2d(w->prec, a, w->coinp, 0, w->stream) : launch_step2d_tb(a, w->coinp, w->stream);
+            };
             if ((err = launch()) != cudaSuccess) break;
             cudaEventRecord(e0, w->stream);
             for (int r = 0; r < 3; ++r) launch();
@@ -1557,6 +1568,7 @@ extern "C" qw_status qw_autotune(qw_walk *w, char *report, size_t report_len) {
             cudaEventElapsedTime(&ms, e0, e1);
             if (ms / (3 * k) < best) { best = ms / (3 * k); best_k = k; }
         }
+        w->sup_mode = sup;
         cudaEventDestroy(e0);
         cudaEventDestroy(e1);
         if (err != cudaSuccess) return cuda_error(w, err, "autotune");
