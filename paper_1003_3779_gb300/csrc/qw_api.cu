@@ -1457,6 +1457,33 @@ void tune_load() {
 // pair rounds about as much as this many steps.
 constexpr int SPEC_MIN_STEPS = 128;
 
+// ms per step of the cycle's stepping plan (state unchanged, the other buffer overwritten)
+cudaError_t time_stepping(qw_walk *w, float &ms) {
+    int k, tile, variant;
+    effective_plan(w, k, tile, variant);
+    Step1DArgs a{};
+    a.n = w->nx; a.shift = w->shift; a.kind = w->kind; a.coins = w->coins_dev;
+    a.variant = variant == 1 && sweep_ok(w, k, tile) ? 1 : 0;
+    a.tile = a.variant == 1 ? tile : tile1d(w->prec, tile, w->kind, 0);
+    a.K = a.variant == 1 ? k : std::min(k, max_k_of_tile(a.tile));
+    a.in = cur_view(w); a.out = next_view(w);
+    launch_gains_1d(w, a.K, 0, a, false);
+    cudaEvent_t e0 = nullptr, e1 = nullptr;
+    cudaError_t e = step1d(w->prec, a, w->coinp, 0, w->stream);
+    if (e == cudaSuccess) e = cudaEventCreate(&e0);
+    if (e == cudaSuccess) e = cudaEventCreate(&e1);
+    if (e == cudaSuccess) e = cudaEventRecord(e0, w->stream);
+    const int reps = 3;
+    for (int r = 0; r < reps && e == cudaSuccess; ++r) e = step1d(w->prec, a, w->coinp, 0, w->stream);
+    if (e == cudaSuccess) e = cudaEventRecord(e1, w->stream);
+    if (e == cudaSuccess) e = cudaEventSynchronize(e1);
+    if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
+    ms /= reps * a.K;
+    if (e0) cudaEventDestroy(e0);
+    if (e1) cudaEventDestroy(e1);
+    return e;
+}
+
 // ms of one momentum-space launch of K steps (state unchanged, a.out overwritten)
 cudaError_t time_spectral(qw_walk *w, Spec1DArgs &a, int K, float &ms) {
     a.K = K;
@@ -1595,36 +1622,38 @@ extern "C" qw_status qw_autotune(qw_walk *w, char *report, size_t report_len) {
     char buf[512];
     spectral_off(w);
     // The momentum-space form, kept beside the stepping plan under its own key
-    // (tile, fewest steps of a call worth a launch; tile 0: never), so that a
-    // tuning file written without it still serves.  ms_step: the stepping plan's.
+    // (tile, fewest steps of a call worth a launch; tile 0: never).  A tuning file
+    // written without it still serves, and so does a plan that was tuned for a coin
+    // without that form: the plan is then timed here (ms_step: its time per step, 0
+    // if it has not been timed).
     auto tune_spectral = [&](float ms_step, std::string &rep) -> cudaError_t {
         const std::string skey = key + "_spectral";
         auto si = g_tune.find(skey);
         cudaError_t err = cudaSuccess;
-        if (si == g_tune.end()) {
+        if (si == g_tune.end() && spectral_walk(w)) {
+            if (!(ms_step > 0) && (err = time_stepping(w, ms_step)) != cudaSuccess) return err;
             int tile = 0, from = 0;
-            if (ms_step > 0 && spectral_walk(w)) {
-                float best = 1e30f;
-                for (int st : {256, 512}) {
-                    const int k = 8 * st;   // a quarter of the block: half its sites are output
-                    if (!spectral1d_ok(w->prec, w->nx, k, st)) continue;
-                    if (spectral_prepare(w, st) != cudaSuccess) { (void)cudaGetLastError(); break; }
-                    Spec1DArgs a{};
-                    a.n = w->nx; a.tile = st; a.shift = w->shift;
-                    a.in = cur_view(w); a.out = next_view(w);
-                    float ms = 0.f, ms_short = 0.f;
-                    if ((err = time_spectral(w, a, k, ms)) != cudaSuccess) return err;
-                    if ((err = time_spectral(w, a, k / 8, ms_short)) != cudaSuccess) return err;
-                    if (ms / k < best) {
-                        best = ms / k;
-                        tile = st;
-                        // the shortest call that gains, and not below SPEC_MIN_STEPS
-                        from = std::max(SPEC_MIN_STEPS, (int)std::min(1e9f, std::ceil(ms_short / ms_step)));
-                    }
+            float best = 1e30f;
+            for (int st : {256, 512}) {
+                const int k = 8 * st;   // a quarter of the block: half its sites are output
+                if (!spectral1d_ok(w->prec, w->nx, k, st)) continue;
+                if (spectral_prepare(w, st) != cudaSuccess) { (void)cudaGetLastError(); break; }
+                Spec1DArgs a{};
+                a.n = w->nx; a.tile = st; a.shift = w->shift;
+                a.in = cur_view(w); a.out = next_view(w);
+                float ms = 0.f, ms_short = 0.f;
+                if ((err = time_spectral(w, a, k, ms)) != cudaSuccess) return err;
+                if ((err = time_spectral(w, a, k / 8, ms_short)) != cudaSuccess) return err;
+                if (ms / k < best) {
+                    best = ms / k;
+                    tile = st;
+                    // the shortest call that gains, and not below SPEC_MIN_STEPS
+                    from = std::max(SPEC_MIN_STEPS, (int)std::min(1e9f, std::ceil(ms_short / ms_step)));
                 }
-                if (!(best < ms_step)) tile = 0;
             }
-            if (ms_step > 0 && spectral_walk(w)) { g_tune[skey] = {tile, from}; tune_save(); }
+            if (!(best < ms_step)) tile = 0;
+            g_tune[skey] = {tile, from};
+            tune_save();
             si = g_tune.find(skey);
         }
         if (si != g_tune.end() && spectral_walk(w) && spectral1d_ok(w->prec, w->nx, 1, si->second.first)) {

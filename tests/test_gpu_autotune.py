@@ -1,11 +1,17 @@
 """What qw_autotune settles on: never a plan that it did not time against the
 kernels that the steps then run, whatever was tuned or cached before."""
+import json
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 
 from paper_1003_3779_gb300 import inputs
 
 pytestmark = pytest.mark.gpu
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
 @pytest.fixture(scope="module")
@@ -45,3 +51,38 @@ def test_general_coins_keep_several_steps_per_launch(qw, shift):
     assert np.array_equal(w.set_state(psi0).step(21).state(np.complex64), v.step(21).state(np.complex64))
     w.close()
     v.close()
+
+
+def tuned(code, env=None):
+    """Run `code` in a process of its own; the JSON lines it prints."""
+    head = "import json, numpy as np\nfrom paper_1003_3779_gb300 import inputs, qw\n"
+    p = subprocess.run([sys.executable, "-c", head + code], cwd=ROOT, env=dict(os.environ, **(env or {})),
+                       capture_output=True, text=True, timeout=600)
+    assert p.returncode == 0, p.stderr[-2000:]
+    return [json.loads(line) for line in p.stdout.splitlines()]
+
+
+TUNE = """
+def tune(coin):
+    w = qw.Walk((1 << 20,), prec="f32").set_coin(coin).set_state(inputs.random_state((2, 1 << 20), seed=1))
+    print(w.autotune())
+    w.close()
+"""
+
+
+def test_a_cache_of_stepping_plans_gets_the_momentum_space_form(qw, tmp_path):
+    """A tuning file that holds the stepping plan alone: the momentum-space form is
+    timed against that plan, used, and added to the file."""
+    path = tmp_path / "tune.json"
+    env = {"QW_TUNE_CACHE": str(path)}
+    (first,) = tuned(TUNE + "tune(inputs.su2(0.3))\n", env)
+    assert not first["cached"] and "spectral" in first
+    path.write_text("".join(line for line in path.read_text().splitlines(True) if "_spectral" not in line))
+    (again,) = tuned(TUNE + "tune(inputs.su2(0.3))\n", env)
+    assert again["cached"] and again["spectral"]["from_steps"] >= 1
+    assert "_spectral" in path.read_text()
+
+
+def test_a_coin_that_is_not_unitary_tuned_first(qw):
+    lossy, unitary = tuned(TUNE + "tune(0.9 * inputs.su2(0.3))\ntune(inputs.su2(0.3))\n")
+    assert "spectral" not in lossy and unitary["cached"] and "spectral" in unitary
