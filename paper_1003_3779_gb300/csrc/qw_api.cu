@@ -1628,16 +1628,20 @@ extern "C" qw_status qw_autotune(qw_walk *w, char *report, size_t report_len) {
     // if it has not been timed).
     auto tune_spectral = [&](float ms_step, std::string &rep) -> cudaError_t {
         const std::string skey = key + "_spectral";
-        auto si = g_tune.find(skey);
+        const auto si = g_tune.find(skey);
+        std::pair<int, int> form{0, 0};
+        if (si != g_tune.end()) form = si->second;
         cudaError_t err = cudaSuccess;
         if (si == g_tune.end() && spectral_walk(w)) {
             if (!(ms_step > 0) && (err = time_stepping(w, ms_step)) != cudaSuccess) return err;
             int tile = 0, from = 0;
+            bool room = true;
             float best = 1e30f;
             for (int st : {256, 512}) {
                 const int k = 8 * st;   // a quarter of the block: half its sites are output
                 if (!spectral1d_ok(w->prec, w->nx, k, st)) continue;
-                if (spectral_prepare(w, st) != cudaSuccess) { (void)cudaGetLastError(); break; }
+                if ((err = spectral_prepare(w, st)) == cudaErrorMemoryAllocation) { (void)cudaGetLastError(); room = false; break; }
+                if (err != cudaSuccess) return err;
                 Spec1DArgs a{};
                 a.n = w->nx; a.tile = st; a.shift = w->shift;
                 a.in = cur_view(w); a.out = next_view(w);
@@ -1652,19 +1656,18 @@ extern "C" qw_status qw_autotune(qw_walk *w, char *report, size_t report_len) {
                 }
             }
             if (!(best < ms_step)) tile = 0;
-            g_tune[skey] = {tile, from};
-            tune_save();
-            si = g_tune.find(skey);
+            form = {tile, from};
+            if (room) { g_tune[skey] = form; tune_save(); }   // (else it says nothing about the next handle)
         }
-        if (si != g_tune.end() && spectral_walk(w) && spectral1d_ok(w->prec, w->nx, 1, si->second.first)) {
-            if ((err = spectral_prepare(w, si->second.first)) == cudaErrorMemoryAllocation) {
+        if (spectral_walk(w) && spectral1d_ok(w->prec, w->nx, 1, form.first)) {
+            if ((err = spectral_prepare(w, form.first)) == cudaErrorMemoryAllocation) {
                 (void)cudaGetLastError();
                 return cudaSuccess;   // no room for the tables: the stepping plan alone
             }
             if (err != cudaSuccess) return err;
-            w->spec_tile = si->second.first;
+            w->spec_tile = form.first;
             w->spec_k = w->spec_tile * 32 / 3;   // a third of the block: more steps leave too few outputs
-            w->spec_min = std::max(1, si->second.second);
+            w->spec_min = std::max(1, form.second);
             char b[96];
             std::snprintf(b, sizeof b, ", \"spectral\": {\"tile\": %d, \"from_steps\": %lld}", w->spec_tile, (long long)w->spec_min);
             rep = b;

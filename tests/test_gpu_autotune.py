@@ -86,3 +86,20 @@ def test_a_cache_of_stepping_plans_gets_the_momentum_space_form(qw, tmp_path):
 def test_a_coin_that_is_not_unitary_tuned_first(qw):
     lossy, unitary = tuned(TUNE + "tune(0.9 * inputs.su2(0.3))\ntune(inputs.su2(0.3))\n")
     assert "spectral" not in lossy and unitary["cached"] and "spectral" in unitary
+
+
+def test_a_failed_allocation_is_not_remembered(qw):
+    """No room for the tables of one handle: it steps; the next one, with room,
+    takes the momentum-space form."""
+    code = """
+import os
+w = [qw.Walk((1 << 20,), prec="f32").set_coin(inputs.su2(0.3)).set_state(inputs.random_state((2, 1 << 20), seed=1)) for _ in range(2)]
+w[0].step(1)
+os.environ["QW_FAULT"] = "alloc"
+qw.lib()
+print(w[0].autotune())
+del os.environ["QW_FAULT"]
+print(w[1].autotune())
+"""
+    starved, fed = tuned(code)
+    assert starved["tuned"] and "spectral" not in starved and "spectral" in fed
