@@ -215,8 +215,9 @@ qw_status qw_get_plan_ex(const qw_walk *w, int *depth_k, int *tile, int *variant
  * many steps) on states that are not clipped; qw_describe reports them as
  * "spectral".  On the torus (FP32) it does the same for the Grover coin with any
  * shift and for H (x) H on the diagonal lattice, for calls of at least 64 steps,
- * in a workspace of 64 MB to 2 GB (four state buffers' worth in between) that
- * the handle keeps; without room for it the steps stay as they are.  1D results are cached per (lattice shape,
+ * in a workspace of 64 MB to 2 GB (four state buffers' worth in between), kept
+ * with the handle where they are faster and given back where not; without room
+ * for it the steps stay as they are.  1D results are cached per (lattice shape,
  * precision, coin kind) in memory and, if the environment variable
  * QW_TUNE_CACHE names a file, in that JSON file.  report (may be NULL)
  * receives a one-line JSON summary, truncated to report_len bytes. */

@@ -1511,13 +1511,14 @@ cudaError_t tune_spectral2d(qw_walk *w, float &ms) {
     const Spec2Plan p = spectral2d_plan(w->nx, w->ny, SPEC2_TUNE_STEPS, true);
     if (p.K < 2) return cudaSuccess;
     if (!w->spec_table) {
-        if (dev_alloc(&w->spec_table, spectral2d_workspace(w->nx, w->ny)) != cudaSuccess) {
+        void *t = nullptr;
+        if (dev_alloc(&t, spectral2d_workspace(w->nx, w->ny)) != cudaSuccess) {
             (void)cudaGetLastError();
-            w->spec_table = nullptr;
             return cudaSuccess;   // no room: the stepping plan alone
         }
-        const cudaError_t e = launch_spectral2d_tables(w->spec_table, w->stream);
-        if (e != cudaSuccess) return e;
+        const cudaError_t e = launch_spectral2d_tables(t, w->stream);
+        if (e != cudaSuccess) { cudaFree(t); return e; }
+        w->spec_table = t;
     }
     Step2DArgs a{};
     a.nx = w->nx; a.ny = w->ny; a.shift = w->shift; a.kind = w->kind; a.K = p.K; a.gain = 1.0;
@@ -1604,8 +1605,12 @@ extern "C" qw_status qw_autotune(qw_walk *w, char *report, size_t report_len) {
         spectral_off(w);
         if (spectral2d_walk(w)) {
             float ms = 0.f;
+            // (a workspace that was there before may be in a captured graph: it stays)
+            const bool fresh = !w->spec_table;
             if ((err = tune_spectral2d(w, ms)) != cudaSuccess) return cuda_error(w, err, "autotune");
-            if (ms > 0 && ms < best * SPEC2_TUNE_STEPS) {
+            if (!(ms > 0 && ms < best * SPEC2_TUNE_STEPS)) {
+                if (fresh) { cudaFree(w->spec_table); w->spec_table = nullptr; }
+            } else {
                 w->spec2 = true;
                 w->spec_min = std::max<int64_t>(SPEC2_MIN_STEPS, (int64_t)std::ceil(ms / best));
                 std::snprintf(sp, sizeof sp, ", \"spectral\": {\"from_steps\": %lld}", (long long)w->spec_min);

@@ -103,3 +103,20 @@ print(w[1].autotune())
 """
     starved, fed = tuned(code)
     assert starved["tuned"] and "spectral" not in starved and "spectral" in fed
+
+
+def test_a_rejected_workspace_is_given_back(qw):
+    """Two sites in x: a block of the transforms holds 128 times the lattice, so the
+    torus goes on being stepped, and keeps none of the transforms' 77 MB."""
+    import torch
+    used = []
+    for _ in range(2):      # (the first handle loads the kernels)
+        w = qw.Walk((2, 300000), prec="f32").set_coin(inputs.grover()).set_state(
+            inputs.random_state((4, 300000, 2), seed=2))
+        w.step(1)
+        w.synchronize()
+        before = torch.cuda.mem_get_info()[0]
+        assert "spectral" not in w.autotune()
+        used.append(before - torch.cuda.mem_get_info()[0])
+        w.close()
+    assert used[1] < 16 << 20
