@@ -124,10 +124,29 @@ template <int INV, class R> __device__ __forceinline__ void dft4(Cx<R> &x0, Cx<R
     x3 = INV ? m : p;
 }
 
+// cos and sin of pi / 8, cos of pi / 4
+template <class R> struct Roots16 {
+    static constexpr R C1 = (R)0.92387953251128675613, S1 = (R)0.38268343236508977173, H = (R)0.70710678118654752440;
+};
+// What the rounding of these constants does to the norm of a 16-point (and, of
+// H alone, an 8-point) transform, as a factor on the amplitudes: all three floats
+// lie below their values, so the float transforms shrink by 1.1e-8 each, always in
+// the same sense.  The launchers undo it in tables that they round themselves (the
+// cycle's matrices, the torus' twiddles).  Change of the norm by one launch, without
+// and with that: cycle -1.6e-7, -2.5e-8; torus 256^2 -2.2e-7, 3.7e-8, 1024^2 -2.6e-7,
+// -5.3e-8, 8192^2 -3.8e-7, -1.6e-8.  A quarter of the points meets w16, w16^3 or
+// w16^9, a quarter H twice.
+template <class R> struct DftGain {
+    static constexpr double rot = (double)Roots16<R>::C1 * Roots16<R>::C1 + (double)Roots16<R>::S1 * Roots16<R>::S1;
+    static constexpr double diag = 2.0 * (double)Roots16<R>::H * Roots16<R>::H;
+    static constexpr double of16 = 1.0 + 0.5 * ((rot - 1.0) + (diag - 1.0)) / 4;
+    static constexpr double of8 = 1.0 + 0.5 * (diag - 1.0) / 4;
+};
+
 // 16-point transform of x (index n) as 4 x 4; output k is left in x[out16(k)].
 __host__ __device__ constexpr int out16(int k) { return 4 * (k & 3) + (k >> 2); }
 template <int INV, class R> __device__ __forceinline__ void dft16(Cx<R> (&x)[16]) {
-    constexpr R C1 = (R)0.92387953251128675613, S1 = (R)0.38268343236508977173, H = (R)0.70710678118654752440;
+    constexpr R C1 = Roots16<R>::C1, S1 = Roots16<R>::S1, H = Roots16<R>::H;
 #pragma unroll
     for (int b = 0; b < 4; ++b) dft4<INV>(x[b], x[4 + b], x[8 + b], x[12 + b]);
     const R g = INV ? (R)-1 : (R)1;   // w16 = C1 - i g S1

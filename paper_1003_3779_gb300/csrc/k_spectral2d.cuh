@@ -75,7 +75,7 @@ __host__ __device__ inline int spec2_place(int L, int f) {   // place of momentu
 __device__ __forceinline__ int spec2_at(int p) { return p + (p >> 4); }   // one pad slot per 16
 
 template <int INV, class R> __device__ __forceinline__ void dft8(Cx<R> (&x)[8]) {
-    constexpr R H = (R)0.70710678118654752440;
+    constexpr R H = Roots16<R>::H;
     const R g = INV ? (R)-1 : (R)1;
     dft4<INV>(x[0], x[2], x[4], x[6]);
     dft4<INV>(x[1], x[3], x[5], x[7]);

@@ -1503,9 +1503,14 @@ cudaError_t time_spectral(qw_walk *w, Spec1DArgs &a, int K, float &ms) {
     return e;
 }
 
+// Torus calls of fewer steps than this are stepped whatever their time.  Relative
+// errors of a launch in momentum space, dense states of 256^2 to 1024^2: amplitudes
+// 2.0e-7 to 2.4e-7, P 1.4e-7 to 1.8e-7; of 64 steps: 3.1e-7 to 3.7e-7, 2.0e-7 to 2.7e-7.
+constexpr int SPEC2_MIN_STEPS = 64;
+
 // ms of SPEC2_TUNE_STEPS steps of the torus in momentum space (0: no room for
 // them); the state is unchanged, the other buffer overwritten.
-constexpr int SPEC2_TUNE_STEPS = 256, SPEC2_MIN_STEPS = 64;
+constexpr int SPEC2_TUNE_STEPS = 256;
 cudaError_t tune_spectral2d(qw_walk *w, float &ms) {
     ms = 0.f;
     const Spec2Plan p = spectral2d_plan(w->nx, w->ny, SPEC2_TUNE_STEPS, true);

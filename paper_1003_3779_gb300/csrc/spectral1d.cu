@@ -158,6 +158,8 @@ static cudaError_t go_matrices(const Spec1DArgs &a, const double *coin, double s
     SpecCoin c;
     for (int i = 0; i < 4; ++i) { c.re[i] = coin[2 * i]; c.im[i] = coin[2 * i + 1]; }
     const int G = spectral1d_groups(a.tile);
+    // (three 16-point transforms each way, whose norm the matrices put right: DftGain)
+    if (sizeof(R) == sizeof(float)) scale /= std::pow(DftGain<R>::of16, 6);
     k_spec_matrices<R, N><<<G * SPEC_POINTS / 32, 32, 0, s>>>(static_cast<SpecPair<R> *>(a.table), c, G, a.K,
                                                               a.shift == QW_SHIFT_FLIPFLOP, a.adjoint,
                                                               scale / (G * SPEC_POINTS));

@@ -9,14 +9,24 @@
 
 namespace qw {
 
-// twiddles of every stage length, and the axis tables of both lengths
+// twiddles of every stage length, and the axis tables of both lengths.  The longer
+// stages' twiddles also undo the norm lost by the 16-point transforms (DftGain):
+// their own, and those of the stage of at most 128 (or, after 256, 16) points that
+// follows, whose few twiddles round too alike (half of those of length 32 are 1).
+// Rounded from many values, they do so on average to well below a rounding, which
+// one float factor at the end could not.
 __global__ void k_spec2_twiddles(S2 *tw) {
     const int id = blockIdx.x * blockDim.x + threadIdx.x;
     if (id < 32 || id >= SPEC2_TW) return;
     const int n = 1 << (31 - __clz(id)), i = id - n, k = i / (n / 16), b = i % (n / 16);
+    using Gain = DftGain<float>;
+    double lost = 1.0;
+    if (n >= 256) lost = Gain::of16 * (n <= 2048 ? Gain::of16 : 1.0) * (n == 2048 ? Gain::of8 : 1.0);
+    // (the points with k = 0 are not multiplied, those with b = 0 by 1)
+    const double up = 1.0 + (1.0 / lost - 1.0) / (15.0 / 16 * (1 - 16.0 / n));
     double s, c;
     sincospi(-2.0 * k * b / n, &s, &c);
-    tw[id] = {(float)c, (float)s};
+    tw[id] = {(float)(c * up), (float)(s * up)};
 }
 // momentum / (2 pi) at place p; split: places of the even momenta of a cycle of
 // 2^(L+1), then of the odd ones
