@@ -139,15 +139,22 @@ size_t spectral2d_workspace(int64_t nx, int64_t ny) {
     return TABLE_BYTES + std::min<size_t>(size_t(1) << 31, std::max<size_t>(size_t(1) << 26, want));
 }
 
+// Steps per launch; fewer are only taken by a call of fewer (below, m launches
+// would round more than stepping).
+constexpr int SPEC2_LEAST_STEPS = 64, SPEC2_MOST_STEPS = 4000;
 Spec2Plan spectral2d_plan(int64_t nx, int64_t ny, int64_t T, bool even) {
     // m launches of about T / m steps; a launch costs its points (about 7e8 point
-    // stages per millisecond) and 20 us for its kernels
+    // stages per millisecond) and 20 us for its kernels.  Every m up to 100, then by
+    // 2 %: with m <= 64 calls of more than 256000 steps were stepped, and shorter ones
+    // off powers of two had only launches of deep halos (300 x 200, T = 100000:
+    // 124 -> 27 ms).
     Spec2Plan best;
     const size_t room = spectral2d_workspace(nx, ny) - TABLE_BYTES;
-    for (int64_t m = 1; m <= 64 && m <= T; ++m) {
+    for (int64_t m = (T + SPEC2_MOST_STEPS - 1) / SPEC2_MOST_STEPS; m >= 1 && m <= T; m = std::max(m + 1, m * 102 / 100)) {
         int64_t K = (T + m - 1) / m;
+        if (m > 1 && K < SPEC2_LEAST_STEPS) break;
         if (even) K += K & 1;
-        if (K > 4000) continue;
+        if (K > SPEC2_MOST_STEPS) continue;
         AxisCut x, y;
         if (!cut_axes(nx, ny, (int)K, room, x, y)) continue;
         const double pts = (double)x.blocks * y.blocks * std::ldexp(1.0, x.L + y.L) * (x.L + y.L + 8);

@@ -4,6 +4,7 @@ import json
 import os
 import subprocess
 import sys
+import time
 
 import numpy as np
 import pytest
@@ -120,3 +121,21 @@ def test_a_rejected_workspace_is_given_back(qw):
         used.append(before - torch.cuda.mem_get_info()[0])
         w.close()
     assert used[1] < 16 << 20
+
+
+@pytest.mark.parametrize("nx,ny,T", [(300, 200, 300000), (256, 256, 300000)])
+def test_long_calls_stay_in_momentum_space(qw, nx, ny, T):
+    """Calls of more steps than 64 of the longest launches: less than half the time
+    of stepping them (a tenth to a third is expected)."""
+    w = qw.Walk((nx, ny), prec="f32").set_coin(inputs.grover()).set_state(inputs.random_state((4, ny, nx), seed=3))
+    assert '"spectral"' in w.autotune()
+    v = qw.Walk((nx, ny), prec="f32").set_coin(inputs.grover()).set_plan(8).set_state(inputs.random_state((4, ny, nx), seed=3))
+    took = []
+    for walk in (w, v):
+        walk.step(T).synchronize()
+        t = time.perf_counter()
+        walk.step(T).synchronize()
+        took.append(time.perf_counter() - t)
+        assert abs(walk.norm() - 1) < 1e-3
+        walk.close()
+    assert took[0] < 0.5 * took[1]
