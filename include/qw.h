@@ -242,7 +242,9 @@ qw_status qw_autotune(qw_walk *w, char *report, size_t report_len);
  * The search rides on the copy of a device state that is in the storage format;
  * else it reads the buffer.  Every amplitude equals that of stepping the whole
  * lattice with the same plan, bit for bit (a zero may differ in sign; clipped
- * states are never taken to momentum space).  on = 0 turns it off
+ * states are never taken to momentum space; with bf16 storage this ends at plans of
+ * 128 steps per launch, as a clipped launch, which rounds the state, takes no
+ * more).  on = 0 turns it off
  * (the current state is then stepped in full); on = 1 takes effect at the next
  * qw_set_state.  qw_describe reports the box ("support": [x0, w, y0, h],
  * columns [x0, x0 + w) and rows [y0, y0 + h) modulo the lattice, "full" or

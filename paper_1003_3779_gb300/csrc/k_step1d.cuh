@@ -122,12 +122,15 @@ __device__ __forceinline__ int64_t tile_origin(int64_t out0, int K) {
 // One warp tile: K steps on the 32R sites around the wthis outputs
 // [out0, out0 + wthis), a range inside [0, n).  Called by the cycle kernel
 // below and by the batched kernel (one walk per CTA).
-template <int P, int R, int CK, int FF, int ADJ>
+// MID: several of the plan's launches in one, of `per` steps each: every amplitude
+// takes their factor `mid`, and in bf16 storage its rounding, where they would end.
+template <int P, int R, int CK, int FF, int ADJ, bool MID = false>
 __device__ __forceinline__ void tb_tile(View in, View out, int64_t n, int K, int64_t out0, int wthis, int lane,
                                         const CoinP<typename St<P>::real> &cp,
                                         const Cx<typename St<P>::real> *__restrict__ coins,
                                         typename St<P>::real pre0, typename St<P>::real pre1,
-                                        typename St<P>::real post0, typename St<P>::real post1) {
+                                        typename St<P>::real post0, typename St<P>::real post1, int per = 0,
+                                        typename St<P>::real mid = typename St<P>::real()) {
     using real = typename St<P>::real;
     using C = Cx<real>;
     const int j0 = lane * R;
@@ -159,10 +162,7 @@ __device__ __forceinline__ void tb_tile(View in, View out, int64_t n, int K, int
         }
     }
 
-    // unrolled by two so the register shift of one step is a renaming into the
-    // other step's registers instead of moves at the loop back edge
-#pragma unroll 2
-    for (int t = 0; t < K; ++t) {
+    auto step = [&] {
         if (!ADJ) {
             C p0[R], p1[R];
 #pragma unroll
@@ -206,6 +206,33 @@ __device__ __forceinline__ void tb_tile(View in, View out, int64_t n, int K, int
 #pragma unroll
             for (int i = 0; i < R; ++i) coin2_adj<CK>(cp, &m[(CK == CK_PERSITE) ? 4 * i : 0], b0[i], b1[i], a0[i], a1[i]);
         }
+    };
+    // unrolled by two so the register shift of one step is a renaming into the
+    // other step's registers instead of moves at the loop back edge
+    if constexpr (!MID) {
+#pragma unroll 2
+        for (int t = 0; t < K; ++t) step();
+    } else {
+#pragma unroll 1
+        for (int done = 0;;) {
+            const int n = min(per, K - done);
+#pragma unroll 1
+            for (int t = n >> 1; t > 0; --t) { step(); step(); }
+            if (n & 1) step();
+            done += n;
+            if (done == K) break;
+#pragma unroll
+            for (int i = 0; i < R; ++i) {
+                a0[i] = rmul(mid, a0[i]);
+                a1[i] = rmul(mid, a1[i]);
+                if constexpr (P == P_BF16) {
+                    const float2 u = __bfloat1622float2(__floats2bfloat162_rn(a0[i].re, a0[i].im));
+                    const float2 v = __bfloat1622float2(__floats2bfloat162_rn(a1[i].re, a1[i].im));
+                    a0[i] = {u.x, u.y};
+                    a1[i] = {v.x, v.y};
+                }
+            }
+        }
     }
     if (!is_one(post0)) {
 #pragma unroll
@@ -222,18 +249,18 @@ __device__ __forceinline__ void tb_tile(View in, View out, int64_t n, int K, int
 // W output sites per warp (see tile_origin) over the output range [obeg, oend)
 // inside [0, n) (the whole cycle, or the light-cone window of a localised
 // state); nwarps = ceil((oend - obeg) / W).
-template <int P, int R, int CK, int FF, int ADJ>
+template <int P, int R, int CK, int FF, int ADJ, bool MID>
 __global__ void __launch_bounds__(128)
 k_step1d(View in, View out, int64_t n, int K, int64_t W, int64_t obeg, int64_t oend, int64_t nwarps,
          CoinP<typename St<P>::real> cp, const Cx<typename St<P>::real> *__restrict__ coins,
          typename St<P>::real pre0, typename St<P>::real pre1,
-         typename St<P>::real post0, typename St<P>::real post1) {
+         typename St<P>::real post0, typename St<P>::real post1, int per, typename St<P>::real mid) {
     const int lane = threadIdx.x & 31;
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (warp >= nwarps) return;  // uniform per warp
     const int64_t out0 = obeg + warp * W;
-    tb_tile<P, R, CK, FF, ADJ>(in, out, n, K, out0, (int)min(W, oend - out0), lane, cp, coins, pre0, pre1, post0,
-                               post1);
+    tb_tile<P, R, CK, FF, ADJ, MID>(in, out, n, K, out0, (int)min(W, oend - out0), lane, cp, coins, pre0, pre1, post0,
+                                    post1, per, mid);
 }
 
 // ---------------------------------------------------------------- k = 1

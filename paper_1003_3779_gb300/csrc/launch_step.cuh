@@ -63,6 +63,12 @@ inline int64_t outputs_per_warp(int R, int K) {
     return (32LL * R - 2LL * K - (V - 1)) / V * V;
 }
 
+// The tiles that take factors between their steps (Step1DArgs::per): the widest of
+// FP32 and bf16 storage and FP64's short one, for the coins that have factors.
+template <int P> constexpr bool joins_1d(int R, int kind) {
+    return (kind == CK_SIGN_P || kind == CK_SIGN_M) && (P == P_F64 ? R == WindowTile1D<P>::R : (P != P_COMP && R == Tiles1D<P>::B));
+}
+
 template <int P, int R, int CK, int FF, int ADJ>
 static void go1d(const Step1DArgs &a, const CoinP<typename St<P>::real> &cp, cudaStream_t s) {
     const int64_t W = outputs_per_warp<P>(R, a.K);
@@ -73,11 +79,16 @@ static void go1d(const Step1DArgs &a, const CoinP<typename St<P>::real> &cp, cud
     // its own
     const int wpb = win && nwarps <= 4 * 152 ? 1 : 4;
     const int64_t blocks = (nwarps + wpb - 1) / wpb;
-    k_step1d<P, R, CK, FF, ADJ><<<(unsigned)blocks, 32 * wpb, 0, s>>>(
+    auto kern = k_step1d<P, R, CK, FF, ADJ, false>;
+    if constexpr (joins_1d<P>(R, CK)) {
+        if (a.per) kern = k_step1d<P, R, CK, FF, ADJ, true>;
+    }
+    kern<<<(unsigned)blocks, 32 * wpb, 0, s>>>(
         a.in, a.out, a.n, a.K, W, ob, oe, nwarps, cp,
         static_cast<const Cx<typename St<P>::real> *>(a.coins),
         real_from_double<typename St<P>::real>(a.pre0), real_from_double<typename St<P>::real>(a.pre1),
-        real_from_double<typename St<P>::real>(a.post0), real_from_double<typename St<P>::real>(a.post1));
+        real_from_double<typename St<P>::real>(a.post0), real_from_double<typename St<P>::real>(a.post1),
+        a.per, real_from_double<typename St<P>::real>(a.mid));
 }
 
 template <int P, int R, int ADJ>
@@ -201,7 +212,7 @@ cudaError_t step1d_t(const Step1DArgs &a0, const void *coinp, int adj, cudaStrea
         }
     }
     a.tile = tile1d_effective<P>(a.tile, a.kind, adj);
-    if (a.K < 1 || a.K > max_k_1d(a.tile)) return cudaErrorInvalidValue;
+    if (a.K < 1 || a.K > max_k_1d(a.tile) || (a.per && !joins_1d<P>(a.tile, a.kind))) return cudaErrorInvalidValue;
     const bool ff = a.shift == QW_SHIFT_FLIPFLOP;
     if (a.K == 1 && a.oend <= a.obeg) {   // one step per launch over the whole cycle: the streaming kernel
         const bool ok = adj ? go1d_k1_kind<P, 1>(a, cp, s) : go1d_k1_kind<P, 0>(a, cp, s);

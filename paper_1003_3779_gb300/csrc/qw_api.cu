@@ -293,13 +293,25 @@ static double take_drift(qw_walk *w, int steps, bool last) {
 // Per-step factor for the 2D and generic kernels: drift_gain(w, 1, last).
 static double drift_gain(qw_walk *w, int steps, bool last = true) { return take_drift(w, steps, last); }
 
-// Pre / post per-plane factors of one 1D launch of K steps.
-static void launch_gains_1d(qw_walk *w, int K, int adj, Step1DArgs &a, bool update = true, bool last = true) {
+// Pre / post per-plane factors of one 1D launch of K steps.  block: the steps of the
+// plan's launch, of which `left` remain, at whose end the factors of all of them are
+// applied: a launch that is a piece of it leaves them to the last piece, and one of
+// several blocks applies them after each.  cut: the pieces of a sweep that scales its
+// state by 2^-SIGN_RESCALE_LOG2 every SIGN_RESCALE_STEPS steps do so at the same steps.
+static void launch_gains_1d(qw_walk *w, int K, int adj, Step1DArgs &a, bool update = true, bool last = true, int block = 0,
+                            int left = 0, bool cut = false) {
+    if (!block) block = left = K;
+    const bool ends = K >= left;
+    a.per = 0;
+    a.mid = 1.0;
     if (w->kind == CK_SIGN_P || w->kind == CK_SIGN_M) {
-        // the sweep kernel rescales by 2^-SIGN_RESCALE_LOG2 every SIGN_RESCALE_STEPS steps
-        const int m = a.variant == 1 ? K / SIGN_RESCALE_STEPS : 0;
-        const double mag = feedback_gain(w, std::ldexp(std::pow(w->sign_lambda, (double)K), SIGN_RESCALE_LOG2 * m),
-                                         update);
+        // the sweep kernel scales for itself
+        const int m = a.variant == 1 ? K / SIGN_RESCALE_STEPS : (cut ? (block - 1) / SIGN_RESCALE_STEPS : 0);
+        const double scale = std::ldexp(1.0, -SIGN_RESCALE_LOG2);
+        const double mag = !ends ? (cut ? scale : 1.0)
+                                 : feedback_gain(w, std::ldexp(std::pow(w->sign_lambda, (double)block), SIGN_RESCALE_LOG2 * m), update);
+        if (K > block) { a.per = block; a.mid = mag; }
+        else if (cut && K > SIGN_RESCALE_STEPS) { a.per = SIGN_RESCALE_STEPS; a.mid = scale; }
         const double ak1 = ((K - 1) % 2 == 0 || w->sign_a > 0) ? 1.0 : -1.0;   // a^{K-1}
         if (!adj) {
             a.pre0 = 1.0; a.pre1 = (double)(w->sign_sigma * w->sign_s);
@@ -310,7 +322,7 @@ static void launch_gains_1d(qw_walk *w, int K, int adj, Step1DArgs &a, bool upda
         }
         return;
     }
-    const double g = update ? take_drift(w, K, last) : 1.0;
+    const double g = update && ends ? take_drift(w, block, last) : 1.0;
     a.pre0 = a.pre1 = 1.0;
     a.post0 = a.post1 = g;
 }
@@ -444,30 +456,49 @@ static qw_status clear_next(qw_walk *w) {
 // least time per step, from a launch's fixed cost (about 4800 clocks from one
 // launch to the next) and per step the longer of a warp's own chain and the
 // issue of the warps that share its scheduler (an FP64 instruction holds a
-// scheduler for 64 clocks, a double-float operation is about 12 instructions).
-// With the sweep's depth of 8 and 256 sites per warp, the 2001-site FP64 cycle kept
-// three SMs busy for 17 us per launch of 8 steps.
+// scheduler for 64 clocks).  With the sweep's depth of 8 and 256 sites per warp, the
+// 2001-site FP64 cycle kept three SMs busy for 17 us per launch of 8 steps.
+//
+// The bits are those of the plan's launches: a launch is one of them (`left` steps
+// remain of it), a piece of it, or up to `more` of them, whose factors it applies in
+// between (joins_1d; FP64 coins of other kinds have none).  bf16 storage rounds the
+// state after each, so there they are not cut.
 constexpr int WINDOW_TILE_F64 = 2;   // (WindowTile1D)
 static int max_k_of_tile(int tile) { return tile == WINDOW_TILE_F64 ? 24 : 8 * tile; }
-static void window_plan(const qw_walk *w, int64_t width, int64_t T, int adj, int &tile, int &k) {
+static void window_plan(const qw_walk *w, int64_t width, int left, int64_t more, bool cut, int adj, int &tile, int &k) {
     int tiles[3] = {0, 0, 0};
     tiles_of(w->prec, tiles[0], tiles[1]);
+    const int wide = w->prec == QW_F64 ? WINDOW_TILE_F64 : tiles[1];   // the tile that joins
     for (int &t : tiles)
         if (t) t = tile1d(w->prec, t, w->kind, adj);
-    if (w->prec == QW_F64 && w->kind != CK_PERSITE) tiles[2] = WINDOW_TILE_F64;
-    const double unit = w->prec == QW_F64 ? 64 : (w->prec == QW_F32_COMP ? 12 : 1);
-    const double ops = w->kind == CK_SIGN_P || w->kind == CK_SIGN_M ? 4 : (w->kind == CK_REAL ? 8 : 16);
+    if (w->prec == QW_F64) tiles[2] = WINDOW_TILE_F64;
+    const bool sign = w->kind == CK_SIGN_P || w->kind == CK_SIGN_M;
+    const double unit = w->prec == QW_F64 ? 64 : 1, ops = sign ? 4 : (w->kind == CK_REAL ? 8 : 16);
     const int64_t schedulers = 4 * 152;
     double best = -1;
     for (int r : tiles) {
         if (!r) continue;
-        for (int kk = 8; kk <= max_k_of_tile(r); kk += 8) {
-            const int K = (int)std::min<int64_t>(kk, T);
+        const int most = max_k_of_tile(r);
+        auto consider = [&](int K) {
             const int64_t W = std::max<int64_t>(1, 32LL * r - 2 * K - 3);
             const int64_t warps = (width + 2 * K + W - 1) / W;
             const double chain = r * ops * unit, step = std::max(chain + 40, (double)((warps + schedulers - 1) / schedulers) * chain);
             const double cost = (4800 + K * step) / K;
             if (best < 0 || cost < best) { best = cost; tile = r; k = K; }
+        };
+        if (cut) {
+            consider(std::min(left, SIGN_RESCALE_STEPS));
+            if (r == wide) consider(std::min(left, most));
+        } else if (left > most) {
+            if (w->prec == QW_F32_BF16STORE) continue;
+            const int pieces = (left + most - 1) / most;
+            consider((left + pieces - 1) / pieces);
+        } else {
+            consider(left);
+            if (!(sign ? r == wide : w->prec == QW_F64)) continue;
+            // (a launch of the whole cycle takes no short tiles)
+            for (int64_t j = 2; j <= more && j * left <= most && (r != WINDOW_TILE_F64 || width + 2 * j * left < w->nx); ++j)
+                consider((int)j * left);
         }
     }
 }
@@ -730,17 +761,28 @@ qw_status run_steps(qw_walk *w, int64_t T, int adj) {
         Step1DArgs a{};
         a.n = w->nx; a.shift = w->shift; a.kind = w->kind; a.coins = w->coins_dev;
         const bool spectral = w->spec_tile && spectral_walk(w);
+        int block = 0, left = 0;   // steps of the plan's launch that is under way, those that are left of it
         for (int64_t rem = T; rem > 0;) {
-            a.K = (int)std::min<int64_t>(K, rem);
             const bool clip = w->sup_mode == 2;
-            if (spectral && !clip && rem >= w->spec_min) return run_spectral(w, rem, adj);
-            // the last, shorter launch of a sweep plan falls back to the tile kernel
-            // if needed; a clipped launch always runs the tiles
-            a.variant = (!clip && variant == 1 && sweep_ok(w, a.K, tile)) ? 1 : 0;
+            if (!left) {
+                if (spectral && !clip && rem >= w->spec_min) return run_spectral(w, rem, adj);
+                block = (int)std::min<int64_t>(K, rem);
+                // the last, shorter launch of a sweep plan falls back to the tile kernel
+                // if needed; a clipped launch always runs the tiles, in pieces where
+                // they are shorter than the sweep
+                const bool sweep = variant == 1 && sweep_ok(w, block, tile);
+                if (!sweep || (clip && w->prec == QW_F32_BF16STORE)) block = std::min(block, 8 * teff);
+                left = block;
+            }
+            a.variant = left == block && !clip && variant == 1 && sweep_ok(w, block, tile) ? 1 : 0;
             a.tile = a.variant == 1 ? tile : teff;
-            if (clip && variant == 1 && !w->plan_user) window_plan(w, w->bw, rem, adj, a.tile, a.K);
-            if (a.variant == 0) a.K = std::min(a.K, max_k_of_tile(a.tile));
-            launch_gains_1d(w, a.K, adj, a, true, rem - a.K == 0);
+            a.K = a.variant == 1 ? block : std::min(left, 8 * teff);
+            const bool cut = a.variant != 1 && w->prec == QW_F32 && variant == 1 && block > SIGN_RESCALE_STEPS &&
+                             (w->kind == CK_SIGN_P || w->kind == CK_SIGN_M) && sweep_ok(w, block, tile);
+            if (clip && variant == 1 && !w->plan_user)
+                window_plan(w, w->bw, left, left == block ? rem / block : 1, cut, adj, a.tile, a.K);
+            launch_gains_1d(w, a.K, adj, a, true, rem - a.K == 0, block, left, cut);
+            left = a.K >= left ? 0 : left - a.K;
             a.in = cur_view(w); a.out = next_view(w);
             a.obeg = a.oend = 0;
             const int64_t n = w->nx, len = w->bw + 2 * (int64_t)a.K;

@@ -341,6 +341,8 @@ struct Step1DArgs {
     double post0, post1; // per-plane factors applied before the store
     int variant;         // 0 independent warp tiles (halo recomputed), 1 time-skewed sweep
     int chunks;          // sweep: chunks per warp segment (0 = default)
+    int per;             // warp tiles, sign coins: a factor mid after every per steps (0: none)
+    double mid;
     // output range [obeg, oend) inside [0, n) when oend > obeg (the light-cone
     // window of a localised state: warp tiles only); else the whole cycle
     int64_t obeg, oend;
