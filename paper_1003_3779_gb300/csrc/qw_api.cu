@@ -141,7 +141,14 @@ static void default_plan(const qw_walk *w, int &k, int &tile, int &variant) {
         // 9.3 / 46, 8192^2 105 / 647 (k = 4: 2.2, 2.2, 4.7, 12.4, 174)
         tile = 0;
         k = 1;
-        if (w->bc != QW_BC_PERIODIC || links_on(w) || w->nx < 32 || w->ny < 32) return;
+        if (w->bc != QW_BC_PERIODIC || links_on(w)) return;
+        if (w->nx < 32 || w->ny < 32) {
+            // a side shorter than a tile: only where the other one has work for 16 warps
+            // per SM, in strips of 48 columns and chunks of 64 rows (k = 1 / k = 8, us per
+            // step: 2^20 x 16 164 / 47, 16 x 2^18 324 / 23, 2^18 x 8 25 / 9.7)
+            if (step2d_tb_ok(w->prec, w->kind, 8, w->shift) && ((w->nx + 47) / 48) * ((w->ny + 63) / 64) >= 16 * 152) k = 8;
+            return;
+        }
         // Phase coins run in tiles: 300 x 200 1.4 / 8.3, 1024^2 8.1 / 16.7 (k = 4: 9.3)
         if (step2d_tb_ok(w->prec, w->kind, 8, w->shift) || tile2d_walk(w)) k = 8;
         return;
