@@ -376,7 +376,7 @@ def stepping_roofline(desc, K, tile, t_step, hbm_gbs, sm_max_mhz, peak_src):
         roof = {"bound": "hbm", "achieved": ach_gbs, "peak": hbm_gbs, "unit": "GB/s",
                 "frac": hbm_frac, "traffic": traffic, "peak_source": f"{peak_src} HBM copy",
                 "alu_view": {"achieved_tflops": ach_tflops, "peak_tflops": alu_peak, "frac": alu_frac}}
-    roof.update({"kernel": "%s<f32,R=%d,%s coin>" % (desc["path"], tile, desc["coin_kind"]), "k": K,
+    roof.update({"kernel": "%s<f32,R=%d,%s coin>" % (desc["kernel"], tile, desc["coin_kind"]), "k": K,
                  "flops_per_site_step": flops_site_step, "avg_launch_ms": avg_launch_s * 1e3,
                  "ms_per_T_steps": t_step * 1e3,
                  "site_coin_updates_per_s": 2.0 * N_SITES * T_STEPS / t_step,
@@ -418,7 +418,7 @@ def coin_class_leg(qw, C, dev0, stream, sm_max_mhz, hbm_gbs):
             "coin_kind": desc["coin_kind"], "momentum_space": desc.get("spectral"), "norm_err": abs(norm - 1.0),
             "autotune": tune,
             "stepping": {"site_coin_updates_per_s": 2.0 * N_SITES * T_STEPS / t, "ms_per_T_steps": t * 1e3,
-                         "kernel": desc["path"], "k": K, "tile": tile, "avg_launch_ms": t * 1e3 / launches},
+                         "kernel": desc["kernel"], "k": K, "tile": tile, "avg_launch_ms": t * 1e3 / launches},
             "roofline_stepping": {"bound": "alu", "achieved": ach_inst / 1e12, "peak": issue_peak / 1e12,
                          "unit": "T FP32-instructions/s", "frac": ach_inst / issue_peak,
                          "instructions_per_site_step": inst, "op": op,
@@ -470,7 +470,7 @@ def localized_legs(qw, stream):
             desc = w.describe()
             leg["clipped" if clip else "whole_lattice"] = {
                 "ms": t * 1e3, "dense_site_coin_updates_per_s": d * nsites * T / t,
-                "active_site_coin_updates_per_s": d * cone / t, "kernel": desc["path"], "k": desc["k"],
+                "active_site_coin_updates_per_s": d * cone / t, "kernel": desc["kernel"], "k": desc["k"],
                 "support_after": desc["support"], "norm": w.norm()}
             w.close()
         leg["clipping_speedup"] = leg["whole_lattice"]["ms"] / leg["clipped"]["ms"]
@@ -677,7 +677,7 @@ def run_gpu(args, rank, world, local):
                 ts = a.elapsed_time(b) / 1e3 / 128
                 gbs = 64.0 * L * L / ts / 1e9      # k = 1 algorithmic bytes per site-step (effective above k = 1)
                 torus[f"{name}_k{kk}"] = {"site_coin_updates_per_s": 4.0 * L * L / ts, "ms_per_step": ts * 1e3,
-                                          "kernel": w2.describe()["path"],
+                                          "kernel": w2.describe()["kernel"],
                                           ("hbm_gbs" if kk == 1 else "effective_gbs"): gbs,
                                           "frac_of_measured": gbs / hbm_gbs, "frac_of_8000": gbs / 8000.0}
             w2.close()
@@ -705,7 +705,7 @@ def run_gpu(args, rank, world, local):
             ts = a.elapsed_time(b) / 1e3 / 64
             gbs = nbytes * L * L / ts / 1e9
             torus[name] = {"site_coin_updates_per_s": 4.0 * L * L / ts, "ms_per_step": ts * 1e3,
-                           "kernel": w2.describe()["path"], "bytes_per_site_step_at_k1": nbytes,
+                           "kernel": w2.describe()["kernel"], "bytes_per_site_step_at_k1": nbytes,
                            "effective_gbs": gbs, "frac_of_measured": gbs / hbm_gbs, "norm": w2.norm()}
             w2.close()
         del z, mask
@@ -720,7 +720,7 @@ def run_gpu(args, rank, world, local):
         torch.cuda.synchronize()
         ts = a.elapsed_time(b) / 1e3 / 64
         torus["cycle_2e27_segment_hadamard"] = {
-            "site_coin_updates_per_s": 2.0 * N_SITES / ts, "ms_per_step": ts * 1e3, "kernel": ws.describe()["path"],
+            "site_coin_updates_per_s": 2.0 * N_SITES / ts, "ms_per_step": ts * 1e3, "kernel": ws.describe()["kernel"],
             "bytes_per_site_step_at_k1": 32.0, "effective_gbs": 32.0 * N_SITES / ts / 1e9,
             "frac_of_measured": 32.0 * N_SITES / ts / 1e9 / hbm_gbs, "norm": ws.norm()}
         ws.close()
@@ -886,7 +886,7 @@ def run_gpu(args, rank, world, local):
                 t1 = a.elapsed_time(b) / 1e3
                 gbs = 16.0 * N_SITES * T_STEPS / t1 / 1e9
                 forms["bf16_k1"] = {"value": 2.0 * N_SITES * T_STEPS / t1, "unit": UNIT, "k": 1,
-                                    "kernel": wf.describe()["path"], "algorithmic_bytes_per_site_step": 16,
+                                    "kernel": wf.describe()["kernel"], "algorithmic_bytes_per_site_step": 16,
                                     "hbm_gbs": gbs, "frac_of_measured": gbs / hbm_gbs,
                                     "l1_vs_f64": float((Pf - ref).abs().sum()),
                                     "maxabs_p_vs_f64": float((Pf - ref).abs().max())}
@@ -1002,7 +1002,7 @@ def run_case(args):
         w.step(4 * k)
         b.record(stream)
         torch.cuda.synchronize()
-        out.update(n=n, coin=args.coin, plan=list(w.plan_ex()), kernel=w.describe()["path"],
+        out.update(n=n, coin=args.coin, plan=list(w.plan_ex()), kernel=w.describe()["kernel"],
                    ms_per_step=a.elapsed_time(b) / (4 * k), norm=w.norm())
         w.close()
     elif args.case == "torus":
@@ -1020,7 +1020,7 @@ def run_case(args):
         w.step(8 * k)
         b.record(stream)
         torch.cuda.synchronize()
-        out.update(L=L, k=k, shift=args.shift, kernel=w.describe()["path"], ms_per_step=a.elapsed_time(b) / (8 * k))
+        out.update(L=L, k=k, shift=args.shift, kernel=w.describe()["kernel"], ms_per_step=a.elapsed_time(b) / (8 * k))
         w.close()
     elif args.case == "batch":
         N, T, th, x0 = _in.batch_1d_params(nwalks=args.walks)

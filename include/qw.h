@@ -253,8 +253,11 @@ qw_status qw_set_clipping(qw_walk *w, int on);
 
 /* One-line JSON description of the handle: lattice, precision, the coin kind
  * the kernels specialise on ("real", "complex", "grover", "hadamard2",
- * "per_site", "phase", "hadamard_class"), the plan (k, tile), which kernel
- * family runs the step and the bytes of one state buffer.  Truncated to len. */
+ * "per_site", "phase", "hadamard_class"), the plan (k, tile), the route of a step
+ * ("path": "generic" for boundaries, links and the torus' per-site coins, else the
+ * family of the plan), the kernel that the next forward call of at least k steps
+ * launches first ("kernel", momentum-space calls apart) and the bytes of one state
+ * buffer.  Truncated to len. */
 qw_status qw_describe(const qw_walk *w, char *buf, size_t len);
 
 /* Number of sites (N or Lx*Ly). */

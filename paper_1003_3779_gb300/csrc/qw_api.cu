@@ -1419,6 +1419,28 @@ qw_status qw_set_clipping(qw_walk *w, int on) {
     return QW_OK;
 }
 
+// The kernel that the next forward call of at least k steps launches first, by the
+// conditions of run_steps (momentum-space calls apart).
+static const char *forward_kernel(const qw_walk *w, bool generic, int k, int var) {
+    const bool clip = w->sup_mode == 2, axis = w->shift != QW_SHIFT_DIAGONAL, ints = w->nx < (int64_t(1) << 30);
+    if (w->ndim == 1) {
+        if (generic) return axis && ints ? "k_step1d_window" : "k_step_generic";
+        if (!clip && var == 1) return "k_step1d_sweep";
+        return k == 1 && var != 1 && (!clip || w->bw + 2 >= w->nx) ? "k_step1d_k1" : "k_step1d";
+    }
+    if (generic) {
+        if (tile2d_walk(w)) return "k_tile2d";
+        return axis && ints && (w->ny + 7) / 8 <= 65535 ? "k_step_generic_tile" : "k_step_generic";
+    }
+    if (k > 1) {
+        Tile2DArgs box{};
+        tile2d_box(w, k, box);
+        if (tile2d_runs(w, k, box.ow * box.oh)) return "k_tile2d";
+        if (step2d_tb_ok(w->prec, w->kind, k, w->shift)) return "k_step2d_tb";
+    }
+    return "k_step2d";
+}
+
 qw_status qw_describe(const qw_walk *w, char *buf, size_t len) {
     if (!w || !buf || !len) return QW_EINVAL;
     static const char *kinds[] = {"real", "complex", "grover", "hadamard2", "per_site", "phase",
@@ -1448,13 +1470,13 @@ qw_status qw_describe(const qw_walk *w, char *buf, size_t len) {
                       w->spec_tile, (long long)w->spec_min);
     std::snprintf(buf, len,
                   "{\"ndim\": %d, \"sites\": %lld, \"coin_dim\": %d, \"precision\": %d, \"coin_kind\": \"%s\", "
-                  "\"k\": %d, \"tile\": %d, \"path\": \"%s\", \"state_bytes\": %zu, \"clipping\": %d, "
+                  "\"k\": %d, \"tile\": %d, \"path\": \"%s\", \"kernel\": \"%s\", \"state_bytes\": %zu, \"clipping\": %d, "
                   "\"support\": %s%s}",
                   w->ndim, (long long)w->ns, w->d, w->prec, kinds[w->kind], k, t,
                   window ? "k_step1d_window" : generic ? "generic"
                           : (w->ndim == 1 ? (var == 1 && w->sup_mode != 2 ? "k_step1d_sweep" : "k_step1d")
                                           : (k > 1 && step2d_tb_ok(w->prec, w->kind, k, w->shift) ? "k_step2d_tb" : "k_step2d")),
-                  w->state_bytes, (int)w->clip_on, sup, spec);
+                  forward_kernel(w, generic, k, var), w->state_bytes, (int)w->clip_on, sup, spec);
     return QW_OK;
 }
 
