@@ -55,11 +55,9 @@ static cudaError_t go_tile2d(const Tile2DArgs &a, const void *coinp, cudaStream_
 
 template <int P, int SH, bool LINKS>
 static cudaError_t tile2d_kind(int kind, const Tile2DArgs &a, const void *coinp, cudaStream_t s) {
-    if (a.phi) {   // phase coins: the base as the full matrix, row by row as in k_step2d, whose bits these are.  (The
-        // Grover form, sum / 2 - a_r, rounds its sum once for all four rows; a gradient from one site, where
-        // that does not average out, was up to 1.9 times as far off: 256^2, T = 300: 5.1e-6 instead of 2.6e-6)
-        if (kind == CK_COMPLEX) return go_tile2d<P, SH, CK_COMPLEX, true, LINKS>(a, coinp, s);
-        return go_tile2d<P, SH, CK_REAL, true, LINKS>(a, coinp, s);
+    if (a.phi) {   // phase coins: the base matrix in its Grover or its general form
+        if (kind == CK_GROVER) return go_tile2d<P, SH, CK_GROVER, true, LINKS>(a, coinp, s);
+        return go_tile2d<P, SH, CK_COMPLEX, true, LINKS>(a, coinp, s);
     }
     switch (kind) {
         case CK_REAL: return go_tile2d<P, SH, CK_REAL, false, LINKS>(a, coinp, s);
