@@ -1580,9 +1580,10 @@ cudaError_t time_spectral(qw_walk *w, Spec1DArgs &a, int K, float &ms) {
 constexpr int SPEC2_MIN_STEPS = 64;
 
 // ms of SPEC2_TUNE_STEPS steps of the torus in momentum space (0: no room for
-// them); the state is unchanged, the other buffer overwritten.
+// them), and that time over its estimate (spectral2d_plan); the state is
+// unchanged, the other buffer overwritten.
 constexpr int SPEC2_TUNE_STEPS = 256;
-cudaError_t tune_spectral2d(qw_walk *w, float &ms) {
+cudaError_t tune_spectral2d(qw_walk *w, float &ms, double &of_estimate) {
     ms = 0.f;
     const Spec2Plan p = spectral2d_plan(w->nx, w->ny, SPEC2_TUNE_STEPS, true);
     if (p.K < 2) return cudaSuccess;
@@ -1608,6 +1609,7 @@ cudaError_t tune_spectral2d(qw_walk *w, float &ms) {
     if (e == cudaSuccess) e = cudaEventRecord(e1, w->stream);
     if (e == cudaSuccess) e = cudaEventSynchronize(e1);
     if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
+    of_estimate = ms * ((SPEC2_TUNE_STEPS + p.K - 1) / p.K) / p.ms;
     ms *= (float)SPEC2_TUNE_STEPS / p.K;
     if (e0) cudaEventDestroy(e0);
     if (e1) cudaEventDestroy(e1);
@@ -1683,12 +1685,20 @@ extern "C" qw_status qw_autotune(qw_walk *w, char *report, size_t report_len) {
             float ms = 0.f;
             // (a workspace that was there before may be in a captured graph: it stays)
             const bool fresh = !w->spec_table;
-            if ((err = tune_spectral2d(w, ms)) != cudaSuccess) return cuda_error(w, err, "autotune");
+            double of_estimate = 1;
+            if ((err = tune_spectral2d(w, ms, of_estimate)) != cudaSuccess) return cuda_error(w, err, "autotune");
             if (!(ms > 0 && ms < best * SPEC2_TUNE_STEPS)) {
                 if (fresh) { cudaFree(w->spec_table); w->spec_table = nullptr; }
             } else {
                 w->spec2 = true;
-                w->spec_min = std::max<int64_t>(SPEC2_MIN_STEPS, (int64_t)std::ceil(ms / best));
+                // the shortest call whose launches, as estimated, take less time than its
+                // steps.  (By the time of 256 steps, calls of fewer than 108 were stepped at
+                // 700 x 1100: 64 steps 215 us, 128 in momentum space.)
+                const int64_t most = std::max<int64_t>(SPEC2_MIN_STEPS, (int64_t)std::ceil(ms / best));
+                w->spec_min = SPEC2_MIN_STEPS;
+                while (w->spec_min < most &&
+                       !(spectral2d_plan(w->nx, w->ny, w->spec_min, w->kind == CK_GROVER).ms * of_estimate * 1.05 < w->spec_min * best))
+                    ++w->spec_min;
                 std::snprintf(sp, sizeof sp, ", \"spectral\": {\"from_steps\": %lld}", (long long)w->spec_min);
             }
         }

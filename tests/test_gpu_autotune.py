@@ -139,3 +139,13 @@ def test_long_calls_stay_in_momentum_space(qw, nx, ny, T):
         assert abs(walk.norm() - 1) < 1e-3
         walk.close()
     assert took[0] < 0.5 * took[1]
+
+
+@pytest.mark.parametrize("nx,ny", [(300, 200), (700, 1100)])
+def test_short_calls_leave_stepping_as_soon_as_they_gain(qw, nx, ny):
+    """Calls of 64 steps take half the time in momentum space on these tori, where a
+    call of 256 steps takes two launches or deeper halos."""
+    w = qw.Walk((nx, ny), prec="f32").set_coin(inputs.grover()).set_state(inputs.random_state((4, ny, nx), seed=9))
+    w.autotune()
+    assert w.describe()["spectral"]["from_steps"] <= 80
+    w.close()
