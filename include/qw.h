@@ -202,7 +202,7 @@ qw_status qw_get_plan(const qw_walk *w, int *depth_k, int *tile);
  * NaN or an infinity reaches every site whose block holds it (all sites on the
  * torus), not its light cone alone; a
  * clipped state (qw_set_clipping) is therefore still stepped, until its box
- * covers the cycle.  Allocates the tile's table of matrices (at most 0.4 MB), which
+ * covers the cycle.  Allocates the tile's table of matrices (0.5 MB), which
  * the handle keeps. */
 qw_status qw_set_plan_ex(qw_walk *w, int depth_k, int tile, int variant);
 qw_status qw_get_plan_ex(const qw_walk *w, int *depth_k, int *tile, int *variant);
@@ -217,7 +217,9 @@ qw_status qw_get_plan_ex(const qw_walk *w, int *depth_k, int *tile, int *variant
  * shift and for H (x) H on the diagonal lattice, for calls of at least 64 steps,
  * in a workspace of 64 MB to 2 GB (four state buffers' worth in between), kept
  * with the handle where they are faster and given back where not; without room
- * for it the steps stay as they are.  1D results are cached per (lattice shape,
+ * for it the steps stay as they are.  What variant 2 says of zero and tiny
+ * amplitudes, NaN and infinities holds for those calls; qw_set_plan (0, 0) takes a
+ * handle back to stepping.  1D results are cached per (lattice shape,
  * precision, coin kind) in memory and, if the environment variable
  * QW_TUNE_CACHE names a file, in that JSON file.  report (may be NULL)
  * receives a one-line JSON summary, truncated to report_len bytes. */

@@ -537,7 +537,10 @@ static cudaError_t spectral_prepare(qw_walk *w, int tile) {
     void *&table = w->spec_tables[spectral1d_groups(tile) - 1];
     if (table) return cudaSuccess;
     void *t = nullptr;
-    cudaError_t e = dev_alloc(&t, spectral1d_table_bytes(w->prec, tile));
+    // (in whole half megabytes, which the tables of a handle then start on: with the
+    // second at an odd multiple of 2 KB a launch of 2^27 sites took 4.62 instead of 4.50 ms)
+    const size_t unit = size_t(1) << 19;
+    cudaError_t e = dev_alloc(&t, (spectral1d_table_bytes(w->prec, tile) + unit - 1) / unit * unit);
     if (e == cudaSuccess) e = launch_spectral1d_twiddles(w->prec, tile, t, w->stream);
     if (e == cudaSuccess) table = t;
     else cudaFree(t);
