@@ -19,7 +19,7 @@
 // is bound by their issue); this costs about 440 instructions per output site
 // whatever K is, so at K = 4096 it needs 1/40 of them, and a state crosses HBM
 // once per K <= S / 3 steps.  Rounding errors do not grow with K either: one
-// transform pair adds 1.9e-7 (float) or 3.4e-16 (double) of the block's norm,
+// transform pair adds 1.8e-7 (float) or 3.4e-16 (double) of the block's norm,
 // where stepping is 3e-7 / 8e-16 off after 128 steps and 1.7e-6 / 6e-15 after
 // 4096 / 1024 (Hadamard; against 64-bit and long double values).  The matrices
 // U^K are formed in double (float walks) or double-double (double walks) by
