@@ -569,7 +569,7 @@ k_step1d_sweep(View in, View out, int64_t n, int K, int nch, int64_t nseg, CoinP
             }
         };
         C b0[R], b1[R];
-        // blocks of levels; the Hadamard class rescales after each full block of
+        // blocks of levels; the Hadamard class rescales between blocks of
         // SIGN_RESCALE_STEPS (its unnormalised additions grow by sqrt(2) per step)
         constexpr bool SIGN = CK == CK_SIGN_P || CK == CK_SIGN_M;
         const int blk = SIGN ? SIGN_RESCALE_STEPS : K;
@@ -582,7 +582,7 @@ k_step1d_sweep(View in, View out, int64_t n, int K, int nch, int64_t nseg, CoinP
                 level(t, a0, a1, b0, b1);
                 level(t + 1, b0, b1, a0, a1);
             }
-            if (SIGN && t == tb + SIGN_RESCALE_STEPS) {   // 2^-SIGN_RESCALE_LOG2, exact
+            if (SIGN && t == tb + SIGN_RESCALE_STEPS && t < K) {   // 2^-SIGN_RESCALE_LOG2, exact
                 const real sc = (real)(1.0 / (double)(1ull << SIGN_RESCALE_LOG2));
 #pragma unroll
                 for (int i = 0; i < R; ++i) { a0[i] = rmul(sc, a0[i]); a1[i] = rmul(sc, a1[i]); }

@@ -300,10 +300,26 @@ static double take_drift(qw_walk *w, int steps, bool last) {
 // Per-step factor for the 2D and generic kernels: drift_gain(w, 1, last).
 static double drift_gain(qw_walk *w, int steps, bool last = true) { return take_drift(w, steps, last); }
 
+// How many of the next `most` launches of `block` steps take the same factor (rounded
+// to float, it may alternate).
+static int steady_blocks(const qw_walk *w, int block, int64_t most) {
+    if (!rounds_to_float(w)) return (int)most;
+    const double ideal = std::pow(w->sign_lambda, (double)block);
+    double fb = w->gain_fb, first = 0.0;
+    for (int i = 0; i < most; ++i) {
+        const double applied = (double)(float)(ideal / fb);
+        if (i && applied != first) return i;
+        first = applied;
+        fb *= applied / ideal;
+    }
+    return (int)most;
+}
+
 // Pre / post per-plane factors of one 1D launch of K steps.  block: the steps of the
 // plan's launch, of which `left` remain, at whose end the factors of all of them are
 // applied: a launch that is a piece of it leaves them to the last piece, and one of
-// several blocks applies them after each.  cut: the pieces of a sweep that scales its
+// several blocks (steady_blocks), the last of which may be shorter, applies them after
+// each.  cut: the pieces of a sweep that scales its
 // state by 2^-SIGN_RESCALE_LOG2 every SIGN_RESCALE_STEPS steps do so at the same steps.
 static void launch_gains_1d(qw_walk *w, int K, int adj, Step1DArgs &a, bool update = true, bool last = true, int block = 0,
                             int left = 0, bool cut = false) {
@@ -313,12 +329,19 @@ static void launch_gains_1d(qw_walk *w, int K, int adj, Step1DArgs &a, bool upda
     a.mid = 1.0;
     if (w->kind == CK_SIGN_P || w->kind == CK_SIGN_M) {
         // the sweep kernel scales for itself
-        const int m = a.variant == 1 ? K / SIGN_RESCALE_STEPS : (cut ? (block - 1) / SIGN_RESCALE_STEPS : 0);
+        const int m = a.variant == 1 || cut ? (block - 1) / SIGN_RESCALE_STEPS : 0;
         const double scale = std::ldexp(1.0, -SIGN_RESCALE_LOG2);
-        const double mag = !ends ? (cut ? scale : 1.0)
-                                 : feedback_gain(w, std::ldexp(std::pow(w->sign_lambda, (double)block), SIGN_RESCALE_LOG2 * m), update);
-        if (K > block) { a.per = block; a.mid = mag; }
-        else if (cut && K > SIGN_RESCALE_STEPS) { a.per = SIGN_RESCALE_STEPS; a.mid = scale; }
+        auto block_gain = [&](int steps) {
+            return feedback_gain(w, std::ldexp(std::pow(w->sign_lambda, (double)steps), SIGN_RESCALE_LOG2 * m), update);
+        };
+        double mag = !ends ? (cut ? scale : 1.0) : block_gain(block);
+        if (K > block) {
+            a.per = block;
+            a.mid = mag;
+            for (int t = 2 * block; t <= K; t += block) mag = block_gain(block);   // (a.mid again: steady_blocks)
+            if (K % block) mag = block_gain(K % block);
+        }
+        if (cut && K > SIGN_RESCALE_STEPS && K <= block) { a.per = SIGN_RESCALE_STEPS; a.mid = scale; }
         const double ak1 = ((K - 1) % 2 == 0 || w->sign_a > 0) ? 1.0 : -1.0;   // a^{K-1}
         if (!adj) {
             a.pre0 = 1.0; a.pre1 = (double)(w->sign_sigma * w->sign_s);
@@ -467,12 +490,13 @@ static qw_status clear_next(qw_walk *w) {
 // 2001-site FP64 cycle kept three SMs busy for 17 us per launch of 8 steps.
 //
 // The bits are those of the plan's launches: a launch is one of them (`left` steps
-// remain of it), a piece of it, or up to `more` of them, whose factors it applies in
-// between (joins_1d; FP64 coins of other kinds have none).  bf16 storage rounds the
-// state after each, so there they are not cut.
+// remain of it), a piece of it, or up to `more` of them and then, if it takes them all,
+// the call's `tail`, whose factors it applies in between (joins_1d; FP64 coins of other
+// kinds have none).  bf16 storage rounds the state after each, so there they are not cut.
 constexpr int WINDOW_TILE_F64 = 2;   // (WindowTile1D)
 static int max_k_of_tile(int tile) { return tile == WINDOW_TILE_F64 ? 24 : 8 * tile; }
-static void window_plan(const qw_walk *w, int64_t width, int left, int64_t more, bool cut, int adj, int &tile, int &k) {
+static void window_plan(const qw_walk *w, int64_t width, int left, int64_t more, int tail, bool cut, int adj, int &tile,
+                        int &k) {
     int tiles[3] = {0, 0, 0};
     tiles_of(w->prec, tiles[0], tiles[1]);
     const int wide = w->prec == QW_F64 ? WINDOW_TILE_F64 : tiles[1];   // the tile that joins
@@ -503,9 +527,14 @@ static void window_plan(const qw_walk *w, int64_t width, int left, int64_t more,
         } else {
             consider(left);
             if (!(sign ? r == wide : w->prec == QW_F64)) continue;
-            // (a launch of the whole cycle takes no short tiles)
-            for (int64_t j = 2; j <= more && j * left <= most && (r != WINDOW_TILE_F64 || width + 2 * j * left < w->nx); ++j)
-                consider((int)j * left);
+            auto fits = [&](int64_t K) {   // (a launch of the whole cycle takes no short tiles)
+                return K <= most && (r != WINDOW_TILE_F64 || width + 2 * K < w->nx);
+            };
+            const int64_t joined = sign ? steady_blocks(w, left, std::min<int64_t>(more, most / left)) : more;
+            for (int64_t j = 1; j <= joined && fits(j * left); ++j) {
+                if (j > 1) consider((int)j * left);
+                if (j == more && tail && fits(j * left + tail)) consider((int)j * left + tail);
+            }
         }
     }
 }
@@ -790,7 +819,8 @@ qw_status run_steps(qw_walk *w, int64_t T, int adj) {
             const bool cut = a.variant != 1 && w->prec == QW_F32 && variant == 1 && block > SIGN_RESCALE_STEPS &&
                              (w->kind == CK_SIGN_P || w->kind == CK_SIGN_M) && sweep_ok(w, block, tile);
             if (clip && variant == 1 && !w->plan_user)
-                window_plan(w, w->bw, left, left == block ? rem / block : 1, cut, adj, a.tile, a.K);
+                window_plan(w, w->bw, left, left == block ? rem / block : 1, left == block ? (int)(rem % block) : 0, cut, adj,
+                            a.tile, a.K);
             launch_gains_1d(w, a.K, adj, a, true, rem - a.K == 0, block, left, cut);
             left = a.K >= left ? 0 : left - a.K;
             a.in = cur_view(w); a.out = next_view(w);

@@ -299,8 +299,10 @@ enum CoinKind {
 // step, so amplitudes grow by sqrt(2) per step; float overflows after about
 // 250 steps.  The sweep kernel, which runs up to 511 steps per launch,
 // multiplies the state by 2^-SIGN_RESCALE_LOG2 (exact) after every
-// SIGN_RESCALE_STEPS steps, and the host folds 2^(SIGN_RESCALE_LOG2 * m), m the
-// number of rescales in the launch, into the launch's lambda^K.
+// SIGN_RESCALE_STEPS steps that others follow, and the host folds
+// 2^(SIGN_RESCALE_LOG2 * m), m the number of rescales in the launch, into the
+// launch's lambda^K.  (Not at its end: a tile launch of as many steps multiplies
+// once, and a denormal would be rounded twice.)
 constexpr int SIGN_RESCALE_STEPS = 64;
 constexpr int SIGN_RESCALE_LOG2 = 32;
 

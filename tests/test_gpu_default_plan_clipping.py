@@ -66,3 +66,25 @@ def test_tuned_plan(qw, prec, coin):
     assert np.array_equal(w.set_state(psi0).step(T).state(), v.set_state(psi0).step(T).state())
     w.close()
     v.close()
+
+
+@pytest.mark.parametrize("prec", ["f64", "f32", "bf16"])
+@pytest.mark.parametrize("scale", [0.97, 1.01])
+def test_coins_of_the_class_that_are_not_unitary(qw, prec, scale):
+    """A factor per launch that is no power of two and, rounded to float, alternates."""
+    N, got = 9000, []
+    for clip in (True, False):
+        w = qw.Walk((N,), prec=prec).set_coin(scale * inputs.hadamard()).set_clipping(clip)
+        w.set_state(inputs.localized_1d(N, N // 3, (0.6, 0.8j)))
+        for T in (300, 5, 12, 20, 70, 127, 129, 200):
+            w.step(T)
+        got.append(w.state())
+        w.close()
+    assert np.array_equal(*got)
+
+
+@pytest.mark.parametrize("prec", ["f64", "f32", "bf16"])
+@pytest.mark.parametrize("coin", list(COINS))
+@pytest.mark.parametrize("adjoint", [False, True])
+def test_short_calls(qw, prec, coin, adjoint):
+    both(qw, 3000, prec, coin, 0, adjoint, [5, 12, 20, 50, 70, 100, 127, 200])
